@@ -51,6 +51,8 @@ struct crkfr_ctx {
   double* d_araw_halo = nullptr;  // 2D slab with the limiter: the neighbours' raw indicator,
                                   // rows -2, -1 (below) and Ey, Ey + 1 (above), [4][Ex]
   double* d_alpha_halo = nullptr; // 2D slab with the limiter: smoothed rows -1, Ey, [2][Ex]
+  double* d_adj_stages = nullptr; // stage values of adj_rows element rows (unrecorded adjoint)
+  int64_t adj_rows = 0;
   double* d_adj_send = nullptr;   // 2D slab adjoint: y-correction sums of ubar1 for the
   double* d_adj_recv = nullptr;   // neighbours / from them, [2][3][Ex][n] each
   double sub_dt = 0.0;            // 1D subdomain: dt of the step between local and faces
@@ -123,6 +125,9 @@ void free_buffers(crkfr_ctx* c) {
   cudaFree(c->d_alpha_halo);
   cudaFree(c->d_adj_send);
   cudaFree(c->d_adj_recv);
+  cudaFree(c->d_adj_stages);
+  c->d_adj_stages = nullptr;
+  c->adj_rows = 0;
   c->d_ghost = c->d_send = c->d_araw_halo = c->d_alpha_halo = nullptr;
   c->d_adj_send = c->d_adj_recv = nullptr;
   c->d_cnode = c->d_alpha_raw = c->d_alpha = c->d_ulo = c->d_lx = c->d_ly = nullptr;
@@ -267,6 +272,7 @@ Launch2D make2d(crkfr_ctx* c) {
   L.periodic_y = c->subdomain ? 0 : 1;
   L.row_begin = 0;
   L.row_end = c->Ey;
+  L.stage_rows = c->Ey;
   return L;
 }
 
@@ -1276,8 +1282,32 @@ crkfr_status ensure_adjoint_sums(crkfr_ctx* c) {
   return CRKFR_OK;
 }
 
+// The local kernel in its residual form (no time bookkeeping) on the element
+// rows [row0, row1) of u: the traces of u^n, and with `stages` the inner stage
+// values, [S-1][3][row1 - row0][Ex][n][n].
+crkfr_status launch_local_for_adjoint(crkfr_ctx* c, const double* u, double dt, int64_t row0,
+                                      int64_t row1, double* stages, cudaStream_t s) {
+  StepCtl ctl{};
+  ctl.dt_fixed = dt;
+  ctl.residual = 1;
+  Launch2D L = make2d(c);
+  L.ctl = ctl;
+  L.u_in = u;
+  L.row_begin = row0;
+  L.row_end = row1;
+  L.stages = stages;
+  L.stage_row0 = row0;
+  L.stage_rows = row1 - row0;
+  int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s,
+                [&] { return stages ? launch_local_2d_stages(L, s) : launch_local_2d(L, s); });
+  if (e) return cuda_fail(c, e, "2D local kernel");
+  c->launches += 1;
+  return CRKFR_OK;
+}
+
 // The adjoint kernels of one step whose forward traces of u^n are in
-// (trx, try_) and whose stage values are in `stages` (null: recomputed).
+// (trx, try_) and whose stage values are in `stages`.  Null: the stage values
+// are recomputed by the local kernel, adj_rows element rows at a time.
 crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, double* ubar0,
                             double* bbar, double dt, const double* trx, const double* try_,
                             const double* stages, cudaStream_t s) {
@@ -1297,15 +1327,43 @@ crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, 
   A.atrx = c->d_atrx;
   A.atry = c->d_atry;
   A.gbar = c->d_gbar;
-  A.stages = stages;
   if (c->subdomain) {
     A.sums_below = c->d_adj_recv;
     A.sums_above = c->d_adj_recv + 3 * c->Ex * c->basis.n;
   }
   A.tab = c->tab;
-  int e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] { return launch_adjoint_2d(A, s); });
-  if (e) return cuda_fail(c, e, "2D adjoint kernels");
-  c->launches += 2;
+  int e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] { return launch_adjoint_faces_2d(A, s); });
+  if (e) return cuda_fail(c, e, "2D adjoint face kernel");
+  c->launches += 1;
+  const int64_t chunk = stages ? c->Ey : c->adj_rows;
+  A.stages = stages ? stages : c->d_adj_stages;
+  for (int64_t r = 0; r < c->Ey; r += chunk) {
+    A.row_begin = r;
+    A.row_end = std::min(r + chunk, c->Ey);
+    if (!stages) {
+      crkfr_status st = launch_local_for_adjoint(c, u, dt, r, A.row_end, c->d_adj_stages, s);
+      if (st != CRKFR_OK) return st;
+    }
+    e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] { return launch_adjoint_local_2d(A, s); });
+    if (e) return cuda_fail(c, e, "2D adjoint local kernel");
+    c->launches += 1;
+  }
+  return CRKFR_OK;
+}
+
+// The buffer of recomputed stage values: the whole mesh if that takes at most
+// a GiB, else as many element rows as do.
+crkfr_status ensure_adjoint_stages(crkfr_ctx* c) {
+  if (c->d_adj_stages) return CRKFR_OK;
+  const int64_t n = c->basis.n;
+  const int64_t row = (int64_t)(tab_stages(c->cfg.degree) - 1) * 3 * c->Ex * n * n;
+  const int64_t rows = std::max<int64_t>(1, std::min(c->Ey, ((int64_t)1 << 27) / row));
+  if (cudaMalloc(&c->d_adj_stages, sizeof(double) * row * rows) != cudaSuccess) {
+    c->d_adj_stages = nullptr;
+    cudaGetLastError();
+    return fail(c, CRKFR_ERR_ALLOC, "device allocation failed");
+  }
+  c->adj_rows = rows;
   return CRKFR_OK;
 }
 
@@ -1339,18 +1397,13 @@ crkfr_status crkfr_step_adjoint(crkfr_ctx* c, const double* u, const double* uba
   if (st == CRKFR_OK) st = adjoint_args(c, u, ubar1, ubar0, bbar, dt);
   if (st != CRKFR_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  // forward traces of u^n: the local kernel in its residual form (same traces,
-  // no time bookkeeping)
-  StepCtl ctl{};
-  ctl.dt_fixed = dt;
-  ctl.residual = 1;
-  Launch2D L = make2d(c);
-  L.ctl = ctl;
-  L.u_in = u;
-  int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s, [&] { return launch_local_2d(L, s); });
-  if (e) return cuda_fail(c, e, "2D local kernel");
-  c->launches += 1;
-  return launch_adjoint(c, u, ubar1, ubar0, bbar, dt, c->d_trx, c->d_try, nullptr, s);
+  st = ensure_adjoint_stages(c);
+  if (st != CRKFR_OK) return st;
+  // forward traces of u^n, and the stage values if those of the whole mesh fit
+  double* stages = c->adj_rows >= c->Ey ? c->d_adj_stages : nullptr;
+  st = launch_local_for_adjoint(c, u, dt, 0, c->Ey, stages, s);
+  if (st != CRKFR_OK) return st;
+  return launch_adjoint(c, u, ubar1, ubar0, bbar, dt, c->d_trx, c->d_try, stages, s);
 }
 
 // The adjoint step of a 2D slab in phases.  Each slab recomputes the face
@@ -1368,19 +1421,12 @@ crkfr_status crkfr_adjoint_local(crkfr_ctx* c, const double* u, const double* ub
   st = ensure_adjoint_sums(c);
   if (st != CRKFR_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  // forward traces of u^n (the local kernel in its residual form) and the
-  // sums the neighbouring slabs need
-  StepCtl ctl{};
-  ctl.dt_fixed = dt;
-  ctl.residual = 1;
-  Launch2D L = make2d(c);
-  L.ctl = ctl;
-  L.u_in = u;
-  int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s, [&] { return launch_local_2d(L, s); });
-  if (e) return cuda_fail(c, e, "2D local kernel");
-  e = launch_adjoint_sums_2d(c->cfg.degree, c->Ex, c->Ey, ubar1, c->tab, c->d_adj_send, s);
+  // forward traces of u^n and the sums the neighbouring slabs need
+  st = launch_local_for_adjoint(c, u, dt, 0, c->Ey, nullptr, s);
+  if (st != CRKFR_OK) return st;
+  int e = launch_adjoint_sums_2d(c->cfg.degree, c->Ex, c->Ey, ubar1, c->tab, c->d_adj_send, s);
   if (e) return cuda_fail(c, e, "adjoint sums kernel");
-  c->launches += 2;
+  c->launches += 1;
   return CRKFR_OK;
 }
 
@@ -1405,6 +1451,8 @@ crkfr_status crkfr_adjoint_faces(crkfr_ctx* c, const double* u, const double* ub
   if (st == CRKFR_OK) st = adjoint_args(c, u, ubar1, ubar0, bbar, dt);
   if (st != CRKFR_OK) return st;
   if (!c->d_adj_send) return fail(c, CRKFR_ERR_STATE, "crkfr_adjoint_local first");
+  st = ensure_adjoint_stages(c);
+  if (st != CRKFR_OK) return st;
   return launch_adjoint(c, u, ubar1, ubar0, bbar, dt, c->d_trx, c->d_try, nullptr,
                         (cudaStream_t)stream);
 }

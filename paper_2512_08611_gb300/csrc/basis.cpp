@@ -192,6 +192,25 @@ bool build_basis(int N, bool gll, HostBasis* out) {
   return true;
 }
 
+namespace {
+
+// Fixed-point form of coefficients (fixed_point.cuh): x as hi * 2^30 + lo in
+// units of 2^-s.
+void fx_coef(double x, int s, int32_t* hi, int32_t* lo) {
+  const int64_t v = std::llrint(std::ldexp(x, s));
+  *hi = (int32_t)((v + ((int64_t)1 << 29)) >> 30);
+  *lo = (int32_t)(v - ((int64_t)*hi << 30));
+}
+
+// the largest s with sum * 2^s <= 2^61 (sum > 0)
+int fx_scale(double sum) {
+  int e = 0;
+  const double m = std::frexp(sum, &e);   // sum = m 2^e, 1/2 <= m < 1
+  return m > 0.0 ? 61 - e : 0;
+}
+
+}  // namespace
+
 void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool imex,
                  double src_coef, Tables* T) {
   std::memset(T, 0, sizeof(*T));
@@ -221,6 +240,34 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
   T->sqrt_gravity = gravity > 0.0 ? std::sqrt(gravity) : 0.0;
   for (int q = 0; q < n; ++q)
     for (int p = 0; p < n; ++p) T->w2[q][p] = b.w[q] * b.w[p];
+  double rx = 0.0, ry = 0.0, rl = 0.0, sl0 = 0.0, sl1 = 0.0;
+  for (int i = 0; i < n; ++i) {
+    // rows and columns: the adjoint contracts with the transposes
+    double ax = 0.0, ay = 0.0, cx = 0.0, cy = 0.0;
+    for (int j = 0; j < n; ++j) {
+      ax += std::fabs(T->Dx[i][j]);
+      ay += std::fabs(T->Dy[i][j]);
+      cx += std::fabs(T->Dx[j][i]);
+      cy += std::fabs(T->Dy[j][i]);
+    }
+    rx = std::fmax(rx, std::fmax(ax, cx));
+    ry = std::fmax(ry, std::fmax(ay, cy));
+    sl0 += std::fabs(T->l0[i]);
+    sl1 += std::fabs(T->l1[i]);
+  }
+  rl = std::fmax(sl0, sl1);
+  const int sD = fx_scale(rx + ry), sL = fx_scale(rl);
+  FxTables& F = T->fx;
+  F.kD = 123 - sD;
+  F.kL = 123 - sL;
+  for (int i = 0; i < n; ++i) {
+    for (int j = 0; j < n; ++j) {
+      fx_coef(T->Dx[i][j], sD, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);
+      fx_coef(T->Dy[i][j], sD, &F.Dy_hi[i][j], &F.Dy_lo[i][j]);
+    }
+    fx_coef(T->l0[i], sL, &F.l0_hi[i], &F.l0_lo[i]);
+    fx_coef(T->l1[i], sL, &F.l1_hi[i], &F.l1_lo[i]);
+  }
   T->src_coef = src_coef;
   // smoothness indicator (Hennemann et al. 2021): inverse Vandermonde of the
   // orthonormal Legendre polynomials sqrt((2j+1)/2) P_j(2 xi - 1) at the

@@ -21,6 +21,17 @@ inline bool sys_is_2d(int s) { return s == CRKFR_SYS_SWE_2D || s == CRKFR_SYS_SW
 inline int sys_vars(int s) { return s == CRKFR_SYS_VARADV_1D ? 1 : sys_is_2d(s) ? 3 : 2; }
 inline bool sys_valid(int s) { return s >= CRKFR_SYS_VARADV_1D && s <= CRKFR_SYS_SWE_2D_WB; }
 
+// The matrices of the contractions as fixed-point integers hi * 2^30 + lo
+// (-2^29 <= lo < 2^29) in units of 2^-s, s such that the largest row sum of
+// magnitudes (of D / dx and D / dy together) is at most 2^61; kD, kL = 123 - s
+// of the differentiation matrices and of the end-point rows (fixed_point.cuh).
+struct FxTables {
+  int32_t Dx_hi[kMaxNodes][kMaxNodes], Dx_lo[kMaxNodes][kMaxNodes];
+  int32_t Dy_hi[kMaxNodes][kMaxNodes], Dy_lo[kMaxNodes][kMaxNodes];
+  int32_t l0_hi[kMaxNodes], l0_lo[kMaxNodes], l1_hi[kMaxNodes], l1_lo[kMaxNodes];
+  int32_t kD, kL;
+};
+
 // Reference-element and mesh tables passed to every kernel by value, so they
 // live in the kernel parameter bank (read through the constant cache) and
 // several contexts with different degrees or meshes can coexist.
@@ -38,7 +49,7 @@ struct Tables {
   double inv_dx, inv_dy;
   double gravity, half_gravity;
   // The kernels accumulate time averages with the weights b_i / b_ref, b_ref
-  // the first non-zero weight of the tableau (so that stage is a copy);
+  // the common unit of the tableau's weights (so the weights are integers);
   // b_ref multiplies dt instead, and the fluctuation term, which is not a
   // time average, uses g / b_ref.
   double b0;       // b_ref
@@ -52,6 +63,7 @@ struct Tables {
   // in the orthonormal Legendre basis, threshold T(N) and s / T
   double Vinv[kMaxNodes][kMaxNodes];
   double ind_T, ind_sharp;
+  FxTables fx;
 };
 
 // Subcell blending limiter of a 1D step (kernels_limit.cu).
@@ -242,8 +254,10 @@ struct Launch2D {
   // or Ey): the whole mesh by default
   int64_t row_begin, row_end;
   // recorded steps (crkfr_step_record): the local kernel also stores the
-  // inner stage values 1..S-1, [S-1][3][Ey][Ex][n][n]
+  // inner stage values 1..S-1 of the element rows [stage_row0, stage_row0 +
+  // stage_rows), [S-1][3][stage_rows][Ex][n][n]
   double* stages;
+  int64_t stage_row0, stage_rows;
   // local operator of the first stage computed ahead (the host-buffer step
   // overlaps it with the upload of the state): 1 = compute L(u^n) only and
   // store it in w; 2 = the step, reading L(u^n) from w (standard form only)
@@ -266,9 +280,11 @@ struct Launch2DAdj {
   double* atrx;          // adjoint traces [7][2][Ey][Ex][n]
   double* atry;          // adjoint traces [Ey][2][7][Ex][n]
   double* gbar;          // adjoint of the face jumps: [Ey][Ex][n] x faces, [Ey][Ex][n] y faces
-  // stage values 1..S-1 of the step from u^n, [S-1][3][Ey][Ex][n][n], as the
-  // forward local kernel stored them (crkfr_step_record); null: recompute
+  // stage values 1..S-1 of the step from u^n at the element rows [row_begin,
+  // row_end) the adjoint local kernel takes, [S-1][3][rows][Ex][n][n], as the
+  // forward local kernel stored them
   const double* stages;
+  int64_t row_begin, row_end;
   // slab of a larger mesh (null: periodic in y): the y-correction sums of
   // ubar1 of the element rows next to the slab, [3][Ex][n] each: below, the
   // sums of its top row's columns with g_R'; above, of its bottom row's
@@ -285,7 +301,8 @@ int launch_adjoint_sums_2d(int N, int64_t Ex, int64_t Ey, const double* ubar1, c
 // the forward local kernel (standard form, GL or GLL, no source) that also
 // stores the inner stage values into L.stages (kernels_adj2d.cu)
 int launch_local_2d_stages(const Launch2D& L, void* stream);
-int launch_adjoint_2d(const Launch2DAdj& A, void* stream);   // A.stages null or not
+int launch_adjoint_faces_2d(const Launch2DAdj& A, void* stream);
+int launch_adjoint_local_2d(const Launch2DAdj& A, void* stream);
 
 int launch_local_2d(const Launch2D& L, void* stream);   // L.pre 0 or 2
 int launch_local_2d_first(const Launch2D& L, void* stream);   // L_0 only (pre = 1)

@@ -1,0 +1,136 @@
+// Block fixed-point contractions with the constant matrices of the scheme
+// (differentiation matrix, end-point interpolation) on the integer pipe.
+//
+// On GB300 an FP64 instruction holds its SM sub-partition's FP64 pipe for 64
+// cycles per warp (two FP64 lanes per SM), an IMAD.WIDE takes 2 and a shift or
+// logic instruction 2 (measured).  The steps are bound by that pipe, and more
+// than half of their FP64 instructions are products with constant matrices.
+// Those are done here in 60-bit block fixed point instead: the operands of a
+// contraction are scaled by one power of two per element and field group,
+// split into two 30-bit halves, and multiplied into two 64-bit accumulators
+// with three IMAD.WIDE per term (6 cycles against 64); the sum is rounded to
+// FP64 once.
+//
+// Accuracy: operands are truncated 2^-kFxBits below the power of two above
+// the group's largest magnitude, coefficients are integers of a row sum up to
+// 2^61, and the dropped product of the lower halves is below 2^-57 of the
+// row's full scale (sum of |coefficient| times the largest operand).  An
+// FP64 FMA chain rounds every partial sum, 2^-53 of the partial sums each.
+//
+// Values too small for the group's scale vanish, exactly as they do against
+// it in an FP64 sum; groups holding an infinity or a NaN give NaN.
+#pragma once
+
+#include <cstdint>
+
+#include "crkfr_internal.h"
+
+namespace crkfr {
+namespace {
+
+// operand value hi * 2^30 + lo (0 <= lo < 2^30 from fx_split)
+struct alignas(8) Fx {
+  int hi, lo;
+};
+
+// added to the biased exponent of a group with a non-finite member: every
+// member then shifts out, and fx_to returns the group's NaN for the zero sums
+constexpr int kFxNonFinite = 4096;
+// smallest biased exponent of a group (zeros and denormals then shift out)
+constexpr int kFxMinExp = 128;
+
+// high word of |x|: its bits 20..30 are the biased exponent, and integer
+// order is magnitude order
+__device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+// biased exponent of a group from the largest fx_mag of its members
+__device__ __forceinline__ int fx_exp(int mag) {
+  const int e = mag >> 20;
+  const int m = e > kFxMinExp ? e : kFxMinExp;
+  return e == 0x7ff ? m + kFxNonFinite : m;
+}
+
+// x as a signed integer of FB bits in units of 2^(E - 1022 - FB), truncated;
+// E at least the biased exponent of x.  The 53-bit significand is shifted
+// into place (PTX shifts of 64 or more give 0) and the sign applied.
+template <int FB>
+__device__ __forceinline__ long long fx_from(double x, int E) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  unsigned long long m =
+      ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | lo) << (FB - 53);
+  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(E - e));
+  const long long s = hi >> 31;
+  return (long long)((m ^ (unsigned long long)s) - (unsigned long long)s);
+}
+
+__device__ __forceinline__ Fx fx_split(long long v) {
+  return Fx{(int)(v >> 30), (int)v & 0x3fffffff};
+}
+
+// arithmetic shift right by s >= 0 (64 or more: the sign)
+__device__ __forceinline__ long long fx_sar(long long v, int s) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+  return r;
+}
+
+// high word of what a zero sum of a group with exponent E stands for: 0, or
+// NaN for a group with a non-finite member
+__device__ __forceinline__ int fx_zero(int E) { return E >= kFxNonFinite ? 0x7ff80000 : 0; }
+
+// R * 2^(eb - 1085) rounded to FP64 (to nearest, ties away from zero); |R| <
+// 2^62; zero = fx_zero of the group.  The leading bit is found by truncating
+// conversions of the two halves to FP32 (2 cycles a warp each; the
+// count-leading-zeros unit takes 8, the 64-bit conversion more than 60).
+// Exponents above the FP64 range give a non-finite value.
+__device__ __forceinline__ double fx_to(long long R, int eb, int zero) {
+  const int rh = (int)(R >> 32);
+  const long long s = rh >> 31;
+  unsigned long long a = (unsigned long long)(R ^ s) - (unsigned long long)s;
+  const float f = __fmaf_rz(__uint2float_rz((unsigned)(a >> 32)), 4294967296.0f,
+                            __uint2float_rz((unsigned)a));
+  const int ex = __float_as_int(f) >> 23;   // 127 + position of the leading bit, 0 for zero
+  const int sh = 189 - ex;                  // leading bit to bit 62
+  asm("shl.b64 %0, %1, %2;" : "=l"(a) : "l"(a), "r"(sh));
+  a += 0x200;
+  const int e = eb - sh;
+  int hi = (int)(a >> 42) + (((e < 2047 ? e : 2047) - 1) << 20);
+  hi |= rh & (int)0x80000000;
+  return __hiloint2double(ex == 0 ? zero : hi, (int)(unsigned)(a >> 10));
+}
+
+// a row of n operands in shared memory (16-byte aligned for even n)
+template <int n>
+__device__ __forceinline__ void fx_row(const Fx* x, Fx (&r)[n]) {
+  if constexpr (n % 2 == 0) {
+#pragma unroll
+    for (int j = 0; j < n; j += 2) {
+      const int4 v = *reinterpret_cast<const int4*>(x + j);
+      r[j] = Fx{v.x, v.y};
+      r[j + 1] = Fx{v.z, v.w};
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < n; ++j) r[j] = x[j];
+  }
+}
+
+// sum of products in units of operand unit x coefficient unit x 2^60
+struct FxAcc {
+  long long a, b;
+};
+__device__ __forceinline__ void fx_mul(FxAcc& s, Fx x, int ch, int cl) {
+  s.a = (long long)x.hi * ch;
+  s.b = (long long)x.hi * cl + (long long)x.lo * ch;
+}
+__device__ __forceinline__ void fx_mad(FxAcc& s, Fx x, int ch, int cl) {
+  s.a += (long long)x.hi * ch;
+  s.b += (long long)x.hi * cl;
+  s.b += (long long)x.lo * ch;
+}
+__device__ __forceinline__ long long fx_sum(const FxAcc& s) { return s.a + (s.b >> 30); }
+
+}  // namespace
+}  // namespace crkfr

@@ -130,7 +130,7 @@ namespace {
 
 template <int N, bool GLL, int PRE>
 int launch_local_pre_t(const Launch2D& L, cudaStream_t s) {
-  constexpr int per_block = kWarpsLocal * (32 / (N + 1));
+  constexpr int per_block = local_elements<N + 1>();
   if (L.row_begin < 0 || L.row_end <= L.row_begin || L.row_end > L.Ey)
     return (int)cudaErrorInvalidValue;
   const int64_t blocks = ((L.row_end - L.row_begin) * L.Ex + per_block - 1) / per_block;

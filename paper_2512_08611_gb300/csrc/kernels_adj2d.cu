@@ -5,7 +5,8 @@
 // and adds (dS/db)^T ubar^{n+1} to bbar.  It is the exact discrete adjoint of
 // the kernels' arithmetic (reverse-mode differentiation written out by hand):
 //
-//  1. k_local_2d (forward, unchanged) recomputes W and the face traces of u^n;
+//  1. k_local_2d (forward) recomputes the face traces of u^n and its stage
+//     values, unless a recorded step kept them;
 //  2. k_face_adj_2d: once per face node, the adjoints of both sides' face
 //     terms follow from the two elements' row (or column) sums of ubar^{n+1}
 //     against the correction tables; they are pulled back through the
@@ -13,8 +14,7 @@
 //     (Sec. 3, Eqs. numflux.cons, combined.wave.speed, good.numflux.non.cons,
 //     total.F.non.cons) to adjoint traces of each side, and to the adjoint of
 //     the static jump g (b+ - b-)/b_0;
-//  3. k_local_adj_2d: per element, the inner stages are recomputed and kept,
-//     then reversed: adjoint traces -> time averages -> stage values ->
+//  3. k_local_adj_2d: per element, the inner stages are reversed: adjoint traces -> time averages -> stage values ->
 //     local operator (transposed D_x, D_y contractions) -> fluxes -> earlier
 //     stages and u^n; the bathymetry enters through g b_x, g b_y and the face
 //     jumps, whose adjoints are mapped back to the nodal b.
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) k_face_adj_2d(const Launch2DAdj A) {
   constexpr int nn = n * n;
   const Tables& T = A.tab;
   const int64_t Ex = A.Ex, Ey = A.Ey, Ne = Ex * Ey, ts = Ne * n, plane = Ex * n;
-  const double dtb0 = A.dt * tab_b(N, 0);
+  const double dtb0 = A.dt * Tab<N, false>::bref();
   const bool slab = A.sums_below != nullptr;
   const int64_t total = Ne * n + (slab ? Ey + 1 : Ey) * plane;   // x faces, y faces
   for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < total;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) k_face_adj_2d(const Launch2DAdj A) {
   }
 }
 
-template <int N, bool LOADED>
+template <int N>
 __global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A) {
   constexpr int n = N + 1;
   constexpr int nn = n * n;
@@ -196,15 +196,16 @@ __global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int le = lane / n, q = lane - le * n;
   const int64_t Ex = A.Ex, Ey = A.Ey, Ne = Ex * Ey, ts = Ne * n, plane = Ex * n;
+  const int64_t r0 = A.row_begin * Ex, Nr = (A.row_end - A.row_begin) * Ex;
   const int64_t g = ((int64_t)blockIdx.x * kWarpsAdj + warp) * EPW + le;
   const bool lane_ok = le < EPW;
-  const bool active = lane_ok && g < Ne;
-  const int64_t ge = active ? g : 0;
+  const bool active = lane_ok && g < Nr;
+  const int64_t gr = active ? g : 0, ge = r0 + gr;
   const int lec = lane_ok ? le : 0;
   double (*X)[n][n] = reinterpret_cast<double (*)[n][n]>(&sm[warp][lec * ES]);
   const int64_t ey = ge / Ex, ex = ge - ey * Ex;
   const double dt = A.dt;
-  constexpr double b0 = tab_b(N, 0);
+  constexpr double b0 = Tab<N, false>::bref();
   const double dtb0 = dt * b0;
 
   double u0[3][n], gbx[n], gby[n];
@@ -218,79 +219,19 @@ __global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A)
     gby[p] = A.snode[(Ne + ge) * nn + q * n + p];
   }
 
-  // ---- stage values (row q): loaded from the recorded step, or recomputed --
+  // ---- stage values (row q) as the forward local kernel stored them ---------
   double cur[S][3][n];
-  if constexpr (LOADED) {
+#pragma unroll
+  for (int v = 0; v < 3; ++v)
+#pragma unroll
+    for (int p = 0; p < n; ++p) cur[0][v][p] = u0[v][p];
+#pragma unroll
+  for (int i = 1; i < S; ++i)
 #pragma unroll
     for (int v = 0; v < 3; ++v)
 #pragma unroll
-      for (int p = 0; p < n; ++p) cur[0][v][p] = u0[v][p];
-#pragma unroll
-    for (int i = 1; i < S; ++i)
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p)
-          cur[i][v][p] = A.stages[(((int64_t)(i - 1) * 3 + v) * Ne + ge) * nn + q * n + p];
-  } else {
-    double Lp[S][3][n];
-#pragma unroll
-    for (int i = 0; i < S; ++i) {
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          double acc = u0[v][p];
-#pragma unroll
-          for (int j = 0; j < i; ++j)
-            if (tab_a(N, i, j) != 0.0) acc = fma(-(dt * tab_a(N, i, j)), Lp[j][v][p], acc);
-          cur[i][v][p] = acc;
-        }
-      if (i == S - 1) break;   // the last stage's operator is not needed here
-      double f2[n], f3[n], g3[n];
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        const double h = cur[i][0][p], mx = cur[i][1][p], my = cur[i][2][p];
-        const double r = drcp(h);
-        const double vx = mx * r, vy = my * r;
-        const double ph = (h * h) * T.half_gravity;
-        f2[p] = fma(mx, vx, ph);
-        f3[p] = mx * vy;
-        g3[p] = fma(my, vy, ph);
-      }
-      __syncwarp();
-      if (lane_ok) {
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          X[0][q][p] = cur[i][2][p];
-          X[1][q][p] = f3[p];
-          X[2][q][p] = g3[p];
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        double a0 = T.Dy[q][0] * X[0][0][p];
-        double a1 = fma(cur[i][0][p], gbx[p], T.Dy[q][0] * X[1][0][p]);
-        double a2 = fma(cur[i][0][p], gby[p], T.Dy[q][0] * X[2][0][p]);
-#pragma unroll
-        for (int j = 1; j < n; ++j) {
-          a0 = fma(T.Dy[q][j], X[0][j][p], a0);
-          a1 = fma(T.Dy[q][j], X[1][j][p], a1);
-          a2 = fma(T.Dy[q][j], X[2][j][p], a2);
-        }
-#pragma unroll
-        for (int j = 0; j < n; ++j) {
-          a0 = fma(T.Dx[p][j], cur[i][1][j], a0);
-          a1 = fma(T.Dx[p][j], f2[j], a1);
-          a2 = fma(T.Dx[p][j], f3[j], a2);
-        }
-        Lp[i][0][p] = a0;
-        Lp[i][1][p] = a1;
-        Lp[i][2][p] = a2;
-      }
-    }
-  }
+      for (int p = 0; p < n; ++p)
+        cur[i][v][p] = A.stages[(((int64_t)(i - 1) * 3 + v) * Nr + gr) * nn + q * n + p];
 
   // ---- adjoints of the time averages from W and the face traces ------------
   // W = u0 - dt b0 V  ->  ubar0 = Wbar,  Vbar = -dt b0 Wbar
@@ -359,7 +300,7 @@ __global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A)
 
 #pragma unroll
   for (int i = S - 1; i >= 0; --i) {
-    const double wi = tab_b(N, i) / tab_b(N, 0);
+    const double wi = tab_weight(N, i);
     double cb[3][n];   // adjoint of the stage value
 #pragma unroll
     for (int v = 0; v < 3; ++v)
@@ -498,20 +439,10 @@ __global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A)
   }
 }
 
-template <int N>
-void launch_adjoint_t(const Launch2DAdj& A, unsigned fblocks, unsigned lblocks, cudaStream_t s) {
-  static_assert(Tab<N, false>::S == tab_stages(N), "one stage count for both kernels");
-  k_face_adj_2d<N><<<fblocks, 256, 0, s>>>(A);
-  if (A.stages)
-    k_local_adj_2d<N, true><<<lblocks, kBlockAdj, 0, s>>>(A);
-  else
-    k_local_adj_2d<N, false><<<lblocks, kBlockAdj, 0, s>>>(A);
-}
-
 template <int N, bool GLL>
 int launch_local_stages_t(const Launch2D& L, cudaStream_t s) {
-  constexpr int per_block = kWarpsLocal * (32 / (N + 1));
-  const int64_t blocks = (L.Ex * L.Ey + per_block - 1) / per_block;
+  constexpr int per_block = local_elements<N + 1>();
+  const int64_t blocks = ((L.row_end - L.row_begin) * L.Ex + per_block - 1) / per_block;
   if (blocks > 0x7fffffff) return (int)cudaErrorInvalidConfiguration;
   if (L.ctl.residual)
     k_local_2d<N, GLL, true, false, false, false, true><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
@@ -553,28 +484,43 @@ int launch_adjoint_sums_2d(int N, int64_t Ex, int64_t Ey, const double* ubar1, c
   return (int)cudaGetLastError();
 }
 
-int launch_adjoint_2d(const Launch2DAdj& A, void* stream) {
+int launch_adjoint_faces_2d(const Launch2DAdj& A, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t Ne = A.Ex * A.Ey;
   const int n = A.N + 1;
-  const int64_t faces = Ne * n + (A.sums_below ? A.Ey + 1 : A.Ey) * A.Ex * n;
-  const unsigned fblocks = (unsigned)std::min<int64_t>((faces + 255) / 256, 152 * 16);
-  const int per_block = kWarpsAdj * (32 / n);
-  const unsigned lblocks = (unsigned)((Ne + per_block - 1) / per_block);
+  const int64_t faces = A.Ex * A.Ey * n + (A.sums_below ? A.Ey + 1 : A.Ey) * A.Ex * n;
+  const unsigned blocks = (unsigned)std::min<int64_t>((faces + 255) / 256, 152 * 16);
   switch (A.N) {
-    case 1: launch_adjoint_t<1>(A, fblocks, lblocks, s); break;
-    case 2: launch_adjoint_t<2>(A, fblocks, lblocks, s); break;
-    case 3: launch_adjoint_t<3>(A, fblocks, lblocks, s); break;
-    case 4: launch_adjoint_t<4>(A, fblocks, lblocks, s); break;
-    default:
-      return (int)cudaErrorInvalidValue;
+    case 1: k_face_adj_2d<1><<<blocks, 256, 0, s>>>(A); break;
+    case 2: k_face_adj_2d<2><<<blocks, 256, 0, s>>>(A); break;
+    case 3: k_face_adj_2d<3><<<blocks, 256, 0, s>>>(A); break;
+    case 4: k_face_adj_2d<4><<<blocks, 256, 0, s>>>(A); break;
+    default: return (int)cudaErrorInvalidValue;
+  }
+  return (int)cudaGetLastError();
+}
+
+int launch_adjoint_local_2d(const Launch2DAdj& A, void* stream) {
+  cudaStream_t s = (cudaStream_t)stream;
+  if (A.row_begin < 0 || A.row_end <= A.row_begin || A.row_end > A.Ey || !A.stages)
+    return (int)cudaErrorInvalidValue;
+  const int per_block = kWarpsAdj * (32 / (A.N + 1));
+  const unsigned blocks =
+      (unsigned)(((A.row_end - A.row_begin) * A.Ex + per_block - 1) / per_block);
+  switch (A.N) {
+    case 1: k_local_adj_2d<1><<<blocks, kBlockAdj, 0, s>>>(A); break;
+    case 2: k_local_adj_2d<2><<<blocks, kBlockAdj, 0, s>>>(A); break;
+    case 3: k_local_adj_2d<3><<<blocks, kBlockAdj, 0, s>>>(A); break;
+    case 4: k_local_adj_2d<4><<<blocks, kBlockAdj, 0, s>>>(A); break;
+    default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();
 }
 
 int launch_local_2d_stages(const Launch2D& L, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  if (L.row_begin != 0 || L.row_end != L.Ey || !L.stages) return (int)cudaErrorInvalidValue;
+  if (L.row_begin < L.stage_row0 || L.row_end <= L.row_begin ||
+      L.row_end > L.stage_row0 + L.stage_rows || L.row_end > L.Ey || !L.stages)
+    return (int)cudaErrorInvalidValue;
   switch (L.N * 2 + (L.gll ? 1 : 0)) {
     case 2: return launch_local_stages_t<1, false>(L, s);
     case 3: return launch_local_stages_t<1, true>(L, s);

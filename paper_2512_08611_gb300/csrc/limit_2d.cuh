@@ -19,7 +19,11 @@ namespace crkfr {
 namespace {
 
 constexpr int kLimFields = 8;     // limiter face data: u (3), c, inner flux (3), trace of c
-constexpr int kLimRowFields = 7;  // shared-memory row fields: u (3), c, y parts (3)
+constexpr int kLimExchange = 22;  // shared-memory fields per node (limit_local_2d)
+template <int D>
+struct LimDir {
+  static constexpr int value = D;
+};
 
 // Per-node parts of a first-order flux in direction DIR (0: x, 1: y): the
 // spectral radius |v_n| + sqrt(g h), the normal momentum's flux (with the
@@ -71,188 +75,114 @@ __device__ __forceinline__ void lo_flux_2d(const double* uL, const double* uR, d
   lo_flux_nodes<DIR, WB>(uL, uR, cL, cR, sL, sR, fnL, fnR, ftL, ftR, g, fm, fp);
 }
 
-// The first-order part of the local kernel for row q of element ge (lanes
-// of one element exchange rows through X, [fields][row][column]).  u0: row
-// q of u^n.  Every lane of the warp calls it (it synchronises the warp).
-template <int N, bool GLL, bool WB>
-__device__ __forceinline__ void limit_local_2d(const Launch2D& L, const double (&u0)[3][N + 1],
-                                               double (*X)[N + 1][N + 1], int q, bool lane_ok,
-                                               bool active, int64_t ge, double dt) {
+// The first-order part of the local kernel, one thread per node (node = q n +
+// p of element ge).  u0: u^n at the node; x: the element's exchange area
+// (kLimExchange fields); sync: the element's barrier, which every thread of
+// the block (or warp) reaches.  The area holds, per node: 0..2 u^n, 3 c, 4..6
+// the x parts and 7..9 the y parts of the node's first-order flux; 10..12 and
+// 13..15 the minus- and plus-side fluxes of the x subface to its right, 16..18
+// and 19..21 of the y subface above it.
+template <int N, bool GLL, bool WB, class Sync>
+__device__ __forceinline__ void limit_local_2d(const Launch2D& L, const double (&u0)[3], double* x,
+                                               int node, bool lane_ok, bool active, int64_t ge,
+                                               double dt, Sync sync) {
   constexpr int n = N + 1;
   constexpr int nn = n * n;
   const Tables& T = L.tab;
   const double g = T.gravity;
   const int64_t Ne = L.Ex * L.Ey;
   const int64_t tstride = Ne * n;
+  const int q = node / n, p = node - q * n;
+  auto X = [x](int f, int k) -> double& { return x[f * nn + k]; };
 
-  double cn[n];
+  if (lane_ok) {
+    // the per-node parts of both directions (one reciprocal, one root)
+    const double ih = drcp(u0[0]), a = dsqrt_pos(g * u0[0]);
+    const double vx = u0[1] * ih, vy = u0[2] * ih;
 #pragma unroll
-  for (int p = 0; p < n; ++p) cn[p] = L.lim.cnode[ge * nn + q * n + p];
-  // row q into shared memory (u, c, and the per-node parts of the y fluxes);
-  // x: inner subfaces of row q from the per-node x parts, node by node
-  double fxm[3][N], fxp[3][N];
-  __syncwarp();
-  {
-    double s0 = 0.0, fn0 = 0.0, ft0 = 0.0;
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      const double u[3] = {u0[0][p], u0[1][p], u0[2][p]};
-      // the per-node parts of both directions (one reciprocal, one root)
-      const double ih = drcp(u[0]), a = dsqrt_pos(g * u[0]);
-      const double vx = u[1] * ih, vy = u[2] * ih;
-      const double s1 = fabs(vx) + a, sy = fabs(vy) + a;
-      const double fn1 = WB ? u[1] * vx : fma(0.5 * g * u[0], u[0], u[1] * vx);
-      const double fny = WB ? u[2] * vy : fma(0.5 * g * u[0], u[0], u[2] * vy);
-      const double ft1 = u[2] * vx, fty = u[1] * vy;
-      if (lane_ok) {
-        X[0][q][p] = u[0];
-        X[1][q][p] = u[1];
-        X[2][q][p] = u[2];
-        X[3][q][p] = cn[p];
-        X[4][q][p] = sy;
-        X[5][q][p] = fny;
-        X[6][q][p] = fty;
-      }
-      if (p > 0) {
-        const double ul[3] = {u0[0][p - 1], u0[1][p - 1], u0[2][p - 1]};
-        double fm_[3], fp_[3];
-        lo_flux_nodes<0, WB>(ul, u, cn[p - 1], cn[p], s0, s1, fn0, fn1, ft0, ft1, g, fm_, fp_);
-#pragma unroll
-        for (int v = 0; v < 3; ++v) {
-          fxm[v][p > 0 ? p - 1 : 0] = fm_[v];
-          fxp[v][p > 0 ? p - 1 : 0] = fp_[v];
-        }
-      }
-      s0 = s1;
-      fn0 = fn1;
-      ft0 = ft1;
-    }
+    for (int v = 0; v < 3; ++v) X(v, node) = u0[v];
+    X(3, node) = L.lim.cnode[ge * nn + node];
+    X(4, node) = fabs(vx) + a;
+    X(5, node) = WB ? u0[1] * vx : fma(0.5 * g * u0[0], u0[0], u0[1] * vx);
+    X(6, node) = u0[2] * vx;
+    X(7, node) = fabs(vy) + a;
+    X(8, node) = WB ? u0[2] * vy : fma(0.5 * g * u0[0], u0[0], u0[2] * vy);
+    X(9, node) = u0[1] * vy;
   }
-  __syncwarp();
-  // column q: nodal state and c at the bottom and top nodes, traces of c at
-  // the bottom and top faces
-  double uB[3], uT[3];
-#pragma unroll
-  for (int v = 0; v < 3; ++v) {
-    uB[v] = X[v][0][q];
-    uT[v] = X[v][N][q];
-  }
-  const double cB = X[3][0][q], cT = X[3][N][q];
-  double ctrB, ctrT;
-  if (GLL) {
-    ctrB = cB;
-    ctrT = cT;
-  } else {
-    ctrB = T.l0[0] * X[3][0][q];
-    ctrT = T.l1[0] * X[3][0][q];
-#pragma unroll
-    for (int j = 1; j < n; ++j) {
-      ctrB = fma(T.l0[j], X[3][j][q], ctrB);
-      ctrT = fma(T.l1[j], X[3][j][q], ctrT);
-    }
-  }
-  // y: subface between rows q and q+1 (rows q < N), column p
-  const int qa = q < N ? q + 1 : q;
-  double fym[3][n], fyp[3][n];
-#pragma unroll
-  for (int p = 0; p < n; ++p) {
-    const double a[3] = {u0[0][p], u0[1][p], u0[2][p]};
-    const double b[3] = {X[0][qa][p], X[1][qa][p], X[2][qa][p]};
-    double fm_[3], fp_[3];
-    lo_flux_nodes<1, WB>(a, b, cn[p], X[3][qa][p], X[4][q][p], X[4][qa][p], X[5][q][p],
-                         X[5][qa][p], X[6][q][p], X[6][qa][p], g, fm_, fp_);
+  sync();
+  // the subfaces to the right of and above the node
+  auto subface = [&](auto dir, int nb) {
+    constexpr int D = decltype(dir)::value;
+    double a[3], b[3], fm[3], fp[3];
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
-      fym[v][p] = fm_[v];
-      fyp[v][p] = fp_[v];
+      a[v] = u0[v];
+      b[v] = X(v, nb);
     }
-  }
-  // round B: the plus-side flux of each inner y-subface to the row above
-  __syncwarp();
-  if (lane_ok && q < N) {
+    lo_flux_nodes<D, WB>(a, b, X(3, node), X(3, nb), X(4 + 3 * D, node), X(4 + 3 * D, nb),
+                         X(5 + 3 * D, node), X(5 + 3 * D, nb), X(6 + 3 * D, node),
+                         X(6 + 3 * D, nb), g, fm, fp);
 #pragma unroll
-    for (int p = 0; p < n; ++p) {
-      X[0][q][p] = fyp[0][p];
-      X[1][q][p] = fyp[1][p];
-      X[2][q][p] = fyp[2][p];
+    for (int v = 0; v < 3; ++v) {
+      X(10 + 6 * D + v, node) = fm[v];
+      X(13 + 6 * D + v, node) = fp[v];
     }
+  };
+  if (lane_ok) {
+    if (p < N) subface(LimDir<0>{}, node + 1);
+    if (q < N) subface(LimDir<1>{}, node + n);
   }
-  __syncwarp();
-  const int qb = q > 0 ? q - 1 : 0;
-  double fyl[3][n];   // subface between rows q-1 and q, seen by row q
-  double fTin[3];     // column q: the left flux of the top node (rows N-1 | N)
+  sync();
+  if (!active) return;
+  // first-order update of the node without the element-face terms
+  const double cx = dt * T.inv_dx * T.inv_w[p], cy = dt * T.inv_dy * T.inv_w[q];
 #pragma unroll
   for (int v = 0; v < 3; ++v) {
-#pragma unroll
-    for (int p = 0; p < n; ++p) fyl[v][p] = X[v][qb][p];
-    fTin[v] = X[v][N - 1][q];
+    const double r = p < N ? X(10 + v, node) : 0.0;
+    const double l = p > 0 ? X(13 + v, node - 1) : 0.0;
+    const double t = q < N ? X(16 + v, node) : 0.0;
+    const double b = q > 0 ? X(19 + v, node - n) : 0.0;
+    L.lim.ulo[(v * Ne + ge) * nn + node] = u0[v] - cx * (r - l) - cy * (t - b);
   }
-  // round C: the minus-side flux of the bottom inner subface, by column
-  __syncwarp();
-  if (lane_ok && q == 0) {
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      X[0][0][p] = fym[0][p];
-      X[1][0][p] = fym[1][p];
-      X[2][0][p] = fym[2][p];
-    }
-  }
-  __syncwarp();
-  double fBin[3];     // column q: the right flux of the bottom node (rows 0 | 1)
-#pragma unroll
-  for (int v = 0; v < 3; ++v) fBin[v] = X[v][0][q];
-
-  if (!active) return;
-  // first-order update of row q without the element-face terms
-  const double cx = dt * T.inv_dx, cy = dt * T.inv_dy * T.inv_w[q];
-#pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      const double r = p < N ? fxm[v][p < N ? p : 0] : 0.0;
-      const double l = p > 0 ? fxp[v][p > 0 ? p - 1 : 0] : 0.0;
-      const double t = q < N ? fym[v][p] : 0.0;
-      const double b = q > 0 ? fyl[v][p] : 0.0;
-      L.lim.ulo[(v * Ne + ge) * nn + q * n + p] =
-          u0[v][p] - (cx * T.inv_w[p]) * (r - l) - cy * (t - b);
-    }
-  // x-face data of row q: left side (node 0), right side (node N)
-  double ctrL, ctrR;
-  if (GLL) {
-    ctrL = cn[0];
-    ctrR = cn[N];
-  } else {
-    ctrL = T.l0[0] * cn[0];
-    ctrR = T.l1[0] * cn[0];
-#pragma unroll
-    for (int p = 1; p < n; ++p) {
-      ctrL = fma(T.l0[p], cn[p], ctrL);
-      ctrR = fma(T.l1[p], cn[p], ctrR);
-    }
-  }
-  const double lx0[kLimFields] = {u0[0][0], u0[1][0], u0[2][0], cn[0],
-                                  fxm[0][0], fxm[1][0], fxm[2][0], ctrL};
-  const double lx1[kLimFields] = {u0[0][N], u0[1][N], u0[2][N], cn[N],
-                                  fxp[0][N - 1], fxp[1][N - 1], fxp[2][N - 1], ctrR};
-#pragma unroll
-  for (int f = 0; f < kLimFields; ++f) {
-    L.lim.lx[(2 * f + 0) * tstride + ge * n + q] = lx0[f];
-    L.lim.lx[(2 * f + 1) * tstride + ge * n + q] = lx1[f];
-  }
-  // y-face data of column q: bottom side (row 0), top side (row N); buffer
-  // rows as the y traces (halo rows 0 and Ey+1 filled in a periodic mesh)
-  const double ly0[kLimFields] = {uB[0], uB[1], uB[2], cB, fBin[0], fBin[1], fBin[2], ctrB};
-  const double ly1[kLimFields] = {uT[0], uT[1], uT[2], cT, fTin[0], fTin[1], fTin[2], ctrT};
-  const int64_t row = ge / L.Ex + 1, col = ge - (row - 1) * L.Ex;
+  // face data: the nodal state and c next to the face, the inner flux of that
+  // node on its far side, the trace of c; the 4 n face nodes as the traces
   const int64_t plane = L.Ex * n;
+  const int64_t row = ge / L.Ex + 1, col = ge - (row - 1) * L.Ex;
 #pragma unroll
-  for (int f = 0; f < kLimFields; ++f) {
-    L.lim.ly[((row * 2 + 0) * kLimFields + f) * plane + col * n + q] = ly0[f];
-    L.lim.ly[((row * 2 + 1) * kLimFields + f) * plane + col * n + q] = ly1[f];
-    if (L.periodic_y && row == 1)
-      L.lim.ly[(((L.Ey + 1) * 2 + 0) * kLimFields + f) * plane + col * n + q] = ly0[f];
-    if (L.periodic_y && row == L.Ey)
-      L.lim.ly[((0 * 2 + 1) * kLimFields + f) * plane + col * n + q] = ly1[f];
+  for (int j0 = 0; j0 < 4 * n; j0 += nn) {
+    const int job = j0 + node;
+    if (4 * n % nn != 0 && job >= 4 * n) break;
+    const int dir = job / (2 * n), side = job / n & 1, r = job % n;
+    const int step = dir ? n : 1, base = dir ? r : r * n;
+    const int at = base + (side ? N * step : 0);          // the node next to the face
+    const int sub = side ? at - step : at;                // its inner subface
+    double d[kLimFields];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      d[v] = X(v, at);
+      d[4 + v] = X(10 + 6 * dir + 3 * side + v, sub);
+    }
+    d[3] = X(3, at);
+    if (GLL) {
+      d[7] = d[3];
+    } else {
+      double c = (side ? T.l1[0] : T.l0[0]) * X(3, base);
+#pragma unroll
+      for (int j = 1; j < n; ++j) c = fma(side ? T.l1[j] : T.l0[j], X(3, base + j * step), c);
+      d[7] = c;
+    }
+    // y: buffer rows as the y traces (halo rows 0 and Ey+1 filled in a
+    // periodic mesh)
+    double* out = dir ? L.lim.ly + (row * 2 + side) * kLimFields * plane + col * n + r
+                      : L.lim.lx + side * tstride + ge * n + r;
+    const int64_t ostep = dir ? plane : 2 * tstride;
+    const bool wrap = dir && L.periodic_y && row == (side ? L.Ey : 1);
+    double* halo = L.lim.ly + (side ? 1 : (L.Ey + 1) * 2) * kLimFields * plane + col * n + r;
+#pragma unroll
+    for (int f = 0; f < kLimFields; ++f) {
+      out[f * ostep] = d[f];
+      if (wrap) halo[f * plane] = d[f];
+    }
   }
 }
 

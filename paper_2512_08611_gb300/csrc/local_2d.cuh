@@ -3,18 +3,29 @@
 // treated implicitly, Sec. 2 Eqs. crkfr.inner, crkfr, avg.source, with
 // SSP3-IMEX(4,3,3)).
 //
-// n = N+1 threads own one element, one row (fixed y-node q) each, so
-// x-derivatives are register-resident FMA chains and y-derivatives read the
-// other rows through shared memory.  All inner stages stay on chip; the
-// kernel writes W = u^n - dt (dloc F + Bloc) [+ dt S] (Eqs. disc.avg.flux,
-// local.time.avg.non.cons, avg.source) and, for every face node, the traces
-// the Riemann problem needs: the time-averaged solution U, the
-// time-averaged normal flux and h^n and the normal momentum at t^n (Eqs.
-// time.avg.soln, combined.wave.speed, good.numflux.non.cons).
+// One thread owns one node: an element's (N+1)^2 threads exchange the fluxes
+// of a stage through shared memory and each takes its node's row of D_x and
+// D_y.  All inner stages stay on chip; the kernel writes W = u^n - dt (dloc F
+// + Bloc) [+ dt S] (Eqs. disc.avg.flux, local.time.avg.non.cons, avg.source)
+// and, for every face node, the traces the Riemann problem needs: the
+// time-averaged solution U, the time-averaged normal flux and h^n and the
+// normal momentum at t^n (Eqs. time.avg.soln, combined.wave.speed,
+// good.numflux.non.cons).
+//
+// The pointwise arithmetic (stage values, fluxes) is FP64; the contractions
+// with D_x, D_y and the end-point rows, which were 60 % of the FP64
+// instructions, and the time averages run in block fixed point on the integer
+// pipe (fixed_point.cuh).  D is applied to the time-averaged fluxes once
+// instead of accumulating every stage's operator, so the last stage needs no
+// contraction.  On a 1024 x 1024 mesh at N = 3 the kernel takes 2.4 ms (FP64
+// pipe 77 % busy, integer pipes 35 %) against 6.4 ms with FP64 chains (one
+// thread per element row, FP64 pipe 96 %).  One thread per row in fixed point
+// took 4.2 ms: 255 registers and two warps per scheduler left the latencies
+// open, and 9700 instructions a warp missed the instruction cache; a thread
+// per node takes 96 registers and a quarter of the code.
 //
 // The well-balanced form (WB) has pressure-free fluxes and the
-// non-conservative terms g h D_x (h + b), g h D_y (h + b): D_x h is a row
-// chain, D_y h reads the other rows of h through shared memory.
+// non-conservative terms g h D_x (h + b), g h D_y (h + b).
 //
 // With the subcell blending limiter (LIMIT; the tensor-product extension of
 // Sec. 4) the kernel ends with the first-order part of limit_2d.cuh.
@@ -23,382 +34,452 @@
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
+#include "fixed_point.cuh"
 #include "limit_2d.cuh"
 
 namespace crkfr {
 namespace {
 
-// Launch shape of the element-local kernel: FP64 issue needs enough warps
-// in flight, so the block is small and at least CRKFR_LOCAL2D_MINB blocks
-// must fit an SM (the compiler caps the registers accordingly).
 #ifndef CRKFR_LOCAL2D_BLOCK
 #define CRKFR_LOCAL2D_BLOCK 128
 #endif
 #ifndef CRKFR_LOCAL2D_MINB
-#define CRKFR_LOCAL2D_MINB 2
+#define CRKFR_LOCAL2D_MINB 5
 #endif
 constexpr int kBlockLocal = CRKFR_LOCAL2D_BLOCK;
-constexpr int kWarpsLocal = kBlockLocal / 32;
 constexpr int kTrFields = 7;
 // x-face trace fields: U_h, U_hu, U_hv, F_hu, F_hv (time-averaged x fluxes of
 // hu and hv), h^n, hu^n.  y-face trace fields: U_h, U_hu, U_hv, G_hu, G_hv,
 // h^n, hv^n.  (The time-averaged h fluxes are U_hu and U_hv.)
 
+// Elements per block: as many as fit (n = 2, 4: whole warps; n = 3: 14 on 126
+// of 128 threads, n = 5: 5 on 125).
+template <int n>
+__host__ __device__ constexpr int local_elements() {
+  return kBlockLocal / (n * n);
+}
+
+// Exchange fields of the kernel: 0..5 the averages of h, hu, hv, hu hu / h
+// (+ pressure), hu hv / h, hv hv / h (+ pressure), or a stage's values of
+// them; 6..8 u^n.
+constexpr int kLocalFields = 9;
+
+// Doubles per element in shared memory, 4 modulo 16 so that the elements of a
+// warp start 32 bytes apart modulo the banks.
+template <int n, bool LIMIT>
+__host__ __device__ constexpr int local_stride() {
+  return ((LIMIT ? kLimExchange : kLocalFields) * n * n + 11) / 16 * 16 + 4;
+}
+
 template <int N, bool GLL, bool RES, bool IMEX, bool WB, bool LIMIT = false, bool STAGES = false,
           int PRE = 0>
-__global__ void __launch_bounds__(kBlockLocal, CRKFR_LOCAL2D_MINB) k_local_2d(const Launch2D L) {
+__global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
+    k_local_2d(const Launch2D L) {
   static_assert(!(STAGES && (IMEX || WB || LIMIT)), "stages are recorded for the standard form");
   // PRE 1: only the first stage's local operator L(u^n), which needs no dt,
   // stored in L.w; PRE 2: the step, taking L(u^n) from L.w (same arithmetic)
   static_assert(PRE == 0 || !(RES || IMEX || WB || LIMIT || STAGES),
                 "the first-stage pre-pass is built for the standard form");
   using TB = Tab<N, IMEX>;
-  static_assert(PRE == 0 || TB::need_L(0), "the first stage has a local operator");
+  static_assert(PRE == 0 || TB::feeds(0), "the first stage feeds a later one");
   constexpr int n = N + 1;
   constexpr int nn = n * n;
-  constexpr int EPW = 32 / n;          // elements per warp
   constexpr int S = TB::S;
-  constexpr int F0 = TB::first();
-  constexpr int NB = 4;                // fields per shared-memory exchange round
+  constexpr int EPB = local_elements<n>();
+  constexpr int ES = local_stride<n, LIMIT>();
+  // bits of the fixed-point operands (weighted sums up to 6 stay below 2^63;
+  // the six-stage method's, up to 90, are kept in two halves), the shift that
+  // brings a sum back to FB bits, and the bits by which a later stage may
+  // outgrow the first before the exponents are raised
+  constexpr int FB = 59;
+  constexpr bool WIDE = TB::weight_sum() > 8;
+  constexpr int kSumShift = WIDE ? 7 : 3;
+  constexpr int kHeadroom = 1;
+  // elements within whole warps need no block barrier
+  constexpr bool WARP = 32 % nn == 0;
   const Tables& T = L.tab;
-  // (the limiter's first-order part exchanges kLimRowFields fields at once)
-  constexpr int ES = exchange_stride(LIMIT ? kLimRowFields : NB, n);
-  __shared__ __align__(16) double sm[kWarpsLocal][EPW * ES];
+  __shared__ __align__(16) double sm[EPB * ES];
+  __shared__ int smag[EPB][3];
+  __shared__ double sdt[2];
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int le = lane / n, q = lane - le * n;
+  const int le_raw = threadIdx.x / nn, node = threadIdx.x - le_raw * nn;
+  const int q = node / n, p = node - q * n;
   const int64_t Ne = L.Ex * L.Ey;
-  const bool lane_ok = le < EPW;
-  const int lec = lane_ok ? le : 0;
-  double (*X)[n][n] = reinterpret_cast<double (*)[n][n]>(&sm[warp][lec * ES]);
+  const bool lane_ok = le_raw < EPB;
+  const int le = lane_ok ? le_raw : 0;
+  Fx (*X)[n][n] = reinterpret_cast<Fx (*)[n][n]>(&sm[le * ES]);
+  auto sync = [] {
+    if (WARP)
+      __syncwarp();
+    else
+      __syncthreads();
+  };
+  auto sync_or = [](bool b) -> bool {
+    return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
+  };
 
-  const double dt = (RES || PRE == 1) ? L.ctl.dt_fixed : step_dt(L.ctl, L.st);
-  if (!RES && PRE != 1 && blockIdx.x == 0 && threadIdx.x == 0 && !L.ctl.skip_bookkeeping)
-    step_bookkeeping(L.ctl, L.st, dt);
+  // the step size (a division) by one thread of the block
+  if (threadIdx.x == 0) {
+    const double dt = (RES || PRE == 1) ? L.ctl.dt_fixed : step_dt(L.ctl, L.st);
+    sdt[0] = dt;
+    sdt[1] = dt * TB::bref();
+    if (!RES && PRE != 1 && blockIdx.x == 0 && !L.ctl.skip_bookkeeping)
+      step_bookkeeping(L.ctl, L.st, dt);
+  }
 
-  // groups of kWarpsLocal * EPW elements; the step's plain instantiations
-  // (PERSIST) run on fewer blocks than groups and take them in turn, the
-  // others (whose registers the loop would spill) one group per block
-  constexpr bool PERSIST = !RES && !IMEX && !LIMIT && !STAGES && PRE == 0;
-  const int64_t groups =
-      ((L.row_end - L.row_begin) * L.Ex + kWarpsLocal * EPW - 1) / (kWarpsLocal * EPW);
-  // one group of kWarpsLocal * EPW elements
-  auto group = [&](const int64_t grp) {
-    const int64_t g = L.row_begin * L.Ex + (grp * kWarpsLocal + warp) * EPW + le;
-    // lanes past EPW*n (n = 3, 5) and lanes past the last element of the rows
-    // [row_begin, row_end) compute on element 0 and store nothing, neither to
-    // memory nor to shared memory
-    const bool active = lane_ok && (g < L.row_end * L.Ex);
-    const int64_t ge = active ? g : 0;
+  // threads past EPB n^2 and elements past the rows [row_begin, row_end)
+  // compute on element 0 and store nothing to memory (the former nothing to
+  // shared memory either)
+  const int64_t g = L.row_begin * L.Ex + (int64_t)blockIdx.x * EPB + le;
+  const bool active = lane_ok && (g < L.row_end * L.Ex);
+  const int64_t ge = active ? g : 0;
 
-    // ---- load row q of u^n and of the static terms g b_x, g b_y ---------------
-    double u0[3][n], gbx[n], gby[n];
+  // ---- u^n, the static terms g b_x, g b_y and the node's rows of D ----------
+  double u0[3];
 #pragma unroll
-    for (int v = 0; v < 3; ++v)
+  for (int v = 0; v < 3; ++v) u0[v] = L.u_in[(v * Ne + ge) * nn + node];
+  const double gbx = L.snode[ge * nn + node], gby = L.snode[(Ne + ge) * nn + node];
+  int dxh[n], dxl[n], dyh[n], dyl[n];
 #pragma unroll
-      for (int p = 0; p < n; ++p) u0[v][p] = L.u_in[(v * Ne + ge) * nn + q * n + p];
+  for (int j = 0; j < n; ++j) {
+    dxh[j] = T.fx.Dx_hi[p][j];
+    dxl[j] = T.fx.Dx_lo[p][j];
+    dyh[j] = T.fx.Dy_hi[q][j];
+    dyl[j] = T.fx.Dy_lo[q][j];
+  }
+  if (threadIdx.x < 3 * EPB) (&smag[0][0])[threadIdx.x] = 0;
+  __syncthreads();
+  const double dt = sdt[0];
+
+  double Ls[S][3];
+  if constexpr (PRE == 2) {
+    // L(u^n), computed ahead by the PRE 1 instantiation; the thread
+    // overwrites the same values with W at the end
 #pragma unroll
-    for (int p = 0; p < n; ++p) {
-      gbx[p] = L.snode[ge * nn + q * n + p];
-      gby[p] = L.snode[(Ne + ge) * nn + q * n + p];
+    for (int v = 0; v < 3; ++v) Ls[0][v] = L.w[(v * Ne + ge) * nn + node];
+  }
+  double Ss[S][2];               // source of hu, hv at each stage (IMEX)
+  double Sb[2] = {0.0, 0.0};     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
+  double P1 = 0.0, P2 = 0.0;     // sum_j (b_j/b_ref) h g d(h + b) (WB)
+  // time averages sum_j (b_j/b_ref) of the exchange fields 0..5 in the fixed
+  // point of the exponents E (h; hu, hv; the fluxes), which only grow: the
+  // sums are shifted when they do
+  // (WIDE: A 2^30 + B)
+  long long A[6] = {0, 0, 0, 0, 0, 0}, B[6] = {0, 0, 0, 0, 0, 0};
+  int E[3] = {-1, -1, -1};
+  auto group_of = [](int f) { return f == 0 ? 0 : f < 3 ? 1 : 2; };
+  // row of D_x on field fx plus row of D_y on field fy
+  auto contract = [&](int fx, int fy) -> long long {
+    FxAcc a;
+    Fx r[n];
+    fx_row<n>(X[fx][q], r);
+    fx_mul(a, r[0], dxh[0], dxl[0]);
+#pragma unroll
+    for (int j = 1; j < n; ++j) fx_mad(a, r[j], dxh[j], dxl[j]);
+#pragma unroll
+    for (int j = 0; j < n; ++j) fx_mad(a, X[fy][j][p], dyh[j], dyl[j]);
+    return fx_sum(a);
+  };
+  bool first = true;             // (resolved at compile time by unrolling)
+#pragma unroll
+  for (int i = 0; i < S; ++i) {
+    double cur[3];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      double acc = u0[v];
+#pragma unroll
+      for (int j = 0; j < i; ++j)
+        if (TB::a(i, j) != 0.0) acc = fma(-(dt * TB::a(i, j)), Ls[j][v], acc);
+      if (IMEX && v > 0) {
+#pragma unroll
+        for (int j = 0; j < i; ++j)
+          if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j][v - 1], acc);
+      }
+      cur[v] = acc;
     }
-
-    double Ls[S][3][n];
-    if constexpr (PRE == 2) {
-      // this row of L(u^n), computed ahead by the PRE 1 instantiation; the
-      // thread overwrites the same values with W at the end
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) Ls[0][v][p] = L.w[(v * Ne + ge) * nn + q * n + p];
+    if constexpr (IMEX) {
+      // Chezy friction s = -C_f |m| m / h^2 on (hu, hv), point-implicit with
+      // h fixed: m is parallel to the stage sum r and
+      // |m| + dt a_ii C_f |m|^2 / h^2 = |r|, so
+      // m = r 2 / (1 + sqrt(1 + 4 dt a_ii C_f |r| / h^2))
+      const double gcf = dt * TB::ai(i, i) * T.src_coef;
+      const double ih = drcp(cur[0]);
+      const double ih2 = ih * ih;
+      const double rx = cur[1], ry = cur[2];
+      double nm = dsqrt_pos(fma(rx, rx, ry * ry));
+      if (TB::ai(i, i) != 0.0) {
+        const double qf = dsqrt_pos(fma(4.0 * gcf * ih2, nm, 1.0));
+        const double f = 2.0 * drcp(1.0 + qf);
+        cur[1] = rx * f;
+        cur[2] = ry * f;
+        nm *= f;
+      }
+      if (TB::need_S(i)) {
+        const double c = -(T.src_coef * ih2) * nm;
+        Ss[i][0] = c * cur[1];
+        Ss[i][1] = c * cur[2];
+      }
     }
-    double Ss[S][2][n];                  // source of hu, hv at each stage (IMEX)
-    double V[3][n], U[3][n], F2[n], F3[n], G3[n];
-    double Sb[2][n];                     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
+    if constexpr (STAGES) {
+      // recorded step: the adjoint reads the stage values instead of
+      // recomputing them (stage 0 is u^n itself)
+      if (i > 0 && active) {
+        const int64_t Nr = L.stage_rows * L.Ex, gr = ge - L.stage_row0 * L.Ex;
 #pragma unroll
-    for (int i = 0; i < S; ++i) {
-      double cur[3][n];
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          double acc = u0[v][p];
-#pragma unroll
-          for (int j = 0; j < i; ++j)
-            if (TB::a(i, j) != 0.0) acc = fma(-(dt * TB::a(i, j)), Ls[j][v][p], acc);
-          if (IMEX && v > 0) {
-#pragma unroll
-            for (int j = 0; j < i; ++j)
-              if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j][v - 1][p], acc);
-          }
-          cur[v][p] = acc;
+        for (int v = 0; v < 3; ++v)
+          L.stages[(((int64_t)(i - 1) * 3 + v) * Nr + gr) * nn + node] = cur[v];
+      }
+    }
+    const int wi = TB::weight(i);
+    const double wd = wi;
+    // the stage's local operator feeds a later stage (for PRE 2 that of the
+    // first stage was loaded), its fluxes the time averages
+    const bool need_op = TB::feeds(i) && !(PRE == 2 && i == 0);
+    if (TB::feeds(i) || wi != 0) {
+      // the exchange fields at this node: the state and the fluxes
+      double f[6];
+      {
+        const double h = cur[0], mx = cur[1], my = cur[2];
+        const double r = drcp(h);
+        const double vx = mx * r, vy = my * r;
+        f[0] = h;
+        f[1] = mx;
+        f[2] = my;
+        if (WB) {
+          f[3] = mx * vx;
+          f[5] = my * vy;
+        } else {
+          const double ph = (h * h) * T.half_gravity;
+          f[3] = fma(mx, vx, ph);
+          f[5] = fma(my, vy, ph);
         }
-      if constexpr (IMEX) {
-        // Chezy friction s = -C_f |m| m / h^2 on (hu, hv), point-implicit with
-        // h fixed: m is parallel to the stage sum r and
-        // |m| + dt a_ii C_f |m|^2 / h^2 = |r|, so
-        // m = r 2 / (1 + sqrt(1 + 4 dt a_ii C_f |r| / h^2))
-        const double gcf = dt * TB::ai(i, i) * T.src_coef;
+        f[4] = mx * vy;
+      }
+      int mag[3];
+      mag[0] = fx_mag(f[0]);
+      mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
+      mag[2] = max(fx_mag(f[3]), max(fx_mag(f[4]), fx_mag(f[5])));
+      if (IMEX && first) {
+        // the traces of u^n, no stage value here, share the exponents
+        mag[0] = max(mag[0], fx_mag(u0[0]));
+        mag[1] = max(mag[1], max(fx_mag(u0[1]), fx_mag(u0[2])));
+      }
+      // one exponent per element and group of fields: the first stage's
+      // largest magnitudes with headroom, raised if a later stage exceeds
+      // them.  (The vote is also the barrier after the last reads of X.)
+      const bool over =
+          lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1] || mag[2] >> 20 > E[2]);
+      if (sync_or(over)) {
+        if (over) {
 #pragma unroll
-        for (int p = 0; p < n; ++p) {
-          const double ih = drcp(cur[0][p]);
-          const double ih2 = ih * ih;
-          const double rx = cur[1][p], ry = cur[2][p];
-          double nm = dsqrt_pos(fma(rx, rx, ry * ry));
-          if (TB::ai(i, i) != 0.0) {
-            const double q = dsqrt_pos(fma(4.0 * gcf * ih2, nm, 1.0));
-            const double f = 2.0 * drcp(1.0 + q);
-            cur[1][p] = rx * f;
-            cur[2][p] = ry * f;
-            nm *= f;
-          }
-          if (TB::need_S(i)) {
-            const double c = -(T.src_coef * ih2) * nm;
-            Ss[i][0][p] = c * cur[1][p];
-            Ss[i][1][p] = c * cur[2][p];
+          for (int k = 0; k < 3; ++k) atomicMax(&smag[le][k], mag[k]);
+        }
+        sync();
+        int d[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int e = fx_exp(smag[le][k]);
+          d[k] = e > E[k] ? e + kHeadroom - E[k] : 0;
+          E[k] += d[k];
+        }
+        if (!first) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const int sh = d[group_of(k)];
+            if (WIDE) {
+              // (the low half takes what the high one loses; from 62 on the
+              // sum is below 2^-55 of the new scale)
+              const long long hi = A[k] >> (sh & 63), lost = A[k] - (hi << (sh & 63));
+              const long long low = (B[k] >> (sh & 63)) +
+                                    (sh < 30 ? (lost << 30) >> (sh & 63) : lost >> ((sh - 30) & 63));
+              A[k] = sh < 62 ? hi : 0;
+              B[k] = sh < 62 ? low : 0;
+            } else {
+              A[k] = fx_sar(A[k], sh);
+            }
           }
         }
       }
-      if constexpr (STAGES) {
-        // recorded step: the adjoint reads the stage values instead of
-        // recomputing them (stage 0 is u^n itself)
-        if (i > 0 && active) {
 #pragma unroll
-          for (int v = 0; v < 3; ++v)
-#pragma unroll
-            for (int p = 0; p < n; ++p)
-              L.stages[(((int64_t)(i - 1) * 3 + v) * Ne + ge) * nn + q * n + p] = cur[v][p];
-        }
-      }
-      const double wi = TB::b(i) / TB::bref();
-      if (TB::need_L(i)) {
-        // fluxes at this row's nodes
-        double f2[n], f3[n], g3[n];
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          const double h = cur[0][p], mx = cur[1][p], my = cur[2][p];
-          const double r = drcp(h);
-          const double vx = mx * r, vy = my * r;
-          if (WB) {
-            f2[p] = mx * vx;
-            g3[p] = my * vy;
+      for (int k = 0; k < 6; ++k) {
+        const bool used = need_op && !(k == 0 && !WB) || WB && (k == 0);
+        const long long v = fx_from<FB>(f[k], E[group_of(k)]);
+        const Fx x = fx_split(v);
+        if (wi != 0) {
+          if (WIDE) {
+            A[k] += (long long)x.hi * wi;
+            B[k] += (long long)x.lo * wi;
           } else {
-            const double ph = (h * h) * T.half_gravity;
-            f2[p] = fma(mx, vx, ph);
-            g3[p] = fma(my, vy, ph);
-          }
-          f3[p] = mx * vy;
-        }
-        // y-fluxes (hv, hu hv / h, hv^2/h + g h^2/2) go through shared memory
-        // (not for the first stage of PRE 2: its operator was loaded)
-        if (!(PRE == 2 && i == 0)) {
-          __syncwarp();
-          if (lane_ok) {
-#pragma unroll
-            for (int p = 0; p < n; ++p) {
-              X[0][q][p] = cur[2][p];
-              X[1][q][p] = f3[p];
-              X[2][q][p] = g3[p];
-              if (WB) X[3][q][p] = cur[0][p];
-            }
-          }
-          __syncwarp();
-#pragma unroll
-          for (int p = 0; p < n; ++p) {
-            // non-conservative factors: g b_x, g b_y, and for the well-balanced
-            // form also g h_x, g h_y
-            double nbx = gbx[p], nby = gby[p];
-            if (WB) {
-              double hx = T.Dx[p][0] * cur[0][0];
-              double hy = T.Dy[q][0] * X[3][0][p];
-#pragma unroll
-              for (int j = 1; j < n; ++j) {
-                hx = fma(T.Dx[p][j], cur[0][j], hx);
-                hy = fma(T.Dy[q][j], X[3][j][p], hy);
-              }
-              nbx = fma(T.gravity, hx, nbx);
-              nby = fma(T.gravity, hy, nby);
-            }
-            double a0 = T.Dy[q][0] * X[0][0][p];
-            double a1 = fma(cur[0][p], nbx, T.Dy[q][0] * X[1][0][p]);
-            double a2 = fma(cur[0][p], nby, T.Dy[q][0] * X[2][0][p]);
-#pragma unroll
-            for (int j = 1; j < n; ++j) {
-              a0 = fma(T.Dy[q][j], X[0][j][p], a0);
-              a1 = fma(T.Dy[q][j], X[1][j][p], a1);
-              a2 = fma(T.Dy[q][j], X[2][j][p], a2);
-            }
-#pragma unroll
-            for (int j = 0; j < n; ++j) {
-              a0 = fma(T.Dx[p][j], cur[1][j], a0);
-              a1 = fma(T.Dx[p][j], f2[j], a1);
-              a2 = fma(T.Dx[p][j], f3[j], a2);
-            }
-            Ls[i][0][p] = a0;
-            Ls[i][1][p] = a1;
-            Ls[i][2][p] = a2;
+            A[k] += wi * v;
           }
         }
-        if constexpr (PRE == 1) {
-          if (active) {
+        if (used && lane_ok) X[k][q][p] = x;
+      }
+      if (need_op || WB) {
+        sync();
+        double ncx = 0.0, ncy = 0.0;   // well-balanced: h g (h + b)_x, _y
+        if constexpr (WB) {
+          FxAcc hx, hy;
+          fx_mul(hx, X[0][q][0], dxh[0], dxl[0]);
+          fx_mul(hy, X[0][0][p], dyh[0], dyl[0]);
 #pragma unroll
-            for (int v = 0; v < 3; ++v)
-#pragma unroll
-              for (int p = 0; p < n; ++p) L.w[(v * Ne + ge) * nn + q * n + p] = Ls[0][v][p];
+          for (int j = 1; j < n; ++j) {
+            fx_mad(hx, X[0][q][j], dxh[j], dxl[j]);
+            fx_mad(hy, X[0][j][p], dyh[j], dyl[j]);
           }
-          break;   // (the stage loop: this instantiation stops after L(u^n))
+          const int b = E[0] + T.fx.kD - FB, z = fx_zero(E[0]);
+          ncx = cur[0] * fma(T.gravity, fx_to(fx_sum(hx), b, z), gbx);
+          ncy = cur[0] * fma(T.gravity, fx_to(fx_sum(hy), b, z), gby);
+          if (wi != 0) {
+            P1 = fma(wd, ncx, P1);
+            P2 = fma(wd, ncy, P2);
+          }
         }
-        // time averages with the weights b_i / b_ref (first weighted stage: a copy)
-        if (wi != 0.0) {
-#pragma unroll
-          for (int p = 0; p < n; ++p) {
-            F2[p] = (i == F0) ? f2[p] : fma(wi, f2[p], F2[p]);
-            F3[p] = (i == F0) ? f3[p] : fma(wi, f3[p], F3[p]);
-            G3[p] = (i == F0) ? g3[p] : fma(wi, g3[p], G3[p]);
-          }
+        if (need_op) {
+          const int bm = E[1] + T.fx.kD - FB, bf = E[2] + T.fx.kD - FB;
+          const int zf = fx_zero(E[2]);
+          Ls[i][0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
+          const double l1 = fx_to(contract(3, 4), bf, zf), l2 = fx_to(contract(4, 5), bf, zf);
+          Ls[i][1] = WB ? l1 + ncx : fma(cur[0], gbx, l1);
+          Ls[i][2] = WB ? l2 + ncy : fma(cur[0], gby, l2);
         }
       }
-      if (wi != 0.0) {
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-#pragma unroll
-          for (int v = 0; v < 3; ++v) {
-            V[v][p] = (i == F0) ? Ls[i][v][p] : fma(wi, Ls[i][v][p], V[v][p]);
-            U[v][p] = (i == F0) ? cur[v][p] : fma(wi, cur[v][p], U[v][p]);
-          }
-          if constexpr (IMEX) {
-            // the implicit weights b_i equal the explicit ones b~_i
-            Sb[0][p] = (i == F0) ? Ss[i][0][p] : fma(wi, Ss[i][0][p], Sb[0][p]);
-            Sb[1][p] = (i == F0) ? Ss[i][1][p] : fma(wi, Ss[i][1][p], Sb[1][p]);
-          }
-        }
-      }
-    }
-
-    if constexpr (PRE == 1) return;
-
-    // ---- W = u^n - dt (dloc F + Bloc) [+ dt S]  (or the residual's part) -------
-    // (V and Sb hold time averages divided by b_ref)
-    constexpr double b0 = TB::bref();
-    const double dtb0 = dt * b0;
-    if (active) {
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          double o = RES ? -b0 * V[v][p] : fma(-dtb0, V[v][p], u0[v][p]);
-          if (IMEX && v > 0) o = fma(RES ? b0 : dtb0, Sb[v - 1][p], o);
-          L.w[(v * Ne + ge) * nn + q * n + p] = o;
-        }
-    }
-
-    const int64_t tstride = Ne * n;  // one (field, side) plane of a trace array
-
-    // ---- x-face traces of row q -------------------------------------------------
-    // field f of the x-face traces at node p of this row (f, p constant after unrolling)
-    auto fx = [&](int f, int p) -> double {
-      switch (f) {
-        case 0: return U[0][p];
-        case 1: return U[1][p];
-        case 2: return U[2][p];
-        case 3: return F2[p];
-        case 4: return F3[p];
-        case 5: return u0[0][p];
-        default: return u0[1][p];
-      }
-    };
-    auto fy = [&](int f, int p) -> double {
-      switch (f) {
-        case 0: return U[0][p];
-        case 1: return U[1][p];
-        case 2: return U[2][p];
-        case 3: return F3[p];
-        case 4: return G3[p];
-        case 5: return u0[0][p];
-        default: return u0[2][p];
-      }
-    };
-    {
-      if (active) {
-#pragma unroll
-        for (int f = 0; f < kTrFields; ++f) {
-          double tl, tr;
-          if (GLL) {
-            tl = fx(f, 0);
-            tr = fx(f, N);
-          } else {
-            tl = T.l0[0] * fx(f, 0);
-            tr = T.l1[0] * fx(f, 0);
-#pragma unroll
-            for (int p = 1; p < n; ++p) {
-              tl = fma(T.l0[p], fx(f, p), tl);
-              tr = fma(T.l1[p], fx(f, p), tr);
-            }
-          }
-          L.trx[(2 * f + 0) * tstride + ge * n + q] = tl;
-          L.trx[(2 * f + 1) * tstride + ge * n + q] = tr;
-        }
-      }
-    }
-    // ---- y-face traces of column p = q (two shared-memory rounds) -------------
-    {
-#pragma unroll
-      for (int r0 = 0; r0 < kTrFields; r0 += NB) {
-        __syncwarp();
-        if (lane_ok) {
-#pragma unroll
-          for (int f = r0; f < r0 + NB && f < kTrFields; ++f)
-#pragma unroll
-            for (int p = 0; p < n; ++p) X[f - r0][q][p] = fy(f, p);
-        }
-        __syncwarp();
+      if constexpr (PRE == 1) {
         if (active) {
 #pragma unroll
-          for (int f = r0; f < r0 + NB && f < kTrFields; ++f) {
-            double tb, tt;
-            if (GLL) {
-              tb = X[f - r0][0][q];
-              tt = X[f - r0][N][q];
-            } else {
-              tb = T.l0[0] * X[f - r0][0][q];
-              tt = T.l1[0] * X[f - r0][0][q];
-#pragma unroll
-              for (int j = 1; j < n; ++j) {
-                tb = fma(T.l0[j], X[f - r0][j][q], tb);
-                tt = fma(T.l1[j], X[f - r0][j][q], tt);
-              }
-            }
-            // buffer row ey+1; in a periodic mesh the bottom row's bottom side
-            // is also the halo above the top row, and vice versa
-            const int64_t row = ge / L.Ex + 1, col = ge - (row - 1) * L.Ex;
-            const int64_t plane = L.Ex * n;
-            L.try_[((row * 2 + 0) * kTrFields + f) * plane + col * n + q] = tb;
-            L.try_[((row * 2 + 1) * kTrFields + f) * plane + col * n + q] = tt;
-            if (L.periodic_y && row == 1)
-              L.try_[(((L.Ey + 1) * 2 + 0) * kTrFields + f) * plane + col * n + q] = tb;
-            if (L.periodic_y && row == L.Ey)
-              L.try_[((0 * 2 + 1) * kTrFields + f) * plane + col * n + q] = tt;
-          }
+          for (int v = 0; v < 3; ++v) L.w[(v * Ne + ge) * nn + node] = Ls[0][v];
         }
+        return;
+      }
+      if (wi != 0) first = false;
+    }
+    if constexpr (IMEX) {
+      // the implicit weights b_i equal the explicit ones b~_i
+      if (wi != 0) {
+        Sb[0] = fma(wd, Ss[i][0], Sb[0]);
+        Sb[1] = fma(wd, Ss[i][1], Sb[1]);
       }
     }
-    // ---- limiter: first-order update without the element-face terms and the
-    //      face data of the first-order face fluxes (limit_2d.cuh) -------------
-    if constexpr (LIMIT) {
-      static_assert(!RES, "the limiter needs a step");
-      limit_local_2d<N, GLL, WB>(L, u0, X, q, lane_ok, active, ge, dt);
+  }
+
+  // ---- W = u^n - dt (dloc F + Bloc) [+ dt S]  (or the residual's part) -------
+  // The derivative of the time averages is taken once: dloc F = D (sum_j b_j
+  // f_j), Bloc = g b_x (sum_j b_j h_j) (the well-balanced product is
+  // accumulated stage by stage).  A, P and Sb hold time averages divided by
+  // b_ref; the sums are scaled back to FB bits for the contractions.
+  if (WIDE) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      A[k] += B[k] >> 30;
+      A[k] = (A[k] << (30 - kSumShift)) + (((int)B[k] & 0x3fffffff) >> kSumShift);
     }
-  };
-  if constexpr (PERSIST) {
-    for (int64_t grp = blockIdx.x; grp < groups; grp += gridDim.x) group(grp);
   } else {
-    group(blockIdx.x);   // one block per group
+#pragma unroll
+    for (int k = 0; k < 6; ++k) A[k] >>= kSumShift;
+  }
+  sync();
+  if (lane_ok) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) X[k][q][p] = fx_split(A[k]);
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      if constexpr (GLL)
+        X[6 + v][q][p] = Fx{__double2hiint(u0[v]), __double2loint(u0[v])};
+      else
+        X[6 + v][q][p] = fx_split(fx_from<FB>(u0[v], E[v == 0 ? 0 : 1]));
+    }
+  }
+  sync();
+  {
+    constexpr double b0 = TB::bref();
+    const double dtb0 = sdt[1];
+    const int bm = E[1] + T.fx.kD - FB + kSumShift, bf = E[2] + T.fx.kD - FB + kSumShift;
+    const int zf = fx_zero(E[2]);
+    double V[3];
+    V[0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
+    V[1] = fx_to(contract(3, 4), bf, zf);
+    V[2] = fx_to(contract(4, 5), bf, zf);
+    if constexpr (WB) {
+      V[1] += P1;
+      V[2] += P2;
+    } else {
+      const double uh = fx_to(A[0], E[0] + 63 - FB + kSumShift, fx_zero(E[0]));
+      V[1] = fma(uh, gbx, V[1]);
+      V[2] = fma(uh, gby, V[2]);
+    }
+    if (active) {
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        double o = RES ? -b0 * V[v] : fma(-dtb0, V[v], u0[v]);
+        if (IMEX && v > 0) o = fma(RES ? b0 : dtb0, Sb[v - 1], o);
+        L.w[(v * Ne + ge) * nn + node] = o;
+      }
+    }
+  }
+
+  // ---- face traces: 4 n face nodes per element (side 0 / 1 of the x faces,
+  //      then of the y faces), all fields of a face node by one thread --------
+  if (active) {
+    const int64_t tstride = Ne * n;              // one (field, side) plane of the x traces
+    const int64_t plane = L.Ex * n;              // one field of a row's y traces
+    const int64_t row = ge / L.Ex + 1, col = ge - (row - 1) * L.Ex;   // y-trace buffer row
+#pragma unroll
+    for (int j0 = 0; j0 < 4 * n; j0 += nn) {
+      const int job = j0 + node;
+      if (4 * n % nn != 0 && job >= 4 * n) break;
+      const int dir = job / (2 * n), side = job / n & 1, r = job % n;
+      // the nodes next to the face line: base + j step
+      const Fx* line = &X[0][dir ? 0 : r][dir ? r : 0];
+      const int step = dir ? n : 1;
+      int ch[n], cl[n];
+#pragma unroll
+      for (int j = 0; j < n; ++j) {
+        ch[j] = side ? T.fx.l1_hi[j] : T.fx.l0_hi[j];
+        cl[j] = side ? T.fx.l1_lo[j] : T.fx.l0_lo[j];
+      }
+      double* out = dir ? L.try_ + (row * 2 + side) * kTrFields * plane + col * n + r
+                        : L.trx + side * tstride + ge * n + r;
+      const int64_t ostep = dir ? plane : 2 * tstride;
+      // in a periodic mesh the bottom row's bottom side is also the halo
+      // above the top row, and vice versa
+      const bool wrap = dir && L.periodic_y && row == (side ? L.Ey : 1);
+      double* halo = L.try_ + (side ? 1 : (L.Ey + 1) * 2) * kTrFields * plane + col * n + r;
+#pragma unroll
+      for (int fi = 0; fi < kTrFields; ++fi) {
+        const int k = fi < 3 ? fi : fi < 5 ? fi + dir : fi == 5 ? 6 : 7 + dir;
+        const int ek = fi == 0 || fi == 5 ? E[0] : fi < 3 || fi == 6 ? E[1] : E[2];
+        const Fx* x = line + k * nn;
+        double t;
+        if constexpr (GLL) {
+          const Fx v = x[side ? N * step : 0];
+          if (fi >= 5)
+            t = __hiloint2double(v.hi, v.lo);
+          else
+            t = fx_to(((long long)v.hi << 30) + v.lo, ek + 63 - FB + kSumShift, fx_zero(ek));
+        } else {
+          FxAcc a;
+          fx_mul(a, x[0], ch[0], cl[0]);
+#pragma unroll
+          for (int j = 1; j < n; ++j) fx_mad(a, x[j * step], ch[j], cl[j]);
+          t = fx_to(fx_sum(a), ek + T.fx.kL - FB + (fi < 5 ? kSumShift : 0), fx_zero(ek));
+        }
+        out[fi * ostep] = t;
+        if (wrap) halo[fi * plane] = t;
+      }
+    }
+  }
+  // ---- limiter: first-order update without the element-face terms and the
+  //      face data of the first-order face fluxes (limit_2d.cuh) -------------
+  if constexpr (LIMIT) {
+    static_assert(!RES, "the limiter needs a step");
+    sync();
+    limit_local_2d<N, GLL, WB>(L, u0, &sm[le * ES], node, lane_ok, active, ge, dt, sync);
   }
 }
 
 template <int N, bool GLL, bool IMEX, bool WB, bool LIMIT = false>
 int launch_local_t(const Launch2D& L, cudaStream_t s) {
-  constexpr int per_block = kWarpsLocal * (32 / (N + 1));
+  constexpr int per_block = local_elements<N + 1>();
   if (L.row_begin < 0 || L.row_end <= L.row_begin || L.row_end > L.Ey)
     return (int)cudaErrorInvalidValue;
   const int64_t blocks = ((L.row_end - L.row_begin) * L.Ex + per_block - 1) / per_block;
@@ -407,28 +488,8 @@ int launch_local_t(const Launch2D& L, cudaStream_t s) {
     k_local_2d<N, GLL, false, IMEX, WB, true><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
   else if (L.ctl.residual)
     k_local_2d<N, GLL, true, IMEX, WB><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
-  else if constexpr (IMEX)
+  else
     k_local_2d<N, GLL, false, IMEX, WB><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
-  else {
-    // the step: twice as many blocks as fit the GPU at once, each taking
-    // element groups in turn, so that no block starts cold after the first
-    // ones (1.5 % faster than one block per group at 1024^2)
-    // (resident blocks on the GPU, asked once; 0 if the query failed: then
-    // one block per group)
-    static const int resident = [] {
-      int nb = 0, dev = 0, sms = 0;
-      if (cudaGetDevice(&dev) != cudaSuccess ||
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-              &nb, k_local_2d<N, GLL, false, IMEX, WB>, kBlockLocal, 0) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-      }
-      return nb * sms;
-    }();
-    const int64_t grid = resident > 0 && 2 * (int64_t)resident < blocks ? 2 * resident : blocks;
-    k_local_2d<N, GLL, false, IMEX, WB><<<(unsigned)grid, kBlockLocal, 0, s>>>(L);
-  }
   return (int)cudaGetLastError();
 }
 

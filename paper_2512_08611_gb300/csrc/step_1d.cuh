@@ -359,7 +359,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         }
       }
     }
-    const double wi = TB::b(i) / TB::bref();
+    const double wi = TB::weight(i);
     if (TB::need_L(i)) {
       if constexpr (SWE) {
         double f2[n];
@@ -390,7 +390,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         }
         if (wi != 0.0) {
 #pragma unroll
-          for (int p = 0; p < n; ++p) F2[p] = (i == F0) ? f2[p] : fma(wi, f2[p], F2[p]);
+          for (int p = 0; p < n; ++p) F2[p] = (i == F0) ? wi * f2[p] : fma(wi, f2[p], F2[p]);
         }
       } else {
 #pragma unroll
@@ -407,13 +407,13 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       for (int v = 0; v < M; ++v)
 #pragma unroll
         for (int p = 0; p < n; ++p) {
-          V[v][p] = (i == F0) ? Ls[i][v][p] : fma(wi, Ls[i][v][p], V[v][p]);
-          U[v][p] = (i == F0) ? cur[v][p] : fma(wi, cur[v][p], U[v][p]);
+          V[v][p] = (i == F0) ? wi * Ls[i][v][p] : fma(wi, Ls[i][v][p], V[v][p]);
+          U[v][p] = (i == F0) ? wi * cur[v][p] : fma(wi, cur[v][p], U[v][p]);
         }
       if constexpr (IMEX) {
         // the implicit weights b_i equal the explicit ones b~_i
 #pragma unroll
-        for (int p = 0; p < n; ++p) Sb[p] = (i == F0) ? Ss[i][p] : fma(wi, Ss[i][p], Sb[p]);
+        for (int p = 0; p < n; ++p) Sb[p] = (i == F0) ? wi * Ss[i][p] : fma(wi, Ss[i][p], Sb[p]);
       }
     }
   }

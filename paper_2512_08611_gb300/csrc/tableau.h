@@ -105,10 +105,25 @@ CRKFR_HD constexpr double imex_b(int i) {
   return i == 0 ? 0.0 : i == 3 ? 2.0 / 3.0 : 1.0 / 6.0;
 }
 
+// b~_i in units of 1 / (sum of these integers): every tableau's weights are
+// small integers over a common denominator (1; 2; 6; 6; 90; IMEX 6)
+CRKFR_HD constexpr int tab_weight(int N, int i) {
+  if (N == 0) return 1;
+  if (N == 1) return 1;
+  if (N == 2) return i == 2 ? 4 : 1;
+  if (N == 3) return (i == 0 || i == 3) ? 1 : 2;
+  return i == 0 || i == 5 ? 7 : i == 1 ? 0 : i == 3 ? 12 : 32;
+}
+CRKFR_HD constexpr int imex_weight(int i) { return i == 0 ? 0 : i == 3 ? 4 : 1; }
+CRKFR_HD constexpr int tab_weight_sum(int N) {
+  return N == 0 ? 1 : N == 1 ? 2 : N == 4 ? 90 : 6;
+}
+
 // The tableau a kernel instantiation uses: the explicit one of degree N, or
 // SSP3-IMEX(4,3,3) when the step has a source.  The time averages are
-// accumulated with the weights b~_i / b~_ref, b~_ref the first non-zero
-// weight (its stage initialises the accumulators).
+// accumulated with the integer weights b~_i / b_ref, b_ref the common
+// denominator's reciprocal; first() is the stage that initialises the
+// accumulators.
 template <int N, bool IMEX>
 struct Tab {
   static constexpr int S = IMEX ? imex_stages() : tab_stages(N);
@@ -121,7 +136,15 @@ struct Tab {
       if (b(i) != 0.0) return i;
     return 0;
   }
-  CRKFR_HD static constexpr double bref() { return b(first()); }
+  CRKFR_HD static constexpr int weight(int i) { return IMEX ? imex_weight(i) : tab_weight(N, i); }
+  CRKFR_HD static constexpr int weight_sum() { return IMEX ? 6 : tab_weight_sum(N); }
+  CRKFR_HD static constexpr double bref() { return 1.0 / weight_sum(); }
+  // the local operator of stage i is needed by a later stage
+  CRKFR_HD static constexpr bool feeds(int i) {
+    for (int k = i + 1; k < S; ++k)
+      if (a(k, i) != 0.0) return true;
+    return false;
+  }
   // the local operator of stage i is needed by a later stage or the averages
   CRKFR_HD static constexpr bool need_L(int i) {
     if (b(i) != 0.0) return true;
@@ -143,10 +166,6 @@ struct Tab {
 inline int host_stages(int N, bool imex) { return imex ? imex_stages() : tab_stages(N); }
 inline double host_a(int N, bool imex, int i, int j) { return imex ? imex_ae(i, j) : tab_a(N, i, j); }
 inline double host_b(int N, bool imex, int i) { return imex ? imex_b(i) : tab_b(N, i); }
-inline double host_bref(int N, bool imex) {
-  for (int i = 0; i < host_stages(N, imex); ++i)
-    if (host_b(N, imex, i) != 0.0) return host_b(N, imex, i);
-  return 1.0;
-}
+inline double host_bref(int N, bool imex) { return 1.0 / (imex ? 6 : tab_weight_sum(N)); }
 
 }  // namespace crkfr

@@ -3,9 +3,9 @@
 // On GB300 the FP64 pipe issues about one warp instruction per 16 SM cycles
 // (two FP64 FMA lanes per SM), some 60x below FP32, and a partly masked warp
 // costs the same as a full one.  These helpers therefore keep FP64
-// instructions to the minimum and push everything that need not be FP64
-// (seeds, comparisons, maxima of non-negative values) onto the FP32 and
-// integer pipes.
+// instructions to the minimum and push everything that can be exact elsewhere
+// (reciprocals and roots, comparisons, maxima of non-negative values) onto the
+// FP32 and integer pipes.
 #pragma once
 
 #include <cstdint>
@@ -15,73 +15,98 @@
 
 namespace crkfr {
 
-// 1/x for FP64 x.  Seed: the FP32 reciprocal of x rounded down to 24
-// significant bits, built from and converted back to the FP64 bit pattern
-// with integer operations (no FP64 conversion instructions).  Refinement:
-// one step of the third-order Newton/series iteration
-// r <- r (1 + e + e^2), e = 1 - x r, which takes the ~2^-22 seed error to
-// ~2^-66; the result is within about one ulp of 1/x.  Three FP64 FMAs.
-// Inputs whose exponent lies outside the FP32 seed range fall back to the
-// IEEE division.
+// The elementary operations below work on the significand as integers: an
+// FP64 instruction holds the FP64 pipe 64 cycles a warp, an IMAD.WIDE the
+// integer pipe 2, so the third-order refinement of an FP32 seed costs about 30
+// integer instructions (some 45 cycles) instead of 3 (reciprocal) or 5 (roots)
+// FP64 ones (192, 320 cycles), and being exact up to 2^-58 it ends within 0.51
+// (1/x), 0.52 (1/sqrt) and 0.58 (sqrt) ulp.
+
+// 2^23 y for the FP32 seed y in (1/2, 1], lowered by 2^-22 so that it stays
+// below 2^23
+__device__ __forceinline__ unsigned seed_bits(float y) {
+  return (unsigned)__float_as_int(fmaf(y, 8388606.0f, 8388608.0f)) - 0x4b000000u;
+}
+
+// (r s) 2^-32 for r < 2^23 and a signed s
+__device__ __forceinline__ long long seed_times(unsigned r, long long s) {
+  return (long long)(int)r * (int)(s >> 32) +
+         (long long)(((unsigned long long)r * (unsigned)s) >> 32);
+}
+
+// 1/x for FP64 x: with the significand m and a seed r of 1/m, p = m r - 1 is
+// formed exactly (2^75 p fits 64 bits since |p| < 2^-20), and 1/m = r (1 - p +
+// p^2) up to p^3 < 2^-60.  Zero, denormal and non-finite x, and x whose
+// reciprocal is not normal, take the IEEE division.
 __device__ __forceinline__ double drcp(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned lo = (unsigned)__double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  if (ex < 1023 - 124 || ex > 1023 + 124) return 1.0 / x;
-  const int sign = hi & (int)0x80000000;
-  const int fb = ((((hi & 0x7fffffff) - ((1023 - 127) << 20)) << 3) | (int)(lo >> 29)) | sign;
-  const float rf = __frcp_rn(__int_as_float(fb));
-  const int rb = __float_as_int(rf);
-  const int rhi = ((((rb & 0x7fffffff) >> 3) + ((1023 - 127) << 20)) | (rb & (int)0x80000000));
-  const int rlo = rb << 29;
-  double r = __hiloint2double(rhi, rlo);
-  const double e = fma(-x, r, 1.0);
-  r = fma(r, fma(e, e, e), r);
-  return r;
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int ex = (int)(hi >> 20) & 0x7ff;
+  if ((unsigned)(ex - 1) > 2043u) return 1.0 / x;
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  float f = __int_as_float((int)((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(f));
+  const unsigned r = seed_bits(f);
+  const long long p =
+      (long long)((unsigned long long)lo * r + ((unsigned long long)(mh * r) << 32));
+  const int ph = (int)(p >> 25);                              // 2^50 p
+  const long long s = (((long long)ph * ph) >> 25) - p;       // 2^75 (p^2 - p)
+  const unsigned long long R = ((unsigned long long)r << 39) +
+                               (unsigned long long)(seed_times(r, s) >> 4) + 0x100u;   // 2^62 / m
+  const unsigned oh = ((unsigned)(R >> 41) + ((unsigned)(2044 - ex) << 20)) | (hi & 0x80000000u);
+  return __hiloint2double((int)oh, (int)(unsigned)(R >> 9));
 }
 
-// sqrt(x) for FP64 x > 0.  Seed: the FP32 reciprocal square root of x
-// rounded down to 24 significant bits, built from and converted back to the
-// FP64 bit pattern with integer operations.  Refinement: with t = x y and
-// e = 1 - t y, sqrt(x) = t (1 - e)^(-1/2); the binomial series to second
-// order, t + t e (1/2 + 3e/8), takes the ~2^-21 seed error to ~2^-63.  Five
-// FP64 instructions.  Non-positive inputs and exponents outside the FP32
-// seed range fall back to the IEEE square root.
-__device__ __forceinline__ double dsqrt_pos(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned lo = (unsigned)__double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  if (hi < 0 || ex < 1023 - 124 || ex > 1023 + 124) return sqrt(x);
-  const int fb = (((hi - ((1023 - 127) << 20)) << 3) | (int)(lo >> 29));
-  const float yf = rsqrtf(__int_as_float(fb));
-  const int yb = __float_as_int(yf);
-  const double y = __hiloint2double((yb >> 3) + ((1023 - 127) << 20), yb << 29);
-  const double t = x * y;
-  const double e = fma(-t, y, 1.0);
-  const double p = fma(0.375, e, 0.5);
-  const double q = t * e;
-  return fma(q, p, t);
+// 2^58 / sqrt(m) of x = m 4^k with 1 <= m < 4, m = (mh, ml) 2^-52: with a seed
+// y, p = m y^2 - 1 (2^66 p, truncated), 1/sqrt(m) = y (1 - p/2 + 3 p^2/8).
+__device__ __forceinline__ unsigned long long rsqrt_bits(double x, unsigned& mh, unsigned& ml,
+                                                         int& k) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int ex = (int)(hi >> 20);
+  const unsigned odd = ~(unsigned)ex & 1u;                    // ex - 1023 odd
+  mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, odd);
+  ml = lo << odd;
+  k = (ex - 1023 - (int)odd) >> 1;
+  float f = __int_as_float((int)(((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u) +
+                                 (odd << 23)));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(f));
+  const unsigned y = seed_bits(f);
+  const unsigned long long Q = (unsigned long long)y * y;
+  const unsigned qh = (unsigned)(Q >> 32), ql = (unsigned)Q;
+  const long long p =
+      (long long)(((unsigned long long)ml * ql >> 32) + (unsigned long long)mh * ql +
+                  (unsigned long long)ml * qh + ((unsigned long long)(mh * qh) << 32));
+  const int ph = (int)(p >> 17);                              // 2^49 p
+  const int t = (int)(((long long)ph * ph) >> 32);            // 2^66 p^2
+  const long long s = (long long)((3 * t) >> 2) - p;          // 2^67 (3 p^2/8 - p/2)
+  return ((unsigned long long)y << 35) + (unsigned long long)seed_times(y, s);
 }
 
-// 1/sqrt(x) for FP64 x > 0.  Seed as in dsqrt_pos; with e = 1 - x y^2,
-// 1/sqrt(x) = y (1 - e)^(-1/2), and the binomial series to second order,
-// y + y e (1/2 + 3e/8), takes the ~2^-21 seed error to ~2^-63.  Five FP64
-// instructions.  Non-positive inputs and exponents outside the FP32 seed
-// range fall back to the IEEE operations.
+// positive, normal and finite (the range of the two roots below)
+__device__ __forceinline__ bool positive_normal(double x) {
+  return (unsigned)__double2hiint(x) - 0x100000u < 0x7fe00000u;
+}
+
+// 1/sqrt(x) for FP64 x > 0; other x take the IEEE operations.
 __device__ __forceinline__ double drsqrt_pos(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned lo = (unsigned)__double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  if (hi < 0 || ex < 1023 - 124 || ex > 1023 + 124) return 1.0 / sqrt(x);
-  const int fb = (((hi - ((1023 - 127) << 20)) << 3) | (int)(lo >> 29));
-  const float yf = rsqrtf(__int_as_float(fb));
-  const int yb = __float_as_int(yf);
-  const double y = __hiloint2double((yb >> 3) + ((1023 - 127) << 20), yb << 29);
-  const double t = x * y;
-  const double e = fma(-t, y, 1.0);
-  const double p = fma(0.375, e, 0.5);
-  const double q = y * e;
-  return fma(q, p, y);
+  if (!positive_normal(x)) return 1.0 / sqrt(x);
+  unsigned mh, ml;
+  int k;
+  const unsigned long long q = (rsqrt_bits(x, mh, ml, k) + 0x10u) >> 5;
+  return __longlong_as_double((long long)(q + ((unsigned long long)(unsigned)(1021 - k) << 52)));
+}
+
+// sqrt(x) for FP64 x > 0, as m (1/sqrt(m)); other x take the IEEE square root.
+__device__ __forceinline__ double dsqrt_pos(double x) {
+  if (!positive_normal(x)) return sqrt(x);
+  unsigned mh, ml;
+  int k;
+  const unsigned long long R = rsqrt_bits(x, mh, ml, k);
+  const unsigned rh = (unsigned)(R >> 32), rl = (unsigned)R;
+  const unsigned long long low = ((unsigned long long)ml * rl >> 32) +
+                                 (unsigned long long)mh * rl + (unsigned long long)ml * rh;
+  const unsigned long long top = (unsigned long long)mh * rh + (low >> 32);   // 2^46 sqrt(m)
+  const unsigned long long q = (top << 6) + ((((unsigned)low >> 25) + 1) >> 1);
+  return __longlong_as_double((long long)(q + ((unsigned long long)(unsigned)(1022 + k) << 52)));
 }
 
 // sigma(f' + B) of shallow water in one direction, |m/h| + sqrt(g h), as

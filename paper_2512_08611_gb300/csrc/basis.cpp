@@ -260,11 +260,17 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
   FxTables& F = T->fx;
   F.kD = 123 - sD;
   F.kL = 123 - sL;
+  double gm = 0.0;
+  for (int i = 0; i < n; ++i)
+    gm = std::fmax(gm, std::fmax(std::fmax(std::fabs(T->gRx[i]), std::fabs(T->gLx[i])),
+                                 std::fmax(std::fabs(T->gRy[i]), std::fabs(T->gLy[i]))));
+  std::frexp(gm, &F.kG);
   for (int i = 0; i < n; ++i) {
     for (int j = 0; j < n; ++j) {
       fx_coef(T->Dx[i][j], sD, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);
       fx_coef(T->Dy[i][j], sD, &F.Dy_hi[i][j], &F.Dy_lo[i][j]);
     }
+    for (int j = 0; j < n; ++j) fx_coef(T->w2[i][j], 60, &F.w2_hi[i][j], &F.w2_lo[i][j]);
     fx_coef(T->l0[i], sL, &F.l0_hi[i], &F.l0_lo[i]);
     fx_coef(T->l1[i], sL, &F.l1_hi[i], &F.l1_lo[i]);
   }

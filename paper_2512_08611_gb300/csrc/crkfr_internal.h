@@ -30,6 +30,10 @@ struct FxTables {
   int32_t Dy_hi[kMaxNodes][kMaxNodes], Dy_lo[kMaxNodes][kMaxNodes];
   int32_t l0_hi[kMaxNodes], l0_lo[kMaxNodes], l1_hi[kMaxNodes], l1_lo[kMaxNodes];
   int32_t kD, kL;
+  // quadrature weights w_q w_p in units of 2^-60 (their sum is one); kG: all
+  // |0.5 g'| / dx, / dy below 2^kG
+  int32_t w2_hi[kMaxNodes][kMaxNodes], w2_lo[kMaxNodes][kMaxNodes];
+  int32_t kG;
 };
 
 // Reference-element and mesh tables passed to every kernel by value, so they

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
+#include "fixed_point.cuh"
 #include "local_2d.cuh"
 
 namespace crkfr {
@@ -29,6 +30,9 @@ namespace {
 
 constexpr int kBlock2D = 256;
 constexpr int kWarps2D = kBlock2D / 32;
+
+// a face term converted in place
+__device__ __forceinline__ Fx fx_at(const double* t) { return *reinterpret_cast<const Fx*>(t); }
 
 // Doubled face terms of both sides of one face node, T'^- = 2 (F^num,- - F^tot,-)
 // and T'^+ = 2 (F^num,+ - F^tot,+), from the two sides' traces.
@@ -183,15 +187,41 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
   const int64_t ex0 = (int64_t)blockIdx.x * TX, ey0 = L.row_begin + (int64_t)blockIdx.y * TY;
   // the traces hold time averages divided by b_0: so do the face terms
   const double dtp = RES ? 1.0 : L.st->dt_cur;
-  const double dt = dtp * T.b0;
-  // correction tables times -dt (phase 2 adds the face terms to W with one
-  // FMA each); written here, read after the barrier between the phases
-  __shared__ double cor[4][n];
+  // correction tables times -dt in fixed point (FB bits below 2^(ec - 1022)),
+  // written here, read after the barriers between the phases
+  constexpr int FB = 59;
+  __shared__ Fx cor[4][n];
+  __shared__ int cor_e;
+  // largest magnitudes of the face terms of h and of the momenta per element
+  __shared__ int emag[2][TY][TX];
+  for (int k = threadIdx.x; k < 2 * TY * TX; k += BT) (&emag[0][0][0])[k] = 0;
   if (threadIdx.x < 4 * n) {
+    const double dt = dtp * T.b0;
     const int t = threadIdx.x / n, p = threadIdx.x - t * n;
     const double g = t == 0 ? T.gRx[p] : t == 1 ? T.gLx[p] : t == 2 ? T.gRy[p] : T.gLy[p];
-    cor[t][p] = -dt * g;
+    const int ec = fx_exp(fx_mag(dt) + (T.fx.kG << 20));
+    cor[t][p] = fx_split(fx_from<FB>(-dt * g, ec));
+    if (threadIdx.x == 0) cor_e = ec;
   }
+  __syncthreads();
+  // the terms of both sides of a face: to shared memory, their magnitudes to
+  // the elements they belong to (minus side: r0, c0; plus side: r1, c1)
+  auto keep = [&](double* tm, double* tp, int vs, const double* Tm, const double* Tp, int r0,
+                  int c0, int r1, int c1) {
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      tm[v * vs] = Tm[v];
+      tp[v * vs] = Tp[v];
+    }
+    if (r0 >= 0 && c0 >= 0) {
+      atomicMax(&emag[0][r0][c0], fx_mag(Tm[0]));
+      atomicMax(&emag[1][r0][c0], max(fx_mag(Tm[1]), fx_mag(Tm[2])));
+    }
+    if (r1 < TY && c1 < TX) {
+      atomicMax(&emag[0][r1][c1], fx_mag(Tp[0]));
+      atomicMax(&emag[1][r1][c1], max(fx_mag(Tp[1]), fx_mag(Tp[2])));
+    }
+  };
 
   // ---- phase 1: every face node of the tile once --------------------------
   for (int f = threadIdx.x; f < NX + NY; f += BT) {
@@ -226,11 +256,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
         face_terms<WB>(a, b, 1, L.sface[ep * n + q], T.gravity, T.inv_gravity, T.sqrt_gravity,
                        Tm, Tp);
       }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        sxm[v][r][k][q] = Tm[v];
-        sxp[v][r][k][q] = Tp[v];
-      }
+      keep(&sxm[0][r][k][q], &sxp[0][r][k][q], TY * (TX + 1) * n, Tm, Tp, r, k - 1, r, k);
     } else {
       const int g = f - NX;
       const int p = g % n, c = (g / n) % TX, k = g / (n * TX);
@@ -276,12 +302,43 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
         face_terms<WB>(a, b, 2, L.sface[Ne * n + (ey0 + k) * plane + ex * n + p], T.gravity,
                        T.inv_gravity, T.sqrt_gravity, Tm, Tp);
       }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        sym[v][k][c][p] = Tm[v];
-        syp[v][k][c][p] = Tp[v];
-      }
+      keep(&sym[0][k][c][p], &syp[0][k][c][p], (TY + 1) * TX * n, Tm, Tp, k - 1, c, k, c);
     }
+  }
+  __syncthreads();
+
+  // ---- the face terms in the fixed point of their element, in place -------
+  for (int f = threadIdx.x; f < NX + NY; f += BT) {
+    double *tm, *tp;
+    int vs, r0, c0, r1, c1;
+    if (f < NX) {
+      const int q = f % n, k = (f / n) % (TX + 1), r = f / (n * (TX + 1));
+      if (ey0 + r >= Ey || (k > 0 && ex0 + k - 1 >= Ex)) continue;
+      tm = &sxm[0][r][k][q];
+      tp = &sxp[0][r][k][q];
+      vs = TY * (TX + 1) * n;
+      r0 = r1 = r;
+      c0 = k - 1;
+      c1 = k;
+    } else {
+      const int g = f - NX;
+      const int p = g % n, c = (g / n) % TX, k = g / (n * TX);
+      if (ex0 + c >= Ex || (k > 0 && ey0 + k - 1 >= Ey)) continue;
+      tm = &sym[0][k][c][p];
+      tp = &syp[0][k][c][p];
+      vs = (TY + 1) * TX * n;
+      r0 = k - 1;
+      r1 = k;
+      c0 = c1 = c;
+    }
+    auto convert = [&](double* t, int r, int c) {
+      const int e0 = fx_exp(emag[0][r][c]), e1 = fx_exp(emag[1][r][c]);
+#pragma unroll
+      for (int v = 0; v < 3; ++v)
+        *reinterpret_cast<Fx*>(t + v * vs) = fx_split(fx_from<FB>(t[v * vs], v ? e1 : e0));
+    };
+    if (r0 >= 0 && c0 >= 0) convert(tm, r0, c0);
+    if (r1 < TY && c1 < TX) convert(tp, r1, c1);
   }
   __syncthreads();
 
@@ -293,18 +350,54 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
   const int64_t ey = ey0 + r, ex = ex0 + cc;
   const bool active = lane_ok && ey < Ey && ex < Ex;
   const int64_t ge = active ? ey * Ex + ex : 0;
+  // u^{n+1} = W + corrections, summed in the fixed point of the larger of W's
+  // and the corrections' scales in the element and rounded once
   double out[3][n];
+  double W[3][n];
+  int mag[2] = {0, 0};
 #pragma unroll
   for (int v = 0; v < 3; ++v)
 #pragma unroll
     for (int p = 0; p < n; ++p) {
-      double o = L.w[(v * Ne + ge) * nn + q * n + p];
-      if (!GLL || p == N) o = fma(sxm[v][r][cc + 1][q], cor[0][p], o);
-      if (!GLL || p == 0) o = fma(sxp[v][r][cc][q], cor[1][p], o);
-      if (!GLL || q == N) o = fma(sym[v][r + 1][cc][p], cor[2][q], o);
-      if (!GLL || q == 0) o = fma(syp[v][r][cc][p], cor[3][q], o);
-      out[v][p] = o;
+      W[v][p] = L.w[(v * Ne + ge) * nn + q * n + p];
+      mag[v > 0] = max(mag[v > 0], fx_mag(W[v][p]));
     }
+  long long O[3][n];
+  int eo[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    // largest magnitude over the n rows of the element
+    int m = mag[k];
+    if constexpr ((n & (n - 1)) == 0) {
+#pragma unroll
+      for (int o = 1; o < n; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    } else {
+#pragma unroll
+      for (int j = 1; j < n; ++j) {
+        const int src = c * n + ((q + j) % n);
+        m = max(m, __shfl_sync(0xffffffffu, mag[k], src < 32 ? src : lane));
+      }
+    }
+    const int et = fx_exp(emag[k][r][cc]) + cor_e - 1021;   // of the corrections' sums
+    const int e = max(fx_exp(m), et), sh = e - et;
+    eo[k] = e;
+#pragma unroll
+    for (int v = k; v < 1 + 2 * k; ++v) {
+      const Fx tr = fx_at(&sxm[v][r][cc + 1][q]), tl = fx_at(&sxp[v][r][cc][q]);
+      const Fx c2 = cor[2][q], c3 = cor[3][q];
+#pragma unroll
+      for (int p = 0; p < n; ++p) {
+        // (GLL: corrections at the end nodes only; in y by zero coefficients)
+        FxAcc a;
+        fx_mul(a, fx_at(&sym[v][r + 1][cc][p]), c2.hi, c2.lo);
+        fx_mad(a, fx_at(&syp[v][r][cc][p]), c3.hi, c3.lo);
+        if (!GLL || p == N) fx_mad(a, tr, cor[0][p].hi, cor[0][p].lo);
+        if (!GLL || p == 0) fx_mad(a, tl, cor[1][p].hi, cor[1][p].lo);
+        O[v][p] = fx_from<FB>(W[v][p], e) + fx_sar(fx_sum(a), sh);
+        out[v][p] = fx_to(O[v][p], e + 63 - FB, fx_zero(e));
+      }
+    }
+  }
   if constexpr (LIMIT) {
     // first-order subcell update: the local kernel's part plus the
     // element-face fluxes of the face nodes (Eq. low.order.update), the
@@ -385,30 +478,56 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
     // element means (Definition admissibility.preserving.means), then
     // sigma_x/dx + sigma_y/dy (Sec. 5, Eq. time.step.2d)
     double m[3];
+    if constexpr (LIMIT) {
 #pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      double s = T.w2[q][0] * out[v][0];
+      for (int v = 0; v < 3; ++v) {
+        double s = T.w2[q][0] * out[v][0];
 #pragma unroll
-      for (int p = 1; p < n; ++p) s = fma(T.w2[q][p], out[v][p], s);
-      m[v] = s;
-    }
-    // sum over the n rows of the element (lanes c*n .. c*n+n-1): a butterfly
-    // when n is a power of two (every lane ends with the same sum), else the
-    // rows in order
-#pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      double s = m[v];
-      if constexpr ((n & (n - 1)) == 0) {
-#pragma unroll
-        for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      } else {
-#pragma unroll
-        for (int k = 1; k < n; ++k) {
-          const int src = c * n + ((q + k) % n);
-          s += __shfl_sync(0xffffffffu, m[v], src < 32 ? src : lane);
-        }
+        for (int p = 1; p < n; ++p) s = fma(T.w2[q][p], out[v][p], s);
+        m[v] = s;
       }
-      m[v] = s;
+      // sum over the n rows of the element (lanes c*n .. c*n+n-1): a butterfly
+      // when n is a power of two (every lane ends with the same sum), else the
+      // rows in order
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        double s = m[v];
+        if constexpr ((n & (n - 1)) == 0) {
+#pragma unroll
+          for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        } else {
+#pragma unroll
+          for (int k = 1; k < n; ++k) {
+            const int src = c * n + ((q + k) % n);
+            s += __shfl_sync(0xffffffffu, m[v], src < 32 ? src : lane);
+          }
+        }
+        m[v] = s;
+      }
+    } else {
+      // in the fixed point of the update: the row with its weights, then the
+      // rows of the element (integer sums: any order)
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        FxAcc a;
+        fx_mul(a, fx_split(O[v][0]), T.fx.w2_hi[q][0], T.fx.w2_lo[q][0]);
+#pragma unroll
+        for (int p = 1; p < n; ++p)
+          fx_mad(a, fx_split(O[v][p]), T.fx.w2_hi[q][p], T.fx.w2_lo[q][p]);
+        const long long row = fx_sum(a);
+        long long s = row;
+        if constexpr ((n & (n - 1)) == 0) {
+#pragma unroll
+          for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        } else {
+#pragma unroll
+          for (int k = 1; k < n; ++k) {
+            const int src = c * n + ((q + k) % n);
+            s += __shfl_sync(0xffffffffu, row, src < 32 ? src : lane);
+          }
+        }
+        m[v] = fx_to(s, eo[v > 0] + 63 - FB, fx_zero(eo[v > 0]));
+      }
     }
     // the rates: one element per thread of the first TY * TX threads, so that
     // a warp computes 32 of them (from the n lanes of an element only one

@@ -452,15 +452,15 @@ typedef enum {
 } crkfr_limiter;
 crkfr_status crkfr_set_limiter(crkfr_ctx* ctx, int32_t mode, double alpha);
 
-/* Threads per block of the fused 1D step kernel, which gives each element one
- * thread and each block threads - 2 elements between two recomputed
- * neighbours.  0 (the default): chosen per mesh among 64, 96 and 128 so that
- * the busiest SM gets the fewest threads; 64, 96 or 128: that size for every
- * step.  Only the schedule changes, not a bit of the results.  Applies to the
- * unlimited step of 1D contexts (crkfr_step, crkfr_advance, crkfr_step_host,
- * crkfr_step_local); the limited step and crkfr_residual run 128-thread
- * blocks.  CRKFR_ERR_UNSUPPORTED on a 2D context, CRKFR_ERR_ARG for other
- * values; kept across crkfr_set_mesh. */
+/* Threads per block of the fused 1D step kernel, which gives each node one
+ * thread (elements within a warp) and each block all its elements but two
+ * recomputed neighbours.  0 (the default): chosen per mesh among 32, 64, 128
+ * and 256 so that the busiest SM sub-partition gets the fewest warps; 64, 96
+ * or 128: that size for every step.  Only the schedule changes, not a bit of
+ * the results.  Applies to the unlimited step of 1D contexts (crkfr_step,
+ * crkfr_advance, crkfr_step_host, crkfr_step_local); the limited step runs
+ * 128-thread and crkfr_residual 256-thread blocks.  CRKFR_ERR_UNSUPPORTED on a
+ * 2D context, CRKFR_ERR_ARG for other values; kept across crkfr_set_mesh. */
 crkfr_status crkfr_set_tile_1d(crkfr_ctx* ctx, int32_t threads);
 crkfr_status crkfr_limiter_alpha(crkfr_ctx* ctx, double* alpha_dev, void* stream);
 
@@ -577,7 +577,7 @@ crkfr_status crkfr_step_1d_noalloc(const crkfr_config* cfg, int64_t n_elem, doub
  * C_s for all; per instance its own degree, element count, interval,
  * coefficient field and, with the CFL step, its own time step).  A step of
  * the whole ensemble is one kernel launch per degree class over a work list
- * of (instance, 126-element tile) pairs running the same fused step as
+ * of (instance, tile of elements) pairs running the same fused step as
  * crkfr_step (Sec. 3, Eq. crkfr.non.cons.final; Sec. 5, Eq. time.step.2d per
  * instance), so instances of any size share the GPU.  The batching itself
  * has no counterpart in the paper.

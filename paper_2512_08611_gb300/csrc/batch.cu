@@ -377,7 +377,8 @@ crkfr_status crkfr_batch_create(crkfr_batch** out, const crkfr_config* cfg, int3
     b->n_state += b->M * n_elem[i] * nn;
     b->n_coef += n_elem[i] * nn;
     b->n_sface += 2 * n_elem[i];
-    const int64_t tiles = (n_elem[i] + kTile1D - 1) / kTile1D;
+    const int64_t own = tile_elements_1d(kMaxBlock1D, (int)nn);
+    const int64_t tiles = (n_elem[i] + own - 1) / own;
     if (tiles > 0x7fffffff) {
       delete b;
       return CRKFR_ERR_ARG;

@@ -139,6 +139,14 @@ double von_neumann_cfl(const HostBasis& b, bool imex);
 void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool imex,
                  double src_coef, Tables* T);
 
+// Largest block of the 1D step, and the elements a block of `threads` threads
+// owns: n threads per element within its warps, less two halo elements.
+constexpr int kMaxBlock1D = 256;
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int tile_elements_1d(int threads, int n) { return threads / 32 * (32 / n) - 2; }
+
 // Launchers (kernels_1d.cu / kernels_2d.cu).  Return cudaError_t as int.
 struct Launch1D {
   int system;  // crkfr_system
@@ -162,8 +170,8 @@ struct Launch1D {
   // exchanged every step: ghost_dyn_1d(M, n) doubles), then the static node
   // terms [n], the face traces of c [2] and the nodal c [n] (null: periodic)
   const double* ghost;
-  // threads per block of the unlimited step: 0 = chosen per mesh, else 64,
-  // 96 or 128
+  // threads per block of the unlimited step (at most kMaxBlock1D): 0 = chosen
+  // per mesh, else 64, 96 or 128
   int tile_threads;
 };
 #ifdef __CUDACC__
@@ -215,7 +223,6 @@ struct LaunchBatch1D {
 int launch_step_1d_batch(const LaunchBatch1D& B, void* stream);
 int launch_step_1d_batch_imex(const LaunchBatch1D& B, void* stream);   // kernels_imex.cu
 int launch_rate_1d_batch(const LaunchBatch1D& B, int slot, void* stream);
-constexpr int kTile1D = 126;   // elements a 1D block owns (128 threads, 2 halo)
 
 // Subcell blending limiter of a 2D step (kernels_limit2d.cu).
 struct LimitArgs2D {

@@ -142,6 +142,14 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
   return __longlong_as_double(ia > ib ? ia : ib);
 }
 
+// max of the bit patterns: of non-negative values their maximum, and any NaN
+// (of either sign) wins
+__device__ __forceinline__ double max_bits(double a, double b) {
+  const unsigned long long ia = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long ib = (unsigned long long)__double_as_longlong(b);
+  return __longlong_as_double((long long)(ia > ib ? ia : ib));
+}
+
 // true if x > 0 and finite (integer test on the bit pattern)
 __device__ __forceinline__ bool positive_finite(double x) {
   const long long ix = __double_as_longlong(x);
@@ -180,6 +188,19 @@ __device__ __forceinline__ double theta_lin(double eps, double Pa, double Pb) {
   if (!(Pb < eps)) return 1.0;
   const double den = Pb - Pa;
   return den != 0.0 ? fmin(1.0, fabs((eps - Pa) / den)) : 1.0;
+}
+
+// Max of a non-negative double over the warps that hold one above zero, then
+// one atomicMax on the bit pattern per such warp.
+__device__ __forceinline__ void block_max_atomic_1d(double v, unsigned long long* slot) {
+  unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  if (!__any_sync(0xffffffffu, b != 0)) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    unsigned long long other = __shfl_xor_sync(0xffffffffu, b, o);
+    b = other > b ? other : b;
+  }
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, b);
 }
 
 // Block-wide max of a non-negative double, then one atomicMax on the bit

@@ -101,6 +101,42 @@ __device__ __forceinline__ double fx_to(long long R, int eb, int zero) {
   return __hiloint2double(ex == 0 ? zero : hi, (int)(unsigned)(a >> 10));
 }
 
+// Weighted sums of operands: with weights up to 6 in all one 64-bit sum A holds
+// them; WIDE (up to 90) keeps the halves' sums apart, A 2^30 + B.
+template <bool WIDE>
+__device__ __forceinline__ void fx_accumulate(long long& A, long long& B, long long v, Fx x,
+                                              int w) {
+  if (WIDE) {
+    A += (long long)x.hi * w;
+    B += (long long)x.lo * w;
+  } else {
+    A += w * v;
+  }
+}
+
+// the sum in units 2^sh larger
+template <bool WIDE>
+__device__ __forceinline__ void fx_rescale(long long& A, long long& B, int sh) {
+  if (WIDE) {
+    // (the low half takes what the high one loses; from 62 on the sum is below
+    // 2^-55 of the new scale)
+    const long long hi = A >> (sh & 63), lost = A - (hi << (sh & 63));
+    const long long low = (B >> (sh & 63)) +
+                          (sh < 30 ? (lost << 30) >> (sh & 63) : lost >> ((sh - 30) & 63));
+    A = sh < 62 ? hi : 0;
+    B = sh < 62 ? low : 0;
+  } else {
+    A = fx_sar(A, sh);
+  }
+}
+
+// the sum shifted back to operand size
+template <bool WIDE, int SHIFT>
+__device__ __forceinline__ long long fx_average(long long A, long long B) {
+  if (!WIDE) return A >> SHIFT;
+  return ((A + (B >> 30)) << (30 - SHIFT)) + (((int)B & 0x3fffffff) >> SHIFT);
+}
+
 // a row of n operands in shared memory (16-byte aligned for even n)
 template <int n>
 __device__ __forceinline__ void fx_row(const Fx* x, Fx (&r)[n]) {

@@ -9,13 +9,15 @@
 namespace crkfr {
 namespace {
 
+constexpr int kBlockRate = 128;
+
 // max_e sigma(ubar_e)/dx of a state into one rate slot (Sec. 5, Eq. time.step.2d)
 template <int SYS, int N>
-__global__ void __launch_bounds__(kBlock1D) k_rate_1d(const Launch1D L, int slot) {
+__global__ void __launch_bounds__(kBlockRate) k_rate_1d(const Launch1D L, int slot) {
   constexpr int n = N + 1;
   constexpr bool SWE = (SYS == CRKFR_SYS_SWE_1D);
   const Tables& T = L.tab;
-  const int64_t e = (int64_t)blockIdx.x * kBlock1D + threadIdx.x;
+  const int64_t e = (int64_t)blockIdx.x * kBlockRate + threadIdx.x;
   double rate = 0.0;
   if (e < L.E) {
     if constexpr (SWE) {
@@ -33,7 +35,7 @@ __global__ void __launch_bounds__(kBlock1D) k_rate_1d(const Launch1D L, int slot
       rate = fabs(ab) * L.xs;
     }
   }
-  block_max_atomic<kBlock1D>(rate, &L.st->rate[slot]);
+  block_max_atomic<kBlockRate>(rate, &L.st->rate[slot]);
 }
 
 // Static coefficient terms: per node the factor of the local non-conservative
@@ -72,16 +74,17 @@ __global__ void k_coef_1d(int64_t E, const double* __restrict__ c, double* __res
 // ---- ragged ensembles -----------------------------------------------------
 // rate of each instance's state (the owned elements of each tile)
 template <int SYS, int N>
-__global__ void __launch_bounds__(kBlock1D) k_rate_1d_batch(const LaunchBatch1D B, int slot) {
+__global__ void __launch_bounds__(kBlockRate) k_rate_1d_batch(const LaunchBatch1D B, int slot) {
   constexpr int n = N + 1;
   const WorkItem w = B.work[blockIdx.x];
   const BatchInstance I = B.inst[w.inst];
   const Tables& T = B.tab;
-  const int t = threadIdx.x;
-  const int64_t e = (int64_t)w.tile * (kBlock1D - 2) + t - 1;
+  constexpr int own = tile_elements_1d(kBlock1D, n);
+  const double* u = B.u_in + I.u_off;
   double rate = 0.0;
-  if (t >= 1 && t <= kBlock1D - 2 && e < I.E) {
-    const double* u = B.u_in + I.u_off;
+  for (int k = threadIdx.x; k < own; k += kBlockRate) {
+    const int64_t e = (int64_t)w.tile * own + k;
+    if (e >= I.E) break;
     if constexpr (SYS == CRKFR_SYS_SWE_1D) {
       double hb = 0.0, mb = 0.0;
 #pragma unroll
@@ -89,15 +92,15 @@ __global__ void __launch_bounds__(kBlock1D) k_rate_1d_batch(const LaunchBatch1D 
         hb = fma(T.w[p], u[e * n + p], hb);
         mb = fma(T.w[p], u[(I.E + e) * n + p], mb);
       }
-      rate = swe_speed(hb, mb, T.sqrt_gravity) * I.xs;
+      rate = max_bits(rate, swe_speed(hb, mb, T.sqrt_gravity) * I.xs);
     } else {
       double ab = 0.0;
 #pragma unroll
       for (int p = 0; p < n; ++p) ab = fma(T.w[p], B.snode[I.sn_off + e * n + p], ab);
-      rate = fabs(ab) * I.xs;
+      rate = max_bits(rate, fabs(ab) * I.xs);
     }
   }
-  block_max_atomic<kBlock1D>(rate, &I.st->rate[slot]);
+  block_max_atomic<kBlockRate>(rate, &I.st->rate[slot]);
 }
 
 template <int SYS>
@@ -105,11 +108,11 @@ int launch_batch_rate_sys(const LaunchBatch1D& B, int slot, cudaStream_t s) {
   if (B.nwork <= 0) return 0;
   const unsigned blocks = (unsigned)B.nwork;
   switch (B.N) {
-    case 0: k_rate_1d_batch<SYS, 0><<<blocks, kBlock1D, 0, s>>>(B, slot); break;
-    case 1: k_rate_1d_batch<SYS, 1><<<blocks, kBlock1D, 0, s>>>(B, slot); break;
-    case 2: k_rate_1d_batch<SYS, 2><<<blocks, kBlock1D, 0, s>>>(B, slot); break;
-    case 3: k_rate_1d_batch<SYS, 3><<<blocks, kBlock1D, 0, s>>>(B, slot); break;
-    case 4: k_rate_1d_batch<SYS, 4><<<blocks, kBlock1D, 0, s>>>(B, slot); break;
+    case 0: k_rate_1d_batch<SYS, 0><<<blocks, kBlockRate, 0, s>>>(B, slot); break;
+    case 1: k_rate_1d_batch<SYS, 1><<<blocks, kBlockRate, 0, s>>>(B, slot); break;
+    case 2: k_rate_1d_batch<SYS, 2><<<blocks, kBlockRate, 0, s>>>(B, slot); break;
+    case 3: k_rate_1d_batch<SYS, 3><<<blocks, kBlockRate, 0, s>>>(B, slot); break;
+    case 4: k_rate_1d_batch<SYS, 4><<<blocks, kBlockRate, 0, s>>>(B, slot); break;
     default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();
@@ -117,13 +120,13 @@ int launch_batch_rate_sys(const LaunchBatch1D& B, int slot, cudaStream_t s) {
 
 template <int SYS>
 int launch_rate_sys(const Launch1D& L, int slot, cudaStream_t s) {
-  const unsigned blocks = (unsigned)((L.E + kBlock1D - 1) / kBlock1D);
+  const unsigned blocks = (unsigned)((L.E + kBlockRate - 1) / kBlockRate);
   switch (L.N) {
-    case 0: k_rate_1d<SYS, 0><<<blocks, kBlock1D, 0, s>>>(L, slot); break;
-    case 1: k_rate_1d<SYS, 1><<<blocks, kBlock1D, 0, s>>>(L, slot); break;
-    case 2: k_rate_1d<SYS, 2><<<blocks, kBlock1D, 0, s>>>(L, slot); break;
-    case 3: k_rate_1d<SYS, 3><<<blocks, kBlock1D, 0, s>>>(L, slot); break;
-    case 4: k_rate_1d<SYS, 4><<<blocks, kBlock1D, 0, s>>>(L, slot); break;
+    case 0: k_rate_1d<SYS, 0><<<blocks, kBlockRate, 0, s>>>(L, slot); break;
+    case 1: k_rate_1d<SYS, 1><<<blocks, kBlockRate, 0, s>>>(L, slot); break;
+    case 2: k_rate_1d<SYS, 2><<<blocks, kBlockRate, 0, s>>>(L, slot); break;
+    case 3: k_rate_1d<SYS, 3><<<blocks, kBlockRate, 0, s>>>(L, slot); break;
+    case 4: k_rate_1d<SYS, 4><<<blocks, kBlockRate, 0, s>>>(L, slot); break;
     default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();

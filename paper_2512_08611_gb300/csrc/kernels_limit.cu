@@ -17,12 +17,14 @@
 namespace crkfr {
 namespace {
 
+constexpr int kBlockAlpha = 128;
+
 template <int N>
-__global__ void __launch_bounds__(kBlock1D) k_alpha_1d(int64_t E, const double* __restrict__ u,
+__global__ void __launch_bounds__(kBlockAlpha) k_alpha_1d(int64_t E, const double* __restrict__ u,
                                                        const Tables T,
                                                        double* __restrict__ alpha_raw) {
   constexpr int n = N + 1;
-  const int64_t e = (int64_t)blockIdx.x * kBlock1D + threadIdx.x;
+  const int64_t e = (int64_t)blockIdx.x * kBlockAlpha + threadIdx.x;
   if (e >= E) return;
   double x[n];
 #pragma unroll
@@ -65,8 +67,9 @@ __global__ void __launch_bounds__(kBlock1D) k_alpha_1d(int64_t E, const double* 
 
 template <int SYS, int N, bool GLL, bool IMEX>
 int launch_limit_t(const Launch1D& L, cudaStream_t s) {
-  const int64_t blocks = (L.E + kBlock1D - 3) / (kBlock1D - 2);
-  k_step_1d<SYS, N, GLL, false, IMEX, true><<<(unsigned)blocks, kBlock1D, 0, s>>>(L);
+  const unsigned blocks = tiles_1d(L.E, kBlockLimit1D, N + 1);
+  if (!blocks) return (int)cudaErrorInvalidConfiguration;
+  k_step_1d<SYS, N, GLL, false, IMEX, true><<<blocks, kBlockLimit1D, 0, s>>>(L);
   return (int)cudaGetLastError();
 }
 
@@ -104,12 +107,12 @@ int launch_step_1d_limit(const Launch1D& L, void* stream) {
 
 int launch_alpha_1d(const Launch1D& L, double* alpha_raw, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  const unsigned blocks = (unsigned)((L.E + kBlock1D - 1) / kBlock1D);
+  const unsigned blocks = (unsigned)((L.E + kBlockAlpha - 1) / kBlockAlpha);
   switch (L.N) {
-    case 1: k_alpha_1d<1><<<blocks, kBlock1D, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
-    case 2: k_alpha_1d<2><<<blocks, kBlock1D, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
-    case 3: k_alpha_1d<3><<<blocks, kBlock1D, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
-    case 4: k_alpha_1d<4><<<blocks, kBlock1D, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
+    case 1: k_alpha_1d<1><<<blocks, kBlockAlpha, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
+    case 2: k_alpha_1d<2><<<blocks, kBlockAlpha, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
+    case 3: k_alpha_1d<3><<<blocks, kBlockAlpha, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
+    case 4: k_alpha_1d<4><<<blocks, kBlockAlpha, 0, s>>>(L.E, L.u_in, L.tab, alpha_raw); break;
     default: return (int)cudaErrorInvalidValue;
   }
   return (int)cudaGetLastError();

@@ -164,7 +164,6 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
   // time averages sum_j (b_j/b_ref) of the exchange fields 0..5 in the fixed
   // point of the exponents E (h; hu, hv; the fluxes), which only grow: the
   // sums are shifted when they do
-  // (WIDE: A 2^30 + B)
   long long A[6] = {0, 0, 0, 0, 0, 0}, B[6] = {0, 0, 0, 0, 0, 0};
   int E[3] = {-1, -1, -1};
   auto group_of = [](int f) { return f == 0 ? 0 : f < 3 ? 1 : 2; };
@@ -284,20 +283,7 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
         }
         if (!first) {
 #pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const int sh = d[group_of(k)];
-            if (WIDE) {
-              // (the low half takes what the high one loses; from 62 on the
-              // sum is below 2^-55 of the new scale)
-              const long long hi = A[k] >> (sh & 63), lost = A[k] - (hi << (sh & 63));
-              const long long low = (B[k] >> (sh & 63)) +
-                                    (sh < 30 ? (lost << 30) >> (sh & 63) : lost >> ((sh - 30) & 63));
-              A[k] = sh < 62 ? hi : 0;
-              B[k] = sh < 62 ? low : 0;
-            } else {
-              A[k] = fx_sar(A[k], sh);
-            }
-          }
+          for (int k = 0; k < 6; ++k) fx_rescale<WIDE>(A[k], B[k], d[group_of(k)]);
         }
       }
 #pragma unroll
@@ -305,14 +291,7 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
         const bool used = need_op && !(k == 0 && !WB) || WB && (k == 0);
         const long long v = fx_from<FB>(f[k], E[group_of(k)]);
         const Fx x = fx_split(v);
-        if (wi != 0) {
-          if (WIDE) {
-            A[k] += (long long)x.hi * wi;
-            B[k] += (long long)x.lo * wi;
-          } else {
-            A[k] += wi * v;
-          }
-        }
+        if (wi != 0) fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
         if (used && lane_ok) X[k][q][p] = x;
       }
       if (need_op || WB) {
@@ -367,16 +346,8 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
   // f_j), Bloc = g b_x (sum_j b_j h_j) (the well-balanced product is
   // accumulated stage by stage).  A, P and Sb hold time averages divided by
   // b_ref; the sums are scaled back to FB bits for the contractions.
-  if (WIDE) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      A[k] += B[k] >> 30;
-      A[k] = (A[k] << (30 - kSumShift)) + (((int)B[k] & 0x3fffffff) >> kSumShift);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) A[k] >>= kSumShift;
-  }
+  for (int k = 0; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
   sync();
   if (lane_ok) {
 #pragma unroll

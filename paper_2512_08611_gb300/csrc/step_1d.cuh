@@ -2,24 +2,27 @@
 // single-mesh kernel, the ragged-ensemble kernel and their source-term (IMEX)
 // instantiations, which live in different translation units.
 //
-// Mapping: one thread owns one element and keeps its N+1 nodes of every
-// variable, all inner stages and all time averages in registers (Sec. 3,
-// Eq. crkfr.non.cons.final, inner stages; Eqs. disc.avg.flux,
-// time.avg.soln, local.time.avg.non.cons).  A block of B threads updates
-// B - 2 consecutive elements (B = 128, or 64 or 96 where those tiles spread
-// more evenly over the SMs); its first and last threads recompute the stages
-// of the two neighbouring elements (2 of 128 threads, 1.6% extra FP64) so
-// that the only inter-element coupling, one Riemann problem per face
-// (Eqs. numflux.cons, combined.wave.speed, good.numflux.non.cons,
-// total.F.non.cons), is solved from face traces exchanged through shared
-// memory, and u is read and written once per step.  The step therefore
-// reads u^n from one buffer and writes u^{n+1} to another.
+// Mapping: one thread owns one node; an element's N+1 threads lie in one warp
+// and exchange the fluxes of a stage through shared memory (Sec. 3,
+// Eq. crkfr.non.cons.final, inner stages; Eqs. disc.avg.flux, time.avg.soln,
+// local.time.avg.non.cons).  The pointwise arithmetic is FP64; the products
+// with D and the end-point rows and the time averages run in block fixed point
+// on the integer pipe (fixed_point.cuh), and D is applied to the averages once
+// instead of accumulating every stage's operator.  A block updates all its
+// elements but the first and the last, whose stages it recomputes for their
+// neighbours (4 % of a 256-thread block at N = 4), so that the only
+// inter-element coupling, one Riemann problem per face (Eqs. numflux.cons,
+// combined.wave.speed, good.numflux.non.cons, total.F.non.cons), is solved
+// from face traces exchanged through shared memory, and u is read and written
+// once per step.  The step therefore reads u^n from one buffer and writes
+// u^{n+1} to another.  Face terms and the next time step's rates are one
+// thread per element, packed into the block's first warps (an FP64
+// instruction costs the same for one lane as for 32).
 //
 // Face terms are carried doubled, T' = 2 (F^num,+- - F^tot,+-), and the
 // correction tables hold 0.5 g'(xi_p)/dx, which saves two FP64 multiplies
 // per face.  For GLL nodes the traces are the end values and g_L', g_R'
-// vanish away from the end nodes (App. B, under Eq. fr.gll), which the
-// GLL instantiation uses at compile time.
+// vanish away from the end nodes (App. B, under Eq. fr.gll).
 //
 // With a source term (IMEX = true; Sec. 2, Eqs. crkfr.inner, crkfr,
 // avg.source) the stages follow SSP3-IMEX(4,3,3): the implicit source terms
@@ -46,46 +49,32 @@
 #include <cuda_runtime.h>
 
 #include "device_common.cuh"
+#include "fixed_point.cuh"
 
 namespace crkfr {
 namespace {
 
-constexpr int kBlock1D = 128;
+constexpr int kBlock1D = kMaxBlock1D;   // of the residual and the ensemble steps
+constexpr int kBlockLimit1D = 128;      // of the limited step (its shared memory)
 
 template <int SYS>
 struct Sys1D;
 template <>
 struct Sys1D<CRKFR_SYS_VARADV_1D> {
   static constexpr int M = 1;
-  static constexpr int NLEFT = 2;   // left-trace fields exchanged: V, a
+  static constexpr int K = 1;       // exchange fields of a stage: v
+  static constexpr int NT = 1;      // traces from nodal values: V (and then a)
   static constexpr int SV = 0;      // variable carrying the source (v)
 };
 template <>
 struct Sys1D<CRKFR_SYS_SWE_1D> {
   static constexpr int M = 2;
-  static constexpr int NLEFT = 6;   // H, M (time averages), F_m, h^n, m^n, b
+  static constexpr int K = 3;       // h, hu, the momentum flux
+  static constexpr int NT = 5;      // H, M (time averages), F_m, h^n, m^n (and then b)
   static constexpr int SV = 1;      // variable carrying the source (hu)
 };
 template <>
 struct Sys1D<CRKFR_SYS_SWE_1D_WB> : Sys1D<CRKFR_SYS_SWE_1D> {};
-
-template <int N, bool GLL>
-__device__ __forceinline__ double trace_r(const Tables& T, const double* X) {
-  if (GLL) return X[N];
-  double s = T.l1[0] * X[0];
-#pragma unroll
-  for (int p = 1; p <= N; ++p) s = fma(T.l1[p], X[p], s);
-  return s;
-}
-
-template <int N, bool GLL>
-__device__ __forceinline__ double trace_l(const Tables& T, const double* X) {
-  if (GLL) return X[0];
-  double s = T.l0[0] * X[0];
-#pragma unroll
-  for (int p = 1; p <= N; ++p) s = fma(T.l0[p], X[p], s);
-  return s;
-}
 
 // First-order non-conservative Rusanov fluxes (Eq. combined.num.flux) between
 // the nodal states L and R: fm = f^num + B(w_L) w^num, fp = f^num + B(w_R) w^num,
@@ -162,13 +151,25 @@ __device__ __forceinline__ void lo_source(const Tables& T, double dt, double* u)
   }
 }
 
-// One tile (BLOCK - 2 elements plus a halo element on each side) of the fused
-// 1D step of one mesh.  T holds reference-element tables (dx = 1: D, l(0),
-// l(1), 0.5 g'); xs = 1/dx scales the local operator and the corrections
-// through the scalar coefficients only (stage coefficients dt a_ij xs, update
-// coefficient dt b_ref xs), so one table serves meshes of any dx.  Every
-// element's arithmetic is the same for any BLOCK.
-template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false, int BLOCK = kBlock1D>
+// Minimum over the n lanes of an element.
+template <int n>
+__device__ __forceinline__ double element_min(double v, int le, int p, int lane) {
+  double m = v;
+#pragma unroll
+  for (int k = 1; k < n; ++k) {
+    const int r = p + k < n ? p + k : p + k - n, src = le * n + r;
+    m = fmin(m, __shfl_sync(0xffffffffu, v, src < 32 ? src : lane));
+  }
+  return m;
+}
+
+// One tile (tile_elements_1d(blockDim.x, n) elements plus a halo element on
+// each side) of the fused 1D step of one mesh.  T holds reference-element
+// tables (dx = 1: D, l(0), l(1), 0.5 g'); xs = 1/dx scales the local operator
+// and the corrections through the scalar coefficients only (stage coefficients
+// dt a_ij xs, update coefficient dt b_ref xs), so one table serves meshes of
+// any dx.  Every element's arithmetic is the same for any block size.
+template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
 __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
                                              const double* __restrict__ u_in,
                                              double* __restrict__ u_out,
@@ -178,76 +179,85 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
                                              bool first_tile, const LimitArgs& LA = LimitArgs{},
                                              const double* __restrict__ ghost = nullptr) {
   using TB = Tab<N, IMEX>;
+  using SY = Sys1D<SYS>;
   constexpr int n = N + 1;
-  constexpr int M = Sys1D<SYS>::M;
-  constexpr int NL = Sys1D<SYS>::NLEFT;
-  constexpr int SV = Sys1D<SYS>::SV;
+  constexpr int M = SY::M, K = SY::K, NT = SY::NT, SV = SY::SV;
   constexpr int S = TB::S;
-  constexpr int F0 = TB::first();
   constexpr bool SWE = (SYS == CRKFR_SYS_SWE_1D || SYS == CRKFR_SYS_SWE_1D_WB);
   constexpr bool WB = (SYS == CRKFR_SYS_SWE_1D_WB);
-  const int t = threadIdx.x;
-  const int64_t e_raw = tile * (BLOCK - 2) + t - 1;
+  constexpr int EPW = 32 / n;                       // elements per warp
+  constexpr int NE = (LIMIT ? kBlockLimit1D : kMaxBlock1D) / 32 * EPW;   // of the largest block
+  constexpr int KX = SWE ? 5 : 1;                   // exchange fields per node
+  // fixed point: operand bits, shift of the weighted sums back to them, and
+  // the bits a later stage may outgrow the first (as in local_2d.cuh)
+  constexpr int FB = 59;
+  constexpr bool WIDE = TB::weight_sum() > 8;
+  constexpr int kSumShift = WIDE ? 7 : 3;
+  constexpr int kHeadroom = 1;
+
+  const int t = threadIdx.x, lane = t & 31;
+  const int le = lane / n, p = lane - le * n;
+  const bool lane_ok = le < EPW;
+  const int ne = (int)(blockDim.x >> 5) * EPW;      // elements of this block
+  const int slot = (t >> 5) * EPW + (lane_ok ? le : 0);
+  const int64_t e_raw = tile * (ne - 2) + slot - 1;
   int64_t e = e_raw % E;
   if (e < 0) e += E;
-  const bool owner = (t >= 1) && (t <= BLOCK - 2) && (e_raw < E);
+  const bool owner = lane_ok && slot >= 1 && slot <= ne - 2 && e_raw < E;
 
-  __shared__ double sm_left[NL][BLOCK];
-  __shared__ double sm_T[M][BLOCK];
+  __shared__ __align__(16) Fx sx[NE][KX][n];
+  __shared__ double str[2][NT + 1][NE];             // traces at the left / right end
+  __shared__ double sT[2][M][NE];                   // face terms: right face, left face
+  __shared__ int smag[NE][K];
+  __shared__ double sdt[2];
+  Fx (*X)[n] = sx[slot];
 
-  const double dt = RES ? ctl.dt_fixed : step_dt(ctl, st);
-  if (!RES && first_tile && t == 0) step_bookkeeping(ctl, st, dt);
-  const double dtx = dt * xs;
+  if (t == 0) {
+    // the step size (a division) by one thread of the block
+    const double dt = RES ? ctl.dt_fixed : step_dt(ctl, st);
+    sdt[0] = dt;
+    sdt[1] = dt * xs;
+    if (!RES && first_tile) step_bookkeeping(ctl, st, dt);
+  }
+  for (int k = t; k < ne * K; k += blockDim.x) (&smag[0][0])[k] = 0;
 
-  // ---- load u^n and the static coefficient terms of this element ----------
+  // ---- u^n and the static coefficient terms of this node -------------------
   // (on a subdomain the elements beyond its ends are the neighbours' ghosts)
-  double u0[M][n];
-  double sn[n];
-  double c_l, c_r;
+  double u0[M], sn;
   const bool from_ghost = ghost != nullptr && (e_raw < 0 || e_raw >= E);
   constexpr int GD = ghost_dyn_1d(M, n);   // static part of a ghost after GD doubles
+  const double* gs = ghost + (e_raw < 0 ? 0 : ghost_stride_1d(M, n));
   if (from_ghost) {
-    const double* gs = ghost + (e_raw < 0 ? 0 : ghost_stride_1d(M, n));
 #pragma unroll
-    for (int v = 0; v < M; ++v)
-#pragma unroll
-      for (int p = 0; p < n; ++p) u0[v][p] = gs[v * n + p];
-#pragma unroll
-    for (int p = 0; p < n; ++p) sn[p] = gs[GD + p];
-    c_l = gs[GD + n];
-    c_r = gs[GD + n + 1];
+    for (int v = 0; v < M; ++v) u0[v] = gs[v * n + p];
+    sn = gs[GD + p];
   } else {
 #pragma unroll
-    for (int v = 0; v < M; ++v)
+    for (int v = 0; v < M; ++v) u0[v] = u_in[((int64_t)v * E + e) * n + p];
+    sn = snode[e * n + p];
+  }
+  if (lane_ok && p == 0) {
+    str[0][NT][slot] = from_ghost ? gs[GD + n] : sface[2 * e];
+    str[1][NT][slot] = from_ghost ? gs[GD + n + 1] : sface[2 * e + 1];
+  }
+  int dh[n], dl[n];                        // the node's row of D
 #pragma unroll
-      for (int p = 0; p < n; ++p) u0[v][p] = u_in[((int64_t)v * E + e) * n + p];
-#pragma unroll
-    for (int p = 0; p < n; ++p) sn[p] = snode[e * n + p];
-    c_l = sface[2 * e];
-    c_r = sface[2 * e + 1];
+  for (int j = 0; j < n; ++j) {
+    dh[j] = T.fx.Dx_hi[p][j];
+    dl[j] = T.fx.Dx_lo[p][j];
   }
 
   // ---- limiter: alpha_e, nodal c, first-order fluxes of the inner subfaces --
   static_assert(!LIMIT || (N >= 1 && !RES), "the limiter needs N >= 1 and a step");
-  constexpr int LM = LIMIT ? M : 1, LN = LIMIT ? N : 1, LB = LIMIT ? BLOCK : 1;
+  constexpr int LM = LIMIT ? M : 1, LE = LIMIT ? NE : 1, Ln = LIMIT ? n : 1;
   double alpha = 0.0;
-  double cn[n];
-  double fim[LM][LN];   // right flux of node p (B at node p)
-  double fip[LM][LN];   // left flux of node p+1 (B at node p+1)
-  __shared__ double sm_u0[LM][LB];
-  __shared__ double sm_fi0[LM][LB];
-  __shared__ double sm_c0[LB];
-  __shared__ double sm_al[LB];
-  __shared__ double sm_F[LM][LB];
+  __shared__ double lu[LM][LE][Ln], lc[LE][Ln], ls[LE][Ln], lf[LE][Ln];
+  __shared__ double lim[LM][LE][Ln];   // right flux of node p (B at node p), p < N
+  __shared__ double lip[LM][LE][Ln];   // left flux of node p+1 (B at node p+1)
+  __shared__ double lF[2][LM][LE];     // limited fluxes F^- of the right, F^+ of the left face
+  __shared__ double la[LE];
   if constexpr (LIMIT) {
-    if (from_ghost) {
-      const double* gs = ghost + (e_raw < 0 ? 0 : ghost_stride_1d(M, n));
-#pragma unroll
-      for (int p = 0; p < n; ++p) cn[p] = gs[GD + n + 2 + p];
-    } else {
-#pragma unroll
-      for (int p = 0; p < n; ++p) cn[p] = LA.cnode[e * n + p];
-    }
+    const double cn = from_ghost ? gs[GD + n + 2 + p] : LA.cnode[e * n + p];
     if (LA.mode == 2) {
       alpha = LA.alpha_fixed;
     } else if (ghost) {
@@ -268,184 +278,233 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       const double rn = fmax(LA.alpha_raw[em], LA.alpha_raw[ep]);
       alpha = fmax(r0, 0.5 * rn);
     }
-    // inner subfaces p | p+1 from per-node parts (shallow water: one
-    // reciprocal and one root per node instead of per subface side)
-    double sp[n], fp2[n];
-    if constexpr (SWE) {
+    if (lane_ok) {
 #pragma unroll
-      for (int p = 0; p < n; ++p) lo_node_1d<SYS>(u0[0][p], u0[1][p], T.gravity, sp[p], fp2[p]);
+      for (int v = 0; v < M; ++v) lu[v][slot][p] = u0[v];
+      lc[slot][p] = cn;
+      if (p == 0) la[slot] = alpha;
+      // per-node parts (shallow water: one reciprocal and one root per node
+      // instead of per subface side)
+      if constexpr (SWE) lo_node_1d<SYS>(u0[0], u0[1], T.gravity, ls[slot][p], lf[slot][p]);
     }
+    __syncwarp();
+    if (lane_ok && p < N) {
+      double b[M], fm_[M], fp_[M];
 #pragma unroll
-    for (int p = 0; p < LN; ++p) {
-      double a[M], b[M], fm_[M], fp_[M];
-#pragma unroll
-      for (int v = 0; v < M; ++v) {
-        a[v] = u0[v][p];
-        b[v] = u0[v][p + 1];
-      }
+      for (int v = 0; v < M; ++v) b[v] = lu[v][slot][p + 1];
       if constexpr (SWE)
-        lo_flux_nodes_1d<SYS>(a, b, cn[p], cn[p + 1], sp[p], sp[p + 1], fp2[p], fp2[p + 1],
-                              T.gravity, fm_, fp_);
+        lo_flux_nodes_1d<SYS>(u0, b, cn, lc[slot][p + 1], ls[slot][p], ls[slot][p + 1],
+                              lf[slot][p], lf[slot][p + 1], T.gravity, fm_, fp_);
       else
-        lo_flux<SYS>(a, b, cn[p], cn[p + 1], T, fm_, fp_);
+        lo_flux<SYS>(u0, b, cn, lc[slot][p + 1], T, fm_, fp_);
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        fim[v][p] = fm_[v];
-        fip[v][p] = fp_[v];
+        lim[v][slot][p] = fm_[v];
+        lip[v][slot][p] = fp_[v];
       }
     }
-#pragma unroll
-    for (int v = 0; v < M; ++v) {
-      sm_u0[v][t] = u0[v][0];
-      sm_fi0[v][t] = fim[v][0];
-    }
-    sm_c0[t] = cn[0];
-    sm_al[t] = alpha;
   }
+  __syncthreads();
+  const double dt = sdt[0], dtx = sdt[1];
 
   // ---- inner stages (element-local) ----------------------------------------
-  // Time averages are accumulated with the weights b_j / b_ref (the first
-  // weighted stage is a copy); b_ref is applied to dt in the update, and the
-  // fluctuation, the one face term that is not a time average, uses
-  // g / b_ref.
-  double Ls[S][M][n];            // local operator at each stage
-  double Ss[S][n];               // source of variable SV at each stage (IMEX)
-  double V[M][n];                // sum_j (b_j/b_ref) L_j
-  double U[M][n];                // sum_j (b_j/b_ref) u^(j)
-  double F2[n];                  // sum_j (b_j/b_ref) f_2(u^(j)) (shallow water momentum flux)
-  double Sb[n];                  // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
+  // Time averages are integer sums with the weights b_j / b_ref; b_ref is
+  // applied to dt in the update, and the fluctuation, the one face term that
+  // is not a time average, uses g / b_ref.
+  double Ls[S][M];                     // local operator at each stage
+  double Ss[S];                        // source of variable SV at each stage (IMEX)
+  double Sb = 0.0;                     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
+  double Pb = 0.0;                     // sum_j (b_j/b_ref) h g d(h + b) (WB)
+  long long A[K], B[K];                // sum_j (b_j/b_ref) of the exchange fields (WIDE: A 2^30 + B)
+  int Ex[K];                           // their exponents
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    A[k] = B[k] = 0;
+    Ex[k] = -1;
+  }
+  // row of D on an exchange field
+  auto contract = [&](int k) -> long long {
+    FxAcc a;
+    Fx r[n];
+    fx_row<n>(X[k], r);
+    fx_mul(a, r[0], dh[0], dl[0]);
+#pragma unroll
+    for (int j = 1; j < n; ++j) fx_mad(a, r[j], dh[j], dl[j]);
+    return fx_sum(a);
+  };
+  bool first = true;                   // (resolved at compile time by unrolling)
 #pragma unroll
   for (int i = 0; i < S; ++i) {
-    double cur[M][n];
+    double cur[M];
 #pragma unroll
-    for (int v = 0; v < M; ++v)
+    for (int v = 0; v < M; ++v) {
+      double acc = u0[v];
 #pragma unroll
-      for (int p = 0; p < n; ++p) {
-        double acc = u0[v][p];
+      for (int j = 0; j < i; ++j)
+        if (TB::a(i, j) != 0.0) acc = fma(-(dtx * TB::a(i, j)), Ls[j][v], acc);
+      if (IMEX && v == SV) {
 #pragma unroll
         for (int j = 0; j < i; ++j)
-          if (TB::a(i, j) != 0.0) acc = fma(-(dtx * TB::a(i, j)), Ls[j][v][p], acc);
-        if (IMEX && v == SV) {
-#pragma unroll
-          for (int j = 0; j < i; ++j)
-            if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j][p], acc);
-        }
-        cur[v][p] = acc;
+          if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j], acc);
       }
+      cur[v] = acc;
+    }
     if constexpr (IMEX) {
       // point-implicit source of this stage: cur - dt a_ii s(cur) = r
       const double gam = dt * TB::ai(i, i);
       if constexpr (SWE) {
         // s = -C_f |m| m / h^2 with h fixed: |m| + gam C_f |m|^2 / h^2 = |r|
         const double gcf = gam * T.src_coef;
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          const double ih = drcp(cur[0][p]);
-          const double ih2 = ih * ih;
-          if (TB::ai(i, i) != 0.0) {
-            const double r = cur[1][p];
-            const double q = dsqrt_pos(fma(4.0 * gcf * ih2, fabs(r), 1.0));
-            cur[1][p] = r * (2.0 * drcp(1.0 + q));
-          }
-          if (TB::need_S(i)) Ss[i][p] = -(T.src_coef * ih2) * fabs(cur[1][p]) * cur[1][p];
+        const double ih = drcp(cur[0]);
+        const double ih2 = ih * ih;
+        if (TB::ai(i, i) != 0.0) {
+          const double r = cur[1];
+          const double qf = dsqrt_pos(fma(4.0 * gcf * ih2, fabs(r), 1.0));
+          cur[1] = r * (2.0 * drcp(1.0 + qf));
         }
+        if (TB::need_S(i)) Ss[i] = -(T.src_coef * ih2) * fabs(cur[1]) * cur[1];
       } else {
         // s = -K v
-        const double inv = (TB::ai(i, i) != 0.0) ? drcp(fma(gam, T.src_coef, 1.0)) : 1.0;
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          if (TB::ai(i, i) != 0.0) cur[0][p] *= inv;
-          if (TB::need_S(i)) Ss[i][p] = -T.src_coef * cur[0][p];
-        }
+        if (TB::ai(i, i) != 0.0) cur[0] *= drcp(fma(gam, T.src_coef, 1.0));
+        if (TB::need_S(i)) Ss[i] = -T.src_coef * cur[0];
       }
     }
-    const double wi = TB::weight(i);
-    if (TB::need_L(i)) {
+    const int wi = TB::weight(i);
+    const double wd = wi;
+    const bool need_op = TB::feeds(i);
+    if (need_op || wi != 0) {
+      double f[K];
+      f[0] = cur[0];
       if constexpr (SWE) {
-        double f2[n];
+        const double vel = cur[1] * drcp(cur[0]);
+        f[1] = cur[1];
+        f[2] = WB ? cur[1] * vel : fma(cur[0] * cur[0], T.half_gravity, cur[1] * vel);
+      }
+      int mag[K];
+      bool over = false;
 #pragma unroll
-        for (int p = 0; p < n; ++p) {
-          const double h = cur[0][p], m = cur[1][p];
-          const double vel = m * drcp(h);
-          f2[p] = WB ? m * vel : fma(h * h, T.half_gravity, m * vel);
+      for (int k = 0; k < K; ++k) {
+        mag[k] = fx_mag(f[k]);
+        // (IMEX: the traces of u^n, no stage value here, share the exponents)
+        if (IMEX && first && k < M) mag[k] = max(mag[k], fx_mag(u0[k]));
+        over = over || (lane_ok && mag[k] >> 20 > Ex[k]);
+      }
+      // exponents as in local_2d.cuh; the vote is also the barrier after the
+      // last reads of X
+      if (__any_sync(0xffffffffu, over)) {
+        if (over) {
+#pragma unroll
+          for (int k = 0; k < K; ++k) atomicMax(&smag[slot][k], mag[k]);
         }
+        __syncwarp();
 #pragma unroll
-        for (int p = 0; p < n; ++p) {
-          double a0 = T.Dx[p][0] * cur[1][0];
-          double nc = sn[p];   // g D b, and for the well-balanced form + g D h
-          if (WB) {
-            double dh = T.Dx[p][0] * cur[0][0];
-#pragma unroll
-            for (int j = 1; j < n; ++j) dh = fma(T.Dx[p][j], cur[0][j], dh);
-            nc = fma(T.gravity, dh, nc);
-          }
-          double a1 = fma(cur[0][p], nc, T.Dx[p][0] * f2[0]);
-#pragma unroll
-          for (int j = 1; j < n; ++j) {
-            a0 = fma(T.Dx[p][j], cur[1][j], a0);
-            a1 = fma(T.Dx[p][j], f2[j], a1);
-          }
-          Ls[i][0][p] = a0;
-          Ls[i][1][p] = a1;
-        }
-        if (wi != 0.0) {
-#pragma unroll
-          for (int p = 0; p < n; ++p) F2[p] = (i == F0) ? wi * f2[p] : fma(wi, f2[p], F2[p]);
-        }
-      } else {
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          double a0 = T.Dx[p][0] * cur[0][0];
-#pragma unroll
-          for (int j = 1; j < n; ++j) a0 = fma(T.Dx[p][j], cur[0][j], a0);
-          Ls[i][0][p] = sn[p] * a0;
+        for (int k = 0; k < K; ++k) {
+          const int ek = fx_exp(smag[slot][k]);
+          const int d = ek > Ex[k] ? ek + kHeadroom - Ex[k] : 0;
+          Ex[k] += d;
+          if (!first) fx_rescale<WIDE>(A[k], B[k], d);
         }
       }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const long long v = fx_from<FB>(f[k], Ex[k]);
+        const Fx x = fx_split(v);
+        if (wi != 0) fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
+        // (h is contracted in the well-balanced form only)
+        if ((SWE && k == 0 ? WB : need_op) && lane_ok) X[k][p] = x;
+      }
+      if (need_op || WB) {
+        __syncwarp();
+        double nc = 0.0;
+        if constexpr (WB) {
+          nc = cur[0] * fma(T.gravity, fx_to(contract(0), Ex[0] + T.fx.kD - FB, fx_zero(Ex[0])), sn);
+          if (wi != 0) Pb = fma(wd, nc, Pb);
+        }
+        if (need_op) {
+          const int k0 = SWE ? 1 : 0;
+          const double l0 = fx_to(contract(k0), Ex[k0] + T.fx.kD - FB, fx_zero(Ex[k0]));
+          if constexpr (SWE) {
+            const double l1 = fx_to(contract(2), Ex[2] + T.fx.kD - FB, fx_zero(Ex[2]));
+            Ls[i][0] = l0;
+            Ls[i][1] = WB ? l1 + nc : fma(cur[0], sn, l1);
+          } else {
+            Ls[i][0] = sn * l0;
+          }
+        }
+      }
+      if (wi != 0) first = false;
     }
-    if (wi != 0.0) {
-#pragma unroll
-      for (int v = 0; v < M; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          V[v][p] = (i == F0) ? wi * Ls[i][v][p] : fma(wi, Ls[i][v][p], V[v][p]);
-          U[v][p] = (i == F0) ? wi * cur[v][p] : fma(wi, cur[v][p], U[v][p]);
-        }
-      if constexpr (IMEX) {
-        // the implicit weights b_i equal the explicit ones b~_i
-#pragma unroll
-        for (int p = 0; p < n; ++p) Sb[p] = (i == F0) ? wi * Ss[i][p] : fma(wi, Ss[i][p], Sb[p]);
-      }
+    if constexpr (IMEX) {
+      // the implicit weights b_i equal the explicit ones b~_i
+      if (wi != 0) Sb = fma(wd, Ss[i], Sb);
     }
   }
 
-  // ---- face traces ----------------------------------------------------------
-  double tr_r[NL];  // right (xi = 1) traces, same field order as sm_left
+  // ---- the averages' derivative and the face traces --------------------------
+#pragma unroll
+  for (int k = 0; k < K; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  __syncwarp();
+  if (lane_ok) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) X[k][p] = fx_split(A[k]);
+    if constexpr (SWE) {
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+        X[3 + v][p] = GLL ? Fx{__double2hiint(u0[v]), __double2loint(u0[v])}
+                          : fx_split(fx_from<FB>(u0[v], Ex[v]));
+    }
+  }
+  __syncwarp();
+  double V[M];                         // sum_j (b_j/b_ref) L_j
   if constexpr (SWE) {
-    tr_r[0] = trace_r<N, GLL>(T, U[0]);
-    tr_r[1] = trace_r<N, GLL>(T, U[1]);
-    tr_r[2] = trace_r<N, GLL>(T, F2);
-    tr_r[3] = trace_r<N, GLL>(T, u0[0]);
-    tr_r[4] = trace_r<N, GLL>(T, u0[1]);
-    tr_r[5] = c_r;
-    sm_left[0][t] = trace_l<N, GLL>(T, U[0]);
-    sm_left[1][t] = trace_l<N, GLL>(T, U[1]);
-    sm_left[2][t] = trace_l<N, GLL>(T, F2);
-    sm_left[3][t] = trace_l<N, GLL>(T, u0[0]);
-    sm_left[4][t] = trace_l<N, GLL>(T, u0[1]);
-    sm_left[5][t] = c_l;
+    V[0] = fx_to(contract(1), Ex[1] + T.fx.kD - FB + kSumShift, fx_zero(Ex[1]));
+    V[1] = fx_to(contract(2), Ex[2] + T.fx.kD - FB + kSumShift, fx_zero(Ex[2]));
+    if (WB)
+      V[1] += Pb;
+    else
+      V[1] = fma(fx_to(A[0], Ex[0] + 63 - FB + kSumShift, fx_zero(Ex[0])), sn, V[1]);
   } else {
-    tr_r[0] = trace_r<N, GLL>(T, U[0]);
-    tr_r[1] = c_r;
-    sm_left[0][t] = trace_l<N, GLL>(T, U[0]);
-    sm_left[1][t] = c_l;
+    V[0] = sn * fx_to(contract(0), Ex[0] + T.fx.kD - FB + kSumShift, fx_zero(Ex[0]));
+  }
+  // traces: 2 NT of them, shared out over the element's threads
+  if (lane_ok) {
+#pragma unroll
+    for (int j0 = 0; j0 < 2 * NT; j0 += n) {
+      const int job = j0 + p;
+      if (2 * NT % n != 0 && job >= 2 * NT) break;
+      const int side = job >= NT, fi = side ? job - NT : job;
+      const int ex = !SWE || fi == 0 || fi == 3 ? Ex[0] : fi == 2 ? Ex[K - 1] : Ex[K > 1 ? 1 : 0];
+      const int avg = fi < 3 ? kSumShift : 0;
+      double tr;
+      if constexpr (GLL) {
+        const Fx v = X[fi][side ? N : 0];
+        tr = fi >= 3 ? __hiloint2double(v.hi, v.lo)
+                     : fx_to(((long long)v.hi << 30) + v.lo, ex + 63 - FB + avg, fx_zero(ex));
+      } else {
+        FxAcc a;
+        Fx r[n];
+        fx_row<n>(X[fi], r);
+        fx_mul(a, r[0], side ? T.fx.l1_hi[0] : T.fx.l0_hi[0], side ? T.fx.l1_lo[0] : T.fx.l0_lo[0]);
+#pragma unroll
+        for (int j = 1; j < n; ++j)
+          fx_mad(a, r[j], side ? T.fx.l1_hi[j] : T.fx.l0_hi[j],
+                 side ? T.fx.l1_lo[j] : T.fx.l0_lo[j]);
+        tr = fx_to(fx_sum(a), ex + T.fx.kL - FB + avg, fx_zero(ex));
+      }
+      str[side][fi][slot] = tr;
+    }
   }
   __syncthreads();
 
-  // ---- Riemann problem at the right face (t | t+1), both sides -------------
-  double Tm[M];        // doubled face term on this element's right face (minus side)
-  double Fm_lim[LM];   // limiter: blended, limited flux F^- of that face
-  if constexpr (LIMIT) {
-    if (t < BLOCK - 1) {
+  // ---- Riemann problem at the right face of slot f (f | f+1), both sides ----
+  for (int f = t; f < ne - 1; f += blockDim.x) {
+    double tm[NT + 1], tp[NT + 1];
+#pragma unroll
+    for (int k = 0; k <= NT; ++k) {
+      tm[k] = str[1][k][f];
+      tp[k] = str[0][k][f + 1];
+    }
+    if constexpr (LIMIT) {
       // time-averaged numerical and total fluxes in the units of the time
       // averages (divided by b_ref), Eqs. numflux.cons, good.numflux.non.cons,
       // total.F.non.cons; the first-order face flux from the nodal values next
@@ -453,10 +512,8 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       constexpr double b0 = TB::bref();
       double FHm[M], FHp[M], FTm[M], FTp[M];
       if constexpr (SWE) {
-        const double Hm = tr_r[0], Mm = tr_r[1], Fm = tr_r[2], hm = tr_r[3], mm = tr_r[4],
-                     bm = tr_r[5];
-        const double Hp = sm_left[0][t + 1], Mp = sm_left[1][t + 1], Fp = sm_left[2][t + 1],
-                     hp = sm_left[3][t + 1], mp = sm_left[4][t + 1], bp = sm_left[5][t + 1];
+        const double Hm = tm[0], Mm = tm[1], Fm = tm[2], hm = tm[3], mm = tm[4], bm = tm[5];
+        const double Hp = tp[0], Mp = tp[1], Fp = tp[2], hp = tp[3], mp = tp[4], bp = tp[5];
         const double g = T.gravity;
         const double lam =
             max_nonneg(swe_speed(hm, mm, T.sqrt_gravity), swe_speed(hp, mp, T.sqrt_gravity));
@@ -476,8 +533,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         FTm[1] = Fm + g * hm * Wm;
         FTp[1] = Fp + g * hp * Wp;
       } else {
-        const double Vm = tr_r[0], am = tr_r[1];
-        const double Vp = sm_left[0][t + 1], ap = sm_left[1][t + 1];
+        const double Vm = tm[0], am = tm[1], Vp = tp[0], ap = tp[1];
         const double lam = max_nonneg(fabs(am), fabs(ap));
         const double Fn = -0.5 * lam * (Vp - Vm);
         const double Vn = 0.5 * (Vm + Vp);
@@ -487,17 +543,17 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         FTp[0] = ap * Vp;
       }
       double uN[M], u0R[M], fLm[M], fLp[M];
-  #pragma unroll
+#pragma unroll
       for (int v = 0; v < M; ++v) {
-        uN[v] = u0[v][N];
-        u0R[v] = sm_u0[v][t + 1];
+        uN[v] = lu[v][f][N];
+        u0R[v] = lu[v][f + 1][0];
       }
-      lo_flux<SYS>(uN, u0R, cn[N], sm_c0[t + 1], T, fLm, fLp);
-      const double af = 0.5 * (alpha + sm_al[t + 1]);
+      lo_flux<SYS>(uN, u0R, lc[f][N], lc[f + 1][0], T, fLm, fLp);
+      const double af = 0.5 * (la[f] + la[f + 1]);
       // (af = 0 and theta = 1 are the common cases: there the blends reduce
       // to their first terms and are skipped)
       double Fm_[M], Fp_[M];
-  #pragma unroll
+#pragma unroll
       for (int v = 0; v < M; ++v) {
         Fm_[v] = b0 * FHm[v];
         Fp_[v] = b0 * FHp[v];
@@ -508,14 +564,14 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       }
       if constexpr (SWE) {
         const double c0 = dtx * T.inv_w[0], cN = dtx * T.inv_w[N];
-        const double fi0R = sm_fi0[0][t + 1], fiNL = fip[0][LN - 1];
+        const double fi0R = lim[0][f + 1][0], fiNL = lip[0][f][N > 0 ? N - 1 : 0];
         const double low0 = u0R[0] - c0 * (fi0R - fLp[0]);
         const double lowN = uN[0] - cN * (fLm[0] - fiNL);
         const double t0 = u0R[0] - c0 * (fi0R - Fp_[0]);
         const double tN = uN[0] - cN * (Fm_[0] - fiNL);
         const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
         if (th < 1.0) {
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < M; ++v) {
             Fm_[v] = th * Fm_[v] + (1.0 - th) * fLm[v];
             Fp_[v] = th * Fp_[v] + (1.0 - th) * fLp[v];
@@ -523,162 +579,129 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         }
       }
       // face terms in the doubled units of the corrections: 2 (F - F^tot) / b_ref
-  #pragma unroll
+#pragma unroll
       for (int v = 0; v < M; ++v) {
-        Fm_lim[v] = Fm_[v];
-        Tm[v] = 2.0 * (Fm_[v] * T.inv_b0 - FTm[v]);
-        sm_T[v][t + 1] = 2.0 * (Fp_[v] * T.inv_b0 - FTp[v]);
-        sm_F[v][t + 1] = Fp_[v];
+        lF[0][v][f] = Fm_[v];
+        lF[1][v][f + 1] = Fp_[v];
+        sT[0][v][f] = 2.0 * (Fm_[v] * T.inv_b0 - FTm[v]);
+        sT[1][v][f + 1] = 2.0 * (Fp_[v] * T.inv_b0 - FTp[v]);
       }
-    }
-  } else {
-    if (t < BLOCK - 1) {
-      if constexpr (SWE) {
-        const double Hm = tr_r[0], Mm = tr_r[1], Fm = tr_r[2], hm = tr_r[3], mm = tr_r[4],
-                     bm = tr_r[5];
-        const double Hp = sm_left[0][t + 1], Mp = sm_left[1][t + 1], Fp = sm_left[2][t + 1],
-                     hp = sm_left[3][t + 1], mp = sm_left[4][t + 1], bp = sm_left[5][t + 1];
-        const double lam =
-            max_nonneg(swe_speed(hm, mm, T.sqrt_gravity), swe_speed(hp, mp, T.sqrt_gravity));
-        // F_h = U_m (the h flux is the momentum)
-        const double dFh = Mp - Mm;
-        const double dFm = Fp - Fm, dUm = Mp - Mm;
-        // jump of the dissipated and fluctuating state: h, or eta = h + b for
-        // the well-balanced form (b is static, so in the units of the time
-        // averages, divided by b_ref, its jump carries 1 / b_ref)
-        const double dUh = WB ? fma(T.inv_b0, bp - bm, Hp - Hm) : Hp - Hm;
-        const double gdb = WB ? T.gravity * dUh : T.face_g * (bp - bm);
-        Tm[0] = fma(-lam, dUh, dFh);
-        Tm[1] = fma(hm, gdb, fma(-lam, dUm, dFm));
-        const double Tp0 = -fma(lam, dUh, dFh);
-        const double Tp1 = -fma(hp, gdb, fma(lam, dUm, dFm));
-        sm_T[0][t + 1] = Tp0;
-        sm_T[1][t + 1] = Tp1;
-      } else {
-        const double Vm = tr_r[0], am = tr_r[1];
-        const double Vp = sm_left[0][t + 1], ap = sm_left[1][t + 1];
-        const double lam = max_nonneg(fabs(am), fabs(ap));
-        const double dU = Vp - Vm;
-        Tm[0] = (am - lam) * dU;
-        sm_T[0][t + 1] = -(lam + ap) * dU;
-      }
+    } else if constexpr (SWE) {
+      const double lam =
+          max_nonneg(swe_speed(tm[3], tm[4], T.sqrt_gravity), swe_speed(tp[3], tp[4], T.sqrt_gravity));
+      // F_h = U_m (the h flux is the momentum)
+      const double dFm = tp[2] - tm[2], dUm = tp[1] - tm[1];
+      // jump of the dissipated and fluctuating state: h, or eta = h + b for
+      // the well-balanced form (b is static, so in the units of the time
+      // averages, divided by b_ref, its jump carries 1 / b_ref)
+      const double db = tp[5] - tm[5];
+      const double dUh = WB ? fma(T.inv_b0, db, tp[0] - tm[0]) : tp[0] - tm[0];
+      const double gdb = WB ? T.gravity * dUh : T.face_g * db;
+      sT[0][0][f] = fma(-lam, dUh, dUm);
+      sT[0][M - 1][f] = fma(tm[3], gdb, fma(-lam, dUm, dFm));
+      sT[1][0][f + 1] = -fma(lam, dUh, dUm);
+      sT[1][M - 1][f + 1] = -fma(tp[3], gdb, fma(lam, dUm, dFm));
+    } else {
+      const double lam = max_nonneg(fabs(tm[1]), fabs(tp[1]));
+      const double dU = tp[0] - tm[0];
+      sT[0][0][f] = (tm[1] - lam) * dU;
+      sT[1][0][f + 1] = -(lam + tp[1]) * dU;
     }
   }
   __syncthreads();
 
   // ---- correction and update (owners only) --------------------------------
-  double rate = 0.0;
-  bool bad = false;
-  if (owner) {
-    double Tp[M];
+  constexpr double b0 = TB::bref();
+  const double dtb0 = dtx * b0;
+  const double dts = dt * b0;
+  double out[M];
 #pragma unroll
-    for (int v = 0; v < M; ++v) Tp[v] = sm_T[v][t];
-    constexpr double b0 = TB::bref();
-    const double dtb0 = dtx * b0;
-    const double dts = dt * b0;
-    double out[M][n];
+  for (int v = 0; v < M; ++v) {
+    double R = V[v];
+    if (!GLL || p == N) R = fma(sT[0][v][slot], T.gRx[p], R);
+    if (!GLL || p == 0) R = fma(sT[1][v][slot], T.gLx[p], R);
+    double o = RES ? -(b0 * xs) * R : fma(-dtb0, R, u0[v]);
+    if (IMEX && v == SV) o = fma(RES ? b0 : dts, Sb, o);
+    out[v] = o;
+  }
+  if constexpr (LIMIT) {
+    // first-order subcell update (Eq. low.order.update), then
+    // Eq. blended.scheme and Algorithm 2 (h > 0)
+    double lo[M];
+    const double cw = dtx * T.inv_w[p];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      const double right = p < N ? lim[v][slot][p] : lF[0][v][slot];
+      const double left = p > 0 ? lip[v][slot][p > 0 ? p - 1 : 0] : lF[1][v][slot];
+      lo[v] = u0[v] - cw * (right - left);
+    }
+    if constexpr (IMEX) lo_source<SYS>(T, dt, lo);
 #pragma unroll
     for (int v = 0; v < M; ++v)
+      if (alpha != 0.0) out[v] = (1.0 - alpha) * out[v] + alpha * lo[v];
+    if constexpr (SWE) {
+      const double eps = 0.1 * element_min<n>(lo[0], le, p, lane);
+      const double th = element_min<n>(theta_lin(eps, lo[0], out[0]), le, p, lane);
+      if (th < 1.0) {
 #pragma unroll
-      for (int p = 0; p < n; ++p) {
-        double R = V[v][p];
-        if (!GLL || p == N) R = fma(Tm[v], T.gRx[p], R);
-        if (!GLL || p == 0) R = fma(Tp[v], T.gLx[p], R);
-        double o = RES ? -(b0 * xs) * R : fma(-dtb0, R, u0[v][p]);
-        if (IMEX && v == SV) o = fma(RES ? b0 : dts, Sb[p], o);
-        out[v][p] = o;
-        if (!LIMIT) u_out[((int64_t)v * E + e) * n + p] = o;
-      }
-    if constexpr (LIMIT) {
-      // first-order subcell update (Eq. low.order.update), then
-      // Eq. blended.scheme and Algorithm 2 (h > 0)
-      double lo[M][n];
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        double x[M];
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          const double right = p < N ? fim[v][p < N ? p : 0] : Fm_lim[v];
-          const double left = p > 0 ? fip[v][p > 0 ? p - 1 : 0] : sm_F[v][t];
-          x[v] = u0[v][p] - (dtx * T.inv_w[p]) * (right - left);
-        }
-        if constexpr (IMEX) lo_source<SYS>(T, dt, x);
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          lo[v][p] = x[v];
-          if (alpha != 0.0) out[v][p] = (1.0 - alpha) * out[v][p] + alpha * x[v];
-        }
-      }
-      if constexpr (SWE) {
-        double lmin = lo[0][0];
-#pragma unroll
-        for (int p = 1; p < n; ++p) lmin = fmin(lmin, lo[0][p]);
-        const double eps = 0.1 * lmin;
-        double th = 1.0;
-#pragma unroll
-        for (int p = 0; p < n; ++p) th = fmin(th, theta_lin(eps, lo[0][p], out[0][p]));
-        if (th < 1.0) {
-#pragma unroll
-          for (int v = 0; v < M; ++v)
-#pragma unroll
-            for (int p = 0; p < n; ++p) out[v][p] = th * out[v][p] + (1.0 - th) * lo[v][p];
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < M; ++v)
-#pragma unroll
-        for (int p = 0; p < n; ++p) u_out[((int64_t)v * E + e) * n + p] = out[v][p];
-      LA.alpha_out[e] = alpha;
-    }
-    if (!RES) {
-      if constexpr (SWE) {
-#pragma unroll
-        for (int p = 0; p < n; ++p) bad |= !positive_finite(out[0][p]) || !finite(out[1][p]);
-      } else {
-#pragma unroll
-        for (int p = 0; p < n; ++p) bad |= !finite(out[0][p]);
-      }
-      if (ctl.want_rate) {
-        double hb = T.w[0] * out[0][0];
-#pragma unroll
-        for (int p = 1; p < n; ++p) hb = fma(T.w[p], out[0][p], hb);
-        if constexpr (SWE) {
-          double mb = T.w[0] * out[1][0];
-#pragma unroll
-          for (int p = 1; p < n; ++p) mb = fma(T.w[p], out[1][p], mb);
-          rate = swe_speed(hb, mb, T.sqrt_gravity) * xs;
-        } else {
-          // the speed of advection is |a| averaged over the element
-          double ab = T.w[0] * sn[0];
-#pragma unroll
-          for (int p = 1; p < n; ++p) ab = fma(T.w[p], sn[p], ab);
-          rate = fabs(ab) * xs;
-        }
+        for (int v = 0; v < M; ++v) out[v] = th * out[v] + (1.0 - th) * lo[v];
       }
     }
+    if (owner && p == 0) LA.alpha_out[e] = alpha;
   }
-  if (!RES) {
-    if (bad) atomicOr(&st->status, 1u);
-    if (ctl.want_rate) block_max_atomic<BLOCK>(rate, &st->rate[ctl.slot_write]);
+  if (owner) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) u_out[((int64_t)v * E + e) * n + p] = out[v];
   }
+  if (RES) return;
+  bool bad = false;
+  if (owner) bad = SWE ? !positive_finite(out[0]) || !finite(out[M - 1]) : !finite(out[0]);
+  if (bad) atomicOr(&st->status, 1u);
+  if (!ctl.want_rate) return;
+  // the next step's rate: element means by one thread per element (the speed
+  // of advection is |a| averaged over the element)
+  double* sm = reinterpret_cast<double*>(&X[0][0]);
+  if (lane_ok) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) sm[v * n + p] = SWE ? out[v] : sn;
+  }
+  __syncthreads();
+  double rate = 0.0;
+  for (int k = t; k < ne; k += blockDim.x) {
+    if (k < 1 || k > ne - 2 || tile * (ne - 2) + k - 1 >= E) continue;
+    const double* x = reinterpret_cast<const double*>(&sx[k][0][0]);
+    double m[M];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      m[v] = T.w[0] * x[v * n];
+#pragma unroll
+      for (int j = 1; j < n; ++j) m[v] = fma(T.w[j], x[v * n + j], m[v]);
+    }
+    if constexpr (SWE)
+      rate = max_bits(rate, swe_speed(m[0], m[M - 1], T.sqrt_gravity) * xs);
+    else
+      rate = max_bits(rate, fabs(m[0]) * xs);
+  }
+  block_max_atomic_1d(rate, &st->rate[ctl.slot_write]);
 }
 
-template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false, int BLOCK = kBlock1D>
-__global__ void __launch_bounds__(BLOCK) k_step_1d(const Launch1D L) {
-  step_1d_tile<SYS, N, GLL, RES, IMEX, LIMIT, BLOCK>(L.tab, L.xs, L.u_in, L.u_out, L.snode,
-                                                     L.sface, L.E, blockIdx.x, L.st, L.ctl,
-                                                     blockIdx.x == 0, L.lim, L.ghost);
+// registers for 24 warps per SM (limited: 16)
+template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
+__global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D, LIMIT ? 4 : 3) k_step_1d(const Launch1D L) {
+  step_1d_tile<SYS, N, GLL, RES, IMEX, LIMIT>(L.tab, L.xs, L.u_in, L.u_out, L.snode, L.sface, L.E,
+                                              blockIdx.x, L.st, L.ctl, blockIdx.x == 0, L.lim,
+                                              L.ghost);
 }
 
 // ragged ensembles: (instance, tile) pairs of a work list, a block taking
 // items blockIdx.x, blockIdx.x + gridDim.x, ... (the grid size is a tuning
-// parameter; the tile body's shared-memory phases are separated by barriers,
-// so a block may run several tiles in turn)
+// parameter; the tile body's shared-memory phases are separated by barriers)
 template <int SYS, int N, bool GLL, bool IMEX>
-__global__ void __launch_bounds__(kBlock1D) k_step_1d_batch(const LaunchBatch1D B) {
+__global__ void __launch_bounds__(kBlock1D, 3) k_step_1d_batch(const LaunchBatch1D B) {
   for (int64_t wi = blockIdx.x; wi < B.nwork; wi += gridDim.x) {
     const WorkItem w = B.work[wi];
     const BatchInstance I = B.inst[w.inst];
+    if (wi != blockIdx.x) __syncthreads();   // the previous tile's last reads
     step_1d_tile<SYS, N, GLL, false, IMEX>(B.tab, I.xs, B.u_in + I.u_off, B.u_out + I.u_off,
                                            B.snode + I.sn_off, B.sface + I.sf_off, I.E, w.tile,
                                            I.st, B.ctl, w.tile == 0);
@@ -686,80 +709,62 @@ __global__ void __launch_bounds__(kBlock1D) k_step_1d_batch(const LaunchBatch1D 
 }
 
 // Threads per block of the step, chosen per mesh among kTileBlocks.  A block
-// updates BLOCK - 2 elements, one per thread, and every thread does the same
-// work, so the step's time follows the busiest SM's thread count,
-// BLOCK x ceil(tiles / SMs).  At 1e5 elements 128-thread tiles (794) put 6
-// blocks = 768 threads on some SMs, 96-thread tiles (1064) 7 blocks = 672
-// threads on every SM: 8% faster.  Among block sizes within 2% of the least
-// such count the one with the most resident threads per SM, then the larger,
-// is taken (on large meshes 128: fewer halo elements, as many warps).
-// crkfr_set_tile_1d can fix the size instead.
-constexpr int kTileBlocks[3] = {64, 96, 128};
+// recomputes two halo elements, so large meshes take the largest block; a
+// small mesh is spread over the SMs in smaller ones, since an SM sub-partition
+// runs its warps' FP64 instructions one after the other: the step's time
+// follows the warps of the busiest sub-partition, ceil(tiles / SMs) blocks of
+// threads / 32 warps over four, and no less than one.  The larger block is
+// taken among those within 2 % of the least such time.  crkfr_set_tile_1d can
+// fix the size instead.
+constexpr int kTileBlocks[4] = {32, 64, 128, 256};
 
-inline int pick_tile_block(int64_t E, int sms, const int* resident) {
-  int64_t cost[3];
-  int64_t best = -1;
-  for (int i = 0; i < 3; ++i) {
-    const int64_t B = kTileBlocks[i];
-    const int64_t tiles = (E + B - 3) / (B - 2);
-    cost[i] = B * ((tiles + sms - 1) / sms);
-    if (best < 0 || cost[i] < best) best = cost[i];
+inline int pick_tile_block(int64_t E, int n, int sms) {
+  double cost[4], best = 0.0;
+  for (int i = 0; i < 4; ++i) {
+    const int64_t own = tile_elements_1d(kTileBlocks[i], n);
+    const int64_t tiles = (E + own - 1) / own;
+    const double warps = (double)((tiles + sms - 1) / sms) * (kTileBlocks[i] / 32) / 4.0;
+    cost[i] = warps < 1.0 ? 1.0 : warps;
+    if (i == 0 || cost[i] < best) best = cost[i];
   }
-  int pick = 2;
-  for (int i = 0; i < 3; ++i) {
-    if (50 * cost[i] > 51 * best) continue;
-    const int64_t ri = (int64_t)resident[i] * kTileBlocks[i];
-    const int64_t rp = (int64_t)resident[pick] * kTileBlocks[pick];
-    if (50 * cost[pick] > 51 * best || ri > rp || (ri == rp && i > pick)) pick = i;
-  }
+  int pick = 0;
+  for (int i = 1; i < 4; ++i)
+    if (cost[i] <= 1.02 * best || cost[pick] > 1.02 * best) pick = i;
   return kTileBlocks[pick];
 }
 
-template <int SYS, int N, bool GLL, bool IMEX, int BLOCK>
-int launch_step_block(const Launch1D& L, cudaStream_t s) {
-  const int64_t blocks = (L.E + BLOCK - 3) / (BLOCK - 2);
-  if (blocks > 0x7fffffff) return (int)cudaErrorInvalidConfiguration;
-  k_step_1d<SYS, N, GLL, false, IMEX, false, BLOCK><<<(unsigned)blocks, BLOCK, 0, s>>>(L);
-  return (int)cudaGetLastError();
+// threads of the block, elements of the mesh: blocks of the launch (0: none fit)
+inline unsigned tiles_1d(int64_t E, int threads, int n) {
+  const int64_t own = tile_elements_1d(threads, n);
+  const int64_t blocks = (E + own - 1) / own;
+  return blocks > 0x7fffffff ? 0u : (unsigned)blocks;
 }
 
 template <int SYS, int N, bool GLL, bool IMEX>
 int launch_step_t(const Launch1D& L, cudaStream_t s) {
   if (L.ctl.residual) {
-    const int64_t blocks = (L.E + kBlock1D - 3) / (kBlock1D - 2);
-    if (blocks > 0x7fffffff) return (int)cudaErrorInvalidConfiguration;
-    k_step_1d<SYS, N, GLL, true, IMEX><<<(unsigned)blocks, kBlock1D, 0, s>>>(L);
+    const unsigned blocks = tiles_1d(L.E, kBlock1D, N + 1);
+    if (!blocks) return (int)cudaErrorInvalidConfiguration;
+    k_step_1d<SYS, N, GLL, true, IMEX><<<blocks, kBlock1D, 0, s>>>(L);
     return (int)cudaGetLastError();
   }
-  // SMs and resident blocks per SM of each block size (the occupancy API,
-  // asked once; if the query failed, 128-thread tiles)
-  struct Occ {
-    int sms = 0;
-    int resident[3] = {0, 0, 0};
-  };
-  static const Occ occ = [] {
-    Occ o;
-    int dev = 0;
+  // SMs of the GPU (asked once; 0 if the query failed: then the largest block)
+  static const int sms = [] {
+    int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&o.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &o.resident[0], k_step_1d<SYS, N, GLL, false, IMEX, false, 64>, 64, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &o.resident[1], k_step_1d<SYS, N, GLL, false, IMEX, false, 96>, 96, 0) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &o.resident[2], k_step_1d<SYS, N, GLL, false, IMEX, false, 128>, 128, 0) !=
-            cudaSuccess) {
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       cudaGetLastError();
-      o.sms = 0;
+      return 0;
     }
-    return o;
+    return v;
   }();
-  if (L.tile_threads <= 0 && occ.sms <= 0) return launch_step_block<SYS, N, GLL, IMEX, 128>(L, s);
-  switch (L.tile_threads > 0 ? L.tile_threads : pick_tile_block(L.E, occ.sms, occ.resident)) {
-    case 64: return launch_step_block<SYS, N, GLL, IMEX, 64>(L, s);
-    case 96: return launch_step_block<SYS, N, GLL, IMEX, 96>(L, s);
-  }
-  return launch_step_block<SYS, N, GLL, IMEX, 128>(L, s);
+  const int threads = L.tile_threads > 0 ? L.tile_threads
+                      : sms > 0          ? pick_tile_block(L.E, N + 1, sms)
+                                         : kBlock1D;
+  const unsigned blocks = tiles_1d(L.E, threads, N + 1);
+  if (!blocks) return (int)cudaErrorInvalidConfiguration;
+  k_step_1d<SYS, N, GLL, false, IMEX><<<blocks, (unsigned)threads, 0, s>>>(L);
+  return (int)cudaGetLastError();
 }
 
 template <int SYS, bool IMEX>

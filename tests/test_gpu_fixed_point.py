@@ -68,6 +68,41 @@ def test_block_edges_and_growing_momentum(crk, N, family, Ex, Ey, still):
     assert rel_l2(got, sch.step(u, b, dt)) < TOL
 
 
+def case_1d(N, family, E, still=False, seed=0):
+    from oracle.crkfr import Scheme1D
+    from oracle.systems import ShallowWater1D
+    L = 10.0
+    sch = Scheme1D(ShallowWater1D(G), N, L / E, family=family)
+    x = (np.arange(E)[:, None] + sch.basis.xi[None, :]) * (L / E)
+    a = np.random.default_rng(seed).uniform(0, 2 * np.pi, 4)
+    k = 2 * np.pi / L
+    b = 0.2 * np.sin(k * x + a[0])
+    h = 1.0 + 0.1 * np.sin(k * x + a[1]) - b
+    return sch, np.stack([h, (0.0 if still else 0.3) * h * np.cos(k * x + a[2])]), b, L
+
+
+# elements a block owns, threads / 32 * (32 / n) - 2: N = 1: 14 (32 threads) ..
+# 126 (256), N = 2: 8 .. 78, N = 3: 6 .. 62, N = 4: 4 .. 46
+@pytest.mark.parametrize("N,family,E", [
+    (0, "gl", 1), (0, "gl", 31), (0, "gl", 255), (1, "gl", 1), (1, "gll", 15), (1, "gl", 127),
+    (2, "gl", 2), (2, "gll", 9), (2, "gl", 79), (3, "gl", 1), (3, "gll", 7), (3, "gl", 63),
+    (4, "gl", 1), (4, "gll", 5), (4, "gl", 47), (4, "gl", 20011)])
+@pytest.mark.parametrize("still", [False, True])
+def test_block_edges_1d(crk, N, family, E, still):
+    sch, u, b, L = case_1d(N, family, E, still)
+    dt = sch.compute_dt(u, b, golden_cfl(N, family), 0.5)
+    want = sch.step(u, b, dt)
+    s = crk.Solver("swe1d", N, nodes=family, gravity=G, cfl_safety=0.5,
+                   cfl_number=golden_cfl(N, family))
+    s.set_mesh([E], [0.0], [L])
+    s.set_coefficients(to_dev(b))
+    for threads in (0, 64, 96, 128):
+        s.set_tile_1d(threads)
+        d = to_dev(u)
+        s.step(d, dt, 1)
+        assert rel_l2(to_host(d), want) < TOL
+
+
 @pytest.mark.parametrize("N", [1, 2, 3, 4])
 @pytest.mark.parametrize("scale", [1e-12, 1e9])
 def test_scales(crk, N, scale):

@@ -182,6 +182,43 @@ __device__ __forceinline__ void step_bookkeeping(const StepCtl& c, DevState* st,
   if (dt > 0.0) st->nadv += 1ull;
 }
 
+// The step size and its products with the tableau's coefficients, by the
+// block's first warp (each product once, in one lane, instead of in every
+// thread: an FP64 instruction costs the same for one lane as for 32): dt;
+// e[i][j] = -(dt a~_ij xs); im[i][j] = dt a_ij; dt b_ref xs and dt b_ref.
+template <class TB>
+struct StepSizes {
+  double dt, dtb_x, dtb;
+  double e[TB::S][TB::S], im[TB::S][TB::S];
+};
+template <class TB, bool IMEX>
+__device__ __forceinline__ void fill_step_sizes(StepSizes<TB>& s, double dt, double xs) {
+  constexpr int S = TB::S;
+  const int lane = threadIdx.x;
+  const double dtx = dt * xs;
+#pragma unroll
+  for (int k0 = 0; k0 < S * S; k0 += 32) {
+    double a = 0.0, ai = 0.0;
+    const int k = k0 + lane;
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) {
+        if (TB::a(i, j) != 0.0 && k == i * S + j) a = TB::a(i, j);
+        if (IMEX && TB::ai(i, j) != 0.0 && k == i * S + j) ai = TB::ai(i, j);
+      }
+    if (k < S * S) {
+      (&s.e[0][0])[k] = -(dtx * a);
+      if (IMEX) (&s.im[0][0])[k] = dt * ai;
+    }
+  }
+  if (lane == 0) {
+    s.dt = dt;
+    s.dtb_x = dtx * TB::bref();
+    s.dtb = dt * TB::bref();
+  }
+}
+
 // Weight of the candidate b in theta b + (1 - theta) a for the linear
 // constraint P (Eq. theta.formula): 1 unless P(b) < eps.
 __device__ __forceinline__ double theta_lin(double eps, double Pa, double Pb) {

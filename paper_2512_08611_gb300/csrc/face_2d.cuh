@@ -143,16 +143,19 @@ __device__ __forceinline__ void face_limited(const double* tm, const double* tp,
   }
 }
 
-// Tile rows of the face kernel: the limited kernel keeps twice the face data
-// in shared memory and takes half the rows.
-template <int N, bool LIMIT>
+// Tile rows (warps) of the face kernel: 8, or 4 limited (its face data takes
+// twice the shared memory); 2 on meshes whose tiles of that height would leave
+// SMs without a block, where the step is latency and an SM sub-partition runs
+// its warps' FP64 instructions one after the other (small: 65 x 47 elements at
+// N = 2 have 42 tiles of 8 rows, 168 of 2).
+template <int N, bool LIMIT, bool SMALL>
 struct FaceShape {
-  static constexpr int TY = LIMIT ? 4 : kWarps2D;   // tile rows (warps)
+  static constexpr int TY = SMALL ? 2 : LIMIT ? 4 : kWarps2D;
   static constexpr int block = TY * 32;
   // resident blocks per SM the register allocation must allow (the plain
-  // kernel: 4 x 8 warps, half the SM's warp slots, to hide the shared-memory
+  // kernel: 40 warps, 32 at N = 4, to hide the barriers and the shared-memory
   // latency of the face terms)
-  static constexpr int min_blocks = LIMIT ? 1 : 4;
+  static constexpr int min_blocks = LIMIT ? 1 : SMALL ? 8 : N >= 4 ? 4 : 5;
 };
 
 // Face kernel on tiles of TY x EPW elements (one tile row per warp).
@@ -161,15 +164,17 @@ struct FaceShape {
 // warp of the loop pays for idle lanes) and keeps both sides' terms in shared
 // memory; phase 2 applies them along the rows and columns of each element.
 
-template <int N, bool GLL, bool RES, bool WB, bool LIMIT = false, bool IMEX = false>
-__global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT>::min_blocks)
+template <int N, bool GLL, bool RES, bool WB, bool LIMIT = false, bool IMEX = false,
+          bool SMALL = false>
+__global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
+                                  FaceShape<N, LIMIT, SMALL>::min_blocks)
     k_face_2d(const Launch2D L) {
   static_assert(!(LIMIT && RES), "the limiter needs a step");
   constexpr int n = N + 1;
   constexpr int nn = n * n;
   constexpr int TX = 32 / n;        // elements per tile row (= per warp)
-  constexpr int TY = FaceShape<N, LIMIT>::TY;
-  constexpr int BT = FaceShape<N, LIMIT>::block;
+  constexpr int TY = FaceShape<N, LIMIT, SMALL>::TY;
+  constexpr int BT = FaceShape<N, LIMIT, SMALL>::block;
   constexpr int NX = TY * (TX + 1) * n;
   constexpr int NY = (TY + 1) * TX * n;
   constexpr int LY = LIMIT ? TY : 1, LX = LIMIT ? TX : 1;
@@ -549,23 +554,34 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT>::block, FaceShape<N, LIMIT
   }
 }
 
-template <int N, bool GLL, bool WB, bool LIMIT = false, bool IMEX = false>
-int launch_face_t(const Launch2D& L, cudaStream_t s) {
+template <int N, bool GLL, bool WB, bool LIMIT, bool IMEX, bool SMALL>
+int launch_face_shape(const Launch2D& L, cudaStream_t s) {
   constexpr int TX = 32 / (N + 1);
-  constexpr int TY = FaceShape<N, LIMIT>::TY, BT = FaceShape<N, LIMIT>::block;
+  constexpr int TY = FaceShape<N, LIMIT, SMALL>::TY, BT = FaceShape<N, LIMIT, SMALL>::block;
   const dim3 grid((unsigned)((L.Ex + TX - 1) / TX),
                   (unsigned)((L.row_end - L.row_begin + TY - 1) / TY));
+  if (grid.y > 65535u) return (int)cudaErrorInvalidConfiguration;
+  if constexpr (LIMIT)
+    k_face_2d<N, GLL, false, WB, true, IMEX, SMALL><<<grid, BT, 0, s>>>(L);
+  else if (L.ctl.residual)
+    k_face_2d<N, GLL, true, WB><<<dim3(grid.x, (grid.y * TY + kWarps2D - 1) / kWarps2D), kBlock2D, 0,
+                                  s>>>(L);
+  else
+    k_face_2d<N, GLL, false, WB, false, false, SMALL><<<grid, BT, 0, s>>>(L);
+  return (int)cudaGetLastError();
+}
+
+template <int N, bool GLL, bool WB, bool LIMIT = false, bool IMEX = false>
+int launch_face_t(const Launch2D& L, cudaStream_t s) {
   if (L.row_begin % 8 != 0 || L.row_end <= L.row_begin || L.row_end > L.Ey ||
       (L.row_end % 8 != 0 && L.row_end != L.Ey))
     return (int)cudaErrorInvalidValue;
-  if (grid.y > 65535u) return (int)cudaErrorInvalidConfiguration;
-  if constexpr (LIMIT)
-    k_face_2d<N, GLL, false, WB, true, IMEX><<<grid, BT, 0, s>>>(L);
-  else if (L.ctl.residual)
-    k_face_2d<N, GLL, true, WB><<<grid, BT, 0, s>>>(L);
-  else
-    k_face_2d<N, GLL, false, WB><<<grid, BT, 0, s>>>(L);
-  return (int)cudaGetLastError();
+  // small: fewer tiles than the GB300's 152 SMs
+  constexpr int TX = 32 / (N + 1), TY = FaceShape<N, LIMIT, false>::TY;
+  const int64_t tiles =
+      ((L.Ex + TX - 1) / TX) * ((L.row_end - L.row_begin + TY - 1) / TY);
+  return tiles < 152 ? launch_face_shape<N, GLL, WB, LIMIT, IMEX, true>(L, s)
+                     : launch_face_shape<N, GLL, WB, LIMIT, IMEX, false>(L, s);
 }
 
 template <bool WB, bool LIMIT = false, bool IMEX = false>

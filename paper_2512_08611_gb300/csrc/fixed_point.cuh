@@ -57,12 +57,16 @@ template <int FB>
 __device__ __forceinline__ long long fx_from(double x, int E) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  unsigned long long m =
-      ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | lo) << (FB - 53);
-  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(E - e));
-  const long long s = hi >> 31;
-  return (long long)((m ^ (unsigned long long)s) - (unsigned long long)s);
+  const int e = (hi & 0x7fffffff) >> 20;
+  long long m = (long long)(((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32 | lo)
+                            << (FB - 53));
+  // (a predicated negation: two integer adds instead of a mask, two xors and
+  // two subtractions)
+  asm("{\n\t.reg .pred n;\n\tshr.u64 %0, %0, %1;\n\tsetp.lt.s32 n, %2, 0;\n\t"
+      "@n neg.s64 %0, %0;\n\t}"
+      : "+l"(m)
+      : "r"(E - e), "r"(hi));
+  return m;
 }
 
 __device__ __forceinline__ Fx fx_split(long long v) {
@@ -87,8 +91,10 @@ __device__ __forceinline__ int fx_zero(int E) { return E >= kFxNonFinite ? 0x7ff
 // Exponents above the FP64 range give a non-finite value.
 __device__ __forceinline__ double fx_to(long long R, int eb, int zero) {
   const int rh = (int)(R >> 32);
-  const long long s = rh >> 31;
-  unsigned long long a = (unsigned long long)(R ^ s) - (unsigned long long)s;
+  unsigned long long a = (unsigned long long)R;
+  asm("{\n\t.reg .pred n;\n\tsetp.lt.s32 n, %1, 0;\n\t@n neg.s64 %0, %0;\n\t}"
+      : "+l"(a)
+      : "r"(rh));
   const float f = __fmaf_rz(__uint2float_rz((unsigned)(a >> 32)), 4294967296.0f,
                             __uint2float_rz((unsigned)a));
   const int ex = __float_as_int(f) >> 23;   // 127 + position of the leading bit, 0 for zero
@@ -110,7 +116,8 @@ __device__ __forceinline__ void fx_accumulate(long long& A, long long& B, long l
     A += (long long)x.hi * w;
     B += (long long)x.lo * w;
   } else {
-    A += w * v;
+    A += (long long)((unsigned long long)(unsigned)v * (unsigned)w) +
+         (long long)((unsigned long long)(unsigned)((int)(v >> 32) * w) << 32);
   }
 }
 
@@ -126,7 +133,7 @@ __device__ __forceinline__ void fx_rescale(long long& A, long long& B, int sh) {
     A = sh < 62 ? hi : 0;
     B = sh < 62 ? low : 0;
   } else {
-    A = fx_sar(A, sh);
+    A = sh < 62 ? A >> (sh & 63) : 0;
   }
 }
 

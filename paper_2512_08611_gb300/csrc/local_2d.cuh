@@ -43,9 +43,6 @@ namespace {
 #ifndef CRKFR_LOCAL2D_BLOCK
 #define CRKFR_LOCAL2D_BLOCK 128
 #endif
-#ifndef CRKFR_LOCAL2D_MINB
-#define CRKFR_LOCAL2D_MINB 5
-#endif
 constexpr int kBlockLocal = CRKFR_LOCAL2D_BLOCK;
 constexpr int kTrFields = 7;
 // x-face trace fields: U_h, U_hu, U_hv, F_hu, F_hv (time-averaged x fluxes of
@@ -59,10 +56,55 @@ __host__ __device__ constexpr int local_elements() {
   return kBlockLocal / (n * n);
 }
 
+// Stage loop unrolled, with the earlier stages' operators and sources in
+// registers (short tableaux and friction: 512 x 512 with friction 2.50 ms for
+// two steps, 2.65 ms rolled), or rolled (unrolled, the kernel of N = 3 misses
+// the instruction cache, hit rate 86 %: 1024 x 1024 5.67 ms for two steps, 5.47
+// ms rolled; 401 x 307 at N = 4 2.25 and 2.07 ms), which also leaves room for
+// 28 instead of 20 warps per SM.
+template <int N, bool IMEX>
+__host__ __device__ constexpr bool local_unrolled() {
+  return IMEX || N <= 2;
+}
+template <int N, bool IMEX, bool LIMIT>
+__host__ __device__ constexpr int local_min_blocks() {
+  return LIMIT ? 3 : local_unrolled<N, IMEX>() ? 5 : 7;
+}
+
 // Exchange fields of the kernel: 0..5 the averages of h, hu, hv, hu hu / h
 // (+ pressure), hu hv / h, hv hv / h (+ pressure), or a stage's values of
 // them; 6..8 u^n.
 constexpr int kLocalFields = 9;
+
+// b~_i / b_ref of a stage counted at run time
+template <class TB>
+__device__ __forceinline__ int local_weight(int i) {
+  unsigned long long w = 0;
+#pragma unroll
+  for (int k = 0; k < TB::S; ++k) w |= (unsigned long long)TB::weight(k) << (8 * k);
+  return (int)(w >> (8 * i)) & 0xff;
+}
+
+// bit 8 i + j: a~_ij is not zero
+template <class TB>
+__device__ __forceinline__ unsigned long long local_nonzero() {
+  unsigned long long m = 0;
+#pragma unroll
+  for (int i = 0; i < TB::S; ++i)
+#pragma unroll
+    for (int j = 0; j < i; ++j)
+      if (TB::a(i, j) != 0.0) m |= 1ull << (8 * i + j);
+  return m;
+}
+
+// every stage sum takes the operator of the stage before it only
+template <class TB>
+__host__ __device__ constexpr bool local_chain() {
+  for (int i = 0; i < TB::S; ++i)
+    for (int j = 0; j + 1 < i; ++j)
+      if (TB::a(i, j) != 0.0) return false;
+  return true;
+}
 
 // Doubles per element in shared memory, 4 modulo 16 so that the elements of a
 // warp start 32 bytes apart modulo the banks.
@@ -73,7 +115,7 @@ __host__ __device__ constexpr int local_stride() {
 
 template <int N, bool GLL, bool RES, bool IMEX, bool WB, bool LIMIT = false, bool STAGES = false,
           int PRE = 0>
-__global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
+__global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>())
     k_local_2d(const Launch2D L) {
   static_assert(!(STAGES && (IMEX || WB || LIMIT)), "stages are recorded for the standard form");
   // PRE 1: only the first stage's local operator L(u^n), which needs no dt,
@@ -100,7 +142,7 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
   const Tables& T = L.tab;
   __shared__ __align__(16) double sm[EPB * ES];
   __shared__ int smag[EPB][3];
-  __shared__ double sdt[2];
+  __shared__ StepSizes<TB> sz;
 
   const int le_raw = threadIdx.x / nn, node = threadIdx.x - le_raw * nn;
   const int q = node / n, p = node - q * n;
@@ -118,15 +160,18 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
     return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
   };
 
-  // the step size (a division) by one thread of the block
-  if (threadIdx.x == 0) {
-    const double dt = (RES || PRE == 1) ? L.ctl.dt_fixed : step_dt(L.ctl, L.st);
-    sdt[0] = dt;
-    sdt[1] = dt * TB::bref();
-    if (!RES && PRE != 1 && blockIdx.x == 0 && !L.ctl.skip_bookkeeping)
-      step_bookkeeping(L.ctl, L.st, dt);
+  // the step size (a division) and its products by the block's first warp;
+  // the others start on the first stage, which needs neither
+  if (threadIdx.x < 32) {
+    double dt = 0.0;
+    if (threadIdx.x == 0) {
+      dt = (RES || PRE == 1) ? L.ctl.dt_fixed : step_dt(L.ctl, L.st);
+      if (!RES && PRE != 1 && blockIdx.x == 0 && !L.ctl.skip_bookkeeping)
+        step_bookkeeping(L.ctl, L.st, dt);
+    }
+    dt = __shfl_sync(0xffffffffu, dt, 0);
+    fill_step_sizes<TB, IMEX>(sz, dt, 1.0);
   }
-
   // threads past EPB n^2 and elements past the rows [row_begin, row_end)
   // compute on element 0 and store nothing to memory (the former nothing to
   // shared memory either)
@@ -147,18 +192,25 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
     dyh[j] = T.fx.Dy_hi[q][j];
     dyl[j] = T.fx.Dy_lo[q][j];
   }
-  if (threadIdx.x < 3 * EPB) (&smag[0][0])[threadIdx.x] = 0;
-  __syncthreads();
-  const double dt = sdt[0];
+  if (lane_ok && node < 3) smag[le][node] = 0;
+  sync();
 
-  double Ls[S][3];
+  // The operators L_j of earlier stages that a stage sum needs: the last one
+  // only (classical RK4), or all of them, in registers or shared memory; the
+  // sources of hu, hv (IMEX) in registers.
+  constexpr bool UNROLL = local_unrolled<N, IMEX>(), CHAIN = !UNROLL && local_chain<TB>();
+  constexpr bool SHARED = !UNROLL && !CHAIN;
+  constexpr int kStageUnroll = UNROLL ? S : 1;
+  static_assert(UNROLL || !IMEX, "the sources are kept in registers");
+  __shared__ double sL[SHARED ? S - 1 : 1][3][SHARED ? kBlockLocal : 1];
+  double rL[UNROLL ? S : 1][3], rS[IMEX ? S : 1][2];
+  double Lp[3] = {0.0, 0.0, 0.0};
   if constexpr (PRE == 2) {
     // L(u^n), computed ahead by the PRE 1 instantiation; the thread
     // overwrites the same values with W at the end
 #pragma unroll
-    for (int v = 0; v < 3; ++v) Ls[0][v] = L.w[(v * Ne + ge) * nn + node];
+    for (int v = 0; v < 3; ++v) Lp[v] = L.w[(v * Ne + ge) * nn + node];
   }
-  double Ss[S][2];               // source of hu, hv at each stage (IMEX)
   double Sb[2] = {0.0, 0.0};     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double P1 = 0.0, P2 = 0.0;     // sum_j (b_j/b_ref) h g d(h + b) (WB)
   // time averages sum_j (b_j/b_ref) of the exchange fields 0..5 in the fixed
@@ -179,44 +231,63 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
     for (int j = 0; j < n; ++j) fx_mad(a, X[fy][j][p], dyh[j], dyl[j]);
     return fx_sum(a);
   };
-  bool first = true;             // (resolved at compile time by unrolling)
-#pragma unroll
+#pragma unroll kStageUnroll
   for (int i = 0; i < S; ++i) {
+    if (i == (IMEX ? 0 : 1)) __syncthreads();   // the step sizes
     double cur[3];
 #pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      double acc = u0[v];
+    for (int v = 0; v < 3; ++v) cur[v] = u0[v];
+    if constexpr (CHAIN) {
+      if (i > 0) {
+        const double c = sz.e[i][i - 1];
 #pragma unroll
-      for (int j = 0; j < i; ++j)
-        if (TB::a(i, j) != 0.0) acc = fma(-(dt * TB::a(i, j)), Ls[j][v], acc);
-      if (IMEX && v > 0) {
-#pragma unroll
-        for (int j = 0; j < i; ++j)
-          if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j][v - 1], acc);
+        for (int v = 0; v < 3; ++v) cur[v] = fma(c, Lp[v], cur[v]);
       }
-      cur[v] = acc;
+    } else if constexpr (SHARED) {
+      for (int j = 0; j < i; ++j) {
+        if (!(local_nonzero<TB>() >> (8 * i + j) & 1)) continue;
+        const double c = sz.e[i][j];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) cur[v] = fma(c, sL[j][v][threadIdx.x], cur[v]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < S; ++j)
+        if (j < i && TB::a(i, j) != 0.0) {
+#pragma unroll
+          for (int v = 0; v < 3; ++v) cur[v] = fma(sz.e[i][j], rL[j][v], cur[v]);
+        }
     }
     if constexpr (IMEX) {
+#pragma unroll
+      for (int j = 0; j < S; ++j)
+        if (j < i && TB::ai(i, j) != 0.0) {
+          cur[1] = fma(sz.im[i][j], rS[j][0], cur[1]);
+          cur[2] = fma(sz.im[i][j], rS[j][1], cur[2]);
+        }
       // Chezy friction s = -C_f |m| m / h^2 on (hu, hv), point-implicit with
       // h fixed: m is parallel to the stage sum r and
       // |m| + dt a_ii C_f |m|^2 / h^2 = |r|, so
       // m = r 2 / (1 + sqrt(1 + 4 dt a_ii C_f |r| / h^2))
-      const double gcf = dt * TB::ai(i, i) * T.src_coef;
+      static_assert(TB::ai(0, 0) == TB::ai(S - 1, S - 1), "one diagonal coefficient");
+      const double gcf = sz.im[0][0] * T.src_coef;
       const double ih = drcp(cur[0]);
       const double ih2 = ih * ih;
       const double rx = cur[1], ry = cur[2];
       double nm = dsqrt_pos(fma(rx, rx, ry * ry));
-      if (TB::ai(i, i) != 0.0) {
-        const double qf = dsqrt_pos(fma(4.0 * gcf * ih2, nm, 1.0));
-        const double f = 2.0 * drcp(1.0 + qf);
-        cur[1] = rx * f;
-        cur[2] = ry * f;
-        nm *= f;
-      }
-      if (TB::need_S(i)) {
-        const double c = -(T.src_coef * ih2) * nm;
-        Ss[i][0] = c * cur[1];
-        Ss[i][1] = c * cur[2];
+      const double qf = dsqrt_pos(fma(4.0 * gcf * ih2, nm, 1.0));
+      const double f = 2.0 * drcp(1.0 + qf);
+      cur[1] = rx * f;
+      cur[2] = ry * f;
+      nm *= f;
+      const double c = -(T.src_coef * ih2) * nm;
+      rS[i][0] = c * cur[1];
+      rS[i][1] = c * cur[2];
+      // the implicit weights b_i equal the explicit ones b~_i
+      const double wd = (double)local_weight<TB>(i);
+      if (wd != 0.0) {
+        Sb[0] = fma(wd, rS[i][0], Sb[0]);
+        Sb[1] = fma(wd, rS[i][1], Sb[1]);
       }
     }
     if constexpr (STAGES) {
@@ -229,115 +300,108 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
           L.stages[(((int64_t)(i - 1) * 3 + v) * Nr + gr) * nn + node] = cur[v];
       }
     }
-    const int wi = TB::weight(i);
-    const double wd = wi;
-    // the stage's local operator feeds a later stage (for PRE 2 that of the
-    // first stage was loaded), its fluxes the time averages
-    const bool need_op = TB::feeds(i) && !(PRE == 2 && i == 0);
-    if (TB::feeds(i) || wi != 0) {
-      // the exchange fields at this node: the state and the fluxes
-      double f[6];
-      {
-        const double h = cur[0], mx = cur[1], my = cur[2];
-        const double r = drcp(h);
-        const double vx = mx * r, vy = my * r;
-        f[0] = h;
-        f[1] = mx;
-        f[2] = my;
-        if (WB) {
-          f[3] = mx * vx;
-          f[5] = my * vy;
-        } else {
-          const double ph = (h * h) * T.half_gravity;
-          f[3] = fma(mx, vx, ph);
-          f[5] = fma(my, vy, ph);
-        }
-        f[4] = mx * vy;
+    // (the first stage of SSP3-IMEX(4,3,3) has neither weight nor successor)
+    if (IMEX && i == 0) continue;
+    const int wi = local_weight<TB>(i);
+    // every stage but the last feeds a later one; the last one's fluxes enter
+    // the averages only
+    const bool need_op = i < S - 1 && !(PRE == 2 && i == 0);
+    // the exchange fields at this node: the state and the fluxes
+    double f[6];
+    {
+      const double h = cur[0], mx = cur[1], my = cur[2];
+      const double r = drcp(h);
+      const double vx = mx * r, vy = my * r;
+      f[0] = h;
+      f[1] = mx;
+      f[2] = my;
+      if (WB) {
+        f[3] = mx * vx;
+        f[5] = my * vy;
+      } else {
+        const double ph = (h * h) * T.half_gravity;
+        f[3] = fma(mx, vx, ph);
+        f[5] = fma(my, vy, ph);
       }
-      int mag[3];
-      mag[0] = fx_mag(f[0]);
-      mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
-      mag[2] = max(fx_mag(f[3]), max(fx_mag(f[4]), fx_mag(f[5])));
-      if (IMEX && first) {
-        // the traces of u^n, no stage value here, share the exponents
-        mag[0] = max(mag[0], fx_mag(u0[0]));
-        mag[1] = max(mag[1], max(fx_mag(u0[1]), fx_mag(u0[2])));
-      }
-      // one exponent per element and group of fields: the first stage's
-      // largest magnitudes with headroom, raised if a later stage exceeds
-      // them.  (The vote is also the barrier after the last reads of X.)
-      const bool over =
-          lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1] || mag[2] >> 20 > E[2]);
-      if (sync_or(over)) {
-        if (over) {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) atomicMax(&smag[le][k], mag[k]);
-        }
-        sync();
-        int d[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int e = fx_exp(smag[le][k]);
-          d[k] = e > E[k] ? e + kHeadroom - E[k] : 0;
-          E[k] += d[k];
-        }
-        if (!first) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) fx_rescale<WIDE>(A[k], B[k], d[group_of(k)]);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const bool used = need_op && !(k == 0 && !WB) || WB && (k == 0);
-        const long long v = fx_from<FB>(f[k], E[group_of(k)]);
-        const Fx x = fx_split(v);
-        if (wi != 0) fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
-        if (used && lane_ok) X[k][q][p] = x;
-      }
-      if (need_op || WB) {
-        sync();
-        double ncx = 0.0, ncy = 0.0;   // well-balanced: h g (h + b)_x, _y
-        if constexpr (WB) {
-          FxAcc hx, hy;
-          fx_mul(hx, X[0][q][0], dxh[0], dxl[0]);
-          fx_mul(hy, X[0][0][p], dyh[0], dyl[0]);
-#pragma unroll
-          for (int j = 1; j < n; ++j) {
-            fx_mad(hx, X[0][q][j], dxh[j], dxl[j]);
-            fx_mad(hy, X[0][j][p], dyh[j], dyl[j]);
-          }
-          const int b = E[0] + T.fx.kD - FB, z = fx_zero(E[0]);
-          ncx = cur[0] * fma(T.gravity, fx_to(fx_sum(hx), b, z), gbx);
-          ncy = cur[0] * fma(T.gravity, fx_to(fx_sum(hy), b, z), gby);
-          if (wi != 0) {
-            P1 = fma(wd, ncx, P1);
-            P2 = fma(wd, ncy, P2);
-          }
-        }
-        if (need_op) {
-          const int bm = E[1] + T.fx.kD - FB, bf = E[2] + T.fx.kD - FB;
-          const int zf = fx_zero(E[2]);
-          Ls[i][0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
-          const double l1 = fx_to(contract(3, 4), bf, zf), l2 = fx_to(contract(4, 5), bf, zf);
-          Ls[i][1] = WB ? l1 + ncx : fma(cur[0], gbx, l1);
-          Ls[i][2] = WB ? l2 + ncy : fma(cur[0], gby, l2);
-        }
-      }
-      if constexpr (PRE == 1) {
-        if (active) {
-#pragma unroll
-          for (int v = 0; v < 3; ++v) L.w[(v * Ne + ge) * nn + node] = Ls[0][v];
-        }
-        return;
-      }
-      if (wi != 0) first = false;
+      f[4] = mx * vy;
     }
-    if constexpr (IMEX) {
-      // the implicit weights b_i equal the explicit ones b~_i
-      if (wi != 0) {
-        Sb[0] = fma(wd, Ss[i][0], Sb[0]);
-        Sb[1] = fma(wd, Ss[i][1], Sb[1]);
+    int mag[3];
+    mag[0] = fx_mag(f[0]);
+    mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
+    mag[2] = max(fx_mag(f[3]), max(fx_mag(f[4]), fx_mag(f[5])));
+    if (IMEX) {
+      // the traces of u^n, no stage value here, share the exponents
+      mag[0] = max(mag[0], fx_mag(u0[0]));
+      mag[1] = max(mag[1], max(fx_mag(u0[1]), fx_mag(u0[2])));
+    }
+    // one exponent per element and group of fields: the first stage's
+    // largest magnitudes with headroom, raised if a later stage exceeds
+    // them.  (The vote is also the barrier after the last reads of X.)
+    const bool over =
+        lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1] || mag[2] >> 20 > E[2]);
+    if (sync_or(over)) {
+      if (over) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) atomicMax(&smag[le][k], mag[k]);
       }
+      sync();
+      int d[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int e = fx_exp(smag[le][k]);
+        d[k] = e > E[k] ? e + kHeadroom - E[k] : 0;
+        E[k] += d[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 6; ++k) fx_rescale<WIDE>(A[k], B[k], d[group_of(k)]);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const long long v = fx_from<FB>(f[k], E[group_of(k)]);
+      const Fx x = fx_split(v);
+      fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
+      // (h is contracted in the well-balanced form only)
+      if ((WB || k > 0) && lane_ok) X[k][q][p] = x;
+    }
+    if (need_op || WB) {
+      sync();
+      double ncx = 0.0, ncy = 0.0;   // well-balanced: h g (h + b)_x, _y
+      if constexpr (WB) {
+        FxAcc hx, hy;
+        fx_mul(hx, X[0][q][0], dxh[0], dxl[0]);
+        fx_mul(hy, X[0][0][p], dyh[0], dyl[0]);
+#pragma unroll
+        for (int j = 1; j < n; ++j) {
+          fx_mad(hx, X[0][q][j], dxh[j], dxl[j]);
+          fx_mad(hy, X[0][j][p], dyh[j], dyl[j]);
+        }
+        const int b = E[0] + T.fx.kD - FB, z = fx_zero(E[0]);
+        ncx = cur[0] * fma(T.gravity, fx_to(fx_sum(hx), b, z), gbx);
+        ncy = cur[0] * fma(T.gravity, fx_to(fx_sum(hy), b, z), gby);
+        const double wd = (double)wi;
+        P1 = fma(wd, ncx, P1);
+        P2 = fma(wd, ncy, P2);
+      }
+      if (need_op) {
+        const int bm = E[1] + T.fx.kD - FB, bf = E[2] + T.fx.kD - FB;
+        const int zf = fx_zero(E[2]);
+        Lp[0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
+        const double l1 = fx_to(contract(3, 4), bf, zf), l2 = fx_to(contract(4, 5), bf, zf);
+        Lp[1] = WB ? l1 + ncx : fma(cur[0], gbx, l1);
+        Lp[2] = WB ? l2 + ncy : fma(cur[0], gby, l2);
+      }
+    }
+    if constexpr (PRE == 1) {
+      if (active) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) L.w[(v * Ne + ge) * nn + node] = Lp[v];
+      }
+      return;
+    }
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      if (UNROLL) rL[i][v] = Lp[v];
+      if (SHARED && i < S - 1) sL[i][v][threadIdx.x] = Lp[v];
     }
   }
 
@@ -363,7 +427,7 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
   sync();
   {
     constexpr double b0 = TB::bref();
-    const double dtb0 = sdt[1];
+    const double dtb0 = sz.dtb;
     const int bm = E[1] + T.fx.kD - FB + kSumShift, bf = E[2] + T.fx.kD - FB + kSumShift;
     const int zf = fx_zero(E[2]);
     double V[3];
@@ -444,7 +508,7 @@ __global__ void __launch_bounds__(kBlockLocal, LIMIT ? 3 : CRKFR_LOCAL2D_MINB)
   if constexpr (LIMIT) {
     static_assert(!RES, "the limiter needs a step");
     sync();
-    limit_local_2d<N, GLL, WB>(L, u0, &sm[le * ES], node, lane_ok, active, ge, dt, sync);
+    limit_local_2d<N, GLL, WB>(L, u0, &sm[le * ES], node, lane_ok, active, ge, sz.dt, sync);
   }
 }
 

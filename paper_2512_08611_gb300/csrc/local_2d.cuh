@@ -35,6 +35,7 @@
 
 #include "device_common.cuh"
 #include "fixed_point.cuh"
+#include "launch.h"
 #include "limit_2d.cuh"
 
 namespace crkfr {
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
   };
 
+  chain_begin();
   // the step size (a division) and its products by the block's first warp;
   // the others start on the first stage, which needs neither
   if (threadIdx.x < 32) {
@@ -519,13 +521,13 @@ int launch_local_t(const Launch2D& L, cudaStream_t s) {
     return (int)cudaErrorInvalidValue;
   const int64_t blocks = ((L.row_end - L.row_begin) * L.Ex + per_block - 1) / per_block;
   if (blocks > 0x7fffffff) return (int)cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)blocks);
   if constexpr (LIMIT)
-    k_local_2d<N, GLL, false, IMEX, WB, true><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
+    return launch_chained(k_local_2d<N, GLL, false, IMEX, WB, true>, grid, kBlockLocal, s, L);
   else if (L.ctl.residual)
-    k_local_2d<N, GLL, true, IMEX, WB><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
+    return launch_chained(k_local_2d<N, GLL, true, IMEX, WB>, grid, kBlockLocal, s, L);
   else
-    k_local_2d<N, GLL, false, IMEX, WB><<<(unsigned)blocks, kBlockLocal, 0, s>>>(L);
-  return (int)cudaGetLastError();
+    return launch_chained(k_local_2d<N, GLL, false, IMEX, WB>, grid, kBlockLocal, s, L);
 }
 
 template <bool IMEX, bool WB, bool LIMIT = false>

@@ -50,6 +50,7 @@
 
 #include "device_common.cuh"
 #include "fixed_point.cuh"
+#include "launch.h"
 
 namespace crkfr {
 namespace {
@@ -168,16 +169,15 @@ __device__ __forceinline__ double element_min(double v, int le, int p, int lane)
 // tables (dx = 1: D, l(0), l(1), 0.5 g'); xs = 1/dx scales the local operator
 // and the corrections through the scalar coefficients only (stage coefficients
 // dt a_ij xs, update coefficient dt b_ref xs), so one table serves meshes of
-// any dx.  Every element's arithmetic is the same for any block size.
+// any dx.  Every element's arithmetic is the same for any block size.  (No
+// __restrict__: the loads must not move above chain_begin().)
 template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
 __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
-                                             const double* __restrict__ u_in,
-                                             double* __restrict__ u_out,
-                                             const double* __restrict__ snode,
-                                             const double* __restrict__ sface, int64_t E,
+                                             const double* u_in, double* u_out,
+                                             const double* snode, const double* sface, int64_t E,
                                              int64_t tile, DevState* st, const StepCtl& ctl,
                                              bool first_tile, const LimitArgs& LA = LimitArgs{},
-                                             const double* __restrict__ ghost = nullptr) {
+                                             const double* ghost = nullptr) {
   using TB = Tab<N, IMEX>;
   using SY = Sys1D<SYS>;
   constexpr int n = N + 1;
@@ -706,6 +706,7 @@ __host__ __device__ constexpr int min_blocks_1d() {
 template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
 __global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D,
                                   LIMIT ? 4 : min_blocks_1d<N>()) k_step_1d(const Launch1D L) {
+  chain_begin();
   step_1d_tile<SYS, N, GLL, RES, IMEX, LIMIT>(L.tab, L.xs, L.u_in, L.u_out, L.snode, L.sface, L.E,
                                               blockIdx.x, L.st, L.ctl, blockIdx.x == 0, L.lim,
                                               L.ghost);
@@ -763,8 +764,7 @@ int launch_step_t(const Launch1D& L, cudaStream_t s) {
   if (L.ctl.residual) {
     const unsigned blocks = tiles_1d(L.E, kBlock1D, N + 1);
     if (!blocks) return (int)cudaErrorInvalidConfiguration;
-    k_step_1d<SYS, N, GLL, true, IMEX><<<blocks, kBlock1D, 0, s>>>(L);
-    return (int)cudaGetLastError();
+    return launch_chained(k_step_1d<SYS, N, GLL, true, IMEX>, dim3(blocks), kBlock1D, s, L);
   }
   // SMs of the GPU (asked once; 0 if the query failed: then the largest block)
   static const int sms = [] {
@@ -781,8 +781,7 @@ int launch_step_t(const Launch1D& L, cudaStream_t s) {
                                          : kBlock1D;
   const unsigned blocks = tiles_1d(L.E, threads, N + 1);
   if (!blocks) return (int)cudaErrorInvalidConfiguration;
-  k_step_1d<SYS, N, GLL, false, IMEX><<<blocks, (unsigned)threads, 0, s>>>(L);
-  return (int)cudaGetLastError();
+  return launch_chained(k_step_1d<SYS, N, GLL, false, IMEX>, dim3(blocks), (unsigned)threads, s, L);
 }
 
 template <int SYS, bool IMEX>

@@ -34,14 +34,10 @@ __device__ __forceinline__ long long seed_times(unsigned r, long long s) {
          (long long)(((unsigned long long)r * (unsigned)s) >> 32);
 }
 
-// 1/x for FP64 x: with the significand m and a seed r of 1/m, p = m r - 1 is
-// formed exactly (2^75 p fits 64 bits since |p| < 2^-20), and 1/m = r (1 - p +
-// p^2) up to p^3 < 2^-60.  Zero, denormal and non-finite x, and x whose
-// reciprocal is not normal, take the IEEE division.
-__device__ __forceinline__ double drcp(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int ex = (int)(hi >> 20) & 0x7ff;
-  if ((unsigned)(ex - 1) > 2043u) return 1.0 / x;
+// 2^62 / m for the significand m in [1, 2) of a normal x = (hi, lo): with a
+// seed r of 1/m, p = m r - 1 is formed exactly (2^75 p fits 64 bits since |p| <
+// 2^-20), and 1/m = r (1 - p + p^2) up to p^3 < 2^-60.
+__device__ __forceinline__ unsigned long long recip_bits(unsigned hi, unsigned lo) {
   const unsigned mh = (hi & 0xfffffu) | 0x100000u;
   float f = __int_as_float((int)((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u));
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(f));
@@ -50,8 +46,16 @@ __device__ __forceinline__ double drcp(double x) {
       (long long)((unsigned long long)lo * r + ((unsigned long long)(mh * r) << 32));
   const int ph = (int)(p >> 25);                              // 2^50 p
   const long long s = (((long long)ph * ph) >> 25) - p;       // 2^75 (p^2 - p)
-  const unsigned long long R = ((unsigned long long)r << 39) +
-                               (unsigned long long)(seed_times(r, s) >> 4) + 0x100u;   // 2^62 / m
+  return ((unsigned long long)r << 39) + (unsigned long long)(seed_times(r, s) >> 4);
+}
+
+// 1/x for FP64 x.  Zero, denormal and non-finite x, and x whose reciprocal is
+// not normal, take the IEEE division.
+__device__ __forceinline__ double drcp(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int ex = (int)(hi >> 20) & 0x7ff;
+  if ((unsigned)(ex - 1) > 2043u) return 1.0 / x;
+  const unsigned long long R = recip_bits(hi, lo) + 0x100u;
   const unsigned oh = ((unsigned)(R >> 41) + ((unsigned)(2044 - ex) << 20)) | (hi & 0x80000000u);
   return __hiloint2double((int)oh, (int)(unsigned)(R >> 9));
 }

@@ -24,6 +24,7 @@
 #include <cstdint>
 
 #include "crkfr_internal.h"
+#include "device_common.cuh"
 
 namespace crkfr {
 namespace {
@@ -67,6 +68,94 @@ __device__ __forceinline__ long long fx_from(double x, int E) {
       : "+l"(m)
       : "r"(E - e), "r"(hi));
   return m;
+}
+
+// |x| = s 2^(e - 1085), s < 2^63 (0 for zeros and denormals); neg the sign bit
+struct FxSig {
+  unsigned long long s;
+  int e, neg;
+};
+__device__ __forceinline__ FxSig fx_sig(double x) {
+  const int hi = __double2hiint(x);
+  const int e = (hi & 0x7fffffff) >> 20;
+  const unsigned mh = (unsigned)((hi & 0xfffff) | 0x100000);
+  const unsigned long long m =
+      ((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << 10;
+  return FxSig{e == 0 ? 0 : m, e, hi};
+}
+
+// m >> sh with the sign bit of neg applied (sh >= 0; 64 or more give 0)
+__device__ __forceinline__ long long fx_signed(unsigned long long m, int sh, int neg) {
+  long long r;
+  asm("{\n\t.reg .pred n;\n\tshr.u64 %0, %1, %2;\n\tsetp.lt.s32 n, %3, 0;\n\t"
+      "@n neg.s64 %0, %0;\n\t}"
+      : "=l"(r)
+      : "l"(m), "r"(sh), "r"(neg));
+  return r;
+}
+
+// (a b) 2^-64 less at most 2, for a and b below 2^63: three IMAD.WIDE
+__device__ __forceinline__ unsigned long long fx_mulhi(unsigned long long a,
+                                                       unsigned long long b) {
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  const unsigned bh = (unsigned)(b >> 32), bl = (unsigned)b;
+  const unsigned long long mid = (unsigned long long)ah * bl + (unsigned long long)al * bh;
+  return (unsigned long long)ah * bh + (mid >> 32);
+}
+__device__ __forceinline__ unsigned long long fx_sqrhi(unsigned long long a) {
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  return (unsigned long long)ah * ah + ((unsigned long long)ah * al >> 31);
+}
+
+// Shallow-water fluxes of a node in the fixed point of their element.  With
+// FP64 products and a conversion each they cost seven FP64 instructions a
+// stage (64 cycles each); the significands of h, hu, hv are at hand for the
+// conversion of the state, a product of two is three IMAD.WIDE, and 1/h stays
+// the integer that the reciprocal ends in.  Nothing is rounded to 53 bits on
+// the way: each product is exact up to 2^-57 of itself and then truncated to
+// the element's fixed point.
+//
+// The exponent is bounded without the products: the bits of a double read as a
+// fixed-point number exceed 1023 + log2 by at most 0 and fall short by at most
+// 0.087 (Mitchell's logarithm), and by another 1/16 cut to 4 fraction bits.
+// fx_flux_mag adds those of the factors: m m / h lies below the sum by at most
+// 2 (0.087 + 1/16) = 0.30, h h g/2 by 0.45; the sum of the two terms adds 1
+// and all of it is covered by 24/16.
+__device__ __forceinline__ int fx_log(double x) { return fx_mag(x) >> 16; }
+
+// magnitude of the group (as fx_mag) for the largest fx_log lm of the momenta;
+// pressure: the fluxes hold h^2 g/2, lhg = fx_log(g/2).  h must be normal for
+// 1/h to be finite: the group counts as non-finite otherwise.
+template <bool PRESSURE>
+__device__ __forceinline__ int fx_flux_mag(double h, int lm, int lhg) {
+  const int lh = fx_log(h);
+  int l = 2 * lm - lh;
+  if (PRESSURE) l = max(l, 2 * lh + lhg - 2 * (1023 << 4));
+  l = min(max(l + 24, 0), 0x7ff0);
+  return ((unsigned)((lh >> 4) - 1) > 2045u ? 0x7ff0 : l) << 16;
+}
+
+// 2^61 |m| / |h| up to their exponents
+__device__ __forceinline__ unsigned long long fx_velocity(unsigned long long R, const FxSig& m) {
+  return fx_mulhi(m.s, R);
+}
+// m v for v = k / h: sign and exponent from m, k, h; FB bits at exponent E.
+// (The product is in units of 2^-60 and at least 1/8 where m, k are not zero,
+// so the bound above leaves the shift non-negative.)
+template <int FB>
+__device__ __forceinline__ long long fx_momentum_flux(const FxSig& m, unsigned long long v,
+                                                      const FxSig& k, const FxSig& h, int E) {
+  return fx_signed(fx_mulhi(m.s, v), 60 - FB + E - (m.e + k.e - h.e + 1), m.neg ^ k.neg ^ h.neg);
+}
+// h^2 g/2
+template <int FB>
+__device__ __forceinline__ long long fx_pressure(const FxSig& h, const FxSig& hg, int E) {
+  return fx_signed(fx_mulhi(fx_sqrhi(h.s), hg.s), 61 - FB + E - (2 * h.e + hg.e - 2044), hg.neg);
+}
+// a value of which fx_sig is at hand
+template <int FB>
+__device__ __forceinline__ long long fx_from(const FxSig& x, int E) {
+  return fx_signed(x.s, 63 - FB + E - x.e, x.neg);
 }
 
 __device__ __forceinline__ Fx fx_split(long long v) {

@@ -12,17 +12,21 @@
 // normal momentum at t^n (Eqs. time.avg.soln, combined.wave.speed,
 // good.numflux.non.cons).
 //
-// The pointwise arithmetic (stage values, fluxes) is FP64; the contractions
-// with D_x, D_y and the end-point rows, which were 60 % of the FP64
-// instructions, and the time averages run in block fixed point on the integer
-// pipe (fixed_point.cuh).  D is applied to the time-averaged fluxes once
-// instead of accumulating every stage's operator, so the last stage needs no
-// contraction.  On a 1024 x 1024 mesh at N = 3 the kernel takes 2.4 ms (FP64
-// pipe 77 % busy, integer pipes 35 %) against 6.4 ms with FP64 chains (one
-// thread per element row, FP64 pipe 96 %).  One thread per row in fixed point
-// took 4.2 ms: 255 registers and two warps per scheduler left the latencies
-// open, and 9700 instructions a warp missed the instruction cache; a thread
-// per node takes 96 registers and a quarter of the code.
+// The stage sums are FP64; the contractions with D_x, D_y and the end-point
+// rows, which were 60 % of the FP64 instructions, the time averages and the
+// fluxes run in block fixed point on the integer pipe (fixed_point.cuh).  D is
+// applied to the time-averaged fluxes once instead of accumulating every
+// stage's operator, so the last stage needs no contraction.  On a 1024 x 1024
+// mesh at N = 3 the kernel takes 1.94 ms (FP64 pipe 33 % busy, the multiplier
+// of the integer products 70 %, 0.64 instructions per cycle and scheduler)
+// against 6.4 ms with FP64 chains (one thread per element row, FP64 pipe 96
+// %).  One thread per row in fixed point took 4.2 ms: 255 registers and two
+// warps per scheduler left the latencies open, and 9700 instructions a warp
+// missed the instruction cache; a thread per node takes a quarter of the
+// code.  With FP64 fluxes, seven FP64 instructions a stage and each result
+// converted, two steps took 5.45 ms (FP64 pipe 77 % busy), with fixed-point
+// ones 5.22 ms; 401 x 307 well-balanced at N = 4 2.08 and 1.95 ms, 640 x 384
+// limited 3.28 and 3.01 ms, 512 x 512 with friction 2.52 and 2.28 ms.
 //
 // The well-balanced form (WB) has pressure-free fluxes and the
 // non-conservative terms g h D_x (h + b), g h D_y (h + b).
@@ -309,28 +313,11 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     // the averages only
     const bool need_op = i < S - 1 && !(PRE == 2 && i == 0);
     // the exchange fields at this node: the state and the fluxes
-    double f[6];
-    {
-      const double h = cur[0], mx = cur[1], my = cur[2];
-      const double r = drcp(h);
-      const double vx = mx * r, vy = my * r;
-      f[0] = h;
-      f[1] = mx;
-      f[2] = my;
-      if (WB) {
-        f[3] = mx * vx;
-        f[5] = my * vy;
-      } else {
-        const double ph = (h * h) * T.half_gravity;
-        f[3] = fma(mx, vx, ph);
-        f[5] = fma(my, vy, ph);
-      }
-      f[4] = mx * vy;
-    }
+    const FxSig sh = fx_sig(cur[0]), sx = fx_sig(cur[1]), sy = fx_sig(cur[2]);
     int mag[3];
-    mag[0] = fx_mag(f[0]);
-    mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
-    mag[2] = max(fx_mag(f[3]), max(fx_mag(f[4]), fx_mag(f[5])));
+    mag[0] = fx_mag(cur[0]);
+    mag[1] = max(fx_mag(cur[1]), fx_mag(cur[2]));
+    mag[2] = fx_flux_mag<!WB>(cur[0], mag[1] >> 16, fx_log(T.half_gravity));
     if (IMEX) {
       // the traces of u^n, no stage value here, share the exponents
       mag[0] = max(mag[0], fx_mag(u0[0]));
@@ -357,9 +344,26 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
 #pragma unroll
       for (int k = 0; k < 6; ++k) fx_rescale<WIDE>(A[k], B[k], d[group_of(k)]);
     }
+    long long f[6];
+    {
+      const unsigned long long R = recip_bits((unsigned)__double2hiint(cur[0]),
+                                              (unsigned)__double2loint(cur[0]));
+      const unsigned long long vx = fx_velocity(R, sx), vy = fx_velocity(R, sy);
+      f[0] = fx_from<FB>(sh, E[0]);
+      f[1] = fx_from<FB>(sx, E[1]);
+      f[2] = fx_from<FB>(sy, E[1]);
+      f[3] = fx_momentum_flux<FB>(sx, vx, sx, sh, E[2]);
+      f[4] = fx_momentum_flux<FB>(sx, vy, sy, sh, E[2]);
+      f[5] = fx_momentum_flux<FB>(sy, vy, sy, sh, E[2]);
+      if (!WB) {
+        const long long ph = fx_pressure<FB>(sh, fx_sig(T.half_gravity), E[2]);
+        f[3] += ph;
+        f[5] += ph;
+      }
+    }
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const long long v = fx_from<FB>(f[k], E[group_of(k)]);
+      const long long v = f[k];
       const Fx x = fx_split(v);
       fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
       // (h is contracted in the well-balanced form only)

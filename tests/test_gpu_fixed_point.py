@@ -130,3 +130,72 @@ def test_non_finite_stays_in_its_neighbourhood(crk, N, value):
     for e in ((3, 4), (2, 4), (4, 4), (3, 3), (3, 5)):
         touched[e] = True
     assert np.array_equal(got[:, ~touched], good[:, ~touched])
+
+
+# The fluxes in the element's fixed point: momenta far below and far above
+# sqrt(g h) h, either sign, and depths spread over a factor of e^4 inside the
+# mesh, so that the bound of the flux exponent is met from both of its terms.
+# Tolerance as for the scales above: |dt R| stays below the state's norm.
+@pytest.mark.parametrize("system", ["swe2d", "swe2d_wb"])
+@pytest.mark.parametrize("N", [1, 3, 4])
+@pytest.mark.parametrize("froude", [1e-9, 1e-2, 1.0, 40.0])
+def test_flux_ratios(crk, system, N, froude):
+    from oracle.crkfr import Scheme2D
+    from oracle.systems import ShallowWater2D, ShallowWater2DWB
+    Ex, Ey = 7, 5
+    sch, u, b, L = case_2d(N, "gl", Ex, Ey)
+    if system == "swe2d_wb":
+        sch = Scheme2D(ShallowWater2DWB(G), N, L / Ex, L / Ey, family="gl")
+    x, y, _, _ = positions_2d(sch.basis, Ex, Ey, L)
+    k = 2 * np.pi / L
+    h = np.exp(2 * np.sin(k * x) * np.sin(k * y + 1.0)) + 0 * b
+    v = froude * np.sqrt(G * h)
+    u = np.stack([h, h * v * np.cos(k * (x + y)), -h * v * np.sin(k * (x - y) + 0.5)])
+    dt = 0.2 * sch.compute_dt(u, b, golden_cfl(N, "gl"), 0.5)
+    s = crk.Solver(system, N, nodes="gl", gravity=G, cfl_safety=0.5,
+                   cfl_number=golden_cfl(N, "gl"))
+    s.set_mesh([Ex, Ey], [0.0, 0.0], [L, L])
+    s.set_coefficients(to_dev(b))
+    d = to_dev(u)
+    s.step(d, dt, 1)
+    got, want = to_host(d), sch.step(u, b, dt)
+    for w in range(3):
+        assert rel_l2(got[w], want[w]) < 10 * TOL
+
+
+# the same for the 1D step
+@pytest.mark.parametrize("system", ["swe1d", "swe1d_wb"])
+@pytest.mark.parametrize("N,E", [(0, 40), (2, 3), (4, 61)])
+@pytest.mark.parametrize("froude", [1e-9, 1.0, 40.0])
+def test_flux_ratios_1d(crk, system, N, E, froude):
+    from oracle.crkfr import Scheme1D
+    from oracle.systems import ShallowWater1D, ShallowWater1DWB
+    L = 10.0
+    sch = Scheme1D((ShallowWater1DWB if system == "swe1d_wb" else ShallowWater1D)(G), N, L / E)
+    x = (np.arange(E)[:, None] + sch.basis.xi[None, :]) * (L / E)
+    k = 2 * np.pi / L
+    b = 0.2 * np.sin(k * x)
+    h = np.exp(2 * np.sin(k * x + 1.0))
+    u = np.stack([h, froude * h * np.sqrt(G * h) * np.cos(k * x)])
+    dt = 0.2 * sch.compute_dt(u, b, golden_cfl(N, "gl"), 0.5)
+    s = crk.Solver(system, N, nodes="gl", gravity=G, cfl_safety=0.5,
+                   cfl_number=golden_cfl(N, "gl"))
+    s.set_mesh([E], [0.0], [L])
+    s.set_coefficients(to_dev(b))
+    d = to_dev(u)
+    s.step(d, dt, 1)
+    got, want = to_host(d), sch.step(u, b, dt)
+    for w in range(2):
+        assert rel_l2(got[w], want[w]) < 10 * TOL
+
+
+# depths that have no finite reciprocal
+@pytest.mark.parametrize("value", [0.0, np.nan, np.inf])
+def test_non_finite_depth(crk, value):
+    sch, u, b, L = case_2d(3, "gl", 5, 5)
+    dt = sch.compute_dt(u, b, golden_cfl(3, "gl"), 0.5)
+    u[0, 2, 2, 1, 1] = value
+    s, got = run(crk, sch, 3, "gl", u, b, L, 5, 5, dt)
+    with pytest.raises(crk.CrkfrError):
+        s.status()
+    assert np.isnan(got[1:, 2, 2]).all()

@@ -142,7 +142,7 @@ def test_non_finite_stays_in_its_neighbourhood(crk, N, value):
 def test_flux_ratios(crk, system, N, froude):
     from oracle.crkfr import Scheme2D
     from oracle.systems import ShallowWater2D, ShallowWater2DWB
-    Ex, Ey = 7, 5
+    Ex, Ey = 27, 25   # (fine enough for positive depths at the faces)
     sch, u, b, L = case_2d(N, "gl", Ex, Ey)
     if system == "swe2d_wb":
         sch = Scheme2D(ShallowWater2DWB(G), N, L / Ex, L / Ey, family="gl")
@@ -159,13 +159,14 @@ def test_flux_ratios(crk, system, N, froude):
     d = to_dev(u)
     s.step(d, dt, 1)
     got, want = to_host(d), sch.step(u, b, dt)
+    assert np.isfinite(want).all()
     for w in range(3):
         assert rel_l2(got[w], want[w]) < 10 * TOL
 
 
 # the same for the 1D step
 @pytest.mark.parametrize("system", ["swe1d", "swe1d_wb"])
-@pytest.mark.parametrize("N,E", [(0, 40), (2, 3), (4, 61)])
+@pytest.mark.parametrize("N,E", [(0, 40), (2, 33), (4, 61)])
 @pytest.mark.parametrize("froude", [1e-9, 1.0, 40.0])
 def test_flux_ratios_1d(crk, system, N, E, froude):
     from oracle.crkfr import Scheme1D
@@ -185,6 +186,7 @@ def test_flux_ratios_1d(crk, system, N, E, froude):
     d = to_dev(u)
     s.step(d, dt, 1)
     got, want = to_host(d), sch.step(u, b, dt)
+    assert np.isfinite(want).all()
     for w in range(2):
         assert rel_l2(got[w], want[w]) < 10 * TOL
 

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <limits>
@@ -499,17 +500,22 @@ crkfr_status run_steps(crkfr_ctx* c, double* u, double dt, int64_t nsteps, doubl
       cur = 1;
     }
     Launch1D L = make1d(c);
-    for (int64_t k = 0; k < nsteps; ++k) {
+    // (a profile has a step's duration per record)
+    const int64_t per = c->prof ? 1 : steps_per_launch_1d(L);
+    for (int64_t k = 0, m; k < nsteps; k += m) {
+      m = std::min(per, nsteps - k);
       ctl.slot_read = (int)(c->nstep % 3);
       ctl.slot_write = (int)((c->nstep + 1) % 3);
       ctl.slot_reset = (int)((c->nstep + 2) % 3);
       ctl.tslot = (int)(c->nstep % 2);
       // (the last step's rate would go unread: every call starts from the
       // rate of its input)
-      ctl.want_rate = cfl_mode && k + 1 < nsteps ? 1 : 0;
+      ctl.want_rate = cfl_mode && k + m < nsteps ? 1 : 0;
       L.ctl = ctl;
       L.u_in = bufs[cur];
       L.u_out = bufs[cur ^ 1];
+      L.steps = (int)m;
+      L.u_next = bufs[cur];
       if (c->limit_mode == CRKFR_LIMITER_BLEND) {
         int ea = timed(c, CRKFR_KERNEL_INDICATOR, s,
                        [&] { return launch_alpha_1d(L, c->d_alpha_raw, s); });
@@ -519,8 +525,8 @@ crkfr_status run_steps(crkfr_ctx* c, double* u, double dt, int64_t nsteps, doubl
       int e = timed(c, CRKFR_KERNEL_STEP_1D, s, [&] { return launch_step_1d(L, s); });
       if (e) return cuda_fail(c, e, "1D step kernel");
       c->launches += 1;
-      c->nstep += 1;
-      cur ^= 1;
+      c->nstep += m;
+      cur ^= (int)(m & 1);
     }
   } else {
     Launch2D L = make2d(c);

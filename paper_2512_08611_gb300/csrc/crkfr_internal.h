@@ -147,6 +147,20 @@ __host__ __device__
 #endif
 constexpr int tile_elements_1d(int threads, int n) { return threads / 32 * (32 / n) - 2; }
 
+// Threads per block of a mesh of E elements that steps as one cluster of at
+// most 8 blocks (the portable size), 0 if it is too large.  More than 128
+// threads would put a second warp on an SM sub-partition, and the step's time
+// is that of a sub-partition's FP64 and integer instructions.
+constexpr int64_t kClusterBlocks = 8;
+constexpr int kMaxClusterThreads = 128;
+// (bounds the time of a launch, some 4 us a step)
+constexpr int64_t kClusterSteps = 1024;
+constexpr int cluster_threads_1d(int64_t E, int n) {
+  for (int t = 32; t <= kMaxClusterThreads; t *= 2)
+    if (tile_elements_1d(t, n) > 0 && E <= kClusterBlocks * tile_elements_1d(t, n)) return t;
+  return 0;
+}
+
 // Launchers (kernels_1d.cu / kernels_2d.cu).  Return cudaError_t as int.
 struct Launch1D {
   int system;  // crkfr_system
@@ -173,7 +187,16 @@ struct Launch1D {
   // threads per block of the unlimited step (at most kMaxBlock1D): 0 = chosen
   // per mesh, else 64, 96 or 128
   int tile_threads;
+  // steps of one launch (at most steps_per_launch_1d; 0 and 1: one step): the
+  // first reads u_in and writes u_out, the next ones alternate between u_next
+  // and u_out.  ctl is the first step's, but for want_rate, the last one's.
+  int steps;
+  double* u_next;
 };
+
+// Steps that one launch may take: 1, or kClusterSteps where the whole mesh is
+// one cluster (launch_steps_t in step_1d.cuh).
+int64_t steps_per_launch_1d(const Launch1D& L);
 #ifdef __CUDACC__
 __host__ __device__
 #endif

@@ -155,6 +155,11 @@ int base_system(int system) {
 
 }  // namespace
 
+int64_t steps_per_launch_1d(const Launch1D& L) {
+  const bool one = L.lim.mode != 0 || L.ghost || L.tile_threads > 0 || L.ctl.residual;
+  return !one && cluster_threads_1d(L.E, L.N + 1) ? kClusterSteps : 1;
+}
+
 int launch_step_1d(const Launch1D& L, void* stream) {
   if (L.lim.mode != 0 && !L.ctl.residual) return launch_step_1d_limit(L, stream);
   if (L.system == CRKFR_SYS_SWE_1D_WB) return launch_step_1d_wb(L, stream);

@@ -12,24 +12,42 @@ namespace crkfr {
 // us of the gap between two kernels: 20 steps of 100 elements 132 -> 109 us, 8
 // steps of 65 x 47 elements (two kernels each) 208 -> 188 us.  In a stream
 // capture the launch is an ordinary one.
+// `cluster`: the grid as one cluster of that many blocks (0: none).
 template <class... P>
-int launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, P... args) {
+int launch_chained_cluster(void (*kernel)(P...), dim3 grid, unsigned block, unsigned cluster,
+                           cudaStream_t s, P... args) {
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   const bool plain = cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
                      capture != cudaStreamCaptureStatusNone;
   if (plain) cudaGetLastError();
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2] = {};
+  unsigned attrs = 0;
+  if (cluster) {
+    attr[attrs].id = cudaLaunchAttributeClusterDimension;
+    attr[attrs].val.clusterDim.x = cluster;
+    attr[attrs].val.clusterDim.y = 1;
+    attr[attrs].val.clusterDim.z = 1;
+    ++attrs;
+  }
+  if (!plain) {
+    attr[attrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[attrs].val.programmaticStreamSerializationAllowed = 1;
+    ++attrs;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = plain ? 0 : 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = attrs;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   const cudaError_t last = cudaGetLastError();
   return (int)(e != cudaSuccess ? e : last);
+}
+
+template <class... P>
+int launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, P... args) {
+  return launch_chained_cluster<P...>(kernel, grid, block, 0, s, args...);
 }
 
 #ifdef __CUDACC__

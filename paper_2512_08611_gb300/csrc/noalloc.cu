@@ -144,7 +144,9 @@ extern "C" crkfr_status crkfr_step_1d_noalloc(const crkfr_config* cfg, int64_t n
   ctl.cs_cfl = cfg->cfl_safety * cfl;
   ctl.t_end = INFINITY;
   ctl.want_rate = cfl_mode ? 1 : 0;
-  for (int64_t k = 0; k < nsteps; ++k) {
+  const int64_t per = steps_per_launch_1d(L);
+  for (int64_t k = 0, m; k < nsteps; k += m) {
+    m = nsteps - k < per ? nsteps - k : per;
     ctl.slot_read = (int)(k % 3);
     ctl.slot_write = (int)((k + 1) % 3);
     ctl.slot_reset = (int)((k + 2) % 3);
@@ -152,9 +154,13 @@ extern "C" crkfr_status crkfr_step_1d_noalloc(const crkfr_config* cfg, int64_t n
     L.ctl = ctl;
     L.u_in = src;
     L.u_out = bufs[cur_dst];
+    L.steps = (int)m;
+    L.u_next = bufs[cur_dst ^ 1];
     if (launch_step_1d(L, s)) return CRKFR_ERR_CUDA;
-    src = bufs[cur_dst];
-    cur_dst ^= 1;
+    // (the last of m steps wrote the first one's target or the other buffer)
+    const int last = m & 1 ? cur_dst : cur_dst ^ 1;
+    src = bufs[last];
+    cur_dst = last ^ 1;
   }
   return CRKFR_OK;
 }

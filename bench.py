@@ -207,13 +207,19 @@ def l2_note(wl):
         size = "%.2f GB" % (ws / 1e9) if ws >= 1e9 else "%.0f MB" % (ws / 1e6)
         return "no flush: state + work buffers (%s) exceed the 129 MB L2" % size
     return ("no flush: state + work buffers (%.0f MB) stay in the 129 MB L2 between steps, as "
-            "in any run on this mesh; the step is FP64-bound" % (ws / 1e6))
+            "in any run on this mesh; the step is bound by arithmetic" % (ws / 1e6))
 
 
 # ---------------------------------------------------------------------------
 # profiles/ summary of the dominant kernel: dram traffic, valid only while the
 # kernel source is unchanged
 # ---------------------------------------------------------------------------
+# what the operation counts mean for these kernels
+FIXED_POINT_NOTE = ("operation count of the FP64 formulation; the products with constant "
+                    "matrices, the time averages and the fluxes run as 60-bit block fixed point "
+                    "on the integer pipe, so the fraction of the FP64 pipe's peak can exceed 1")
+
+
 def kernel_source_hash(files):
     h = hashlib.sha256()
     for f in files:
@@ -539,6 +545,7 @@ def run_ours(args, wl):
                      "traffic": traffic, "avg_launch_ms": avg_ms,
                      "flops_per_launch": flops,
                      "peak_source": "FP64: 152 SMs x 2 FMA/clk x 2 flop x 2070 MHz",
+                     "work_note": FIXED_POINT_NOTE,
                      **({"flops_note": "the unlimited step's operation count: a lower bound "
                                        "of the limited kernel's work"}
                         if wl.limiter and wl.dim == 1 else
@@ -735,7 +742,8 @@ def run_ensemble(args):
                      "traffic": profiled_traffic("k_step_1d_batch__ensemble256.md",
                                                  ["step_1d.cuh", "device_common.cuh", "tableau.h"],
                                                  1.0),
-                     "traffic_unit": "bytes per step (the degree classes' launches)"},
+                     "traffic_unit": "bytes per step (the degree classes' launches)",
+                     "work_note": FIXED_POINT_NOTE},
         "gpu_launches": launches, "clocks": clk}))
 
 

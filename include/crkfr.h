@@ -456,8 +456,10 @@ crkfr_status crkfr_set_limiter(crkfr_ctx* ctx, int32_t mode, double alpha);
  * thread (elements within a warp) and each block all its elements but two
  * recomputed neighbours.  0 (the default): chosen per mesh among 32, 64, 128
  * and 256 so that the busiest SM sub-partition gets the fewest warps; 64, 96
- * or 128: that size for every step.  Only the schedule changes, not a bit of
- * the results.  Applies to the unlimited step of 1D contexts (crkfr_step,
+ * or 128: that size, and a launch for every step (by default the steps of one
+ * call on a mesh of at most 8 blocks of 128 threads are one launch, up to 1024
+ * of them, outside profiling).  Only the schedule changes, not a bit of the
+ * results.  Applies to the unlimited step of 1D contexts (crkfr_step,
  * crkfr_advance, crkfr_step_host, crkfr_step_local); the limited step runs
  * 128-thread and crkfr_residual 256-thread blocks.  CRKFR_ERR_UNSUPPORTED on a
  * 2D context, CRKFR_ERR_ARG for other values; kept across crkfr_set_mesh. */

@@ -238,8 +238,6 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
   T->inv_b0 = 1.0 / T->b0;
   T->inv_gravity = gravity > 0.0 ? 1.0 / gravity : 0.0;
   T->sqrt_gravity = gravity > 0.0 ? std::sqrt(gravity) : 0.0;
-  for (int q = 0; q < n; ++q)
-    for (int p = 0; p < n; ++p) T->w2[q][p] = b.w[q] * b.w[p];
   double rx = 0.0, ry = 0.0, rl = 0.0, sl0 = 0.0, sl1 = 0.0;
   for (int i = 0; i < n; ++i) {
     // rows and columns: the adjoint contracts with the transposes
@@ -270,7 +268,7 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
       fx_coef(T->Dx[i][j], sD, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);
       fx_coef(T->Dy[i][j], sD, &F.Dy_hi[i][j], &F.Dy_lo[i][j]);
     }
-    for (int j = 0; j < n; ++j) fx_coef(T->w2[i][j], 60, &F.w2_hi[i][j], &F.w2_lo[i][j]);
+    for (int j = 0; j < n; ++j) fx_coef(b.w[i] * b.w[j], 60, &F.w2_hi[i][j], &F.w2_lo[i][j]);
     fx_coef(T->l0[i], sL, &F.l0_hi[i], &F.l0_lo[i]);
     fx_coef(T->l1[i], sL, &F.l1_hi[i], &F.l1_lo[i]);
   }

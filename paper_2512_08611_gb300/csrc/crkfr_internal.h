@@ -61,7 +61,6 @@ struct Tables {
   double inv_b0;   // 1 / b_ref
   double inv_gravity;  // 1 / g (0 without gravity)
   double sqrt_gravity; // sqrt(g) (0 without gravity)
-  double w2[kMaxNodes][kMaxNodes];  // w_q w_p (element means of 2D nodal fields)
   double src_coef; // source coefficient: K (linear damping) or C_f (Chezy)
   // smoothness indicator of the subcell limiter: nodal values -> coefficients
   // in the orthonormal Legendre basis, threshold T(N) and s / T

@@ -231,6 +231,38 @@ __device__ __forceinline__ double theta_lin(double eps, double Pa, double Pb) {
   return den != 0.0 ? fmin(1.0, fabs((eps - Pa) / den)) : 1.0;
 }
 
+// x in FP32, cut to 20 fraction bits; NaN beyond the normal range but for zero
+__device__ __forceinline__ float cut_f32(double x) {
+  const int hi = __double2hiint(x), m = hi & 0x7fffffff;
+  const int f = (int)((unsigned)(m - (896 << 20)) << 3) | (hi & (int)0x80000000);
+  const bool in = (unsigned)(m - (897 << 20)) < (254u << 20);
+  return __int_as_float(in ? f : (m | __double2loint(x)) == 0 ? 0 : 0x7fc00000);
+}
+
+// true only if theta_lin(0.1 low, low, t) is 1 for low = a - c (d - fl) and
+// t = a - c (d - fh): t - 0.1 low in FP32 exceeds 2^-16 of the sum of the
+// operands' magnitudes.  Operands are cut by 2^-20 of themselves and the handful
+// of FP32 roundings are 2^-24 each, below 2^-17 of that sum together; the FP64
+// evaluation rounds by 2^-50 of it.  (Six FP64 instructions a face side
+// otherwise, some 400 cycles of their pipe.)
+__device__ __forceinline__ bool theta_one(double a64, double c64, double d64, double fl64,
+                                          double fh64) {
+  const float a = cut_f32(a64), c = cut_f32(c64), d = cut_f32(d64), fl = cut_f32(fl64),
+              fh = cut_f32(fh64);
+  const float low = a - c * (d - fl), t = a - c * (d - fh);
+  const float sum = a + fabsf(c) * (fabsf(d) + fabsf(fl) + fabsf(fh));
+  return a > 1e-30f && t - 0.1f * low > 1.52587890625e-5f * sum;
+}
+
+// true only if theta_lin(0.1 lmin, ., t) is 1 for every t of an element, from the
+// smallest high word of its t and of its first-order values, whose smallest is
+// lmin: no t below an eighth of lmin.  (Positive doubles order as their high
+// words; a negative one, or a NaN with its sign set, fails the comparison, and a
+// positive NaN has theta 1.)
+__device__ __forceinline__ bool theta_one_element(int lmin_hi, int tmin_hi) {
+  return lmin_hi >= 0x400000 && lmin_hi < 0x7ff00000 && tmin_hi > lmin_hi - (3 << 20);
+}
+
 // Max of a non-negative double over the warps that hold one above zero, then
 // one atomicMax on the bit pattern per such warp.
 __device__ __forceinline__ void block_max_atomic_1d(double v, unsigned long long* slot) {

@@ -70,8 +70,8 @@ __device__ __forceinline__ void face_terms(const double* tm, const double* tp, i
 // first-order flux of that node on its far side, trace of c).  af: blending
 // coefficient of the face; c1m, c1p: dt / (w dx) of the two nodes (the doubled
 // step of Algorithm 1's one-direction updates times the half of the doubled
-// fluxes).  Returns the doubled face terms 2 (F^+- / b_ref - F^tot,+-) of the
-// corrections and the doubled fluxes 2 F^-, 2 F^+ of the first-order update.
+// fluxes).  Returns the face terms F^+- / b_ref - F^tot,+- of the corrections (not
+// doubled: that is one in their fixed point's exponent) and the doubled fluxes 2 F^-, 2 F^+ of the first-order update.
 template <int DIR, bool WB>
 __device__ __forceinline__ void face_limited(const double* tm, const double* tp, const double* lm,
                                              const double* lp, double af, double c1m, double c1p,
@@ -126,24 +126,28 @@ __device__ __forceinline__ void face_limited(const double* tm, const double* tp,
     }
   }
   // Algorithm 1 (h > 0): the doubled-dt one-direction first-order updates
-  // of the plus side's node 0 and the minus side's node N
-  const double low0 = lp[0] - c1p * (lp[4] - fLp[0]);
-  const double lowN = lm[0] - c1m * (fLm[0] - lm[4]);
-  const double t0 = lp[0] - c1p * (lp[4] - Fp[0]);
-  const double tN = lm[0] - c1m * (Fm[0] - lm[4]);
-  const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
-  if (th < 1.0) {
+  // of the plus side's node 0 and the minus side's node N, in FP64 only where
+  // FP32 does not show theta = 1
+  if (!(theta_one(lp[0], c1p, lp[4], fLp[0], Fp[0]) &&
+        theta_one(lm[0], -c1m, lm[4], fLm[0], Fm[0]))) {
+    const double low0 = lp[0] - c1p * (lp[4] - fLp[0]);
+    const double lowN = lm[0] - c1m * (fLm[0] - lm[4]);
+    const double t0 = lp[0] - c1p * (lp[4] - Fp[0]);
+    const double tN = lm[0] - c1m * (Fm[0] - lm[4]);
+    const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
+    if (th < 1.0) {
 #pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      Fm[v] = th * Fm[v] + (1.0 - th) * fLm[v];
-      Fp[v] = th * Fp[v] + (1.0 - th) * fLp[v];
+      for (int v = 0; v < 3; ++v) {
+        Fm[v] = th * Fm[v] + (1.0 - th) * fLm[v];
+        Fp[v] = th * Fp[v] + (1.0 - th) * fLp[v];
+      }
     }
   }
   const double hib0 = 0.5 * ib0;
 #pragma unroll
   for (int v = 0; v < 3; ++v) {
-    Tm[v] = 2.0 * fma(Fm[v], hib0, -FTm[v]);
-    Tp[v] = 2.0 * fma(Fp[v], hib0, -FTp[v]);
+    Tm[v] = fma(Fm[v], hib0, -FTm[v]);
+    Tp[v] = fma(Fp[v], hib0, -FTp[v]);
   }
 }
 
@@ -181,6 +185,9 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   constexpr int BT = FaceShape<N, LIMIT, SMALL>::block;
   constexpr int NX = TY * (TX + 1) * n;
   constexpr int NY = (TY + 1) * TX * n;
+  // x faces to whole warps, so that no warp takes both branches of the loops
+  // below (N = 3 limited: 10 passes of a warp instead of 11)
+  constexpr int NXW = (NX + 31) / 32 * 32;
   constexpr int LY = LIMIT ? TY : 1, LX = LIMIT ? TX : 1;
   const Tables& T = L.tab;
   // x faces: [row][face k between elements k-1 and k][node]; y faces:
@@ -240,9 +247,10 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   };
 
   // ---- phase 1: every face node of the tile once --------------------------
-  for (int f = threadIdx.x; f < NX + NY; f += BT) {
+  for (int f = threadIdx.x; f < NXW + NY; f += BT) {
     double a[kTrFields], b[kTrFields], Tm[3], Tp[3];
-    if (f < NX) {
+    if (f < NXW) {
+      if (NXW != NX && f >= NX) continue;
       const int q = f % n, k = (f / n) % (TX + 1), r = f / (n * (TX + 1));
       const int64_t ey = ey0 + r;
       if (ey >= Ey || (k > 0 && ex0 + k - 1 >= Ex)) continue;
@@ -273,7 +281,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
       }
       keep(&sxm[0][r][k][q], &sxp[0][r][k][q], TY * (TX + 1) * n, Tm, Tp, r, k - 1, r, k);
     } else {
-      const int g = f - NX;
+      const int g = f - NXW;
       const int p = g % n, c = (g / n) % TX, k = g / (n * TX);
       const int64_t ex = ex0 + c;
       if (ex >= Ex || (k > 0 && ey0 + k - 1 >= Ey)) continue;
@@ -322,10 +330,11 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   __syncthreads();
 
   // ---- the face terms in the fixed point of their element, in place -------
-  for (int f = threadIdx.x; f < NX + NY; f += BT) {
+  for (int f = threadIdx.x; f < NXW + NY; f += BT) {
     double *tm, *tp;
     int vs, r0, c0, r1, c1;
-    if (f < NX) {
+    if (f < NXW) {
+      if (NXW != NX && f >= NX) continue;
       const int q = f % n, k = (f / n) % (TX + 1), r = f / (n * (TX + 1));
       if (ey0 + r >= Ey || (k > 0 && ex0 + k - 1 >= Ex)) continue;
       tm = &sxm[0][r][k][q];
@@ -335,7 +344,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
       c0 = k - 1;
       c1 = k;
     } else {
-      const int g = f - NX;
+      const int g = f - NXW;
       const int p = g % n, c = (g / n) % TX, k = g / (n * TX);
       if (ex0 + c >= Ex || (k > 0 && ey0 + k - 1 >= Ey)) continue;
       tm = &sym[0][k][c][p];
@@ -378,10 +387,9 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     }
   long long O[3][n];
   int eo[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    // largest magnitude over the n rows of the element
-    int m = mag[k];
+  // largest value over the n rows of the element
+  auto element_max = [&](int v) -> int {
+    int m = v;
     if constexpr ((n & (n - 1)) == 0) {
 #pragma unroll
       for (int o = 1; o < n; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -389,10 +397,16 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
 #pragma unroll
       for (int j = 1; j < n; ++j) {
         const int src = c * n + ((q + j) % n);
-        m = max(m, __shfl_sync(0xffffffffu, mag[k], src < 32 ? src : lane));
+        m = max(m, __shfl_sync(0xffffffffu, v, src < 32 ? src : lane));
       }
     }
-    const int et = fx_exp(emag[k][r][cc]) + cor_e - 1021;   // of the corrections' sums
+    return m;
+  };
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int m = element_max(mag[k]);
+    // of the corrections' sums (limited terms are not doubled)
+    const int et = fx_exp(emag[k][r][cc]) + cor_e - 1021 + (LIMIT ? 1 : 0);
     const int e = max(fx_exp(m), et), sh = e - et;
     eo[k] = e;
 #pragma unroll
@@ -449,30 +463,41 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
         if (alpha != 0.0) out[v][p] = (1.0 - alpha) * out[v][p] + alpha * x[v];
       }
     }
-    // Algorithm 2 over the element's n rows (lanes c*n .. c*n+n-1)
-    double lmin = lo[0][0];
+    // Algorithm 2 over the element's n rows (lanes c*n .. c*n+n-1), in FP64
+    // only where the high words of the smallest depths do not show theta = 1
+    int omin = 0x7fffffff, fmn = 0x7fffffff;
 #pragma unroll
-    for (int p = 1; p < n; ++p) lmin = fmin(lmin, lo[0][p]);
-#pragma unroll
-    for (int k = 1; k < n; ++k) {
-      const int src = c * n + ((q + k) % n);
-      lmin = fmin(lmin, __shfl_sync(0xffffffffu, lmin, src < 32 ? src : lane));
+    for (int p = 0; p < n; ++p) {
+      omin = min(omin, __double2hiint(out[0][p]));
+      fmn = min(fmn, __double2hiint(lo[0][p]));
     }
-    const double eps = 0.1 * lmin;
-    double th = 1.0;
+    omin = ~element_max(~omin);
+    fmn = ~element_max(~fmn);
+    if (__any_sync(0xffffffffu, !theta_one_element(fmn, omin))) {
+      double lmin = lo[0][0];
 #pragma unroll
-    for (int p = 0; p < n; ++p) th = fmin(th, theta_lin(eps, lo[0][p], out[0][p]));
-    double thr = th;
+      for (int p = 1; p < n; ++p) lmin = fmin(lmin, lo[0][p]);
 #pragma unroll
-    for (int k = 1; k < n; ++k) {
-      const int src = c * n + ((q + k) % n);
-      thr = fmin(thr, __shfl_sync(0xffffffffu, th, src < 32 ? src : lane));
-    }
-    if (thr < 1.0) {
+      for (int k = 1; k < n; ++k) {
+        const int src = c * n + ((q + k) % n);
+        lmin = fmin(lmin, __shfl_sync(0xffffffffu, lmin, src < 32 ? src : lane));
+      }
+      const double eps = 0.1 * lmin;
+      double th = 1.0;
 #pragma unroll
-      for (int v = 0; v < 3; ++v)
+      for (int p = 0; p < n; ++p) th = fmin(th, theta_lin(eps, lo[0][p], out[0][p]));
+      double thr = th;
 #pragma unroll
-        for (int p = 0; p < n; ++p) out[v][p] = thr * out[v][p] + (1.0 - thr) * lo[v][p];
+      for (int k = 1; k < n; ++k) {
+        const int src = c * n + ((q + k) % n);
+        thr = fmin(thr, __shfl_sync(0xffffffffu, th, src < 32 ? src : lane));
+      }
+      if (thr < 1.0) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v)
+#pragma unroll
+          for (int p = 0; p < n; ++p) out[v][p] = thr * out[v][p] + (1.0 - thr) * lo[v][p];
+      }
     }
   }
   if (active) {
@@ -493,35 +518,25 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     // element means (Definition admissibility.preserving.means), then
     // sigma_x/dx + sigma_y/dy (Sec. 5, Eq. time.step.2d)
     double m[3];
+    // in the fixed point of the update (of its blended result with the
+    // limiter): the row with its weights, then the rows of the element (integer
+    // sums: any order)
     if constexpr (LIMIT) {
 #pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        double s = T.w2[q][0] * out[v][0];
+      for (int k = 0; k < 2; ++k) {
+        int mg = 0;
 #pragma unroll
-        for (int p = 1; p < n; ++p) s = fma(T.w2[q][p], out[v][p], s);
-        m[v] = s;
+        for (int v = k; v < 1 + 2 * k; ++v)
+#pragma unroll
+          for (int p = 0; p < n; ++p) mg = max(mg, fx_mag(out[v][p]));
+        eo[k] = fx_exp(element_max(mg));
+#pragma unroll
+        for (int v = k; v < 1 + 2 * k; ++v)
+#pragma unroll
+          for (int p = 0; p < n; ++p) O[v][p] = fx_from<FB>(out[v][p], eo[k]);
       }
-      // sum over the n rows of the element (lanes c*n .. c*n+n-1): a butterfly
-      // when n is a power of two (every lane ends with the same sum), else the
-      // rows in order
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        double s = m[v];
-        if constexpr ((n & (n - 1)) == 0) {
-#pragma unroll
-          for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        } else {
-#pragma unroll
-          for (int k = 1; k < n; ++k) {
-            const int src = c * n + ((q + k) % n);
-            s += __shfl_sync(0xffffffffu, m[v], src < 32 ? src : lane);
-          }
-        }
-        m[v] = s;
-      }
-    } else {
-      // in the fixed point of the update: the row with its weights, then the
-      // rows of the element (integer sums: any order)
+    }
+    {
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
         FxAcc a;

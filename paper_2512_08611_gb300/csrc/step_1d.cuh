@@ -155,13 +155,17 @@ __device__ __forceinline__ void lo_source(const Tables& T, double dt, double* u)
 }
 
 // Minimum over the n lanes of an element.
-template <int n>
-__device__ __forceinline__ double element_min(double v, int le, int p, int lane) {
-  double m = v;
+template <int n, class V>
+__device__ __forceinline__ V element_min(V v, int le, int p, int lane) {
+  V m = v;
 #pragma unroll
   for (int k = 1; k < n; ++k) {
     const int r = p + k < n ? p + k : p + k - n, src = le * n + r;
-    m = fmin(m, __shfl_sync(0xffffffffu, v, src < 32 ? src : lane));
+    const V o = __shfl_sync(0xffffffffu, v, src < 32 ? src : lane);
+    if constexpr (sizeof(V) == 8)
+      m = fmin(m, o);
+    else
+      m = min(m, o);
   }
   return m;
 }
@@ -583,16 +587,20 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       if constexpr (SWE) {
         const double c0 = dtx * T.inv_w[0], cN = dtx * T.inv_w[N];
         const double fi0R = lim[0][f + 1][0], fiNL = lip[0][f][N > 0 ? N - 1 : 0];
-        const double low0 = u0R[0] - c0 * (fi0R - fLp[0]);
-        const double lowN = uN[0] - cN * (fLm[0] - fiNL);
-        const double t0 = u0R[0] - c0 * (fi0R - Fp_[0]);
-        const double tN = uN[0] - cN * (Fm_[0] - fiNL);
-        const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
-        if (th < 1.0) {
+        // (in FP64 only where FP32 does not show theta = 1)
+        if (!(theta_one(u0R[0], c0, fi0R, fLp[0], Fp_[0]) &&
+              theta_one(uN[0], -cN, fiNL, fLm[0], Fm_[0]))) {
+          const double low0 = u0R[0] - c0 * (fi0R - fLp[0]);
+          const double lowN = uN[0] - cN * (fLm[0] - fiNL);
+          const double t0 = u0R[0] - c0 * (fi0R - Fp_[0]);
+          const double tN = uN[0] - cN * (Fm_[0] - fiNL);
+          const double th = fmin(theta_lin(0.1 * low0, low0, t0), theta_lin(0.1 * lowN, lowN, tN));
+          if (th < 1.0) {
 #pragma unroll
-          for (int v = 0; v < M; ++v) {
-            Fm_[v] = th * Fm_[v] + (1.0 - th) * fLm[v];
-            Fp_[v] = th * Fp_[v] + (1.0 - th) * fLp[v];
+            for (int v = 0; v < M; ++v) {
+              Fm_[v] = th * Fm_[v] + (1.0 - th) * fLm[v];
+              Fp_[v] = th * Fp_[v] + (1.0 - th) * fLp[v];
+            }
           }
         }
       }
@@ -657,11 +665,16 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
     for (int v = 0; v < M; ++v)
       if (alpha != 0.0) out[v] = (1.0 - alpha) * out[v] + alpha * lo[v];
     if constexpr (SWE) {
-      const double eps = 0.1 * element_min<n>(lo[0], le, p, lane);
-      const double th = element_min<n>(theta_lin(eps, lo[0], out[0]), le, p, lane);
-      if (th < 1.0) {
+      // (in FP64 only where the high words do not show theta = 1)
+      const int lmn = element_min<n>(__double2hiint(lo[0]), le, p, lane);
+      const int omn = element_min<n>(__double2hiint(out[0]), le, p, lane);
+      if (__any_sync(0xffffffffu, !theta_one_element(lmn, omn))) {
+        const double eps = 0.1 * element_min<n>(lo[0], le, p, lane);
+        const double th = element_min<n>(theta_lin(eps, lo[0], out[0]), le, p, lane);
+        if (th < 1.0) {
 #pragma unroll
-        for (int v = 0; v < M; ++v) out[v] = th * out[v] + (1.0 - th) * lo[v];
+          for (int v = 0; v < M; ++v) out[v] = th * out[v] + (1.0 - th) * lo[v];
+        }
       }
     }
     if (owner && p == 0) LA.alpha_out[e] = alpha;

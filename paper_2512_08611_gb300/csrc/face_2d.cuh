@@ -500,6 +500,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
       }
     }
   }
+  chain_end();
   if (active) {
 #pragma unroll
     for (int v = 0; v < 3; ++v)

@@ -458,6 +458,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     }
   }
 
+  chain_end();
   // ---- face traces: 4 n face nodes per element (side 0 / 1 of the x faces,
   //      then of the y faces), all fields of a face node by one thread --------
   if (active) {

@@ -636,6 +636,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   }
   __syncthreads();
 
+  chain_end();
   // ---- correction and update (owners only) --------------------------------
   constexpr double b0 = TB::bref();
   const double dtb0 = sz.dtb_x, dts = sz.dtb;

@@ -263,6 +263,14 @@ __device__ __forceinline__ bool theta_one_element(int lmin_hi, int tmin_hi) {
   return lmin_hi >= 0x400000 && lmin_hi < 0x7ff00000 && tmin_hi > lmin_hi - (3 << 20);
 }
 
+// True in every lane if b is in any; also the warp's barrier.  (A vote alone
+// orders no shared-memory accesses: the reads of the exchange fields before it
+// must not meet the writes of the next stage after it.)
+__device__ __forceinline__ bool warp_barrier_or(bool b) {
+  __syncwarp();
+  return __any_sync(0xffffffffu, b);
+}
+
 // Max of a non-negative double over the warps that hold one above zero, then
 // one atomicMax on the bit pattern per such warp.
 __device__ __forceinline__ void block_max_atomic_1d(double v, unsigned long long* slot) {

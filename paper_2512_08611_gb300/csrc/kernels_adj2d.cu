@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
       __syncthreads();
   };
   auto sync_or = [](bool b) -> bool {
-    return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
+    return WARP ? warp_barrier_or(b) : __syncthreads_or(b);
   };
 
   if (threadIdx.x < 32) fill_step_sizes<TB, false>(sz, A.dt, 1.0);

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
       __syncthreads();
   };
   auto sync_or = [](bool b) -> bool {
-    return WARP ? __any_sync(0xffffffffu, b) : __syncthreads_or(b);
+    return WARP ? warp_barrier_or(b) : __syncthreads_or(b);
   };
 
   chain_begin();
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     }
     // one exponent per element and group of fields: the first stage's
     // largest magnitudes with headroom, raised if a later stage exceeds
-    // them.  (The vote is also the barrier after the last reads of X.)
+    // them.  (sync_or is also the barrier after the last reads of X.)
     const bool over =
         lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1] || mag[2] >> 20 > E[2]);
     if (sync_or(over)) {

@@ -398,9 +398,9 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         if (IMEX && first && k < M) mag[k] = max(mag[k], fx_mag(u0[k]));
         over = over || (lane_ok && mag[k] >> 20 > Ex[k]);
       }
-      // exponents as in local_2d.cuh; the vote is also the barrier after the
-      // last reads of X
-      if (__any_sync(0xffffffffu, over)) {
+      // exponents as in local_2d.cuh, after the barrier that ends the last
+      // stage's reads of X
+      if (warp_barrier_or(over)) {
         if (over) {
 #pragma unroll
           for (int k = 0; k < K; ++k) atomicMax(&smag[slot][k], mag[k]);

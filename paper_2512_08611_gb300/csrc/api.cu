@@ -1290,9 +1290,9 @@ crkfr_status ensure_adjoint_sums(crkfr_ctx* c) {
 
 // The local kernel in its residual form (no time bookkeeping) on the element
 // rows [row0, row1) of u: the traces of u^n, and with `stages` the inner stage
-// values, [S-1][3][row1 - row0][Ex][n][n].
-crkfr_status launch_local_for_adjoint(crkfr_ctx* c, const double* u, double dt, int64_t row0,
-                                      int64_t row1, double* stages, cudaStream_t s) {
+// values, [S-1][3][row1 - row0][Ex][n][n].  Returns a cudaError_t.
+int launch_local_for_adjoint(crkfr_ctx* c, const double* u, double dt, int64_t row0, int64_t row1,
+                             double* stages, cudaStream_t s) {
   StepCtl ctl{};
   ctl.dt_fixed = dt;
   ctl.residual = 1;
@@ -1304,11 +1304,9 @@ crkfr_status launch_local_for_adjoint(crkfr_ctx* c, const double* u, double dt, 
   L.stages = stages;
   L.stage_row0 = row0;
   L.stage_rows = row1 - row0;
-  int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s,
-                [&] { return stages ? launch_local_2d_stages(L, s) : launch_local_2d(L, s); });
-  if (e) return cuda_fail(c, e, "2D local kernel");
-  c->launches += 1;
-  return CRKFR_OK;
+  const int e = stages ? launch_local_2d_stages(L, s) : launch_local_2d(L, s);
+  if (!e) c->launches += 1;
+  return e;
 }
 
 // The adjoint kernels of one step whose forward traces of u^n are in
@@ -1338,22 +1336,22 @@ crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, 
     A.sums_above = c->d_adj_recv + 3 * c->Ex * c->basis.n;
   }
   A.tab = c->tab;
-  int e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] { return launch_adjoint_faces_2d(A, s); });
-  if (e) return cuda_fail(c, e, "2D adjoint face kernel");
-  c->launches += 1;
   const int64_t chunk = stages ? c->Ey : c->adj_rows;
   A.stages = stages ? stages : c->d_adj_stages;
-  for (int64_t r = 0; r < c->Ey; r += chunk) {
-    A.row_begin = r;
-    A.row_end = std::min(r + chunk, c->Ey);
-    if (!stages) {
-      crkfr_status st = launch_local_for_adjoint(c, u, dt, r, A.row_end, c->d_adj_stages, s);
-      if (st != CRKFR_OK) return st;
+  // one record of the profile for the step, as its kind says
+  const int e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] {
+    int err = launch_adjoint_faces_2d(A, s);
+    if (!err) c->launches += 1;
+    for (int64_t r = 0; r < c->Ey && !err; r += chunk) {
+      A.row_begin = r;
+      A.row_end = std::min(r + chunk, c->Ey);
+      if (!stages) err = launch_local_for_adjoint(c, u, dt, r, A.row_end, c->d_adj_stages, s);
+      if (!err) err = launch_adjoint_local_2d(A, s);
+      if (!err) c->launches += 1;
     }
-    e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] { return launch_adjoint_local_2d(A, s); });
-    if (e) return cuda_fail(c, e, "2D adjoint local kernel");
-    c->launches += 1;
-  }
+    return err;
+  });
+  if (e) return cuda_fail(c, e, "2D adjoint kernels");
   return CRKFR_OK;
 }
 
@@ -1407,8 +1405,10 @@ crkfr_status crkfr_step_adjoint(crkfr_ctx* c, const double* u, const double* uba
   if (st != CRKFR_OK) return st;
   // forward traces of u^n, and the stage values if those of the whole mesh fit
   double* stages = c->adj_rows >= c->Ey ? c->d_adj_stages : nullptr;
-  st = launch_local_for_adjoint(c, u, dt, 0, c->Ey, stages, s);
-  if (st != CRKFR_OK) return st;
+  const int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s, [&] {
+    return launch_local_for_adjoint(c, u, dt, 0, c->Ey, stages, s);
+  });
+  if (e) return cuda_fail(c, e, "2D local kernel");
   return launch_adjoint(c, u, ubar1, ubar0, bbar, dt, c->d_trx, c->d_try, stages, s);
 }
 
@@ -1428,9 +1428,11 @@ crkfr_status crkfr_adjoint_local(crkfr_ctx* c, const double* u, const double* ub
   if (st != CRKFR_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   // forward traces of u^n and the sums the neighbouring slabs need
-  st = launch_local_for_adjoint(c, u, dt, 0, c->Ey, nullptr, s);
-  if (st != CRKFR_OK) return st;
-  int e = launch_adjoint_sums_2d(c->cfg.degree, c->Ex, c->Ey, ubar1, c->tab, c->d_adj_send, s);
+  int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s, [&] {
+    return launch_local_for_adjoint(c, u, dt, 0, c->Ey, nullptr, s);
+  });
+  if (e) return cuda_fail(c, e, "2D local kernel");
+  e = launch_adjoint_sums_2d(c->cfg.degree, c->Ex, c->Ey, ubar1, c->tab, c->d_adj_send, s);
   if (e) return cuda_fail(c, e, "adjoint sums kernel");
   c->launches += 1;
   return CRKFR_OK;

@@ -258,11 +258,13 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
   FxTables& F = T->fx;
   F.kD = 123 - sD;
   F.kL = 123 - sL;
-  double gm = 0.0;
-  for (int i = 0; i < n; ++i)
-    gm = std::fmax(gm, std::fmax(std::fmax(std::fabs(T->gRx[i]), std::fabs(T->gLx[i])),
-                                 std::fmax(std::fabs(T->gRy[i]), std::fabs(T->gLy[i]))));
-  std::frexp(gm, &F.kG);
+  double gx = 0.0, gy = 0.0;
+  for (int i = 0; i < n; ++i) {
+    gx = std::fmax(gx, std::fmax(std::fabs(T->gRx[i]), std::fabs(T->gLx[i])));
+    gy = std::fmax(gy, std::fmax(std::fabs(T->gRy[i]), std::fabs(T->gLy[i])));
+  }
+  std::frexp(gx, &F.kG[0]);
+  std::frexp(gy, &F.kG[1]);
   for (int i = 0; i < n; ++i) {
     for (int j = 0; j < n; ++j) {
       fx_coef(T->Dx[i][j], sD, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);

@@ -31,9 +31,9 @@ struct FxTables {
   int32_t l0_hi[kMaxNodes], l0_lo[kMaxNodes], l1_hi[kMaxNodes], l1_lo[kMaxNodes];
   int32_t kD, kL;
   // quadrature weights w_q w_p in units of 2^-60 (their sum is one); kG: all
-  // |0.5 g'| / dx, / dy below 2^kG
+  // |0.5 g'| / dx below 2^kG[0], / dy below 2^kG[1]
   int32_t w2_hi[kMaxNodes][kMaxNodes], w2_lo[kMaxNodes][kMaxNodes];
-  int32_t kG;
+  int32_t kG[2];
 };
 
 // Reference-element and mesh tables passed to every kernel by value, so they

@@ -71,7 +71,8 @@ __device__ __forceinline__ void face_terms(const double* tm, const double* tp, i
 // coefficient of the face; c1m, c1p: dt / (w dx) of the two nodes (the doubled
 // step of Algorithm 1's one-direction updates times the half of the doubled
 // fluxes).  Returns the face terms F^+- / b_ref - F^tot,+- of the corrections (not
-// doubled: that is one in their fixed point's exponent) and the doubled fluxes 2 F^-, 2 F^+ of the first-order update.
+// doubled: that is one in their fixed point's exponent) and the doubled fluxes
+// 2 F^-, 2 F^+ of the first-order update.
 template <int DIR, bool WB>
 __device__ __forceinline__ void face_limited(const double* tm, const double* tp, const double* lm,
                                              const double* lp, double af, double c1m, double c1p,
@@ -204,21 +205,23 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   chain_begin();
   // the traces hold time averages divided by b_0: so do the face terms
   const double dtp = RES ? 1.0 : L.st->dt_cur;
-  // correction tables times -dt in fixed point (FB bits below 2^(ec - 1022)),
-  // written here, read after the barriers between the phases
+  // correction tables times -dt in fixed point (FB bits below 2^(ec - 1022), ec
+  // of the x and of the y tables), written here, read after the barriers
+  // between the phases
   constexpr int FB = 59;
   __shared__ Fx cor[4][n];
-  __shared__ int cor_e;
-  // largest magnitudes of the face terms of h and of the momenta per element
-  __shared__ int emag[2][TY][TX];
-  for (int k = threadIdx.x; k < 2 * TY * TX; k += BT) (&emag[0][0][0])[k] = 0;
+  __shared__ int cor_e[2];
+  // largest magnitudes of each variable's terms on the x and the y faces of an
+  // element
+  __shared__ int emag[2][3][TY][TX];
+  for (int k = threadIdx.x; k < 6 * TY * TX; k += BT) (&emag[0][0][0][0])[k] = 0;
   if (threadIdx.x < 4 * n) {
     const double dt = dtp * T.b0;
     const int t = threadIdx.x / n, p = threadIdx.x - t * n;
     const double g = t == 0 ? T.gRx[p] : t == 1 ? T.gLx[p] : t == 2 ? T.gRy[p] : T.gLy[p];
-    const int ec = fx_exp(fx_mag(dt) + (T.fx.kG << 20));
+    const int ec = fx_exp(fx_mag(dt) + (T.fx.kG[t >> 1] << 20));
     cor[t][p] = fx_split(fx_from<FB>(-dt * g, ec));
-    if (threadIdx.x == 0) cor_e = ec;
+    if (p == 0 && (t & 1) == 0) cor_e[t >> 1] = ec;
   }
   // limiter: dt / (w dx) of the nodes next to a face (0 and N), x and y
   __shared__ double cl[2][2];
@@ -229,20 +232,20 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   __syncthreads();
   // the terms of both sides of a face: to shared memory, their magnitudes to
   // the elements they belong to (minus side: r0, c0; plus side: r1, c1)
-  auto keep = [&](double* tm, double* tp, int vs, const double* Tm, const double* Tp, int r0,
-                  int c0, int r1, int c1) {
+  auto keep = [&](int d, double* tm, double* tp, int vs, const double* Tm, const double* Tp,
+                  int r0, int c0, int r1, int c1) {
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       tm[v * vs] = Tm[v];
       tp[v * vs] = Tp[v];
     }
     if (r0 >= 0 && c0 >= 0) {
-      atomicMax(&emag[0][r0][c0], fx_mag(Tm[0]));
-      atomicMax(&emag[1][r0][c0], max(fx_mag(Tm[1]), fx_mag(Tm[2])));
+#pragma unroll
+      for (int v = 0; v < 3; ++v) atomicMax(&emag[d][v][r0][c0], fx_mag(Tm[v]));
     }
     if (r1 < TY && c1 < TX) {
-      atomicMax(&emag[0][r1][c1], fx_mag(Tp[0]));
-      atomicMax(&emag[1][r1][c1], max(fx_mag(Tp[1]), fx_mag(Tp[2])));
+#pragma unroll
+      for (int v = 0; v < 3; ++v) atomicMax(&emag[d][v][r1][c1], fx_mag(Tp[v]));
     }
   };
 
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
         face_terms<WB>(a, b, 1, L.sface[ep * n + q], T.gravity, T.inv_gravity, T.sqrt_gravity,
                        Tm, Tp);
       }
-      keep(&sxm[0][r][k][q], &sxp[0][r][k][q], TY * (TX + 1) * n, Tm, Tp, r, k - 1, r, k);
+      keep(0, &sxm[0][r][k][q], &sxp[0][r][k][q], TY * (TX + 1) * n, Tm, Tp, r, k - 1, r, k);
     } else {
       const int g = f - NXW;
       const int p = g % n, c = (g / n) % TX, k = g / (n * TX);
@@ -324,12 +327,19 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
         face_terms<WB>(a, b, 2, L.sface[Ne * n + (ey0 + k) * plane + ex * n + p], T.gravity,
                        T.inv_gravity, T.sqrt_gravity, Tm, Tp);
       }
-      keep(&sym[0][k][c][p], &syp[0][k][c][p], (TY + 1) * TX * n, Tm, Tp, k - 1, c, k, c);
+      keep(1, &sym[0][k][c][p], &syp[0][k][c][p], (TY + 1) * TX * n, Tm, Tp, k - 1, c, k, c);
     }
   }
   __syncthreads();
 
-  // ---- the face terms in the fixed point of their element, in place -------
+  // ---- the face terms in fixed point, in place: x and y terms of a variable
+  //      so that their products with the correction tables have one unit per
+  //      element, 2^(unit - 1022 - FB) ------------------------------------------
+  auto unit = [&](int v, int r, int c, int& zero) -> int {
+    const int x = fx_exp(emag[0][v][r][c]), y = fx_exp(emag[1][v][r][c]);
+    zero = fx_zero(max(x, y));
+    return max(x + cor_e[0], y + cor_e[1]);
+  };
   for (int f = threadIdx.x; f < NXW + NY; f += BT) {
     double *tm, *tp;
     int vs, r0, c0, r1, c1;
@@ -354,14 +364,16 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
       r1 = k;
       c0 = c1 = c;
     }
-    auto convert = [&](double* t, int r, int c) {
-      const int e0 = fx_exp(emag[0][r][c]), e1 = fx_exp(emag[1][r][c]);
+    auto convert = [&](double* t, int d, int r, int c) {
 #pragma unroll
-      for (int v = 0; v < 3; ++v)
-        *reinterpret_cast<Fx*>(t + v * vs) = fx_split(fx_from<FB>(t[v * vs], v ? e1 : e0));
+      for (int v = 0; v < 3; ++v) {
+        int zero;
+        *reinterpret_cast<Fx*>(t + v * vs) =
+            fx_split(fx_from<FB>(t[v * vs], unit(v, r, c, zero) - cor_e[d]));
+      }
     };
-    if (r0 >= 0 && c0 >= 0) convert(tm, r0, c0);
-    if (r1 < TY && c1 < TX) convert(tp, r1, c1);
+    if (r0 >= 0 && c0 >= 0) convert(tm, f >= NXW, r0, c0);
+    if (r1 < TY && c1 < TX) convert(tp, f >= NXW, r1, c1);
   }
   __syncthreads();
 
@@ -373,20 +385,7 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
   const int64_t ey = ey0 + r, ex = ex0 + cc;
   const bool active = lane_ok && ey < Ey && ex < Ex;
   const int64_t ge = active ? ey * Ex + ex : 0;
-  // u^{n+1} = W + corrections, summed in the fixed point of the larger of W's
-  // and the corrections' scales in the element and rounded once
   double out[3][n];
-  double W[3][n];
-  int mag[2] = {0, 0};
-#pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int p = 0; p < n; ++p) {
-      W[v][p] = L.w[(v * Ne + ge) * nn + q * n + p];
-      mag[v > 0] = max(mag[v > 0], fx_mag(W[v][p]));
-    }
-  long long O[3][n];
-  int eo[2];
   // largest value over the n rows of the element
   auto element_max = [&](int v) -> int {
     int m = v;
@@ -402,28 +401,28 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     }
     return m;
   };
+  // u^{n+1} = W + corrections: their sum in fixed point, W added with an
+  // exponent of its own (so that a step of zero size leaves it as it is, and
+  // values far below the element's largest keep their bits), rounded once.
+  // Limited terms are not doubled.
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int m = element_max(mag[k]);
-    // of the corrections' sums (limited terms are not doubled)
-    const int et = fx_exp(emag[k][r][cc]) + cor_e - 1021 + (LIMIT ? 1 : 0);
-    const int e = max(fx_exp(m), et), sh = e - et;
-    eo[k] = e;
+  for (int v = 0; v < 3; ++v) {
+    int zero;
+    const int et = unit(v, r, cc, zero) - 1021 + (LIMIT ? 1 : 0);
+    const Fx tr = fx_at(&sxm[v][r][cc + 1][q]), tl = fx_at(&sxp[v][r][cc][q]);
+    const Fx c2 = cor[2][q], c3 = cor[3][q];
 #pragma unroll
-    for (int v = k; v < 1 + 2 * k; ++v) {
-      const Fx tr = fx_at(&sxm[v][r][cc + 1][q]), tl = fx_at(&sxp[v][r][cc][q]);
-      const Fx c2 = cor[2][q], c3 = cor[3][q];
-#pragma unroll
-      for (int p = 0; p < n; ++p) {
-        // (GLL: corrections at the end nodes only; in y by zero coefficients)
-        FxAcc a;
-        fx_mul(a, fx_at(&sym[v][r + 1][cc][p]), c2.hi, c2.lo);
-        fx_mad(a, fx_at(&syp[v][r][cc][p]), c3.hi, c3.lo);
-        if (!GLL || p == N) fx_mad(a, tr, cor[0][p].hi, cor[0][p].lo);
-        if (!GLL || p == 0) fx_mad(a, tl, cor[1][p].hi, cor[1][p].lo);
-        O[v][p] = fx_from<FB>(W[v][p], e) + fx_sar(fx_sum(a), sh);
-        out[v][p] = fx_to(O[v][p], e + 63 - FB, fx_zero(e));
-      }
+    for (int p = 0; p < n; ++p) {
+      // (GLL: corrections at the end nodes only; in y by zero coefficients)
+      FxAcc a;
+      fx_mul(a, fx_at(&sym[v][r + 1][cc][p]), c2.hi, c2.lo);
+      fx_mad(a, fx_at(&syp[v][r][cc][p]), c3.hi, c3.lo);
+      if (!GLL || p == N) fx_mad(a, tr, cor[0][p].hi, cor[0][p].lo);
+      if (!GLL || p == 0) fx_mad(a, tl, cor[1][p].hi, cor[1][p].lo);
+      const double w = L.w[(v * Ne + ge) * nn + q * n + p];
+      const int e = max(fx_exp(fx_mag(w)), et);
+      out[v][p] = fx_to(fx_from<FB>(w, e) + fx_sar(fx_sum(a), e - et), e + 63 - FB,
+                        fx_zero(e) | zero);
     }
   }
   if constexpr (LIMIT) {
@@ -519,46 +518,31 @@ __global__ void __launch_bounds__(FaceShape<N, LIMIT, SMALL>::block,
     // element means (Definition admissibility.preserving.means), then
     // sigma_x/dx + sigma_y/dy (Sec. 5, Eq. time.step.2d)
     double m[3];
-    // in the fixed point of the update (of its blended result with the
-    // limiter): the row with its weights, then the rows of the element (integer
-    // sums: any order)
-    if constexpr (LIMIT) {
+    // in the fixed point of each variable: the row with its weights, then the
+    // rows of the element (integer sums: any order)
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        int mg = 0;
+    for (int v = 0; v < 3; ++v) {
+      int mg = 0;
 #pragma unroll
-        for (int v = k; v < 1 + 2 * k; ++v)
+      for (int p = 0; p < n; ++p) mg = max(mg, fx_mag(out[v][p]));
+      const int eo = fx_exp(element_max(mg));
+      FxAcc a{0, 0};
 #pragma unroll
-          for (int p = 0; p < n; ++p) mg = max(mg, fx_mag(out[v][p]));
-        eo[k] = fx_exp(element_max(mg));
+      for (int p = 0; p < n; ++p)
+        fx_mad(a, fx_split(fx_from<FB>(out[v][p], eo)), T.fx.w2_hi[q][p], T.fx.w2_lo[q][p]);
+      const long long row = fx_sum(a);
+      long long s = row;
+      if constexpr ((n & (n - 1)) == 0) {
 #pragma unroll
-        for (int v = k; v < 1 + 2 * k; ++v)
+        for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      } else {
 #pragma unroll
-          for (int p = 0; p < n; ++p) O[v][p] = fx_from<FB>(out[v][p], eo[k]);
-      }
-    }
-    {
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        FxAcc a;
-        fx_mul(a, fx_split(O[v][0]), T.fx.w2_hi[q][0], T.fx.w2_lo[q][0]);
-#pragma unroll
-        for (int p = 1; p < n; ++p)
-          fx_mad(a, fx_split(O[v][p]), T.fx.w2_hi[q][p], T.fx.w2_lo[q][p]);
-        const long long row = fx_sum(a);
-        long long s = row;
-        if constexpr ((n & (n - 1)) == 0) {
-#pragma unroll
-          for (int o = 1; o < n; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        } else {
-#pragma unroll
-          for (int k = 1; k < n; ++k) {
-            const int src = c * n + ((q + k) % n);
-            s += __shfl_sync(0xffffffffu, row, src < 32 ? src : lane);
-          }
+        for (int k = 1; k < n; ++k) {
+          const int src = c * n + ((q + k) % n);
+          s += __shfl_sync(0xffffffffu, row, src < 32 ? src : lane);
         }
-        m[v] = fx_to(s, eo[v > 0] + 63 - FB, fx_zero(eo[v > 0]));
       }
+      m[v] = fx_to(s, eo + 63 - FB, fx_zero(eo));
     }
     // the rates: one element per thread of the first TY * TX threads, so that
     // a warp computes 32 of them (from the n lanes of an element only one

@@ -254,9 +254,10 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
     sl1 += std::fabs(T->l1[i]);
   }
   rl = std::fmax(sl0, sl1);
-  const int sD = fx_scale(rx + ry), sL = fx_scale(rl);
+  const int sx = fx_scale(rx), sy = fx_scale(ry), sL = fx_scale(rl);
   FxTables& F = T->fx;
-  F.kD = 123 - sD;
+  F.kDx = 123 - sx;
+  F.kDy = 123 - sy;
   F.kL = 123 - sL;
   double gx = 0.0, gy = 0.0;
   for (int i = 0; i < n; ++i) {
@@ -267,8 +268,8 @@ void fill_tables(const HostBasis& b, double dx, double dy, double gravity, bool 
   std::frexp(gy, &F.kG[1]);
   for (int i = 0; i < n; ++i) {
     for (int j = 0; j < n; ++j) {
-      fx_coef(T->Dx[i][j], sD, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);
-      fx_coef(T->Dy[i][j], sD, &F.Dy_hi[i][j], &F.Dy_lo[i][j]);
+      fx_coef(T->Dx[i][j], sx, &F.Dx_hi[i][j], &F.Dx_lo[i][j]);
+      fx_coef(T->Dy[i][j], sy, &F.Dy_hi[i][j], &F.Dy_lo[i][j]);
     }
     for (int j = 0; j < n; ++j) fx_coef(b.w[i] * b.w[j], 60, &F.w2_hi[i][j], &F.w2_lo[i][j]);
     fx_coef(T->l0[i], sL, &F.l0_hi[i], &F.l0_lo[i]);

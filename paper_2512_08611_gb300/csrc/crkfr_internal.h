@@ -22,14 +22,14 @@ inline int sys_vars(int s) { return s == CRKFR_SYS_VARADV_1D ? 1 : sys_is_2d(s) 
 inline bool sys_valid(int s) { return s >= CRKFR_SYS_VARADV_1D && s <= CRKFR_SYS_SWE_2D_WB; }
 
 // The matrices of the contractions as fixed-point integers hi * 2^30 + lo
-// (-2^29 <= lo < 2^29) in units of 2^-s, s such that the largest row sum of
-// magnitudes (of D / dx and D / dy together) is at most 2^61; kD, kL = 123 - s
-// of the differentiation matrices and of the end-point rows (fixed_point.cuh).
+// (-2^29 <= lo < 2^29) in units of 2^-s, s such that the largest row or column
+// sum of magnitudes is at most 2^61; kDx, kDy, kL = 123 - s of D / dx, of D /
+// dy and of the end-point rows (fixed_point.cuh).
 struct FxTables {
   int32_t Dx_hi[kMaxNodes][kMaxNodes], Dx_lo[kMaxNodes][kMaxNodes];
   int32_t Dy_hi[kMaxNodes][kMaxNodes], Dy_lo[kMaxNodes][kMaxNodes];
   int32_t l0_hi[kMaxNodes], l0_lo[kMaxNodes], l1_hi[kMaxNodes], l1_lo[kMaxNodes];
-  int32_t kD, kL;
+  int32_t kDx, kDy, kL;
   // quadrature weights w_q w_p in units of 2^-60 (their sum is one); kG: all
   // |0.5 g'| / dx below 2^kG[0], / dy below 2^kG[1]
   int32_t w2_hi[kMaxNodes][kMaxNodes], w2_lo[kMaxNodes][kMaxNodes];

@@ -6,10 +6,9 @@
 // logic instruction 2 (measured).  The steps are bound by that pipe, and more
 // than half of their FP64 instructions are products with constant matrices.
 // Those are done here in 60-bit block fixed point instead: the operands of a
-// contraction are scaled by one power of two per element and field group,
-// split into two 30-bit halves, and multiplied into two 64-bit accumulators
-// with three IMAD.WIDE per term (6 cycles against 64); the sum is rounded to
-// FP64 once.
+// contraction are scaled by one power of two per element and field, split into
+// two 30-bit halves, and multiplied into two 64-bit accumulators with three
+// IMAD.WIDE per term (6 cycles against 64); the sum is rounded to FP64 once.
 //
 // Accuracy: operands are truncated 2^-kFxBits below the power of two above
 // the group's largest magnitude, coefficients are integers of a row sum up to
@@ -17,8 +16,17 @@
 // row's full scale (sum of |coefficient| times the largest operand).  An
 // FP64 FMA chain rounds every partial sum, 2^-53 of the partial sums each.
 //
-// Values too small for the group's scale vanish, exactly as they do against
-// it in an FP64 sum; groups holding an infinity or a NaN give NaN.
+// A group is one field of one element (a variable, a flux, an adjoint): what
+// enters one sum, so that its errors are those of the sum's own terms.  A value
+// far below the largest of its group loses bits, as its part of an FP64 sum over
+// the element does; sums of different fields are aligned after the contraction.
+// What is not summed over the element has an exponent of its own or stays FP64:
+// the state in the update, the average of h in the source term, the traces of
+// u^n and of that average at GLL nodes.  (The GLL traces of the averaged momenta
+// and fluxes are single values in their field's fixed point: all stages but the
+// first carry the rounding of a row of D on that field anyway.)  Groups whose largest value is below 2^-895 (1e-269) lose bits,
+// below 2^-953 they count as zero; groups holding an infinity or a NaN give
+// non-finite sums.
 #pragma once
 
 #include <cstdint>
@@ -123,16 +131,32 @@ __device__ __forceinline__ unsigned long long fx_sqrhi(unsigned long long a) {
 // and all of it is covered by 24/16.
 __device__ __forceinline__ int fx_log(double x) { return fx_mag(x) >> 16; }
 
-// magnitude of the group (as fx_mag) for the largest fx_log lm of the momenta;
-// pressure: the fluxes hold h^2 g/2, lhg = fx_log(g/2).  h must be normal for
-// 1/h to be finite: the group counts as non-finite otherwise.
+// magnitude of the group (as fx_mag) of m k / h (+ h^2 g/2) with lm, lk the
+// fx_log of the momenta, lhg = fx_log(g/2).  h must be normal for 1/h to be
+// finite, and m, k finite: the group counts as non-finite otherwise.
 template <bool PRESSURE>
-__device__ __forceinline__ int fx_flux_mag(double h, int lm, int lhg) {
+__device__ __forceinline__ int fx_flux_mag(double h, int lm, int lk, int lhg) {
   const int lh = fx_log(h);
-  int l = 2 * lm - lh;
+  int l = lm + lk - lh;
   if (PRESSURE) l = max(l, 2 * lh + lhg - 2 * (1023 << 4));
   l = min(max(l + 24, 0), 0x7ff0);
-  return ((unsigned)((lh >> 4) - 1) > 2045u ? 0x7ff0 : l) << 16;
+  return ((unsigned)((lh >> 4) - 1) > 2045u || max(lm, lk) >= 0x7ff0 ? 0x7ff0 : l) << 16;
+}
+
+// true if h (of the well-balanced form: the pressure-free one), a momentum or a
+// product of a 2D node exceeds the exponents E of its element's fields h, hu,
+// hv, hu hu / h, hu hv / h, hv hv / h
+template <bool PRESSURE>
+__device__ __forceinline__ bool fx_over(double h, int lx, int ly, int lhg, const int (&E)[6]) {
+  const int lh = fx_log(h), x = lx - lh + 24, y = ly - lh + 24;
+  int f3 = lx + x, f5 = ly + y;
+  if (PRESSURE) {
+    const int p = 2 * lh + lhg + 24 - 2 * (1023 << 4);
+    f3 = max(f3, p);
+    f5 = max(f5, p);
+  }
+  return (!PRESSURE && lh >> 4 > E[0]) || lx >> 4 > E[1] || ly >> 4 > E[2] || f3 >> 4 > E[3] ||
+         ly + x >> 4 > E[4] || f5 >> 4 > E[5] || (unsigned)((lh >> 4) - 1) > 2045u;
 }
 
 // 2^61 |m| / |h| up to their exponents
@@ -167,6 +191,22 @@ __device__ __forceinline__ long long fx_sar(long long v, int s) {
   long long r;
   asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
   return r;
+}
+
+// R1 2^(e1 - 1085) + R2 2^(e2 - 1085) in units of the larger exponent e (|R1|,
+// |R2| at most 2^60).  CANCEL: of the other one's where a sum is zero, for rows
+// that annihilate equal values without rounding.
+template <bool CANCEL = false>
+__device__ __forceinline__ long long fx_align(long long R1, int e1, long long R2, int e2,
+                                              int& e) {
+  if (CANCEL) {
+    // (but for groups with a non-finite member, whose sums are zero too)
+    if (R1 == 0 && e1 < 3000) e1 = e2;
+    if (R2 == 0 && e2 < 3000) e2 = e1;
+  }
+  const int d = e1 - e2;
+  e = max(e1, e2);
+  return fx_sar(R1, max(-d, 0)) + fx_sar(R2, max(d, 0));
 }
 
 // high word of what a zero sum of a group with exponent E stands for: 0, or

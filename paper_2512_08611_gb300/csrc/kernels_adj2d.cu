@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
   constexpr int kStageUnroll = UNROLL ? S : 1;
   const Tables& T = A.tab;
   __shared__ __align__(16) double sm[EPB * ES];
-  __shared__ int smag[EPB][5];
+  __shared__ int smag[EPB][2 * kTr];
   __shared__ StepSizes<TB> sz;
   __shared__ double sC[SHARED ? S : 1][3][SHARED ? kBlockAdj : 1];
 
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
 
   if (threadIdx.x < 32) fill_step_sizes<TB, false>(sz, A.dt, 1.0);
   if (lane_ok) {
-    for (int k = node; k < 5; k += nn) smag[le][k] = 0;
+    for (int k = node; k < 2 * kTr; k += nn) smag[le][k] = 0;
   }
   const double gbx = A.snode[ge * nn + node], gby = A.snode[(Ne + ge) * nn + node];
   int dxh[n], dxl[n], dyh[n], dyl[n];   // columns p of D_x, q of D_y
@@ -262,8 +262,7 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
   // A trace field X gets l0[p] tbar_left + l1[p] tbar_right from the x faces
   // of its row and l0[q] tbar_bottom + l1[q] tbar_top from the y faces of its
   // column.  The 4 n face nodes of the element, 7 fields each, one thread per
-  // face node; exponents per group of fields: U_h; U_hu, U_hv; the fluxes;
-  // h^n; the momentum at t^n.
+  // face node; an exponent per direction and field.
   {
     constexpr int J = (4 * n + nn - 1) / nn;
     double t[J][kTr];
@@ -275,23 +274,14 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
       const double* in = dir ? A.atry + (ey * 2 + side) * kTr * plane + ex * n + r
                              : A.atrx + side * ts + ge * n + r;
       const int64_t step = dir ? plane : 2 * ts;
-      int m[5];
 #pragma unroll
-      for (int fi = 0; fi < kTr; ++fi) t[jj][fi] = in[fi * step];
-      m[0] = fx_mag(t[jj][0]);
-      m[1] = max(fx_mag(t[jj][1]), fx_mag(t[jj][2]));
-      m[2] = max(fx_mag(t[jj][3]), fx_mag(t[jj][4]));
-      m[3] = fx_mag(t[jj][5]);
-      m[4] = fx_mag(t[jj][6]);
-      if (lane_ok) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) atomicMax(&smag[le][k], m[k]);
+      for (int fi = 0; fi < kTr; ++fi) {
+        t[jj][fi] = in[fi * step];
+        if (lane_ok) atomicMax(&smag[le][dir * kTr + fi], fx_mag(t[jj][fi]));
       }
     }
     sync();
-    int E[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) E[k] = fx_exp(smag[le][k]);
+    auto E = [&](int k) { return fx_exp(smag[le][k]); };   // k = direction kTr + field
 #pragma unroll
     for (int jj = 0; jj < J; ++jj) {
       const int job = jj * nn + node;
@@ -299,37 +289,43 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
       const int ds = job / n, r = job % n;   // direction and side, node of the face
 #pragma unroll
       for (int fi = 0; fi < kTr; ++fi) {
-        const int k = fi == 0 ? 0 : fi < 3 ? 1 : fi < 5 ? 2 : fi - 2;
-        if (lane_ok) X[(ds * kTr + fi) * n + r] = fx_split(fx_from<FB>(t[jj][fi], E[k]));
+        if (lane_ok)
+          X[(ds * kTr + fi) * n + r] =
+              fx_split(fx_from<FB>(t[jj][fi], E((ds >> 1) * kTr + fi)));
       }
     }
     sync();
     // products of field fx from the x faces, fy from the y faces (negative: none)
-    auto pull = [&](int fx, int fy, int k) -> double {
-      FxAcc a{0, 0};
+    auto pull = [&](int fx, int fy) -> double {
+      FxAcc a{0, 0}, b{0, 0};
+      const int ex = fx >= 0 ? E(fx) : 0, ey = fy >= 0 ? E(kTr + fy) : 0;
       if (fx >= 0) {
         fx_mad(a, X[fx * n + q], T.fx.l0_hi[p], T.fx.l0_lo[p]);
         fx_mad(a, X[(kTr + fx) * n + q], T.fx.l1_hi[p], T.fx.l1_lo[p]);
       }
       if (fy >= 0) {
-        fx_mad(a, X[(2 * kTr + fy) * n + p], T.fx.l0_hi[q], T.fx.l0_lo[q]);
-        fx_mad(a, X[(3 * kTr + fy) * n + p], T.fx.l1_hi[q], T.fx.l1_lo[q]);
+        fx_mad(b, X[(2 * kTr + fy) * n + p], T.fx.l0_hi[q], T.fx.l0_lo[q]);
+        fx_mad(b, X[(3 * kTr + fy) * n + p], T.fx.l1_hi[q], T.fx.l1_lo[q]);
       }
-      return fx_to(fx_sum(a), E[k] + T.fx.kL - FB, fx_zero(E[k]));
+      int e = fx >= 0 ? ex : ey;
+      const long long s = fx < 0   ? fx_sum(b)
+                          : fy < 0 ? fx_sum(a)
+                                   : fx_align(fx_sum(a), ex, fx_sum(b), ey, e);
+      return fx_to(s, e + T.fx.kL - FB, fx_zero(max(ex, ey)));
     };
-    Ub[0] = pull(0, 0, 0);
-    Ub[1] = pull(1, 1, 1);
-    Ub[2] = pull(2, 2, 1);
-    F2b = pull(3, -1, 2);
-    F3b = pull(4, 3, 2);
-    G3b = pull(-1, 4, 2);
-    ub0[0] += pull(5, 5, 3);
-    ub0[1] += pull(6, -1, 4);
-    ub0[2] += pull(-1, 6, 4);
+    Ub[0] = pull(0, 0);
+    Ub[1] = pull(1, 1);
+    Ub[2] = pull(2, 2);
+    F2b = pull(3, -1);
+    F3b = pull(4, 3);
+    G3b = pull(-1, 4);
+    ub0[0] += pull(5, 5);
+    ub0[1] += pull(6, -1);
+    ub0[2] += pull(-1, 6);
   }
   sync();
   if (lane_ok) {
-    for (int k = node; k < 2; k += nn) smag[le][k] = 0;
+    for (int k = node; k < 3; k += nn) smag[le][k] = 0;
   }
   sync();
 
@@ -337,41 +333,47 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
   double gbxb = 0.0, gbyb = 0.0;
   double cb[3] = {0.0, 0.0, 0.0};        // adjoint of the stage value just reversed
   double rC[UNROLL ? S : 1][3];          // of every later stage
-  int E[2] = {-1, -1};                   // exponents of the adjoints of L (h; momenta)
+  int E[3] = {-1, -1, -1};               // exponents of the adjoints of L
   // column p of D_x on exchange field fx plus column q of D_y on field fy
-  auto contract = [&](int fx, int fy) -> long long {
-    FxAcc a{0, 0};
+  // (negative: none)
+  auto contract = [&](int fx, int fy) -> double {
+    FxAcc a{0, 0}, b{0, 0};
+    const int ex = fx >= 0 ? E[fx >= 0 ? fx : 0] : -1, ey = fy >= 0 ? E[fy >= 0 ? fy : 0] : -1;
     if (fx >= 0) {
 #pragma unroll
       for (int j = 0; j < n; ++j) fx_mad(a, X[fx * nn + q * n + j], dxh[j], dxl[j]);
     }
     if (fy >= 0) {
 #pragma unroll
-      for (int j = 0; j < n; ++j) fx_mad(a, X[fy * nn + j * n + p], dyh[j], dyl[j]);
+      for (int j = 0; j < n; ++j) fx_mad(b, X[fy * nn + j * n + p], dyh[j], dyl[j]);
     }
-    return fx_sum(a);
+    int e = fx >= 0 ? ex + T.fx.kDx : ey + T.fx.kDy;
+    const long long s =
+        fx < 0   ? fx_sum(b)
+        : fy < 0 ? fx_sum(a)
+                 : fx_align(fx_sum(a), ex + T.fx.kDx, fx_sum(b), ey + T.fx.kDy, e);
+    return fx_to(s, e - FB, fx_zero(max(ex, ey)));
   };
-  // fields to shared memory in the element's fixed point
+  // fields to shared memory in the fixed point of each field and element
   auto publish = [&](const double (&f)[3]) {
-    int mag[2];
-    mag[0] = fx_mag(f[0]);
-    mag[1] = max(fx_mag(f[1]), fx_mag(f[2]));
-    const bool over = lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1]);
+    bool over = false;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) over = over || (lane_ok && fx_mag(f[k]) >> 20 > E[k]);
     if (sync_or(over)) {
       if (over) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) atomicMax(&smag[le][k], mag[k]);
+        for (int k = 0; k < 3; ++k) atomicMax(&smag[le][k], fx_mag(f[k]));
       }
       sync();
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < 3; ++k) {
         const int e = fx_exp(smag[le][k]);
         E[k] = e > E[k] ? e + kHeadroom : E[k];
       }
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      if (lane_ok) X[k * nn + node] = fx_split(fx_from<FB>(f[k], E[k > 0]));
+      if (lane_ok) X[k * nn + node] = fx_split(fx_from<FB>(f[k], E[k]));
     sync();
   };
 #pragma unroll kStageUnroll
@@ -409,12 +411,10 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
     const double h = stage[0], mx = stage[vstep], my = stage[2 * vstep];
     publish(Lb);
     // local operator L_i = Dx f + Dy g + h (g b_x, g b_y): transposed contractions
-    const int bm = E[0] + T.fx.kD - FB, bf = E[1] + T.fx.kD - FB;
-    const int zm = fx_zero(E[0]), zf = fx_zero(E[1]);
-    const double mxb = fx_to(contract(0, -1), bm, zm), myb = fx_to(contract(-1, 0), bm, zm);
-    const double f2b = fma(wi, F2b, fx_to(contract(1, -1), bf, zf));
-    const double f3b = fma(wi, F3b, fx_to(contract(2, 1), bf, zf));
-    const double g3b = fma(wi, G3b, fx_to(contract(-1, 2), bf, zf));
+    const double mxb = contract(0, -1), myb = contract(-1, 0);
+    const double f2b = fma(wi, F2b, contract(1, -1));
+    const double f3b = fma(wi, F3b, contract(2, 1));
+    const double g3b = fma(wi, G3b, contract(-1, 2));
     // nonconservative terms h g b_x, h g b_y and the fluxes
     // f2 = mx vx + g h^2/2, f3 = mx vy, g3 = my vy + g h^2/2
     gbxb = fma(h, Lb[1], gbxb);
@@ -447,12 +447,12 @@ __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj
   const double gb2[3] = {0.0, gbxb, gbyb};
   sync();
   if (lane_ok) {
-    for (int k = node; k < 2; k += nn) smag[le][k] = 0;
+    for (int k = node; k < 3; k += nn) smag[le][k] = 0;
   }
   sync();
-  E[0] = E[1] = -1;
+  E[0] = E[1] = E[2] = -1;
   publish(gb2);
-  double bb = T.gravity * fx_to(contract(1, 2), E[1] + T.fx.kD - FB, fx_zero(E[1]));
+  double bb = T.gravity * contract(1, 2);
   // face jumps (g / b_0)(b+ - b-): left / right x faces of row q, bottom / top
   // y faces of column p
   {

@@ -78,8 +78,12 @@ __host__ __device__ constexpr int local_min_blocks() {
 
 // Exchange fields of the kernel: 0..5 the averages of h, hu, hv, hu hu / h
 // (+ pressure), hu hv / h, hv hv / h (+ pressure), or a stage's values of
-// them; 6..8 u^n.
+// them; 6..8 u^n.  Each of 0..5 has an exponent of its own per element (a small
+// momentum beside a large one keeps its bits; two terms of one equation are
+// aligned only where their derivatives are added).  The average of h enters
+// the source term node by node, so it is summed in FP64.
 constexpr int kLocalFields = 9;
+constexpr int kLocalGroups = 6;
 
 // b~_i / b_ref of a stage counted at run time
 template <class TB>
@@ -88,6 +92,23 @@ __device__ __forceinline__ int local_weight(int i) {
 #pragma unroll
   for (int k = 0; k < TB::S; ++k) w |= (unsigned long long)TB::weight(k) << (8 * k);
   return (int)(w >> (8 * i)) & 0xff;
+}
+
+// the same in FP64, from the upper halves of the weights' high words (a
+// conversion is an FP64 instruction)
+template <class TB>
+__device__ __forceinline__ double local_weight_fp(int i) {
+  unsigned long long w[2] = {0, 0};
+#pragma unroll
+  for (int k = 0; k < TB::S; ++k) {
+    // m 2^e, m < 2: exponent 1023 + e, four bits of m - 1
+    int m = TB::weight(k), e = 0;
+    while (m >> (e + 1)) ++e;
+    const unsigned long long h = m ? (unsigned)((1023 + e) << 4 | ((m << 4 >> e) & 15)) : 0;
+    w[k / 4] |= h << (16 * (k % 4));
+  }
+  const unsigned long long x = TB::S > 4 && i >= 4 ? w[1] >> (16 * (i - 4)) : w[0] >> (16 * i);
+  return __hiloint2double((int)(unsigned)(x << 16), 0);
 }
 
 // bit 8 i + j: a~_ij is not zero
@@ -146,7 +167,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   constexpr bool WARP = 32 % nn == 0;
   const Tables& T = L.tab;
   __shared__ __align__(16) double sm[EPB * ES];
-  __shared__ int smag[EPB][3];
+  __shared__ int smag[EPB][kLocalGroups];
   __shared__ StepSizes<TB> sz;
 
   const int le_raw = threadIdx.x / nn, node = threadIdx.x - le_raw * nn;
@@ -198,7 +219,9 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     dyh[j] = T.fx.Dy_hi[q][j];
     dyl[j] = T.fx.Dy_lo[q][j];
   }
-  if (lane_ok && node < 3) smag[le][node] = 0;
+  if (lane_ok) {
+    for (int k = node; k < kLocalGroups; k += nn) smag[le][k] = 0;
+  }
   sync();
 
   // The operators L_j of earlier stages that a stage sum needs: the last one
@@ -219,23 +242,37 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   }
   double Sb[2] = {0.0, 0.0};     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double P1 = 0.0, P2 = 0.0;     // sum_j (b_j/b_ref) h g d(h + b) (WB)
-  // time averages sum_j (b_j/b_ref) of the exchange fields 0..5 in the fixed
-  // point of the exponents E (h; hu, hv; the fluxes), which only grow: the
-  // sums are shifted when they do
+  double uh = 0.0;               // sum_j (b_j/b_ref) h
+  // time averages sum_j (b_j/b_ref) of the exchange fields 1..5 in the fixed
+  // point of their exponents E, which only grow: the sums are shifted when
+  // they do
   long long A[6] = {0, 0, 0, 0, 0, 0}, B[6] = {0, 0, 0, 0, 0, 0};
-  int E[3] = {-1, -1, -1};
-  auto group_of = [](int f) { return f == 0 ? 0 : f < 3 ? 1 : 2; };
-  // row of D_x on field fx plus row of D_y on field fy
-  auto contract = [&](int fx, int fy) -> long long {
+  int E[kLocalGroups] = {-1, -1, -1, -1, -1, -1};
+  constexpr int k0 = WB ? 0 : 1;   // (h is contracted in the well-balanced form only)
+  // row of D_x on field f (y: row of D_y)
+  auto row_x = [&](int f) -> long long {
     FxAcc a;
     Fx r[n];
-    fx_row<n>(X[fx][q], r);
+    fx_row<n>(X[f][q], r);
     fx_mul(a, r[0], dxh[0], dxl[0]);
 #pragma unroll
     for (int j = 1; j < n; ++j) fx_mad(a, r[j], dxh[j], dxl[j]);
-#pragma unroll
-    for (int j = 0; j < n; ++j) fx_mad(a, X[fy][j][p], dyh[j], dyl[j]);
     return fx_sum(a);
+  };
+  auto row_y = [&](int f) -> long long {
+    FxAcc a;
+    fx_mul(a, X[f][0][p], dyh[0], dyl[0]);
+#pragma unroll
+    for (int j = 1; j < n; ++j) fx_mad(a, X[f][j][p], dyh[j], dyl[j]);
+    return fx_sum(a);
+  };
+  // row of D_x on field fx plus row of D_y on field fy, in units 2^shift larger
+  // (at N = 1 a row of D is a difference: equal values cancel without rounding)
+  auto contract = [&](int fx, int fy, int shift) -> double {
+    int e;
+    const long long s =
+        fx_align<N == 1>(row_x(fx), E[fx] + T.fx.kDx, row_y(fy), E[fy] + T.fx.kDy, e);
+    return fx_to(s, e - FB + shift, fx_zero(max(E[fx], E[fy])));
   };
 #pragma unroll kStageUnroll
   for (int i = 0; i < S; ++i) {
@@ -290,7 +327,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
       rS[i][0] = c * cur[1];
       rS[i][1] = c * cur[2];
       // the implicit weights b_i equal the explicit ones b~_i
-      const double wd = (double)local_weight<TB>(i);
+      const double wd = local_weight_fp<TB>(i);
       if (wd != 0.0) {
         Sb[0] = fma(wd, rS[i][0], Sb[0]);
         Sb[1] = fma(wd, rS[i][1], Sb[1]);
@@ -312,87 +349,78 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     // every stage but the last feeds a later one; the last one's fluxes enter
     // the averages only
     const bool need_op = i < S - 1 && !(PRE == 2 && i == 0);
+    uh = fma(local_weight_fp<TB>(i), cur[0], uh);
     // the exchange fields at this node: the state and the fluxes
     const FxSig sh = fx_sig(cur[0]), sx = fx_sig(cur[1]), sy = fx_sig(cur[2]);
-    int mag[3];
-    mag[0] = fx_mag(cur[0]);
-    mag[1] = max(fx_mag(cur[1]), fx_mag(cur[2]));
-    mag[2] = fx_flux_mag<!WB>(cur[0], mag[1] >> 16, fx_log(T.half_gravity));
-    if (IMEX) {
-      // the traces of u^n, no stage value here, share the exponents
-      mag[0] = max(mag[0], fx_mag(u0[0]));
-      mag[1] = max(mag[1], max(fx_mag(u0[1]), fx_mag(u0[2])));
-    }
-    // one exponent per element and group of fields: the first stage's
-    // largest magnitudes with headroom, raised if a later stage exceeds
-    // them.  (sync_or is also the barrier after the last reads of X.)
-    const bool over =
-        lane_ok && (mag[0] >> 20 > E[0] || mag[1] >> 20 > E[1] || mag[2] >> 20 > E[2]);
-    if (sync_or(over)) {
-      if (over) {
+    // one exponent per element and field: the first stage's largest
+    // magnitudes with headroom, raised if a later stage exceeds them.
+    // (sync_or is also the barrier after the last reads of X.)
+    const int lx = fx_log(cur[1]), ly = fx_log(cur[2]), lhg = fx_log(T.half_gravity);
+    if (sync_or(lane_ok && fx_over<!WB>(cur[0], lx, ly, lhg, E))) {
+      if (lane_ok) {
+        int mag[kLocalGroups];
+        mag[0] = fx_mag(cur[0]);
+        mag[1] = fx_mag(cur[1]);
+        mag[2] = fx_mag(cur[2]);
+        mag[3] = fx_flux_mag<!WB>(cur[0], lx, lx, lhg);
+        mag[4] = fx_flux_mag<false>(cur[0], lx, ly, lhg);
+        mag[5] = fx_flux_mag<!WB>(cur[0], ly, ly, lhg);
+        if (IMEX) {
+          // the traces of u^n, no stage value here, share the exponents
+          mag[1] = max(mag[1], fx_mag(u0[1]));
+          mag[2] = max(mag[2], fx_mag(u0[2]));
+        }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) atomicMax(&smag[le][k], mag[k]);
+        for (int k = k0; k < kLocalGroups; ++k) atomicMax(&smag[le][k], mag[k]);
       }
       sync();
-      int d[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
+      for (int k = k0; k < kLocalGroups; ++k) {
         const int e = fx_exp(smag[le][k]);
-        d[k] = e > E[k] ? e + kHeadroom - E[k] : 0;
-        E[k] += d[k];
+        const int d = e > E[k] ? e + kHeadroom - E[k] : 0;
+        E[k] += d;
+        if (k > 0) fx_rescale<WIDE>(A[k], B[k], d);
       }
-#pragma unroll
-      for (int k = 0; k < 6; ++k) fx_rescale<WIDE>(A[k], B[k], d[group_of(k)]);
     }
     long long f[6];
     {
       const unsigned long long R = recip_bits((unsigned)__double2hiint(cur[0]),
                                               (unsigned)__double2loint(cur[0]));
       const unsigned long long vx = fx_velocity(R, sx), vy = fx_velocity(R, sy);
-      f[0] = fx_from<FB>(sh, E[0]);
+      if (WB) f[0] = fx_from<FB>(sh, E[0]);
       f[1] = fx_from<FB>(sx, E[1]);
-      f[2] = fx_from<FB>(sy, E[1]);
-      f[3] = fx_momentum_flux<FB>(sx, vx, sx, sh, E[2]);
-      f[4] = fx_momentum_flux<FB>(sx, vy, sy, sh, E[2]);
-      f[5] = fx_momentum_flux<FB>(sy, vy, sy, sh, E[2]);
+      f[2] = fx_from<FB>(sy, E[2]);
+      f[3] = fx_momentum_flux<FB>(sx, vx, sx, sh, E[3]);
+      f[4] = fx_momentum_flux<FB>(sx, vy, sy, sh, E[4]);
+      f[5] = fx_momentum_flux<FB>(sy, vy, sy, sh, E[5]);
       if (!WB) {
-        const long long ph = fx_pressure<FB>(sh, fx_sig(T.half_gravity), E[2]);
-        f[3] += ph;
-        f[5] += ph;
+        const FxSig hg = fx_sig(T.half_gravity);
+        f[3] += fx_pressure<FB>(sh, hg, E[3]);
+        f[5] += fx_pressure<FB>(sh, hg, E[5]);
       }
     }
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const long long v = f[k];
-      const Fx x = fx_split(v);
-      fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
-      // (h is contracted in the well-balanced form only)
-      if ((WB || k > 0) && lane_ok) X[k][q][p] = x;
+    for (int k = k0; k < 6; ++k) {
+      const Fx x = fx_split(f[k]);
+      if (k > 0) fx_accumulate<WIDE>(A[k], B[k], f[k], x, wi);
+      if (lane_ok) X[k][q][p] = x;
     }
     if (need_op || WB) {
       sync();
       double ncx = 0.0, ncy = 0.0;   // well-balanced: h g (h + b)_x, _y
       if constexpr (WB) {
-        FxAcc hx, hy;
-        fx_mul(hx, X[0][q][0], dxh[0], dxl[0]);
-        fx_mul(hy, X[0][0][p], dyh[0], dyl[0]);
-#pragma unroll
-        for (int j = 1; j < n; ++j) {
-          fx_mad(hx, X[0][q][j], dxh[j], dxl[j]);
-          fx_mad(hy, X[0][j][p], dyh[j], dyl[j]);
-        }
-        const int b = E[0] + T.fx.kD - FB, z = fx_zero(E[0]);
-        ncx = cur[0] * fma(T.gravity, fx_to(fx_sum(hx), b, z), gbx);
-        ncy = cur[0] * fma(T.gravity, fx_to(fx_sum(hy), b, z), gby);
-        const double wd = (double)wi;
+        const int z = fx_zero(E[0]);
+        const double hx = fx_to(row_x(0), E[0] + T.fx.kDx - FB, z);
+        const double hy = fx_to(row_y(0), E[0] + T.fx.kDy - FB, z);
+        ncx = cur[0] * fma(T.gravity, hx, gbx);
+        ncy = cur[0] * fma(T.gravity, hy, gby);
+        const double wd = local_weight_fp<TB>(i);
         P1 = fma(wd, ncx, P1);
         P2 = fma(wd, ncy, P2);
       }
       if (need_op) {
-        const int bm = E[1] + T.fx.kD - FB, bf = E[2] + T.fx.kD - FB;
-        const int zf = fx_zero(E[2]);
-        Lp[0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
-        const double l1 = fx_to(contract(3, 4), bf, zf), l2 = fx_to(contract(4, 5), bf, zf);
+        Lp[0] = contract(1, 2, 0);
+        const double l1 = contract(3, 4, 0), l2 = contract(4, 5, 0);
         Lp[1] = WB ? l1 + ncx : fma(cur[0], gbx, l1);
         Lp[2] = WB ? l2 + ncy : fma(cur[0], gby, l2);
       }
@@ -417,34 +445,40 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   // accumulated stage by stage).  A, P and Sb hold time averages divided by
   // b_ref; the sums are scaled back to FB bits for the contractions.
 #pragma unroll
-  for (int k = 0; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  for (int k = 1; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  if constexpr (!GLL) {
+    // the exponent of the traces of h: u^n and its average (in sum units)
+    const int mu = fx_mag(uh);
+    const int m = max(fx_mag(u0[0]), mu >= 0x7ff00000 ? mu : mu - (kSumShift << 20));
+    if (lane_ok) atomicMax(&smag[le][0], m);
+  }
   sync();
+  if (!GLL) E[0] = fx_exp(smag[le][0]);
   if (lane_ok) {
+    X[0][q][p] = GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
+                     : fx_split(fx_from<FB>(uh, E[0] + kSumShift));
 #pragma unroll
-    for (int k = 0; k < 6; ++k) X[k][q][p] = fx_split(A[k]);
+    for (int k = 1; k < 6; ++k) X[k][q][p] = fx_split(A[k]);
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       if constexpr (GLL)
         X[6 + v][q][p] = Fx{__double2hiint(u0[v]), __double2loint(u0[v])};
       else
-        X[6 + v][q][p] = fx_split(fx_from<FB>(u0[v], E[v == 0 ? 0 : 1]));
+        X[6 + v][q][p] = fx_split(fx_from<FB>(u0[v], E[v]));
     }
   }
   sync();
   {
     constexpr double b0 = TB::bref();
     const double dtb0 = sz.dtb;
-    const int bm = E[1] + T.fx.kD - FB + kSumShift, bf = E[2] + T.fx.kD - FB + kSumShift;
-    const int zf = fx_zero(E[2]);
     double V[3];
-    V[0] = fx_to(contract(1, 2), bm, fx_zero(E[1]));
-    V[1] = fx_to(contract(3, 4), bf, zf);
-    V[2] = fx_to(contract(4, 5), bf, zf);
+    V[0] = contract(1, 2, kSumShift);
+    V[1] = contract(3, 4, kSumShift);
+    V[2] = contract(4, 5, kSumShift);
     if constexpr (WB) {
       V[1] += P1;
       V[2] += P2;
     } else {
-      const double uh = fx_to(A[0], E[0] + 63 - FB + kSumShift, fx_zero(E[0]));
       V[1] = fma(uh, gbx, V[1]);
       V[2] = fma(uh, gby, V[2]);
     }
@@ -489,12 +523,14 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
 #pragma unroll
       for (int fi = 0; fi < kTrFields; ++fi) {
         const int k = fi < 3 ? fi : fi < 5 ? fi + dir : fi == 5 ? 6 : 7 + dir;
-        const int ek = fi == 0 || fi == 5 ? E[0] : fi < 3 || fi == 6 ? E[1] : E[2];
+        // (in y the fields after the first three are the next ones)
+        const int ek = fi < 3 ? E[fi] : fi == 3 ? (dir ? E[4] : E[3])
+                     : fi == 4 ? (dir ? E[5] : E[4]) : fi == 5 ? E[0] : (dir ? E[2] : E[1]);
         const Fx* x = line + k * nn;
         double t;
         if constexpr (GLL) {
           const Fx v = x[side ? N * step : 0];
-          if (fi >= 5)
+          if (fi == 0 || fi >= 5)
             t = __hiloint2double(v.hi, v.lo);
           else
             t = fx_to(((long long)v.hi << 30) + v.lo, ek + 63 - FB + kSumShift, fx_zero(ek));

@@ -393,7 +393,8 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         mag[k] = k < M ? fx_mag(cur[k < M ? k : 0])
-                       : fx_flux_mag<!WB>(cur[0], fx_log(cur[M - 1]), fx_log(T.half_gravity));
+                       : fx_flux_mag<!WB>(cur[0], fx_log(cur[M - 1]), fx_log(cur[M - 1]),
+                                          fx_log(T.half_gravity));
         // (IMEX: the traces of u^n, no stage value here, share the exponents)
         if (IMEX && first && k < M) mag[k] = max(mag[k], fx_mag(u0[k]));
         over = over || (lane_ok && mag[k] >> 20 > Ex[k]);
@@ -438,14 +439,14 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         __syncwarp();
         double nc = 0.0;
         if constexpr (WB) {
-          nc = cur[0] * fma(T.gravity, fx_to(contract(0), Ex[0] + T.fx.kD - FB, fx_zero(Ex[0])), sn);
+          nc = cur[0] * fma(T.gravity, fx_to(contract(0), Ex[0] + T.fx.kDx - FB, fx_zero(Ex[0])), sn);
           if (wi != 0) Pb = fma(wd, nc, Pb);
         }
         if (need_op) {
           const int k0 = SWE ? 1 : 0;
-          const double l0 = fx_to(contract(k0), Ex[k0] + T.fx.kD - FB, fx_zero(Ex[k0]));
+          const double l0 = fx_to(contract(k0), Ex[k0] + T.fx.kDx - FB, fx_zero(Ex[k0]));
           if constexpr (SWE) {
-            const double l1 = fx_to(contract(2), Ex[2] + T.fx.kD - FB, fx_zero(Ex[2]));
+            const double l1 = fx_to(contract(2), Ex[2] + T.fx.kDx - FB, fx_zero(Ex[2]));
             Ls[i][0] = l0;
             Ls[i][1] = WB ? l1 + nc : fma(cur[0], sn, l1);
           } else {
@@ -478,14 +479,14 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   __syncwarp();
   double V[M];                         // sum_j (b_j/b_ref) L_j
   if constexpr (SWE) {
-    V[0] = fx_to(contract(1), Ex[1] + T.fx.kD - FB + kSumShift, fx_zero(Ex[1]));
-    V[1] = fx_to(contract(2), Ex[2] + T.fx.kD - FB + kSumShift, fx_zero(Ex[2]));
+    V[0] = fx_to(contract(1), Ex[1] + T.fx.kDx - FB + kSumShift, fx_zero(Ex[1]));
+    V[1] = fx_to(contract(2), Ex[2] + T.fx.kDx - FB + kSumShift, fx_zero(Ex[2]));
     if (WB)
       V[1] += Pb;
     else
       V[1] = fma(fx_to(A[0], Ex[0] + 63 - FB + kSumShift, fx_zero(Ex[0])), sn, V[1]);
   } else {
-    V[0] = sn * fx_to(contract(0), Ex[0] + T.fx.kD - FB + kSumShift, fx_zero(Ex[0]));
+    V[0] = sn * fx_to(contract(0), Ex[0] + T.fx.kDx - FB + kSumShift, fx_zero(Ex[0]));
   }
   // traces: 2 NT of them, shared out over the element's threads
   if (lane_ok) {

@@ -189,11 +189,15 @@ __device__ __forceinline__ void step_bookkeeping(const StepCtl& c, DevState* st,
 // The step size and its products with the tableau's coefficients, by the
 // block's first warp (each product once, in one lane, instead of in every
 // thread: an FP64 instruction costs the same for one lane as for 32): dt;
-// e[i][j] = -(dt a~_ij xs); im[i][j] = dt a_ij; dt b_ref xs and dt b_ref.
+// e[i][j] = -(dt a~_ij xs); im[i][j] = dt a_ij; dt b_ref xs and dt b_ref; avg[j] =
+// sum_i (b_i/b_ref) e[i][j], so that a variable without source has the time
+// average (1/b_ref) u^n + sum_j avg[j] L_j in units of b_ref: one rounding of
+// the size of u^n instead of one per stage.
 template <class TB>
 struct StepSizes {
   double dt, dtb_x, dtb;
-  double e[TB::S][TB::S], im[TB::S][TB::S];
+  double e[TB::S][TB::S], avg[TB::S];   // (filled as one array)
+  double im[TB::S][TB::S];
 };
 template <class TB, bool IMEX>
 __device__ __forceinline__ void fill_step_sizes(StepSizes<TB>& s, double dt, double xs) {
@@ -201,7 +205,7 @@ __device__ __forceinline__ void fill_step_sizes(StepSizes<TB>& s, double dt, dou
   const int lane = threadIdx.x;
   const double dtx = dt * xs;
 #pragma unroll
-  for (int k0 = 0; k0 < S * S; k0 += 32) {
+  for (int k0 = 0; k0 < S * S + S; k0 += 32) {
     double a = 0.0, ai = 0.0;
     const int k = k0 + lane;
 #pragma unroll
@@ -211,10 +215,11 @@ __device__ __forceinline__ void fill_step_sizes(StepSizes<TB>& s, double dt, dou
         if (TB::a(i, j) != 0.0 && k == i * S + j) a = TB::a(i, j);
         if (IMEX && TB::ai(i, j) != 0.0 && k == i * S + j) ai = TB::ai(i, j);
       }
-    if (k < S * S) {
-      (&s.e[0][0])[k] = -(dtx * a);
-      if (IMEX) (&s.im[0][0])[k] = dt * ai;
-    }
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (k == S * S + j) a = TB::avg(j);
+    if (k < S * S + S) (&s.e[0][0])[k] = -(dtx * a);
+    if (IMEX && k < S * S) (&s.im[0][0])[k] = dt * ai;
   }
   if (lane == 0) {
     s.dt = dt;

@@ -81,7 +81,8 @@ __host__ __device__ constexpr int local_min_blocks() {
 // them; 6..8 u^n.  Each of 0..5 has an exponent of its own per element (a small
 // momentum beside a large one keeps its bits; two terms of one equation are
 // aligned only where their derivatives are added).  The average of h enters
-// the source term node by node, so it is summed in FP64.
+// the source term node by node, so it is formed in FP64, from h^n and the
+// stages' operators.
 constexpr int kLocalFields = 9;
 constexpr int kLocalGroups = 6;
 
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   }
   double Sb[2] = {0.0, 0.0};     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double P1 = 0.0, P2 = 0.0;     // sum_j (b_j/b_ref) h g d(h + b) (WB)
-  double uh = 0.0;               // sum_j (b_j/b_ref) h
+  double uh = 0.0;               // sum_j (b_j/b_ref) (h^(j) - h^n), below + h^n / b_ref
   // time averages sum_j (b_j/b_ref) of the exchange fields 1..5 in the fixed
   // point of their exponents E, which only grow: the sums are shifted when
   // they do
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
 #pragma unroll kStageUnroll
   for (int i = 0; i < S; ++i) {
     if (i == (IMEX ? 0 : 1)) __syncthreads();   // the step sizes
+    if (i > 0) uh = fma(sz.avg[i - 1], Lp[0], uh);
     double cur[3];
 #pragma unroll
     for (int v = 0; v < 3; ++v) cur[v] = u0[v];
@@ -349,7 +351,6 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     // every stage but the last feeds a later one; the last one's fluxes enter
     // the averages only
     const bool need_op = i < S - 1 && !(PRE == 2 && i == 0);
-    uh = fma(local_weight_fp<TB>(i), cur[0], uh);
     // the exchange fields at this node: the state and the fluxes
     const FxSig sh = fx_sig(cur[0]), sx = fx_sig(cur[1]), sy = fx_sig(cur[2]);
     // one exponent per element and field: the first stage's largest
@@ -446,6 +447,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   // b_ref; the sums are scaled back to FB bits for the contractions.
 #pragma unroll
   for (int k = 1; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  uh = fma((double)TB::weight_sum(), u0[0], uh);
   if constexpr (!GLL) {
     // the exponent of the traces of h: u^n and its average (in sum units)
     const int mu = fx_mag(uh);

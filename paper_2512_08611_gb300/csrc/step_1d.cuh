@@ -321,15 +321,19 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   __syncwarp();
 
   // ---- inner stages (element-local) ----------------------------------------
-  // Time averages are integer sums with the weights b_j / b_ref; b_ref is
+  // Time averages are integer sums (h: FP64) with the weights b_j / b_ref; b_ref is
   // applied to dt in the update, and the fluctuation, the one face term that
   // is not a time average, uses g / b_ref.
   double Ls[S][M];                     // local operator at each stage
   double Ss[S];                        // source of variable SV at each stage (IMEX)
   double Sb = 0.0;                     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double Pb = 0.0;                     // sum_j (b_j/b_ref) h g d(h + b) (WB)
-  long long A[K], B[K];                // sum_j (b_j/b_ref) of the exchange fields (WIDE: A 2^30 + B)
-  int Ex[K];                           // their exponents
+  // sum_j (b_j/b_ref) (h^(j) - h^n), below + h^n / b_ref: it enters node by node
+  double uh = 0.0;
+  long long A[K], B[K];                // of the other exchange fields (WIDE: A 2^30 + B)
+  int Ex[K];                           // exponents of the exchange fields
+  // shallow water: h is contracted in the well-balanced form only
+  constexpr int kStage0 = SWE && !WB ? 1 : 0, kAvg0 = SWE ? 1 : 0;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     A[k] = B[k] = 0;
@@ -350,6 +354,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   for (int i = 0; i < S; ++i) {
     // (the step sizes: the first stage does without)
     if (i == (IMEX ? 0 : 1)) __syncthreads();
+    if (SWE && i > 0 && TB::feeds(i > 0 ? i - 1 : 0)) uh = fma(sz.avg[i - 1], Ls[i - 1][0], uh);
     double cur[M];
 #pragma unroll
     for (int v = 0; v < M; ++v) {
@@ -391,7 +396,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       int mag[K];
       bool over = false;
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
+      for (int k = kStage0; k < K; ++k) {
         mag[k] = k < M ? fx_mag(cur[k < M ? k : 0])
                        : fx_flux_mag<!WB>(cur[0], fx_log(cur[M - 1]), fx_log(cur[M - 1]),
                                           fx_log(T.half_gravity));
@@ -404,15 +409,15 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       if (warp_barrier_or(over)) {
         if (over) {
 #pragma unroll
-          for (int k = 0; k < K; ++k) atomicMax(&smag[slot][k], mag[k]);
+          for (int k = kStage0; k < K; ++k) atomicMax(&smag[slot][k], mag[k]);
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
+        for (int k = kStage0; k < K; ++k) {
           const int ek = fx_exp(smag[slot][k]);
           const int d = ek > Ex[k] ? ek + kHeadroom - Ex[k] : 0;
           Ex[k] += d;
-          if (!first) fx_rescale<WIDE>(A[k], B[k], d);
+          if (!first && k >= kAvg0) fx_rescale<WIDE>(A[k], B[k], d);
         }
       }
       long long f[K];
@@ -420,7 +425,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         const FxSig sh = fx_sig(cur[0]), sm = fx_sig(cur[1]);
         const unsigned long long R = recip_bits((unsigned)__double2hiint(cur[0]),
                                                 (unsigned)__double2loint(cur[0]));
-        f[0] = fx_from<FB>(sh, Ex[0]);
+        if (WB) f[0] = fx_from<FB>(sh, Ex[0]);
         f[1] = fx_from<FB>(sm, Ex[1]);
         f[2] = fx_momentum_flux<FB>(sm, fx_velocity(R, sm), sm, sh, Ex[2]);
         if (!WB) f[2] += fx_pressure<FB>(sh, fx_sig(T.half_gravity), Ex[2]);
@@ -428,11 +433,10 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
         f[0] = fx_from<FB>(cur[0], Ex[0]);
       }
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
+      for (int k = kStage0; k < K; ++k) {
         const long long v = f[k];
         const Fx x = fx_split(v);
-        if (wi != 0) fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
-        // (h is contracted in the well-balanced form only)
+        if (wi != 0 && k >= kAvg0) fx_accumulate<WIDE>(A[k], B[k], v, x, wi);
         if ((SWE && k == 0 ? WB : need_op) && lane_ok) X[k][p] = x;
       }
       if (need_op || WB) {
@@ -464,12 +468,22 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
 
   // ---- the averages' derivative and the face traces --------------------------
 #pragma unroll
-  for (int k = 0; k < K; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  for (int k = kAvg0; k < K; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  uh = fma((double)TB::weight_sum(), u0[0], uh);
+  if constexpr (SWE && !GLL) {
+    // the exponent of the traces of h: u^n and its average (in sum units)
+    const int mu = fx_mag(uh);
+    const int m = max(fx_mag(u0[0]), mu >= 0x7ff00000 ? mu : mu - (kSumShift << 20));
+    if (lane_ok) atomicMax(&smag[slot][0], m);
+  }
   __syncwarp();
+  if (SWE && !GLL) Ex[0] = fx_exp(smag[slot][0]);
   if (lane_ok) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) X[k][p] = fx_split(A[k]);
+    for (int k = kAvg0; k < K; ++k) X[k][p] = fx_split(A[k]);
     if constexpr (SWE) {
+      X[0][p] = GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
+                    : fx_split(fx_from<FB>(uh, Ex[0] + kSumShift));
 #pragma unroll
       for (int v = 0; v < 2; ++v)
         X[3 + v][p] = GLL ? Fx{__double2hiint(u0[v]), __double2loint(u0[v])}
@@ -484,7 +498,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
     if (WB)
       V[1] += Pb;
     else
-      V[1] = fma(fx_to(A[0], Ex[0] + 63 - FB + kSumShift, fx_zero(Ex[0])), sn, V[1]);
+      V[1] = fma(uh, sn, V[1]);
   } else {
     V[0] = sn * fx_to(contract(0), Ex[0] + T.fx.kDx - FB + kSumShift, fx_zero(Ex[0]));
   }
@@ -500,7 +514,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
       double tr;
       if constexpr (GLL) {
         const Fx v = X[fi][side ? N : 0];
-        tr = fi >= 3 ? __hiloint2double(v.hi, v.lo)
+        tr = fi >= 3 || (SWE && fi == 0) ? __hiloint2double(v.hi, v.lo)
                      : fx_to(((long long)v.hi << 30) + v.lo, ex + 63 - FB + avg, fx_zero(ex));
       } else {
         FxAcc a;

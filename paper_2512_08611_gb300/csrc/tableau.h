@@ -139,6 +139,12 @@ struct Tab {
   CRKFR_HD static constexpr int weight(int i) { return IMEX ? imex_weight(i) : tab_weight(N, i); }
   CRKFR_HD static constexpr int weight_sum() { return IMEX ? 6 : tab_weight_sum(N); }
   CRKFR_HD static constexpr double bref() { return 1.0 / weight_sum(); }
+  // sum_i (b~_i / b_ref) a~_ij
+  CRKFR_HD static constexpr double avg(int j) {
+    double s = 0.0;
+    for (int i = j + 1; i < S; ++i) s += weight(i) * a(i, j);
+    return s;
+  }
   // the local operator of stage i is needed by a later stage
   CRKFR_HD static constexpr bool feeds(int i) {
     for (int k = i + 1; k < S; ++k)

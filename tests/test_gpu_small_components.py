@@ -69,6 +69,24 @@ def test_steps_after_the_end_change_nothing(crk, system, source, N, family):
     assert torch.equal(one, many)
 
 
+@pytest.mark.parametrize("system,source", [("swe2d", None), ("swe2d_wb", None), ("swe2d", "chezy")])
+@pytest.mark.parametrize("N,family", [(1, "gl"), (2, "gll"), (3, "gl"), (4, "gl")])
+def test_a_step_below_the_last_bit_changes_nothing(crk, system, source, N, family):
+    from oracle.basis import Basis
+    Ex, Ey, L = 33, 21, 8.0
+    x, y, _, _ = positions_2d(Basis(N, family), Ex, Ey, L)
+    k = 2 * np.pi / L
+    b = 0.1 * np.sin(k * x) * np.cos(k * y)
+    h = 1.0 + 0.2 * np.cos(k * x + 1.0) * np.sin(2 * k * y) - b
+    u = np.stack([h, h * np.sin(k * x + 2 * k * y + 0.1),
+                  1e-3 * h * np.sin(3 * k * x - k * y + 0.1)])
+    assert (np.abs(u) > 1e-100).all()
+    s = solver(crk, system, N, family, Ex, Ey, L, L, b, source)
+    d = to_dev(u)
+    assert s.advance(d, 1e-200) == 1
+    assert torch.equal(d, to_dev(u))
+
+
 # ---- one momentum far below the other ---------------------------------------
 def aligned_flow(N, family, froude, small, system):
     """h, b, hu and hv functions of x alone, hv `small` times hu."""
@@ -106,7 +124,7 @@ def test_small_transverse_momentum(crk, system, N, family, froude, small):
 
 
 # ---- a depth far below the others, beside a steep bottom ----------------------
-@pytest.mark.parametrize("dim", [2])
+@pytest.mark.parametrize("dim", [1, 2])
 @pytest.mark.parametrize("N", [2, 4])
 def test_shallow_node_on_a_steep_bottom(crk, dim, N):
     # still water; the middle node of a GLL element takes nothing from the faces,

@@ -309,9 +309,9 @@ crkfr_status crkfr_limiter_halo_buffers(crkfr_ctx* ctx, int32_t kind, double** s
 /* Adjoint of the step of Sec. 3, Eq. crkfr.non.cons.final (the paper has
  * no adjoint; it is this library's differentiation path).
  * Adjoint of one 2D shallow-water step with fixed dt > 0 (standard form,
- * GL nodes, no source term, context not in subdomain mode (slabs: the phased form below); otherwise
- * CRKFR_ERR_UNSUPPORTED or CRKFR_ERR_STATE).  With u^{n+1} = S(u^n; b) the step of crkfr_step
- * and a scalar J: given ubar1 = dJ/du^{n+1} (device, state layout), writes
+ * GL nodes, no source term, context not in subdomain mode (slabs: the phased
+ * form below); otherwise CRKFR_ERR_UNSUPPORTED or CRKFR_ERR_STATE).  With
+ * u^{n+1} = S(u^n; b) the step of crkfr_step and a scalar J: given ubar1 = dJ/du^{n+1} (device, state layout), writes
  * ubar0 = (dS/du^n)^T ubar1 and adds (dS/db)^T ubar1 to bbar (device,
  * coefficient layout [Ey][Ex][n][n]), b being the field passed to
  * crkfr_set_coefficients.  The exact discrete adjoint of the kernels'
@@ -319,7 +319,12 @@ crkfr_status crkfr_limiter_halo_buffers(crkfr_ctx* ctx, int32_t kind, double** s
  * maximum of two wave speeds follows the side the forward step selected.
  * u_dev is u^n and is not modified; ubar1 and ubar0 must not overlap.  The
  * simulated time is not changed.  Allocates the adjoint trace buffers on the
- * first call. */
+ * first call, and keeps them until the next crkfr_set_mesh.  The inner stage
+ * values are recomputed into a buffer kept as long: (S - 1) states (S the
+ * stages of the degree), at most 1 GiB, allocated by the first call outside a
+ * stream capture.  Where that much cannot be had, or in a capture before such a
+ * call, a smaller part or the context's work state serves, in more launches, with
+ * the same results bit for bit. */
 crkfr_status crkfr_step_adjoint(crkfr_ctx* ctx, const double* u_dev, const double* ubar1_dev,
                                 double* ubar0_dev, double* bbar_dev, double dt, void* stream);
 
@@ -336,9 +341,10 @@ crkfr_status crkfr_step_adjoint(crkfr_ctx* ctx, const double* u_dev, const doubl
  * crkfr_set_mesh, available after the first crkfr_adjoint_local);
  * crkfr_adjoint_faces (writes ubar0 of the slab's elements and adds the
  * gradient of their bathymetry to bbar, [Ey_local][Ex][n][n]: the halo rows
- * of the coefficient field get none here, their own slab adds it).  Equal
- * bit for bit to crkfr_step_adjoint on the whole mesh, row for row.  Both
- * phases return CRKFR_ERR_STATE on a context that is not a 2D slab. */
+ * of the coefficient field get none here, their own slab adds it; it
+ * recomputes the stage values as crkfr_step_adjoint does, in the same kind of
+ * buffer).  Equal bit for bit to crkfr_step_adjoint on the whole mesh, row for
+ * row.  Both phases return CRKFR_ERR_STATE on a context that is not a 2D slab. */
 crkfr_status crkfr_adjoint_local(crkfr_ctx* ctx, const double* u_dev, const double* ubar1_dev,
                                  double dt, void* stream);
 crkfr_status crkfr_adjoint_halo_buffers(crkfr_ctx* ctx, double** send_bottom, double** send_top,

@@ -52,7 +52,8 @@ struct crkfr_ctx {
   double* d_araw_halo = nullptr;  // 2D slab with the limiter: the neighbours' raw indicator,
                                   // rows -2, -1 (below) and Ey, Ey + 1 (above), [4][Ex]
   double* d_alpha_halo = nullptr; // 2D slab with the limiter: smoothed rows -1, Ey, [2][Ex]
-  double* d_adj_stages = nullptr; // stage values of adj_rows element rows (unrecorded adjoint)
+  double* d_adj_stages = nullptr; // stage values of adj_rows element rows (unrecorded adjoint;
+                                  // null: in d_work, adjoint_stage_buffer)
   int64_t adj_rows = 0;
   double* d_adj_send = nullptr;   // 2D slab adjoint: y-correction sums of ubar1 for the
   double* d_adj_recv = nullptr;   // neighbours / from them, [2][3][Ex][n] each
@@ -156,6 +157,12 @@ cudaEvent_t take_event(crkfr_ctx* c) {
     return nullptr;
   }
   return e;
+}
+
+// Doubles of the stage values of one element row.
+int64_t adjoint_stage_row(const crkfr_ctx* c) {
+  const int64_t n = c->basis.n;
+  return (int64_t)(tab_stages(c->cfg.degree) - 1) * 3 * c->Ex * n * n;
 }
 
 // Runs `launch` (returns a cudaError_t as int); with profiling on, brackets
@@ -744,9 +751,12 @@ crkfr_status crkfr_set_mesh(crkfr_ctx* c, int32_t dim, const int64_t* n_elem, co
     sn = (size_t)2 * Ne * n * n;
     sf = (size_t)(2 * Ne + Ex) * n;
   }
+  // (the adjoint may keep a row of inner stage values in d_work)
+  const size_t nw = dim == 1 ? (size_t)c->n_state
+                             : (size_t)std::max<int64_t>(c->n_state, adjoint_stage_row(c));
   if (cudaMalloc(&c->d_snode, sizeof(double) * sn) != cudaSuccess ||
       cudaMalloc(&c->d_sface, sizeof(double) * sf) != cudaSuccess ||
-      cudaMalloc(&c->d_work, sizeof(double) * c->n_state) != cudaSuccess ||
+      cudaMalloc(&c->d_work, sizeof(double) * nw) != cudaSuccess ||
       cudaMalloc(&c->d_state, sizeof(DevState)) != cudaSuccess) {
     free_buffers(c);
     cudaGetLastError();
@@ -1309,9 +1319,42 @@ int launch_local_for_adjoint(crkfr_ctx* c, const double* u, double dt, int64_t r
   return e;
 }
 
+// Where the adjoint step recomputes stage values, and how many element rows of
+// them at a time.  A buffer of the context's own, allocated by the first call
+// that is not being captured: the whole mesh if that takes at most a GiB, else
+// as many rows as do, or as many as there is memory for.  Without one (in a
+// capture, or with less memory than d_work holds) they go to d_work, which the
+// adjoint does not use otherwise: one row in S - 1, and at least one
+// (crkfr_set_mesh sees to that).  A smaller buffer costs launches and a second
+// pass of the local kernel: 256 x 256 at N = 3, 532 us a step with the whole
+// mesh in the buffer, 706 in d_work.
+double* adjoint_stage_buffer(crkfr_ctx* c, cudaStream_t s, int64_t* rows) {
+  const int64_t row = adjoint_stage_row(c);
+  const int64_t work_rows =
+      std::max<int64_t>(1, std::min(c->Ey, c->Ey / (tab_stages(c->cfg.degree) - 1)));
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  const bool captured = cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
+                        capture != cudaStreamCaptureStatusNone;
+  if (captured) cudaGetLastError();
+  if (!c->d_adj_stages && !captured) {
+    int64_t r = std::min(c->Ey, ((int64_t)1 << 27) / row);
+    for (; r > work_rows && !c->d_adj_stages; r /= 2) {
+      if (cudaMalloc(&c->d_adj_stages, sizeof(double) * row * r) == cudaSuccess) {
+        c->adj_rows = r;
+      } else {
+        c->d_adj_stages = nullptr;
+        cudaGetLastError();
+      }
+    }
+  }
+  *rows = c->d_adj_stages ? c->adj_rows : work_rows;
+  return c->d_adj_stages ? c->d_adj_stages : c->d_work;
+}
+
 // The adjoint kernels of one step whose forward traces of u^n are in
 // (trx, try_) and whose stage values are in `stages`.  Null: the stage values
-// are recomputed by the local kernel, adj_rows element rows at a time.
+// are recomputed by the local kernel, as many element rows at a time as
+// adjoint_stage_buffer holds.
 crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, double* ubar0,
                             double* bbar, double dt, const double* trx, const double* try_,
                             const double* stages, cudaStream_t s) {
@@ -1336,8 +1379,9 @@ crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, 
     A.sums_above = c->d_adj_recv + 3 * c->Ex * c->basis.n;
   }
   A.tab = c->tab;
-  const int64_t chunk = stages ? c->Ey : c->adj_rows;
-  A.stages = stages ? stages : c->d_adj_stages;
+  int64_t chunk = c->Ey;
+  double* buffer = stages ? nullptr : adjoint_stage_buffer(c, s, &chunk);
+  A.stages = stages ? stages : buffer;
   // one record of the profile for the step, as its kind says
   const int e = timed(c, CRKFR_KERNEL_ADJOINT_2D, s, [&] {
     int err = launch_adjoint_faces_2d(A, s);
@@ -1345,29 +1389,13 @@ crkfr_status launch_adjoint(crkfr_ctx* c, const double* u, const double* ubar1, 
     for (int64_t r = 0; r < c->Ey && !err; r += chunk) {
       A.row_begin = r;
       A.row_end = std::min(r + chunk, c->Ey);
-      if (!stages) err = launch_local_for_adjoint(c, u, dt, r, A.row_end, c->d_adj_stages, s);
+      if (buffer) err = launch_local_for_adjoint(c, u, dt, r, A.row_end, buffer, s);
       if (!err) err = launch_adjoint_local_2d(A, s);
       if (!err) c->launches += 1;
     }
     return err;
   });
   if (e) return cuda_fail(c, e, "2D adjoint kernels");
-  return CRKFR_OK;
-}
-
-// The buffer of recomputed stage values: the whole mesh if that takes at most
-// a GiB, else as many element rows as do.
-crkfr_status ensure_adjoint_stages(crkfr_ctx* c) {
-  if (c->d_adj_stages) return CRKFR_OK;
-  const int64_t n = c->basis.n;
-  const int64_t row = (int64_t)(tab_stages(c->cfg.degree) - 1) * 3 * c->Ex * n * n;
-  const int64_t rows = std::max<int64_t>(1, std::min(c->Ey, ((int64_t)1 << 27) / row));
-  if (cudaMalloc(&c->d_adj_stages, sizeof(double) * row * rows) != cudaSuccess) {
-    c->d_adj_stages = nullptr;
-    cudaGetLastError();
-    return fail(c, CRKFR_ERR_ALLOC, "device allocation failed");
-  }
-  c->adj_rows = rows;
   return CRKFR_OK;
 }
 
@@ -1384,6 +1412,9 @@ crkfr_status adjoint_args(crkfr_ctx* c, const double* u, const double* ubar1, do
     if (cudaMalloc(&c->d_atrx, sizeof(double) * tr) != cudaSuccess ||
         cudaMalloc(&c->d_atry, sizeof(double) * tr) != cudaSuccess ||
         cudaMalloc(&c->d_gbar, sizeof(double) * (2 * Ne + c->Ex) * n) != cudaSuccess) {
+      cudaFree(c->d_atrx);
+      cudaFree(c->d_atry);
+      c->d_atrx = c->d_atry = c->d_gbar = nullptr;
       cudaGetLastError();
       return fail(c, CRKFR_ERR_ALLOC, "device allocation failed");
     }
@@ -1401,10 +1432,10 @@ crkfr_status crkfr_step_adjoint(crkfr_ctx* c, const double* u, const double* uba
   if (st == CRKFR_OK) st = adjoint_args(c, u, ubar1, ubar0, bbar, dt);
   if (st != CRKFR_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  st = ensure_adjoint_stages(c);
-  if (st != CRKFR_OK) return st;
   // forward traces of u^n, and the stage values if those of the whole mesh fit
-  double* stages = c->adj_rows >= c->Ey ? c->d_adj_stages : nullptr;
+  int64_t rows;
+  double* stages = adjoint_stage_buffer(c, s, &rows);
+  if (rows < c->Ey) stages = nullptr;
   const int e = timed(c, CRKFR_KERNEL_LOCAL_2D, s, [&] {
     return launch_local_for_adjoint(c, u, dt, 0, c->Ey, stages, s);
   });
@@ -1459,8 +1490,6 @@ crkfr_status crkfr_adjoint_faces(crkfr_ctx* c, const double* u, const double* ub
   if (st == CRKFR_OK) st = adjoint_args(c, u, ubar1, ubar0, bbar, dt);
   if (st != CRKFR_OK) return st;
   if (!c->d_adj_send) return fail(c, CRKFR_ERR_STATE, "crkfr_adjoint_local first");
-  st = ensure_adjoint_stages(c);
-  if (st != CRKFR_OK) return st;
   return launch_adjoint(c, u, ubar1, ubar0, bbar, dt, c->d_trx, c->d_try, nullptr,
                         (cudaStream_t)stream);
 }

@@ -484,7 +484,9 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
       V[1] = fma(uh, gbx, V[1]);
       V[2] = fma(uh, gby, V[2]);
     }
-    if (active) {
+    // (a record alone, without a step, has no use for W: its place may hold the
+    // stage values)
+    if (active && !(STAGES && RES)) {
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
         double o = RES ? -b0 * V[v] : fma(-dtb0, V[v], u0[v]);

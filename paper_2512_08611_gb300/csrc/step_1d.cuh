@@ -175,14 +175,16 @@ __device__ __forceinline__ V element_min(V v, int le, int p, int lane) {
 // tables (dx = 1: D, l(0), l(1), 0.5 g'); xs = 1/dx scales the local operator
 // and the corrections through the scalar coefficients only (stage coefficients
 // dt a_ij xs, update coefficient dt b_ref xs), so one table serves meshes of
-// any dx.  Every element's arithmetic is the same for any block size.  (No
-// __restrict__: the loads must not move above chain_begin().)
+// any dx.  Every element's arithmetic is the same for any block size.  last: the
+// block leaves after this tile (chain_end()).  (No __restrict__: the loads must
+// not move above chain_begin().)
 template <int SYS, int N, bool GLL, bool RES, bool IMEX, bool LIMIT = false>
 __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
                                              const double* u_in, double* u_out,
                                              const double* snode, const double* sface, int64_t E,
                                              int64_t tile, DevState* st, const StepCtl& ctl,
-                                             bool first_tile, const LimitArgs& LA = LimitArgs{},
+                                             bool first_tile, bool last,
+                                             const LimitArgs& LA = LimitArgs{},
                                              const double* ghost = nullptr) {
   using TB = Tab<N, IMEX>;
   using SY = Sys1D<SYS>;
@@ -651,7 +653,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   }
   __syncthreads();
 
-  chain_end();
+  if (last) chain_end();
   // ---- correction and update (owners only) --------------------------------
   constexpr double b0 = TB::bref();
   const double dtb0 = sz.dtb_x, dts = sz.dtb;
@@ -745,8 +747,8 @@ __global__ void __launch_bounds__(LIMIT ? kBlockLimit1D : kMaxBlock1D,
                                   LIMIT ? 4 : min_blocks_1d<N>()) k_step_1d(const Launch1D L) {
   chain_begin();
   step_1d_tile<SYS, N, GLL, RES, IMEX, LIMIT>(L.tab, L.xs, L.u_in, L.u_out, L.snode, L.sface, L.E,
-                                              blockIdx.x, L.st, L.ctl, blockIdx.x == 0, L.lim,
-                                              L.ghost);
+                                              blockIdx.x, L.st, L.ctl, blockIdx.x == 0, true,
+                                              L.lim, L.ghost);
 }
 
 // Several steps of a mesh that one cluster of blocks holds.  A step of a small
@@ -779,7 +781,7 @@ __global__ void __launch_bounds__(kMaxClusterThreads) k_steps_1d(const Launch1D 
     }
     ctl.want_rate = k + 1 < L.steps ? !(ctl.dt_fixed > 0.0) : L.ctl.want_rate;
     step_1d_tile<SYS, N, GLL, false, IMEX>(L.tab, L.xs, in, out, L.snode, L.sface, L.E, blockIdx.x,
-                                           L.st, ctl, blockIdx.x == 0);
+                                           L.st, ctl, blockIdx.x == 0, k + 1 == L.steps);
   }
 }
 
@@ -794,7 +796,7 @@ __global__ void __launch_bounds__(kBlock1D, min_blocks_1d<N>()) k_step_1d_batch(
     if (wi != blockIdx.x) __syncthreads();   // the previous tile's last reads
     step_1d_tile<SYS, N, GLL, false, IMEX>(B.tab, I.xs, B.u_in + I.u_off, B.u_out + I.u_off,
                                            B.snode + I.sn_off, B.sface + I.sf_off, I.E, w.tile,
-                                           I.st, B.ctl, w.tile == 0);
+                                           I.st, B.ctl, w.tile == 0, wi + gridDim.x >= B.nwork);
   }
 }
 

@@ -1,7 +1,7 @@
-"""Votes of the kernels as barriers: a warp vote (__any_sync) orders no memory,
-so the places that vote between reads of shared memory and the writes that
-replace what was read must have a barrier too.  Read from the sources, since a
-missing one need not show in any result."""
+"""Orderings of the kernels that no result need show, read from the sources.  A
+warp vote (__any_sync) orders no memory, so the places that vote between reads
+of shared memory and the writes that replace what was read must have a barrier
+too."""
 import glob
 import os
 import re
@@ -35,3 +35,11 @@ def test_stage_votes_are_barriers():
     for name in ("local_2d.cuh", "step_1d.cuh", "kernels_adj2d.cu"):
         text = open(os.path.join(CSRC, name)).read()
         assert "warp_barrier_or(" in text, name
+
+
+def test_loops_over_tiles_release_the_next_kernel_last():
+    # launch.h: the next kernel of the stream is let in when the blocks are
+    # about to leave, not in the first of many steps or tiles
+    text = open(os.path.join(CSRC, "step_1d.cuh")).read()
+    assert re.findall(r"\n( *.*chain_end\(\);)", text) == ["  if (last) chain_end();"]
+    assert "k + 1 == L.steps)" in text and "wi + gridDim.x >= B.nwork)" in text

@@ -585,12 +585,12 @@ int launch_face_t(const Launch2D& L, cudaStream_t s) {
   if (L.row_begin % 8 != 0 || L.row_end <= L.row_begin || L.row_end > L.Ey ||
       (L.row_end % 8 != 0 && L.row_end != L.Ey))
     return (int)cudaErrorInvalidValue;
-  // small: fewer tiles than the GB300's 152 SMs
+  // small: fewer tiles than SMs
   constexpr int TX = 32 / (N + 1), TY = FaceShape<N, LIMIT, false>::TY;
   const int64_t tiles =
       ((L.Ex + TX - 1) / TX) * ((L.row_end - L.row_begin + TY - 1) / TY);
-  return tiles < 152 ? launch_face_shape<N, GLL, WB, LIMIT, IMEX, true>(L, s)
-                     : launch_face_shape<N, GLL, WB, LIMIT, IMEX, false>(L, s);
+  return tiles < sm_count() ? launch_face_shape<N, GLL, WB, LIMIT, IMEX, true>(L, s)
+                            : launch_face_shape<N, GLL, WB, LIMIT, IMEX, false>(L, s);
 }
 
 template <bool WB, bool LIMIT = false, bool IMEX = false>

@@ -10,8 +10,8 @@
 // two 30-bit halves, and multiplied into two 64-bit accumulators with three
 // IMAD.WIDE per term (6 cycles against 64); the sum is rounded to FP64 once.
 //
-// Accuracy: operands are truncated 2^-kFxBits below the power of two above
-// the group's largest magnitude, coefficients are integers of a row sum up to
+// Accuracy: operands are truncated 2^-59 below the power of two above the
+// group's largest magnitude, coefficients are integers of a row sum up to
 // 2^61, and the dropped product of the lower halves is below 2^-57 of the
 // row's full scale (sum of |coefficient| times the largest operand).  An
 // FP64 FMA chain rounds every partial sum, 2^-53 of the partial sums each.
@@ -24,9 +24,9 @@
 // the state in the update, the average of h in the source term, the traces of
 // u^n and of that average at GLL nodes.  (The GLL traces of the averaged momenta
 // and fluxes are single values in their field's fixed point: all stages but the
-// first carry the rounding of a row of D on that field anyway.)  Groups whose largest value is below 2^-895 (1e-269) lose bits,
-// below 2^-953 they count as zero; groups holding an infinity or a NaN give
-// non-finite sums.
+// first carry the rounding of a row of D on that field anyway.)  Groups whose
+// largest value is below 2^-895 (1e-269) lose bits, below 2^-953 they count as
+// zero; groups holding an infinity or a NaN give non-finite sums.
 #pragma once
 
 #include <cstdint>

@@ -14,10 +14,11 @@
 //     (Sec. 3, Eqs. numflux.cons, combined.wave.speed, good.numflux.non.cons,
 //     total.F.non.cons) to adjoint traces of each side, and to the adjoint of
 //     the static jump g (b+ - b-)/b_0;
-//  3. k_local_adj_2d: per element, the inner stages are reversed: adjoint traces -> time averages -> stage values ->
-//     local operator (transposed D_x, D_y contractions) -> fluxes -> earlier
-//     stages and u^n; the bathymetry enters through g b_x, g b_y and the face
-//     jumps, whose adjoints are mapped back to the nodal b.
+//  3. k_local_adj_2d: per element, the inner stages are reversed: adjoint
+//     traces -> time averages -> stage values -> local operator (transposed D_x,
+//     D_y contractions) -> fluxes -> earlier stages and u^n; the bathymetry
+//     enters through g b_x, g b_y and the face jumps, whose adjoints are mapped
+//     back to the nodal b.
 //
 // Non-smooth points: |m/h| takes sign(0) = 0, and the maximum of the two wave
 // speeds passes its adjoint to the side the forward kernel selected (the

@@ -5,6 +5,20 @@
 
 namespace crkfr {
 
+// SMs of the GPU (asked once; 0 if the query failed)
+inline int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return v;
+  }();
+  return sms;
+}
+
 // A launch that may be scheduled while the kernel before it in the stream
 // finishes (programmatic stream serialization): its blocks take free places
 // once all blocks of that kernel have come to chain_end() (or left) and wait in

@@ -849,16 +849,7 @@ int launch_step_t(const Launch1D& L, cudaStream_t s) {
     return launch_chained(k_step_1d<SYS, N, GLL, true, IMEX>, dim3(blocks), kBlock1D, s, L);
   }
   if (L.steps > 1) return launch_steps_t<SYS, N, GLL, IMEX>(L, s);
-  // SMs of the GPU (asked once; 0 if the query failed: then the largest block)
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    return v;
-  }();
+  const int sms = sm_count();   // (unknown: the largest block)
   const int threads = L.tile_threads > 0 ? L.tile_threads
                       : sms > 0          ? pick_tile_block(L.E, N + 1, sms)
                                          : kBlock1D;

@@ -122,8 +122,7 @@ CRKFR_HD constexpr int tab_weight_sum(int N) {
 // The tableau a kernel instantiation uses: the explicit one of degree N, or
 // SSP3-IMEX(4,3,3) when the step has a source.  The time averages are
 // accumulated with the integer weights b~_i / b_ref, b_ref the common
-// denominator's reciprocal; first() is the stage that initialises the
-// accumulators.
+// denominator's reciprocal.
 template <int N, bool IMEX>
 struct Tab {
   static constexpr int S = IMEX ? imex_stages() : tab_stages(N);
@@ -131,11 +130,6 @@ struct Tab {
   CRKFR_HD static constexpr double b(int i) { return IMEX ? imex_b(i) : tab_b(N, i); }
   CRKFR_HD static constexpr double ai(int i, int j) { return IMEX ? imex_ai(i, j) : 0.0; }
   CRKFR_HD static constexpr double bi(int i) { return IMEX ? imex_b(i) : 0.0; }
-  CRKFR_HD static constexpr int first() {
-    for (int i = 0; i < S; ++i)
-      if (b(i) != 0.0) return i;
-    return 0;
-  }
   CRKFR_HD static constexpr int weight(int i) { return IMEX ? imex_weight(i) : tab_weight(N, i); }
   CRKFR_HD static constexpr int weight_sum() { return IMEX ? 6 : tab_weight_sum(N); }
   CRKFR_HD static constexpr double bref() { return 1.0 / weight_sum(); }
@@ -147,13 +141,6 @@ struct Tab {
   }
   // the local operator of stage i is needed by a later stage
   CRKFR_HD static constexpr bool feeds(int i) {
-    for (int k = i + 1; k < S; ++k)
-      if (a(k, i) != 0.0) return true;
-    return false;
-  }
-  // the local operator of stage i is needed by a later stage or the averages
-  CRKFR_HD static constexpr bool need_L(int i) {
-    if (b(i) != 0.0) return true;
     for (int k = i + 1; k < S; ++k)
       if (a(k, i) != 0.0) return true;
     return false;

@@ -220,6 +220,12 @@ FIXED_POINT_NOTE = ("operation count of the FP64 formulation; the products with 
                     "on the integer pipe, so the fraction of the FP64 pipe's peak can exceed 1")
 
 
+# sources of the dominant kernels, which the summaries' hashes cover
+LOCAL_2D_SOURCES = ["local_2d.cuh", "fixed_point.cuh", "device_common.cuh", "launch.h",
+                    "tableau.h"]
+STEP_1D_SOURCES = ["step_1d.cuh", "fixed_point.cuh", "device_common.cuh", "launch.h", "tableau.h"]
+
+
 def kernel_source_hash(files):
     h = hashlib.sha256()
     for f in files:
@@ -228,19 +234,34 @@ def kernel_source_hash(files):
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(summary, files, scale):
-    """dram bytes per launch from a profiles/ summary, scaled to the bench
-    launch, or None if absent or taken on another version of the sources."""
-    path = os.path.join(ROOT, "profiles", summary)
+def profile_summary(summary, files):
+    """Text of a profiles/ summary, or None if absent or taken on another
+    version of the sources."""
     try:
-        text = open(path).read()
+        text = open(os.path.join(ROOT, "profiles", summary)).read()
     except OSError:
         return None
-    m_hash = re.search(r"source_sha256:\s*([0-9a-f]+)", text)
-    m_bytes = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", text)
-    if not m_hash or not m_bytes or m_hash.group(1) != kernel_source_hash(files):
+    m = re.search(r"source_sha256:\s*([0-9a-f]+)", text)
+    return text if m and m.group(1) == kernel_source_hash(files) else None
+
+
+def profiled_traffic(summary, files, scale):
+    """dram bytes per launch from a profiles/ summary, scaled to the bench
+    launch, or None."""
+    text = profile_summary(summary, files)
+    m = text and re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", text)
+    return float(m.group(1)) * scale if m else None
+
+
+def profiled_pipes(summary, files):
+    """{pipe: % busy} of the dominant kernel from a profiles/ summary, or None.
+    "integer multiplier" is the pipe of the fixed-point products."""
+    text = profile_summary(summary, files)
+    m = text and re.search(r"pipe_busy_pct:\s*(.+)", text)
+    if not m:
         return None
-    return float(m_bytes.group(1)) * scale
+    return {k.strip(): float(v) for k, v in re.findall(r"([a-zA-Z0-9 ]+?) ([0-9.]+)(?:,|$)",
+                                                       m.group(1))}
 
 
 # ---------------------------------------------------------------------------
@@ -504,7 +525,7 @@ def run_ours(args, wl):
     peaks = load_peaks()
     hbm_peak = peaks.get("hbm_gbs", HBM_FALLBACK_GBS)
     if wl.dim == 2:
-        kname, files = "local_2d", ["local_2d.cuh", "device_common.cuh", "tableau.h"]
+        kname, files = "local_2d", LOCAL_2D_SOURCES
         if wl.limiter:
             files = files + ["limit_2d.cuh"]
         summary = ("k_local_2d__swe2d_friction_N3.md" if wl.source else
@@ -512,7 +533,7 @@ def run_ours(args, wl):
                    "k_local_2d__swe2d_N3_limited.md" if wl.limiter else
                    "k_local_2d__swe2d_N3.md")
     else:
-        kname, files = "step_1d", ["step_1d.cuh", "device_common.cuh", "tableau.h"]
+        kname, files = "step_1d", STEP_1D_SOURCES
         summary = "k_step_1d__swe1d_N4_limited.md" if wl.limiter else "k_step_1d__swe1d_N4.md"
     nk, ms_k = prof.get(kname, (0, float("nan")))
     avg_ms = ms_k / max(nk, 1)
@@ -546,6 +567,7 @@ def run_ours(args, wl):
                      "flops_per_launch": flops,
                      "peak_source": "FP64: 152 SMs x 2 FMA/clk x 2 flop x 2070 MHz",
                      "work_note": FIXED_POINT_NOTE,
+                     "pipes_busy_pct": profiled_pipes(summary, files),
                      **({"flops_note": "the unlimited step's operation count: a lower bound "
                                        "of the limited kernel's work"}
                         if wl.limiter and wl.dim == 1 else
@@ -740,8 +762,9 @@ def run_ensemble(args):
                      "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": achieved / FP64_PEAK_TFLOPS,
                      "traffic": profiled_traffic("k_step_1d_batch__ensemble256.md",
-                                                 ["step_1d.cuh", "device_common.cuh", "tableau.h"],
-                                                 1.0),
+                                                 STEP_1D_SOURCES, 1.0),
+                     "pipes_busy_pct": profiled_pipes("k_step_1d_batch__ensemble256.md",
+                                                      STEP_1D_SOURCES),
                      "traffic_unit": "bytes per step (the degree classes' launches)",
                      "work_note": FIXED_POINT_NOTE},
         "gpu_launches": launches, "clocks": clk}))

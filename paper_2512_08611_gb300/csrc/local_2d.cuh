@@ -357,8 +357,11 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
     // magnitudes with headroom, raised if a later stage exceeds them.
     // (sync_or is also the barrier after the last reads of X.)
     const int lx = fx_log(cur[1]), ly = fx_log(cur[2]), lhg = fx_log(T.half_gravity);
-    if (sync_or(lane_ok && fx_over<!WB>(cur[0], lx, ly, lhg, E))) {
-      if (lane_ok) {
+    // (Only the nodes that exceed them enter smag: what an element's exponents
+    // become must not depend on the elements it shares a barrier with.)
+    const bool over = lane_ok && fx_over<!WB>(cur[0], lx, ly, lhg, E);
+    if (sync_or(over)) {
+      if (over) {
         int mag[kLocalGroups];
         mag[0] = fx_mag(cur[0]);
         mag[1] = fx_mag(cur[1]);

@@ -167,7 +167,10 @@ struct FaceShape {
   static constexpr int min_blocks = LIMIT ? 1 : SMALL ? 8 : N >= 4 ? 4 : 5;
 };
 
-// Face kernel on tiles of TY x EPW elements (one tile row per warp).
+// Face kernel on tiles of TY x TX elements (one tile row per warp).  512 x 512 at
+// N = 3: 175 us, bound by the FP64 pipe (58 % busy), issue slots (0.52) and DRAM
+// (38 % of its peak) together; 169 us with one exponent for both momenta and for
+// W, which cut the smaller values of the state.
 // Phase 1 solves every face node of the tile exactly once in a flat loop over
 // the block (warps with no face left issue nothing, so only the last, partial
 // warp of the loop pays for idle lanes) and keeps both sides' terms in shared

@@ -193,8 +193,9 @@ __host__ __device__ constexpr int adjoint_stride() {
 // One thread per node, as k_local_2d: the pointwise reverse arithmetic in FP64
 // (some 30 instructions a stage), the transposed contractions with D and the
 // products with the end-point rows, more than half of the FP64 instructions
-// before, in block fixed point (fixed_point.cuh).  256 x 256 at N = 3: 547 us
-// with a thread per element row and FP64 chains (255 registers).
+// before, in block fixed point (fixed_point.cuh).  256 x 256 at N = 3: 308 us,
+// bound by the FP64 pipe (83 % busy), against 547 us with a thread per element
+// row and FP64 chains (255 registers).
 template <int N>
 __global__ void __launch_bounds__(kBlockAdj, 5) k_local_adj_2d(const Launch2DAdj A) {
   using TB = Tab<N, false>;

@@ -17,16 +17,21 @@
 // fluxes run in block fixed point on the integer pipe (fixed_point.cuh).  D is
 // applied to the time-averaged fluxes once instead of accumulating every
 // stage's operator, so the last stage needs no contraction.  On a 1024 x 1024
-// mesh at N = 3 the kernel takes 1.94 ms (FP64 pipe 33 % busy, the multiplier
-// of the integer products 70 %, 0.64 instructions per cycle and scheduler)
-// against 6.4 ms with FP64 chains (one thread per element row, FP64 pipe 96
-// %).  One thread per row in fixed point took 4.2 ms: 255 registers and two
-// warps per scheduler left the latencies open, and 9700 instructions a warp
-// missed the instruction cache; a thread per node takes a quarter of the
-// code.  With FP64 fluxes, seven FP64 instructions a stage and each result
-// converted, two steps took 5.45 ms (FP64 pipe 77 % busy), with fixed-point
-// ones 5.22 ms; 401 x 307 well-balanced at N = 4 2.08 and 1.95 ms, 640 x 384
-// limited 3.28 and 3.01 ms, 512 x 512 with friction 2.52 and 2.28 ms.
+// mesh at N = 3 the kernel takes 2.17 ms, bound by issue slots and the integer
+// multiplier together (0.63 instructions per cycle and scheduler, multiplier 65
+// % busy, ALU 61 %, FP64 pipe 37 %), against 6.4 ms with FP64 chains (one thread
+// per element row, FP64 pipe 96 %).  One thread per row in fixed point took 4.2
+// ms: 255 registers and two warps per scheduler left the latencies open, and
+// 9700 instructions a warp missed the instruction cache; a thread per node takes
+// a quarter of the code.  FP64 fluxes, seven FP64 instructions a stage and each
+// result converted, cost another 4 to 9 % of a step (two steps on 1024 x 1024
+// 5.45 against 5.22 ms, 512 x 512 with friction 2.52 against 2.28 ms).
+//
+// An exponent per field instead of one for hu and hv and one for all fluxes,
+// and the fields of an equation aligned after their contractions, take 512 x 512
+// at N = 3 from 499 to 541 us and 401 x 307 well-balanced at N = 4 from 819 to 888
+// us: what a small momentum beside a large one needs to keep the precision that
+// FP64 gives it.
 //
 // The well-balanced form (WB) has pressure-free fluxes and the
 // non-conservative terms g h D_x (h + b), g h D_y (h + b).

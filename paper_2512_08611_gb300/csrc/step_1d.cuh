@@ -10,7 +10,9 @@
 // on the integer pipe (fixed_point.cuh), and D is applied to the averages once
 // instead of accumulating every stage's operator.  (Fluxes in fixed point
 // instead of FP64: 1e5 elements at N = 4, four steps, 375 -> 302 us; the
-// ensemble of 256 meshes, two steps, 4.03 -> 3.24 ms.)  A block updates all its
+// ensemble of 256 meshes, two steps, 4.03 -> 3.24 ms.  The average of h in FP64,
+// which a shallow node needs: 311 us, 3.32 ms.)  Bound by the FP64 pipe (67 %
+// busy) and issue slots (0.50) together.  A block updates all its
 // elements but the first and the last, whose stages it recomputes for their
 // neighbours (4 % of a 256-thread block at N = 4), so that the only
 // inter-element coupling, one Riemann problem per face (Eqs. numflux.cons,

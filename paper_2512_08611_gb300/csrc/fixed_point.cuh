@@ -273,6 +273,17 @@ __device__ __forceinline__ long long fx_average(long long A, long long B) {
   return ((A + (B >> 30)) << (30 - SHIFT)) + (((int)B & 0x3fffffff) >> SHIFT);
 }
 
+// The operand of the average w x + inc (inc: FP64, in units 2^SHIFT smaller than
+// the result's) of a value x: what FP64 would round off the sum at x's size is
+// kept.  E at least the biased exponent of x and that of inc less SHIFT.
+template <bool WIDE, int SHIFT, int FB>
+__device__ __forceinline__ long long fx_increment(double x, int w, double inc, int E) {
+  long long A = 0, B = 0;
+  const long long v = fx_from<FB>(x, E);
+  fx_accumulate<WIDE>(A, B, v, fx_split(v), w);
+  return fx_average<WIDE, SHIFT>(A, B) + fx_from<FB>(inc, E + SHIFT);
+}
+
 // a row of n operands in shared memory (16-byte aligned for even n)
 template <int n>
 __device__ __forceinline__ void fx_row(const Fx* x, Fx (&r)[n]) {

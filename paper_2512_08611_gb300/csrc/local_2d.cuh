@@ -87,7 +87,8 @@ __host__ __device__ constexpr int local_min_blocks() {
 // momentum beside a large one keeps its bits; two terms of one equation are
 // aligned only where their derivatives are added).  The average of h enters
 // the source term node by node, so it is formed in FP64, from h^n and the
-// stages' operators.
+// stages' operators; in the well-balanced form, whose source term has the
+// stages' own h, it is for the traces only, and with GL nodes a sum as the others.
 constexpr int kLocalFields = 9;
 constexpr int kLocalGroups = 6;
 
@@ -248,7 +249,8 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   }
   double Sb[2] = {0.0, 0.0};     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double P1 = 0.0, P2 = 0.0;     // sum_j (b_j/b_ref) h g d(h + b) (WB)
-  double uh = 0.0;               // sum_j (b_j/b_ref) (h^(j) - h^n), below + h^n / b_ref
+  constexpr bool FIX_H = WB && !GLL;   // the average of h as field 0's sum
+  double uh = 0.0;               // or sum_j (b_j/b_ref) (h^(j) - h^n), below + h^n / b_ref
   // time averages sum_j (b_j/b_ref) of the exchange fields 1..5 in the fixed
   // point of their exponents E, which only grow: the sums are shifted when
   // they do
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
 #pragma unroll kStageUnroll
   for (int i = 0; i < S; ++i) {
     if (i == (IMEX ? 0 : 1)) __syncthreads();   // the step sizes
-    if (i > 0) uh = fma(sz.avg[i - 1], Lp[0], uh);
+    if (!FIX_H && i > 0) uh = fma(sz.avg[i - 1], Lp[0], uh);
     double cur[3];
 #pragma unroll
     for (int v = 0; v < 3; ++v) cur[v] = u0[v];
@@ -376,6 +378,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
         mag[5] = fx_flux_mag<!WB>(cur[0], ly, ly, lhg);
         if (IMEX) {
           // the traces of u^n, no stage value here, share the exponents
+          mag[0] = max(mag[0], fx_mag(u0[0]));
           mag[1] = max(mag[1], fx_mag(u0[1]));
           mag[2] = max(mag[2], fx_mag(u0[2]));
         }
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
         const int e = fx_exp(smag[le][k]);
         const int d = e > E[k] ? e + kHeadroom - E[k] : 0;
         E[k] += d;
-        if (k > 0) fx_rescale<WIDE>(A[k], B[k], d);
+        if (k > 0 || FIX_H) fx_rescale<WIDE>(A[k], B[k], d);
       }
     }
     long long f[6];
@@ -411,7 +414,7 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
 #pragma unroll
     for (int k = k0; k < 6; ++k) {
       const Fx x = fx_split(f[k]);
-      if (k > 0) fx_accumulate<WIDE>(A[k], B[k], f[k], x, wi);
+      if (k > 0 || FIX_H) fx_accumulate<WIDE>(A[k], B[k], f[k], x, wi);
       if (lane_ok) X[k][q][p] = x;
     }
     if (need_op || WB) {
@@ -454,19 +457,23 @@ __global__ void __launch_bounds__(kBlockLocal, local_min_blocks<N, IMEX, LIMIT>(
   // accumulated stage by stage).  A, P and Sb hold time averages divided by
   // b_ref; the sums are scaled back to FB bits for the contractions.
 #pragma unroll
-  for (int k = 1; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
-  uh = fma((double)TB::weight_sum(), u0[0], uh);
-  if constexpr (!GLL) {
-    // the exponent of the traces of h: u^n and its average (in sum units)
-    const int mu = fx_mag(uh);
+  for (int k = FIX_H ? 0 : 1; k < 6; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
+  const double du = uh;
+  uh = fma((double)TB::weight_sum(), u0[0], du);
+  if constexpr (!GLL && !FIX_H) {
+    // the exponent of the traces of h: u^n and its average's increment (in sum
+    // units)
+    const int mu = fx_mag(du);
     const int m = max(fx_mag(u0[0]), mu >= 0x7ff00000 ? mu : mu - (kSumShift << 20));
     if (lane_ok) atomicMax(&smag[le][0], m);
   }
   sync();
-  if (!GLL) E[0] = fx_exp(smag[le][0]);
+  if (!GLL && !FIX_H) E[0] = fx_exp(smag[le][0]);
   if (lane_ok) {
-    X[0][q][p] = GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
-                     : fx_split(fx_from<FB>(uh, E[0] + kSumShift));
+    X[0][q][p] = FIX_H ? fx_split(A[0])
+                 : GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
+                       : fx_split(fx_increment<WIDE, kSumShift, FB>(u0[0], TB::weight_sum(), du,
+                                                                    E[0]));
 #pragma unroll
     for (int k = 1; k < 6; ++k) X[k][q][p] = fx_split(A[k]);
 #pragma unroll

@@ -332,12 +332,14 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   double Ss[S];                        // source of variable SV at each stage (IMEX)
   double Sb = 0.0;                     // sum_j (b_j/b_ref) s(u^(j)) (IMEX)
   double Pb = 0.0;                     // sum_j (b_j/b_ref) h g d(h + b) (WB)
-  // sum_j (b_j/b_ref) (h^(j) - h^n), below + h^n / b_ref: it enters node by node
+  // the average of h: field 0's sum (FIX_H), or sum_j (b_j/b_ref) (h^(j) - h^n),
+  // below + h^n / b_ref, where it enters node by node (as in local_2d.cuh)
+  constexpr bool FIX_H = WB && !GLL;
   double uh = 0.0;
   long long A[K], B[K];                // of the other exchange fields (WIDE: A 2^30 + B)
   int Ex[K];                           // exponents of the exchange fields
   // shallow water: h is contracted in the well-balanced form only
-  constexpr int kStage0 = SWE && !WB ? 1 : 0, kAvg0 = SWE ? 1 : 0;
+  constexpr int kStage0 = SWE && !WB ? 1 : 0, kAvg0 = SWE && !FIX_H ? 1 : 0;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     A[k] = B[k] = 0;
@@ -358,7 +360,7 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   for (int i = 0; i < S; ++i) {
     // (the step sizes: the first stage does without)
     if (i == (IMEX ? 0 : 1)) __syncthreads();
-    if (SWE && i > 0 && TB::feeds(i > 0 ? i - 1 : 0)) uh = fma(sz.avg[i - 1], Ls[i - 1][0], uh);
+    if (SWE && !FIX_H && i > 0 && TB::feeds(i > 0 ? i - 1 : 0)) uh = fma(sz.avg[i - 1], Ls[i - 1][0], uh);
     double cur[M];
 #pragma unroll
     for (int v = 0; v < M; ++v) {
@@ -473,21 +475,25 @@ __device__ __forceinline__ void step_1d_tile(const Tables& T, double xs,
   // ---- the averages' derivative and the face traces --------------------------
 #pragma unroll
   for (int k = kAvg0; k < K; ++k) A[k] = fx_average<WIDE, kSumShift>(A[k], B[k]);
-  uh = fma((double)TB::weight_sum(), u0[0], uh);
-  if constexpr (SWE && !GLL) {
-    // the exponent of the traces of h: u^n and its average (in sum units)
-    const int mu = fx_mag(uh);
+  const double du = uh;
+  uh = fma((double)TB::weight_sum(), u0[0], du);
+  if constexpr (SWE && !GLL && !FIX_H) {
+    // the exponent of the traces of h: u^n and its average's increment (in sum
+    // units)
+    const int mu = fx_mag(du);
     const int m = max(fx_mag(u0[0]), mu >= 0x7ff00000 ? mu : mu - (kSumShift << 20));
     if (lane_ok) atomicMax(&smag[slot][0], m);
   }
   __syncwarp();
-  if (SWE && !GLL) Ex[0] = fx_exp(smag[slot][0]);
+  if (SWE && !GLL && !FIX_H) Ex[0] = fx_exp(smag[slot][0]);
   if (lane_ok) {
 #pragma unroll
     for (int k = kAvg0; k < K; ++k) X[k][p] = fx_split(A[k]);
     if constexpr (SWE) {
-      X[0][p] = GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
-                    : fx_split(fx_from<FB>(uh, Ex[0] + kSumShift));
+      if (!FIX_H)
+        X[0][p] = GLL ? Fx{__double2hiint(uh), __double2loint(uh)}
+                      : fx_split(fx_increment<WIDE, kSumShift, FB>(u0[0], TB::weight_sum(), du,
+                                                                   Ex[0]));
 #pragma unroll
       for (int v = 0; v < 2; ++v)
         X[3 + v][p] = GLL ? Fx{__double2hiint(u0[v]), __double2loint(u0[v])}

@@ -210,8 +210,8 @@ crkfr_status crkfr_step(crkfr_ctx* ctx, double* u_dev, double dt, int64_t nsteps
                         void* stream);
 
 /* Advance with the step of Eq. time.step.2d until time t_end, shortening the
- * last step to land on t_end exactly (steps after that are no-ops).  Runs
- * chunks of device steps and reads the time back between chunks.  At most
+ * last step to land on t_end exactly (steps after that have size zero: without
+ * the limiter they leave every bit of the state).  Runs chunks of device steps and reads the time back between chunks.  At most
  * max_steps steps; *steps_taken (may be NULL) receives the number of steps
  * that advanced the state.  Returns CRKFR_ERR_ARG if t_end is not reached
  * within max_steps. */
